@@ -42,6 +42,7 @@ namespace {
 // that run on it; plus a per-task overhead.
 constexpr double kFlopPerNs = 7.6 / kCtasPerSm;
 constexpr double kTaskOverheadNs = 2500.0;
+constexpr int kGpuSms = 152;  // of a GB300
 constexpr double kSweepStepNs = 120.0;  // one step of an in-shared-memory triangular sweep
 
 struct Builder {
@@ -83,13 +84,14 @@ struct Builder {
     if (t.prec != PREC_FP64) flops_lowered += sym_block ? 0.5 * f : f;
     sym_block = false;
     if (t.pmode == PM_TRI3) f *= 0.75;
+    if (t.pmode == PM_TRI16) f *= 0.625;
     if (t.prec == PREC_EMU64) f /= 10.0;   // order of the emulated-FP64 speed-up per block
     if (t.prec == PREC_FP32X) f /= 25.0;
     int id = (int)tasks.size();
     tasks.push_back(t);
     // parts run side by side on different CTAs
     cost.push_back(kTaskOverheadNs + f / kFlopPerNs / t.parts +
-                   epi_ns / (t.pmode == PM_ROWS2 ? 2 : t.pmode == PM_ROWS4 ? 4 : 1));
+                   epi_ns / (t.pmode == PM_ROWS2 || t.pmode == PM_ROWS4 || t.pmode == PM_ROWS8 ? t.parts : 1));
     fsegs.insert(fsegs.end(), segs.begin(), segs.end());
     seg_off.push_back((int64_t)fsegs.size());
     fwaits.insert(fwaits.end(), waits.begin(), waits.end());
@@ -116,22 +118,52 @@ struct Builder {
   // (blocks of at most 32 rows or columns) falls back to one part.
   static void split(Task& t, uint8_t mode) {
     if (mode == PM_ROWS2 && t.m > 32) { t.pmode = PM_ROWS2; t.parts = 2; }
-    else if (mode == PM_ROWS4 && t.m > 48) { t.pmode = PM_ROWS4; t.parts = 4; }
-    else if (mode == PM_ROWS4 && t.m > 32) { t.pmode = PM_ROWS2; t.parts = 2; }
+    else if (mode == PM_ROWS4 && t.m > 16) { t.pmode = PM_ROWS4; t.parts = (uint8_t)((t.m + 15) / 16); }
     else if (mode == PM_QUAD4 && t.m > 32 && t.n > 32) { t.pmode = PM_QUAD4; t.parts = 4; }
     else if (mode == PM_TRI3 && t.m > 32 && t.m == t.n) { t.pmode = PM_TRI3; t.parts = 3; }
-    else if (mode == PM_ROWS8 && t.m > 8 && t.m <= 32) { t.pmode = PM_ROWS8; t.parts = (uint8_t)((t.m + 7) / 8); }
-    else if (mode == PM_TRI16 && t.m > 16 && t.m <= 32 && t.m == t.n) { t.pmode = PM_TRI16; t.parts = 3; }
-    else if (mode == PM_QUAD16 && t.m <= 32 && t.n > 16 && t.n <= 32) {
-      t.pmode = PM_QUAD16;
-      t.parts = t.m > 16 ? 4 : 2;  // parts 2 and 3 are the lower row of quadrants
+    else if (mode == PM_ROWS8 && t.m > 8) { t.pmode = PM_ROWS8; t.parts = (uint8_t)((t.m + 7) / 8); }
+    else if (mode == PM_GRID16 && (t.m > 16 || t.n > 16)) {
+      t.pmode = PM_GRID16;
+      t.parts = (uint8_t)((t.m + 15) / 16 * ((t.n + 15) / 16));
+    } else if (mode == PM_TRI16 && t.m > 16 && t.m == t.n) {
+      const int d = (t.m + 15) / 16;
+      t.pmode = PM_TRI16;
+      t.parts = (uint8_t)(d * (d + 1) / 2);
     }
   }
 
-  // Parts of an off-diagonal phase-2 block task (tuning bits 2-3).
-  void split_p2(Task& t) const {
+  // How finely FP64 products are divided. One SM does 2 FP64 multiply-adds per
+  // clock whatever the part's shape, so a 64 x 64 block with an inner length
+  // of 64 takes 63 us on one SM, a 32 x 32 quadrant 16 us, a 16 x 16 part 4 us
+  // plus about 4 us of fixed cost. A step of the factorization or of phase 2
+  // offers a known number of blocks at a time: they are cut until the parts
+  // reach the SMs, and no further (a fuller step is bound by the FP64 pipes, and
+  // smaller parts then only add their fixed cost and operand traffic).
+  // `blocks`: 64 x 64 blocks that are ready at a time; `crowd`: matrices that
+  // share the GPU. Tasks whose products are lowered keep their 32 x 32 parts.
+  int crowd = 1;
+  uint8_t fine_mode(long long blocks, uint8_t coarse) const {
+    blocks *= crowd;
+    return 4 * blocks <= kGpuSms ? (uint8_t)PM_GRID16 : blocks <= kGpuSms ? (uint8_t)PM_QUAD4 : coarse;
+  }
+  // ... of a task, `tri`: only the lower triangle of its (square) block.
+  static void split_fp64(Task& t, uint8_t mode, bool tri) {
+    if (mode == PM_GRID16) split(t, tri ? PM_TRI16 : PM_GRID16);
+    else if (tri) split(t, PM_TRI3);
+    else split(t, mode);
+  }
+  // 64 x 64 blocks of tile column k of L.
+  long long col_blocks(int k) const {
+    long long n = L.nblk(k);
+    if (k < s.nt) n += (long long)L.nsub(k) * L.nblk(0) + (s.a > 0 ? L.nblk(s.nt) : 0);
+    return n;
+  }
+
+  // Parts of an off-diagonal phase-2 block task (tuning bits 2-3), one of
+  // `blocks` ready at a time.
+  void split_p2(Task& t, long long blocks) const {
     const int mode = tune_p2_split(s.tune);
-    if (mode == 0) split(t, PM_QUAD4);
+    if (mode == 0) split_fp64(t, fine_mode(blocks, PM_QUAD4), false);
     else if (mode == 1) split(t, PM_ROWS2);
   }
 
@@ -142,6 +174,11 @@ struct Builder {
   void lower_precision(Task& t) const {
     if (s.prec == PREC_FP64) return;
     t.prec = (uint8_t)s.prec;
+    if (t.pmode == PM_TRI16) {  // its FP64 parts are smaller
+      t.pmode = PM_FULL;
+      t.parts = 1;
+      split(t, PM_TRI3);
+    }
     if (t.pmode != PM_QUAD4 && t.pmode != PM_TRI3) {
       const int pr = t.m > 32 ? 2 : 1, pc = t.n > 32 ? 2 : 1;
       t.pmode = PM_TILE32;
@@ -344,58 +381,32 @@ struct Builder {
       w.push_back({lctr[lidx(i, t.k, r, t.c1)], lfinal[lidx(i, t.k, r, t.c1)]});
       w.push_back({lctr[lidx(kq, t.k, cq, t.c1)], lfinal[lidx(kq, t.k, cq, t.c1)]});
     };
-    const size_t nfused = 0;  // every update runs as its own (split) task
-    size_t nchain = terms.size() - nfused;
     // The critical path's links run as small parts on more CTAs: the FP64
-    // newest update of a diagonal block as three quadrant tasks of 16 x 16
-    // parts, the final TRSM of the block right below a diagonal block as two
-    // tasks of 8-row parts (they write disjoint parts of the block)
-    const bool newest_fp64 = nchain > 0 && (s.prec == PREC_FP64 ||
-                                            (i == kq && terms[nchain - 1].k == kq && !tune_lower_diag(s.tune)));
-    const bool fine_newest = diag && m == n && m > 32 && newest_fp64;
-    const bool fine_final = !diag && dist == 1 && m > 32;
-    // writers of the block's chain counter `me` (strictly ordered); the
-    // quadrant tasks and the two final TRSM halves run side by side and
-    // signal counters of their own
-    int total_writers = (int)nchain + 1 - (fine_newest ? 1 : 0);
+    // newest update of a diagonal block as the 16 x 16 parts of its lower
+    // triangle, the final TRSM of the block right below a diagonal block in
+    // parts of 8 rows.
+    const int total_writers = (int)terms.size() + 1;
     lfinal[lidx(i, kq, r, cq)] = total_writers;
+    // blocks updated by one source block column: the lower triangle over the
+    // blocks of a column of L. The newest terms, one column's, are cut to 16 x 16
+    // as long as that whole step leaves SMs idle (in the reduced precisions, whose
+    // FP64 share is small, as long as their own parts do).
+    const long long W = col_blocks(kq) - cq, step = W * (W + 1) / 2;
+    const uint8_t fine_old = fine_mode(step, PM_FULL);
+    const uint8_t fine_new = (s.prec == PREC_FP64 ? step : 4 * W) * crowd <= kGpuSms ? PM_GRID16 : PM_QUAD4;
     bool written = false;  // the block already holds an update (read it from L, not A)
-    int32_t qctr = -1;     // the quadrant tasks of the newest update
-    for (size_t t = 0; t < nchain; ++t) {
-      if (fine_newest && t + 1 == nchain) {
-        const Seg sg = term_seg(terms[t]);
-        const int qr[3] = {0, 32, 32}, qc[3] = {0, 0, 32};
-        qctr = newctr(false);
-        for (int x = 0; x < 3; ++x) {
-          const int64_t off = qr[x] + (int64_t)qc[x] * ld_i;
-          Task tq = blank(OP_UPD, std::min(32, m - qr[x]), std::min(32, n - qc[x]));
-          tq.out = outref + off;
-          tq.ldo = ld_i;
-          tq.cin = (written ? outref : mkref(BUF_A, L.blk(i, kq, r, cq))) + off;
-          tq.ldc = ld_i;
-          split(tq, x == 1 ? PM_QUAD16 : PM_TRI16);
-          if (grow(i, r) - grow(terms[t].k, terms[t].c1) <= kUrgentReach) tq.flags |= TF_URGENT;
-          Seg sq = sg;
-          sq.a += qr[x];
-          sq.b += qc[x];
-          std::vector<Wait> w;
-          if (nwritten > 0) w.push_back({me, nwritten});
-          if (!written && serve) w.push_back({prep_ctr[kq], 1});
-          term_waits(terms[t], w);
-          emit(tq, {sq}, w, {qctr}, 0.0);
-        }
-        written = true;
-        continue;
-      }
+    for (size_t t = 0; t < terms.size(); ++t) {
       Task tk = blank(OP_UPD, m, n);
       tk.out = outref;
       tk.ldo = ld_i;
       tk.cin = written ? outref : mkref(BUF_A, L.blk(i, kq, r, cq));
       tk.ldc = ld_i;
-      // a diagonal block only needs its lower quadrants; the newest update of
-      // a block gates its TRSM / POTRF on the critical path: split it 4 ways
-      if (diag) split(tk, PM_TRI3);
-      else if (t + 1 == nchain && tune_upd_split(s.tune) == 0) split(tk, PM_QUAD4);
+      const bool newest = t + 1 == terms.size();
+      // a diagonal block only needs its lower part; the newest update of a
+      // block gates its TRSM / POTRF on the critical path
+      if (diag) split_fp64(tk, newest ? (uint8_t)PM_GRID16 : fine_old, true);
+      else if (!newest) split_fp64(tk, fine_old, false);
+      else if (tune_upd_split(s.tune) == 0) split_fp64(tk, fine_new, false);
       if (grow(i, r) - grow(terms[t].k, terms[t].c1) <= kUrgentReach) tk.flags |= TF_URGENT;
       // the diagonal tile's own updates belong to its POTRF, which stays true
       // FP64 unless the tuning code lowers them too
@@ -413,42 +424,9 @@ struct Builder {
     std::vector<Seg> segs;
     std::vector<Wait> w;
     if (nwritten > 0) w.push_back({me, nwritten});
-    if (qctr >= 0) w.push_back({qctr, 3});
     if (!written && serve) w.push_back({prep_ctr[kq], 1});
-    for (size_t t = nchain; t < terms.size(); ++t) {
-      segs.push_back(term_seg(terms[t]));
-      term_waits(terms[t], w);
-    }
-    if (fine_final) {
-      // the two halves signal a counter of their own, which replaces the
-      // block's chain counter for every later reader (both are predecessors)
-      const int32_t dctr = lctr[lidx(kq, kq, cq, cq)];
-      w.push_back({dctr, lfinal[lidx(kq, kq, cq, cq)]});
-      const int32_t fctr = newctr(false);
-      if (kind == PLAN_FUSED) colblocks[kq]++;  // two final tasks signal the column
-      for (int h = 0; h < 2; ++h) {
-        const int r0 = 32 * h;
-        Task tq = blank(OP_TRSM_RLT, std::min(32, m - r0), n);
-        split(tq, PM_ROWS8);
-        tq.flags |= TF_URGENT;
-        tq.out = outref + r0;
-        tq.ldo = ld_i;
-        tq.cin = (written ? outref : mkref(BUF_A, L.blk(i, kq, r, cq))) + r0;
-        tq.ldc = ld_i;
-        tq.aux = mkref(BUF_L, L.blk(kq, kq, cq, cq));
-        tq.ldx = L.rows(kq);
-        std::vector<Seg> sh = segs;
-        for (Seg& g : sh) g.a += r0;
-        std::vector<int32_t> sig{fctr};
-        if (kind == PLAN_FUSED) sig.push_back(colfinal[kq]);
-        emit(tq, sh, w, sig, 2.0 * n * kSweepStepNs);
-      }
-      lctr[lidx(i, kq, r, cq)] = fctr;
-      lfinal[lidx(i, kq, r, cq)] = 2;
-      return;
-    }
     Task tk = blank(diag ? OP_POTRF : OP_TRSM_RLT, m, n);
-    if (!diag) split(tk, PM_ROWS4);
+    if (!diag) split(tk, dist == 1 || W * crowd <= 2 * kUrgentReach ? PM_ROWS8 : PM_ROWS4);
     if (diag || dist <= kUrgentReach) tk.flags |= TF_URGENT;
     tk.out = outref;
     tk.ldo = ld_i;
@@ -459,7 +437,7 @@ struct Builder {
     if (diag) {
       tk.diag = ndiag++;
       tk.gcol = kq * s.b + cq * FB;
-      epi = 3.0 * m * kSweepStepNs;
+      epi = 1.5 * m * kSweepStepNs;
     } else {
       const int32_t dctr = lctr[lidx(kq, kq, cq, cq)];
       w.push_back({dctr, lfinal[lidx(kq, kq, cq, cq)]});
@@ -589,7 +567,8 @@ struct Builder {
       for (int c = 0; c <= r; ++c) {
         const int m = L.bdim(i, r), n = L.bdim(i, c);
         Task t = blank(OP_STORE, m, n);
-        if (r == c) split(t, PM_TRI3);  // only the lower part of a diagonal block is used
+        // only the lower part of a diagonal block is used
+        split_fp64(t, 2LL * R * (R + 1) * crowd <= kGpuSms ? PM_GRID16 : PM_FULL, r == c);
         t.out = mkref(BUF_S, L.blk(i, i, r, c));
         t.ldo = ld;
         std::vector<Wait> w{{linv_ctr(i, r), R - r}, {linv_ctr(i, c), R - c}};
@@ -605,6 +584,7 @@ struct Builder {
         for (int r = 0; r < L.nblk(k); ++r) {
           const int m = L.bdim(k, r), n = L.bdim(i, c);
           Task t = blank(OP_STORE, m, n);
+          split_fp64(t, fine_mode((col_blocks(i) - R) * R, PM_FULL), false);
           t.out = mkref(BUF_W, L.blk(k, i, r, c));
           t.ldo = ldk;
           std::vector<Wait> w;
@@ -629,7 +609,7 @@ struct Builder {
         for (int r = 0; r < L.nblk(j); ++r) {
           const int m = L.bdim(j, r), n = L.bdim(i, c);
           Task t = blank(OP_NEG, m, n);
-          split_p2(t);  // phase 2 is a chain of joins: shorter tasks, shorter steps
+          split_p2(t, (col_blocks(i) - R) * R);  // phase 2 is a chain of joins: shorter tasks, shorter steps
           t.out = mkref(BUF_S, L.blk(j, i, r, c));
           t.ldo = ldj;
           std::vector<Seg> segs;
@@ -662,8 +642,9 @@ struct Builder {
       for (int c = 0; c <= r; ++c) {
         const int m = L.bdim(i, r), n = L.bdim(i, c);
         Task t = blank(OP_SYMUPD, m, n);
-        if (r == c) split(t, PM_TRI3);
-        else split_p2(t);
+        const long long blocks = (long long)R * (R + 1) / 2;
+        if (r == c) split_fp64(t, fine_mode(blocks, PM_QUAD4), true);
+        else split_p2(t, blocks);
         t.out = mkref(BUF_S, L.blk(i, i, r, c));
         t.ldo = ld;
         t.cin = t.out;
@@ -692,6 +673,7 @@ struct Builder {
 
   // ---------------------------------------------------------- schedule ----
   int finish(int workers) {
+    if (tasks.size() > (size_t)kMaxTasks) return STILES_ERR_PLAN;
     const int nt_ = (int)tasks.size();
     // predecessor edges from waits (flat, per task sorted and unique); the
     // emission order must be topological
@@ -801,6 +783,8 @@ struct Builder {
     // write the plan in list-schedule order (the device queue order)
     Plan& p = *out;
     p.tasks.clear(); p.segs.clear(); p.waits.clear(); p.sigs.clear();
+    p.wait_off.assign(1, 0); p.sig_off.assign(1, 0);
+    p.wait_off.reserve(nt_ + 1); p.sig_off.reserve(nt_ + 1);
     p.tasks.reserve(nt_); p.segs.reserve(fsegs.size()); p.waits.reserve(fwaits.size()); p.sigs.reserve(fsigs.size());
     std::vector<int32_t> rank(nt_);
     for (int r = 0; r < nt_; ++r) rank[order[r]] = r;
@@ -809,16 +793,15 @@ struct Builder {
       tk.seg0 = (int32_t)p.segs.size();
       tk.nseg = (int32_t)(seg_off[t + 1] - seg_off[t]);
       p.segs.insert(p.segs.end(), fsegs.begin() + seg_off[t], fsegs.begin() + seg_off[t + 1]);
-      tk.wait0 = (int32_t)p.waits.size();
-      tk.nwait = (int32_t)(wait_off[t + 1] - wait_off[t]);
       p.waits.insert(p.waits.end(), fwaits.begin() + wait_off[t], fwaits.begin() + wait_off[t + 1]);
-      tk.sig0 = (int32_t)p.sigs.size();
-      tk.nsig = (int16_t)(sig_off[t + 1] - sig_off[t]);
+      p.wait_off.push_back((int64_t)p.waits.size());
       p.sigs.insert(p.sigs.end(), fsigs.begin() + sig_off[t], fsigs.begin() + sig_off[t + 1]);
+      p.sig_off.push_back((int64_t)p.sigs.size());
       p.tasks.push_back(tk);
     }
     // successor graph in schedule-order indices
     p.indeg.assign(nt_, 0);
+    p.rem0.assign(nt_, 0);
     p.succ_off.assign(nt_ + 1, 0);
     p.succ.clear();
     p.succ.reserve(succ.size());
@@ -829,29 +812,33 @@ struct Builder {
         p.succ.push_back(rank[succ[e]]);
         p.indeg[rank[succ[e]]]++;
       }
+      Task& tk = p.tasks[r];
+      tk.succ0 = p.succ_off[r];
+      tk.nsucc = (int32_t)p.succ.size() - p.succ_off[r];
+      for (size_t e = p.succ_off[r]; e < p.succ.size(); ++e) p.rem0[p.succ[e]] += counts_parts(tk) ? tk.parts : 1;
     }
     p.succ_off[nt_] = (int32_t)p.succ.size();
     p.nbuckets = (nt_ + kTasksPerBucket - 1) / kTasksPerBucket;
-    p.slots0.assign((size_t)p.nbuckets * kSlotsPerBucket, -1);
+    p.soff.assign(p.nbuckets + 1, 0);
     p.tail0.assign(p.nbuckets, 0);
-    p.bcap.assign(p.nbuckets, 0);
     p.urgent_parts = 0;
     p.urgent_tail0 = 0;
     for (int r = 0; r < nt_; ++r) {
       const int parts = p.tasks[r].parts;
-      if (p.tasks[r].flags & TF_URGENT) {
-        p.urgent_parts += parts;
-        continue;
-      }
+      if (p.tasks[r].flags & TF_URGENT) p.urgent_parts += parts;
+      else p.soff[r / kTasksPerBucket + 1] += parts;
+    }
+    for (int b = 0; b < p.nbuckets; ++b) p.soff[b + 1] += p.soff[b];
+    p.slots0.assign(p.soff[p.nbuckets], -1);
+    for (int r = 0; r < nt_; ++r) {
+      if ((p.tasks[r].flags & TF_URGENT) || p.indeg[r] != 0) continue;
       const int b = r / kTasksPerBucket;
-      p.bcap[b] += parts;
-      if (p.indeg[r] == 0)
-        for (int q = 0; q < parts; ++q) p.slots0[(size_t)b * kSlotsPerBucket + p.tail0[b]++] = 4 * r + q;
+      for (int q = 0; q < p.tasks[r].parts; ++q) p.slots0[p.soff[b] + p.tail0[b]++] = kMaxParts * r + q;
     }
     p.uslots0.assign(std::max(1, p.urgent_parts), -1);
     for (int r = 0; r < nt_; ++r)
       if ((p.tasks[r].flags & TF_URGENT) && p.indeg[r] == 0)
-        for (int q = 0; q < p.tasks[r].parts; ++q) p.uslots0[p.urgent_tail0++] = 4 * r + q;
+        for (int q = 0; q < p.tasks[r].parts; ++q) p.uslots0[p.urgent_tail0++] = kMaxParts * r + q;
     p.nctr = (int32_t)chain.size();
     p.ndiag = ndiag;
     p.flops = flops;
@@ -928,6 +915,7 @@ int build_serve_template(const Shape& s, int workers, Plan* out) {
   if (task_estimate(s) > 4.0e8) return STILES_ERR_INVALID_ARG;
   Builder B(s, PLAN_FUSED, out);
   B.serve = true;
+  B.crowd = 2;  // requests run side by side
   B.build_factor();
   B.build_selinv();
   B.flops = tile_flops(s, PLAN_FUSED);
@@ -949,6 +937,7 @@ int build_batch_plan(const std::vector<Shape>& shapes, const std::vector<int64_t
   diag_base->assign(shapes.size() + 1, 0);
   for (size_t m = 0; m < shapes.size(); ++m) {
     Builder B(shapes[m], PLAN_FUSED, nullptr);
+    B.crowd = (int)shapes.size();
     B.build_factor();
     B.build_selinv();
     const int32_t coff = (int32_t)M.chain.size(), doff = M.ndiag;
@@ -992,21 +981,21 @@ int build_batch_plan(const std::vector<Shape>& shapes, const std::vector<int64_t
 
 int check_plan(const Plan& p) {
   const int64_t ntasks = (int64_t)p.tasks.size();
+  if ((int64_t)p.wait_off.size() != ntasks + 1 || (int64_t)p.sig_off.size() != ntasks + 1) return STILES_ERR_PLAN;
   std::vector<int32_t> seen(p.nctr, 0);  // signals issued by tasks before the current one
   for (int64_t t = 0; t < ntasks; ++t) {
     const Task& tk = p.tasks[t];
-    if (tk.wait0 < 0 || tk.nwait < 0 || (int64_t)tk.wait0 + tk.nwait > (int64_t)p.waits.size()) return STILES_ERR_PLAN;
     if (tk.seg0 < 0 || tk.nseg < 0 || (int64_t)tk.seg0 + tk.nseg > (int64_t)p.segs.size()) return STILES_ERR_PLAN;
-    if (tk.sig0 < 0 || tk.nsig < 0 || (int64_t)tk.sig0 + tk.nsig > (int64_t)p.sigs.size()) return STILES_ERR_PLAN;
+    if (tk.succ0 < 0 || tk.nsucc < 0 || (int64_t)tk.succ0 + tk.nsucc > (int64_t)p.succ.size()) return STILES_ERR_PLAN;
     if (tk.m < 0 || tk.n < 0 || tk.m > FB || tk.n > FB || tk.op > OP_JOIN) return STILES_ERR_PLAN;
-    if (tk.parts < 1 || tk.parts > 4 || tk.pmode > PM_QUAD16 || tk.prec > PREC_FP32X) return STILES_ERR_PLAN;
-    for (int q = 0; q < tk.nwait; ++q) {
-      const Wait& w = p.waits[tk.wait0 + q];
+    if (tk.parts < 1 || tk.parts > kMaxParts || tk.pmode > PM_TRI16 || tk.prec > PREC_FP32X) return STILES_ERR_PLAN;
+    for (int64_t q = p.wait_off[t]; q < p.wait_off[t + 1]; ++q) {
+      const Wait& w = p.waits[q];
       if (w.ctr < 0 || w.ctr >= p.nctr) return STILES_ERR_PLAN;
       if (w.need > seen[w.ctr]) return STILES_ERR_PLAN;  // would wait for a later task: can deadlock
     }
-    for (int q = 0; q < tk.nsig; ++q) {
-      int32_t c = p.sigs[tk.sig0 + q];
+    for (int64_t q = p.sig_off[t]; q < p.sig_off[t + 1]; ++q) {
+      int32_t c = p.sigs[q];
       if (c < 0 || c >= p.nctr) return STILES_ERR_PLAN;
       seen[c]++;
     }
@@ -1066,30 +1055,10 @@ int validate_plan_len(const Plan& p, int64_t lim, int kind) {
       continue;
     }
     for (int q = 0; q < tk.parts; ++q) {
-      int r0 = 0, c0 = 0, rm = tk.m, cn = tk.n;
-      switch (tk.pmode) {
-        case PM_ROWS2: r0 = 32 * q; rm = std::min(32, tk.m - r0); break;
-        case PM_ROWS4: r0 = 16 * q; rm = std::min(16, tk.m - r0); break;
-        case PM_QUAD4: r0 = 32 * (q & 1); c0 = 32 * (q >> 1); break;
-        case PM_TRI3: r0 = q == 0 ? 0 : 32; c0 = q == 2 ? 32 : 0; break;
-        case PM_TILE32: {
-          const int pr = tk.m > 32 ? 2 : 1;
-          r0 = 32 * (q % pr); c0 = 32 * (q / pr);
-          break;
-        }
-        case PM_ROWS8: r0 = 8 * q; rm = std::min(8, tk.m - r0); break;
-        case PM_TRI16: r0 = q == 0 ? 0 : 16; c0 = q == 2 ? 16 : 0; break;
-        case PM_QUAD16: r0 = 16 * (q >> 1); c0 = 16 * (q & 1); break;
-        default: break;
-      }
-      if (tk.pmode == PM_QUAD4 || tk.pmode == PM_TRI3 || tk.pmode == PM_TILE32) {
-        rm = std::min(32, tk.m - r0); cn = std::min(32, tk.n - c0);
-      } else if (tk.pmode == PM_TRI16 || tk.pmode == PM_QUAD16) {
-        rm = std::min(16, tk.m - r0); cn = std::min(16, tk.n - c0);
-      }
-      if ((tk.pmode == PM_ROWS8 && tk.m > 32) || ((tk.pmode == PM_TRI16 || tk.pmode == PM_QUAD16) && (tk.m > 32 || tk.n > 32)))
-        return bad("fine part mode on a block larger than 32", t);
-      if ((tk.pmode == PM_TRI16 || tk.pmode == PM_QUAD16) && tk.prec != PREC_FP64)
+      const Sub sb = part_sub(tk.pmode, tk.m, tk.n, q);
+      const int r0 = sb.r0, c0 = sb.c0, rm = sb.rm, cn = sb.cn;
+      if ((tk.pmode == PM_TRI16 || tk.pmode == PM_TRI3) && tk.m != tk.n) return bad("triangle parts on a block that is not square", t);
+      if ((tk.pmode == PM_TRI16 || tk.pmode == PM_GRID16) && tk.prec != PREC_FP64)
         return bad("16 x 16 parts on a reduced-precision task", t);
       if (tk.prec == PREC_EMU64 && (rm > 32 || cn > 32)) return bad("emulated task part larger than 32 x 32", t);
       if (tk.prec != PREC_FP64 && tk.op != OP_UPD && tk.op != OP_NEG && tk.op != OP_STORE && tk.op != OP_SYMUPD)
@@ -1119,7 +1088,7 @@ int validate_plan_len(const Plan& p, int64_t lim, int kind) {
     }
   }
   // queue emulation: pushes per bucket / urgent queue never exceed capacity
-  std::vector<int> rem(p.indeg), tail(p.tail0), seen(nt, 0);
+  std::vector<int> rem(p.rem0), tail(p.tail0), seen(nt, 0);
   int utail = p.urgent_tail0;
   std::vector<int> stack;
   for (int t = 0; t < nt; ++t)
@@ -1133,7 +1102,8 @@ int validate_plan_len(const Plan& p, int64_t lim, int kind) {
     for (int e = p.succ_off[t]; e < p.succ_off[t + 1]; ++e) {
       const int sc = p.succ[e];
       if (sc < 0 || sc >= nt) return bad("successor out of range", t);
-      if (--rem[sc] == 0) {
+      rem[sc] -= counts_parts(p.tasks[t]) ? p.tasks[t].parts : 1;
+      if (rem[sc] == 0) {
         const int parts = p.tasks[sc].parts;
         if (p.tasks[sc].flags & TF_URGENT) {
           utail += parts;
@@ -1141,7 +1111,7 @@ int validate_plan_len(const Plan& p, int64_t lim, int kind) {
         } else {
           const int b = sc / kTasksPerBucket;
           tail[b] += parts;
-          if (tail[b] > p.bcap[b] || tail[b] > kSlotsPerBucket) return bad("bucket overflow", sc);
+          if (tail[b] > p.soff[b + 1] - p.soff[b]) return bad("bucket overflow", sc);
         }
         stack.push_back(sc);
       }
@@ -1150,7 +1120,7 @@ int validate_plan_len(const Plan& p, int64_t lim, int kind) {
   }
   if (done != nt) return bad("some tasks never become ready", -1);
   for (int b = 0; b < p.nbuckets; ++b)
-    if (tail[b] != p.bcap[b]) return bad("bucket not filled exactly", b * kTasksPerBucket);
+    if (tail[b] != p.soff[b + 1] - p.soff[b]) return bad("bucket not filled exactly", b * kTasksPerBucket);
   if (utail != p.urgent_parts) return bad("urgent queue not filled exactly", -1);
   return 0;
 }
@@ -1173,38 +1143,6 @@ int validate_plan_len(const Plan& p, int64_t lim, int kind) {
 // first race printed to stderr) or STILES_ERR_INVALID_ARG.
 namespace {
 
-struct PartRect {
-  int r0, c0, rm, cn;
-};
-
-PartRect part_rect(const Task& tk, int q) {
-  PartRect x{0, 0, tk.m, tk.n};
-  switch (tk.pmode) {
-    case PM_ROWS2: x.r0 = 32 * q; x.rm = std::min(32, tk.m - x.r0); break;
-    case PM_ROWS4: x.r0 = 16 * q; x.rm = std::min(16, tk.m - x.r0); break;
-    case PM_ROWS8: x.r0 = 8 * q; x.rm = std::min(8, tk.m - x.r0); break;
-    case PM_QUAD4: x.r0 = 32 * (q & 1); x.c0 = 32 * (q >> 1); break;
-    case PM_TRI3: x.r0 = q == 0 ? 0 : 32; x.c0 = q == 2 ? 32 : 0; break;
-    case PM_TRI16: x.r0 = q == 0 ? 0 : 16; x.c0 = q == 2 ? 16 : 0; break;
-    case PM_QUAD16: x.r0 = 16 * (q >> 1); x.c0 = 16 * (q & 1); break;
-    case PM_TILE32: {
-      const int pr = tk.m > 32 ? 2 : 1;
-      x.r0 = 32 * (q % pr);
-      x.c0 = 32 * (q / pr);
-      break;
-    }
-    default: break;
-  }
-  if (tk.pmode == PM_QUAD4 || tk.pmode == PM_TRI3 || tk.pmode == PM_TILE32) {
-    x.rm = std::min(32, tk.m - x.r0);
-    x.cn = std::min(32, tk.n - x.c0);
-  } else if (tk.pmode == PM_TRI16 || tk.pmode == PM_QUAD16) {
-    x.rm = std::min(16, tk.m - x.r0);
-    x.cn = std::min(16, tk.n - x.c0);
-  }
-  return x;
-}
-
 class RaceCheck {
  public:
   RaceCheck(const Plan& p, int64_t lim, const std::vector<std::vector<int32_t>>& preds, bool serve)
@@ -1224,13 +1162,13 @@ class RaceCheck {
   }
   bool before(int a, int b) const { return (anc_[(size_t)b * words_ + (a >> 6)] >> (a & 63)) & 1; }
 
-  // one access of part `id` (4 task + part) to element `off` of buffer `buf`
+  // one access of part `id` (kMaxParts task + part) to element `off` of buffer `buf`
   bool access(int buf, int64_t off, int id, bool write) {
     if (serve_ && buf == BUF_A) buf = BUF_L;  // a served request's A is built in place in L
     if (buf < 0 || buf > 3 || off < 0 || off >= lim_) return fail("access outside the buffers", id, -1, buf, off);
-    const int t = id >> 2;
+    const int t = id / kMaxParts;
     const int w = lw_[buf][off];
-    if (w >= 0 && w != id && !before(w >> 2, t)) return fail(write ? "unordered writes" : "read not ordered after the write", w, id, buf, off);
+    if (w >= 0 && w != id && !before(w / kMaxParts, t)) return fail(write ? "unordered writes" : "read not ordered after the write", w, id, buf, off);
     if (!write) {
       // readers since the last write; one the new reader descends from is dropped
       // (a writer ordered after the new reader is ordered after it too)
@@ -1238,7 +1176,7 @@ class RaceCheck {
       while (*link >= 0) {
         const int r = pool_[*link].first;
         if (r == id) return true;
-        if (r >> 2 != t && before(r >> 2, t)) *link = pool_[*link].second;
+        if (r / kMaxParts != t && before(r / kMaxParts, t)) *link = pool_[*link].second;
         else link = &pool_[*link].second;
       }
       pool_.push_back({id, head_[buf][off]});
@@ -1247,7 +1185,7 @@ class RaceCheck {
     }
     for (int e = head_[buf][off]; e >= 0; e = pool_[e].second) {
       const int r = pool_[e].first;
-      if (r != id && !before(r >> 2, t)) return fail("write not ordered after a read", r, id, buf, off);
+      if (r != id && !before(r / kMaxParts, t)) return fail("write not ordered after a read", r, id, buf, off);
     }
     head_[buf][off] = -1;
     lw_[buf][off] = id;
@@ -1265,7 +1203,7 @@ class RaceCheck {
   }
   bool task_part(int t, int q) {
     const Task& tk = p_.tasks[t];
-    const int id = 4 * t + q;
+    const int id = kMaxParts * t + q;
     if (tk.op == OP_JOIN) return true;
     if (tk.op == OP_ZERO) return rect(tk.out, tk.ldo, -tk.zrows, tk.zrows, 0, tk.n, id, true);
     if (tk.op == OP_PREP) {  // the tile column of L (its base-value reads are outside the launch's buffers)
@@ -1273,7 +1211,7 @@ class RaceCheck {
       const int64_t len = (tk.flags & TF_CORNER) ? a * a : (1 + (int64_t)tk.zrows) * b * b + a * b;
       return len > 0 ? rect(tk.out, (int)len, 0, (int)len, 0, 1, id, true) : true;
     }
-    const PartRect x = part_rect(tk, q);
+    const Sub x = part_sub(tk.pmode, tk.m, tk.n, q);
     if (x.rm <= 0 || x.cn <= 0) return true;
     for (int g = tk.seg0; g < tk.seg0 + tk.nseg; ++g) {
       const Seg& sg = p_.segs[g];
@@ -1298,9 +1236,9 @@ class RaceCheck {
     return true;
   }
   bool fail(const char* what, int a, int b, int buf, int64_t off) {
-    const int ta = a >= 0 ? a >> 2 : -1, tb = b >= 0 ? b >> 2 : -1;
+    const int ta = a >= 0 ? a / kMaxParts : -1, tb = b >= 0 ? b / kMaxParts : -1;
     fprintf(stderr, "race_check: %s: task %d part %d (op %d) and task %d part %d (op %d), buffer %d element %lld\n",
-            what, ta, a & 3, ta >= 0 ? (int)p_.tasks[ta].op : -1, tb, b & 3, tb >= 0 ? (int)p_.tasks[tb].op : -1,
+            what, ta, a % kMaxParts, ta >= 0 ? (int)p_.tasks[ta].op : -1, tb, b % kMaxParts, tb >= 0 ? (int)p_.tasks[tb].op : -1,
             buf, (long long)off);
     return false;
   }

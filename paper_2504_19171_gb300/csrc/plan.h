@@ -14,6 +14,7 @@
 // consumer flags of Algorithm 3, one per block or block panel instead of one
 // per tile).
 #pragma once
+#include <stddef.h>
 #include <stdint.h>
 
 namespace stiles {
@@ -51,11 +52,11 @@ enum PartMode : uint8_t {
   PM_ROWS2 = 1,  // rows [0,32) and [32,64)
   PM_QUAD4 = 2,  // the four 32 x 32 quadrants
   PM_TRI3 = 3,   // quadrants (0,0), (1,0), (1,1): a diagonal block's lower part
-  PM_ROWS4 = 4,  // rows [0,16), [16,32), [32,48), [48,64)
+  PM_ROWS4 = 4,  // rows [0,16), [16,32), ..
   PM_TILE32 = 5, // a grid of at most 2 x 2 sub-tiles of at most 32 x 32 (parts = row tiles x column tiles)
-  PM_ROWS8 = 6,  // rows [0,8), [8,16), [16,24), [24,32) of a block of at most 32 rows
-  PM_TRI16 = 7,  // quadrants (0,0), (1,0), (1,1) of 16 x 16: the lower part of a square block of at most 32
-  PM_QUAD16 = 8, // the 16 x 16 quadrants (0,0), (0,1), (1,0), (1,1) of a block of at most 32 x 32
+  PM_ROWS8 = 6,  // rows [0,8), [8,16), ..
+  PM_GRID16 = 7, // a grid of at most 4 x 4 sub-tiles of at most 16 x 16 (parts = row tiles x column tiles)
+  PM_TRI16 = 8,  // the sub-tiles of that grid on or below the diagonal of a square block, row by row
 };
 
 // Arithmetic of a task's block products (its epilogue is always FP64).
@@ -74,6 +75,52 @@ enum TaskFlag : uint8_t {
   TF_CORNER = 4,    // OP_PREP of the arrow corner column
 };
 
+// Sub-tile of part q of an m x n block (rm or cn <= 0: nothing to do).
+struct Sub {
+  int r0, c0, rm, cn;
+};
+
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline Sub part_sub(int pmode, int m, int n, int q) {
+  Sub s{0, 0, m, n};
+  int dim = 0;  // sub-tile order of the grid modes
+  switch (pmode) {
+    case PM_ROWS2: s.r0 = 32 * q; s.rm = 32; break;
+    case PM_ROWS4: s.r0 = 16 * q; s.rm = 16; break;
+    case PM_ROWS8: s.r0 = 8 * q; s.rm = 8; break;
+    case PM_QUAD4: dim = 32; s.r0 = 32 * (q & 1); s.c0 = 32 * (q >> 1); break;
+    case PM_TRI3: dim = 32; s.r0 = q == 0 ? 0 : 32; s.c0 = q == 2 ? 32 : 0; break;
+    case PM_TILE32: {
+      const int pr = m > 32 ? 2 : 1;
+      dim = 32;
+      s.r0 = 32 * (q % pr);
+      s.c0 = 32 * (q / pr);
+      break;
+    }
+    case PM_GRID16: {
+      const int pr = (m + 15) / 16;
+      dim = 16;
+      s.r0 = 16 * (q % pr);
+      s.c0 = 16 * (q / pr);
+      break;
+    }
+    case PM_TRI16: {
+      const int r = q >= 6 ? 3 : q >= 3 ? 2 : q >= 1 ? 1 : 0;
+      dim = 16;
+      s.r0 = 16 * r;
+      s.c0 = 16 * (q - r * (r + 1) / 2);
+      break;
+    }
+    default: break;
+  }
+  if (dim) s.rm = s.cn = dim;
+  if (s.rm > m - s.r0) s.rm = m - s.r0;
+  if (s.cn > n - s.c0) s.cn = n - s.c0;
+  return s;
+}
+
 struct Seg {       // acc += op(A) (m x k) * op(B) (k x n)
   int64_t a, b;    // buffer refs (mkref) of element (0,0) of the stored operands
   int32_t lda, ldb;
@@ -86,26 +133,24 @@ struct Wait {
   int32_t need;    // wait until counter >= need
 };
 
-struct Task {        // 64 bytes
+struct Task {        // 80 bytes
   int64_t out;       // ref of the output block
   int64_t cin;       // ref of the input block (OP_UPD/POTRF/TRSM_RLT/SYMUPD) or -1
   int64_t aux;       // ref of the triangular block (TRSM/TRTRI) or the mirror block (SYMUPD) or -1
   int32_t ldo, ldc, ldx;
   int16_t m, n;      // output rows / columns (<= FB)
   int32_t seg0, nseg;
-  int32_t wait0, nwait;
-  int32_t sig0;      // signals: sig[sig0 .. sig0+nsig)
-  int16_t nsig;
-  uint8_t op;
-  uint8_t flags;     // TaskFlag bits
+  int32_t succ0, nsucc;  // its successors: succ[succ0 .. succ0 + nsucc) (who counts it off them: counts_parts)
   int32_t diag;      // POTRF: index of its logdet partial sum
   int32_t zrows;     // ZERO: rows above the block in its tile column to zero (L's strict upper part)
   int32_t gcol;      // POTRF: 0-based global column of the block's first pivot
-  uint8_t parts;     // 1..4 queue entries (see PartMode)
+  uint8_t op;        // op, flags, parts and pmode share one aligned 32-bit word (read on
+  uint8_t flags;     // their own by the finisher of a predecessor); flags: TaskFlag bits
+  uint8_t parts;     // 1..16 queue entries (see PartMode)
   uint8_t pmode;
   uint8_t prec;      // Precision of the block products
 };
-static_assert(sizeof(Task) == 80, "task layout");
+static_assert(sizeof(Task) == 80 && offsetof(Task, op) % 4 == 0, "task layout");
 
 }  // namespace stiles
 
@@ -144,25 +189,38 @@ struct Shape {
   int sel0 = 0;          // selected inversion of tile columns >= sel0 only (their phase 1 and 2)
 };
 
-// Dynamic schedule: a task becomes ready when its last predecessor finishes
-// (device counter rem[t], initialised to indeg[t]) and is pushed into the
-// bucket of its expected start time in the list schedule; workers pop from the
-// earliest non-empty bucket. Buckets hold kTasksPerBucket consecutive tasks of
-// the list-schedule order.
+// A task with few successors is counted off them by each of its parts as it
+// finishes (one atomic per successor and part, no join of the parts on the
+// critical path); one with many by the last of its parts.
+constexpr int kPartSucc = 16;
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline bool counts_parts(const Task& t) { return t.nsucc <= kPartSucc; }
+
+// Dynamic schedule: a task becomes ready when the last part of its last
+// predecessor finishes (device counter rem[t], initialised to rem0[t]) and is
+// pushed into the bucket of its expected start time in the list schedule;
+// workers pop from the earliest non-empty bucket. Buckets hold kTasksPerBucket
+// consecutive tasks of the list-schedule order.
 constexpr int kTasksPerBucket = 64;
-constexpr int kSlotsPerBucket = 4 * kTasksPerBucket;  // up to 4 parts per task
+constexpr int kMaxParts = 16;  // parts of one task; a queue entry is kMaxParts * task + part
+constexpr int kMaxTasks = (1 << 27) - 1;  // entries stay positive 32-bit integers
 
 struct Plan {
   std::vector<Task> tasks;  // in list-schedule order
   std::vector<Seg> segs;
   std::vector<Wait> waits;  // counter form of the dependencies (host checks)
   std::vector<int32_t> sigs;
+  std::vector<int64_t> wait_off;  // waits of task t: waits[wait_off[t] .. wait_off[t+1])
+  std::vector<int64_t> sig_off;   // signalled counters of task t: sigs[sig_off[t] .. sig_off[t+1])
   std::vector<int32_t> indeg;     // predecessors per task
+  std::vector<int32_t> rem0;      // device counter's start value: predecessors, those that count parts by their parts
   std::vector<int32_t> succ_off;  // successors: succ[succ_off[t] .. succ_off[t+1])
   std::vector<int32_t> succ;
+  std::vector<int32_t> soff;      // slots of bucket b: [soff[b], soff[b+1]) (one per part)
   std::vector<int32_t> slots0;    // initial bucket slots: ready tasks at the front, -1 elsewhere
   std::vector<int32_t> tail0;     // initial ready parts per bucket
-  std::vector<int32_t> bcap;      // parts per bucket (a bucket is finished when all were popped)
   std::vector<int32_t> uslots0;   // initial urgent queue (ready urgent parts first, -1 elsewhere)
   int32_t urgent_parts = 0;       // capacity of the urgent queue
   int32_t urgent_tail0 = 0;

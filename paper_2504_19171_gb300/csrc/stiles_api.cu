@@ -22,23 +22,24 @@ namespace {
 struct DevPlan {
   Task* tasks = nullptr;
   Seg* segs = nullptr;
-  int32_t* succ_off = nullptr;
   int32_t* succ = nullptr;
-  int32_t* bcap = nullptr;
+  int32_t* soff = nullptr;
   int32_t* image = nullptr;  // initial scheduler state (copied to scratch before each launch)
   size_t image_ints = 0;
   int ntasks = 0;
   int nbuckets = 0;
+  int nslots = 0;
   int ucap = 0;
 };
 
-// Initial scheduler state of a plan: rem = indeg, slots = slots0, tail = tail0,
+// Initial scheduler state of a plan: rem = rem0, slots = slots0, tail = tail0,
 // head = 0, gcnt = ready tasks per group of 32 buckets, lo = 0.
 std::vector<int32_t> sched_image(const Plan& p) {
   const int nt = (int)p.tasks.size(), nb = p.nbuckets;
-  std::vector<int32_t> img(sched_state_ints(nt, nb, p.urgent_parts), 0);
-  SchedState q = sched_state_at(img.data(), nt, nb, p.urgent_parts);
-  for (int t = 0; t < nt; ++t) q.rem[t] = p.indeg[t];
+  const int ns = (int)p.slots0.size();
+  std::vector<int32_t> img(sched_state_ints(nt, nb, ns, p.urgent_parts), 0);
+  SchedState q = sched_state_at(img.data(), nt, nb, ns, p.urgent_parts);
+  for (int t = 0; t < nt; ++t) q.rem[t] = p.rem0[t];
   for (size_t i = 0; i < p.slots0.size(); ++i) q.slots[i] = p.slots0[i];
   for (int b = 0; b < nb; ++b) {
     q.tail[b] = p.tail0[b];
@@ -117,9 +118,8 @@ static void free_handle(stiles_handle* h) {
   for (auto& d : h->dev) {
     cudaFree(d.tasks);
     cudaFree(d.segs);
-    cudaFree(d.succ_off);
     cudaFree(d.succ);
-    cudaFree(d.bcap);
+    cudaFree(d.soff);
     cudaFree(d.image);
   }
   cudaFree(h->dstatus);
@@ -172,14 +172,14 @@ static int create_handle(int nt, int b, int band, int arrow, int precision, int 
     Plan& p = h->plans[k];
     rc = upload(p.tasks, &h->dev[k].tasks);
     if (!rc) rc = upload(p.segs, &h->dev[k].segs);
-    if (!rc) rc = upload(p.succ_off, &h->dev[k].succ_off);
     if (!rc) rc = upload(p.succ, &h->dev[k].succ);
-    if (!rc) rc = upload(p.bcap, &h->dev[k].bcap);
+    if (!rc) rc = upload(p.soff, &h->dev[k].soff);
     std::vector<int32_t> img = sched_image(p);
     if (!rc) rc = upload(img, &h->dev[k].image);
     h->dev[k].image_ints = img.size();
     h->dev[k].ntasks = (int)p.tasks.size();
     h->dev[k].nbuckets = p.nbuckets;
+    h->dev[k].nslots = (int)p.slots0.size();
     h->dev[k].ucap = p.urgent_parts;
     if (img.size() > h->state_ints_max) h->state_ints_max = img.size();
     if (p.ndiag > h->ndiag) h->ndiag = p.ndiag;
@@ -232,13 +232,12 @@ static int launch(stiles_t h, int kind, const double* A, double* L, double* S, v
   KParams p{};
   p.tasks = d.tasks;
   p.segs = d.segs;
-  p.succ_off = d.succ_off;
   p.succ = d.succ;
-  p.bcap = d.bcap;
+  p.soff = d.soff;
   p.ntasks = d.ntasks;
   p.nbuckets = d.nbuckets;
   p.ucap = d.ucap;
-  p.q = sched_state_at(state, d.ntasks, d.nbuckets, d.ucap);
+  p.q = sched_state_at(state, d.ntasks, d.nbuckets, d.nslots, d.ucap);
   p.st = ds;
   p.logdet_part = h->dlogdet;
   p.buf[BUF_A] = const_cast<double*>(A);
@@ -538,13 +537,9 @@ extern "C" int stiles_debug_check_corrupted(int nt, int b, int band, int arrow, 
     case 1: p.waits.back().ctr = p.nctr; break;
     case 2: p.waits.back().need += 1000000; break;
     case 3: {  // make the first task that waits depend on the last task's signal
-      const Task& last = p.tasks.back();
-      if (last.nsig < 1) return STILES_ERR_INVALID_ARG;
-      for (Task& t : p.tasks)
-        if (t.nwait > 0) {
-          p.waits[t.wait0] = Wait{p.sigs[last.sig0], 1 << 20};
-          break;
-        }
+      const size_t nt_ = p.tasks.size();
+      if (p.sig_off[nt_] <= p.sig_off[nt_ - 1]) return STILES_ERR_INVALID_ARG;
+      p.waits.front() = Wait{p.sigs[p.sig_off[nt_ - 1]], 1 << 20};
       break;
     }
     default: return STILES_ERR_INVALID_ARG;
@@ -558,11 +553,11 @@ extern "C" int stiles_debug_break_plan(stiles_t h, int which) {
   // the first task with a predecessor now waits for one more that never comes
   for (size_t t = 0; t < p.tasks.size(); ++t)
     if (p.indeg[t] > 0) {
-      const int32_t v = p.indeg[t] + 1;
+      const int32_t v = p.rem0[t] + 1;
       if (cudaSetDevice(h->device) != cudaSuccess) return STILES_ERR_CUDA;
       if (cudaMemcpy(h->dev[which].image + t, &v, sizeof(int32_t), cudaMemcpyHostToDevice) != cudaSuccess)
         return STILES_ERR_CUDA;
-      p.indeg[t] = v;
+      p.rem0[t] = v;
       return STILES_OK;
     }
   return STILES_ERR_INVALID_ARG;
@@ -642,9 +637,8 @@ static void free_batch(stiles_batch* h) {
   if (h->graph) cudaGraphDestroy(h->graph);
   cudaFree(h->dev.tasks);
   cudaFree(h->dev.segs);
-  cudaFree(h->dev.succ_off);
   cudaFree(h->dev.succ);
-  cudaFree(h->dev.bcap);
+  cudaFree(h->dev.soff);
   cudaFree(h->dev.image);
   cudaFree(h->dstatus);
   cudaFree(h->dlogdet);
@@ -688,9 +682,8 @@ extern "C" int stiles_batch_create(int count, const int* nt, const int* b, const
   Plan& p = h->plan;
   rc = upload(p.tasks, &h->dev.tasks);
   if (!rc) rc = upload(p.segs, &h->dev.segs);
-  if (!rc) rc = upload(p.succ_off, &h->dev.succ_off);
   if (!rc) rc = upload(p.succ, &h->dev.succ);
-  if (!rc) rc = upload(p.bcap, &h->dev.bcap);
+  if (!rc) rc = upload(p.soff, &h->dev.soff);
   {
     std::vector<int32_t> img = sched_image(p);
     if (!rc) rc = upload(img, &h->dev.image);
@@ -698,6 +691,7 @@ extern "C" int stiles_batch_create(int count, const int* nt, const int* b, const
   }
   h->dev.ntasks = (int)p.tasks.size();
   h->dev.nbuckets = p.nbuckets;
+  h->dev.nslots = (int)p.slots0.size();
   h->dev.ucap = p.urgent_parts;
   h->ndiag = p.ndiag;
   if (!rc) rc = dev_malloc((void**)&h->dstatus, sizeof(DevStatus));
@@ -715,7 +709,9 @@ extern "C" int stiles_batch_create(int count, const int* nt, const int* b, const
   p.tasks.clear(); p.tasks.shrink_to_fit();
   p.segs.clear(); p.segs.shrink_to_fit();
   p.waits.clear(); p.waits.shrink_to_fit();
+  p.wait_off.clear(); p.wait_off.shrink_to_fit();
   p.sigs.clear(); p.sigs.shrink_to_fit();
+  p.sig_off.clear(); p.sig_off.shrink_to_fit();
   p.succ.clear(); p.succ.shrink_to_fit();
   p.succ_off.clear(); p.succ_off.shrink_to_fit();
   p.slots0.clear(); p.slots0.shrink_to_fit();
@@ -753,13 +749,12 @@ static int build_batch_graph(stiles_batch* h, const double* A, double* L, double
   p = KParams{};
   p.tasks = h->dev.tasks;
   p.segs = h->dev.segs;
-  p.succ_off = h->dev.succ_off;
   p.succ = h->dev.succ;
-  p.bcap = h->dev.bcap;
+  p.soff = h->dev.soff;
   p.ntasks = h->dev.ntasks;
   p.nbuckets = h->dev.nbuckets;
   p.ucap = h->dev.ucap;
-  p.q = sched_state_at(state, h->dev.ntasks, h->dev.nbuckets, h->dev.ucap);
+  p.q = sched_state_at(state, h->dev.ntasks, h->dev.nbuckets, h->dev.nslots, h->dev.ucap);
   p.st = h->dstatus;
   p.logdet_part = h->dlogdet;
   p.badpiv = h->dbad;

@@ -21,9 +21,9 @@ struct DevStatus {
 
 // Per-launch scheduler state, one contiguous int32 block in the caller's
 // scratch, reset before every launch from a device image built at create:
-//   rem[ntasks]      predecessors not yet finished (image: indeg)
+//   rem[ntasks]      predecessors, or their parts, not yet finished (image: rem0)
 //   pdone[ntasks]    parts of the task finished so far
-//   slots[nb*kSlotsPerBucket]  bucket b owns slots [b*kSlotsPerBucket, +kSlotsPerBucket)
+//   slots[nslots]    bucket b owns slots [soff[b], soff[b + 1])
 //   tail[nbuckets]   slots reserved by pushes into the bucket so far
 //   head[nbuckets]   slots claimed by pops so far
 //   avail[nbuckets]  parts pushed and not yet claimed (a pop claims one by
@@ -32,7 +32,8 @@ struct DevStatus {
 //   scnt[nsuper]     ready parts per super-group of 32 groups (a scan hint)
 //   uslots[ucap]     urgent queue (critical-path tasks), popped before any bucket
 //   lo[32]           lo[0]: every bucket below it is finished (all popped);
-//                    lo[8]: urgent tail, lo[16]: urgent head, lo[24]: urgent avail
+//                    lo[8]: urgent tail, lo[16]: urgent head, lo[24]: urgent avail,
+//                    lo[20]: urgent parts that their releaser ran itself
 struct SchedState {
   int* rem;
   int* pdone;
@@ -46,18 +47,18 @@ struct SchedState {
   int* lo;
 };
 
-inline size_t sched_state_ints(int ntasks, int nbuckets, int ucap) {
+inline size_t sched_state_ints(int ntasks, int nbuckets, int nslots, int ucap) {
   const int ngroups = (nbuckets + 31) / 32, nsuper = (ngroups + 31) / 32;
-  return 2 * (size_t)ntasks + (size_t)nbuckets * kSlotsPerBucket + 3 * (size_t)nbuckets + (size_t)ngroups +
+  return 2 * (size_t)ntasks + (size_t)nslots + 3 * (size_t)nbuckets + (size_t)ngroups +
          (size_t)nsuper + (size_t)(ucap > 0 ? ucap : 1) + 32;
 }
 
-inline SchedState sched_state_at(int* base, int ntasks, int nbuckets, int ucap) {
+inline SchedState sched_state_at(int* base, int ntasks, int nbuckets, int nslots, int ucap) {
   SchedState s;
   s.rem = base;
   s.pdone = s.rem + ntasks;
   s.slots = s.pdone + ntasks;
-  s.tail = s.slots + (size_t)nbuckets * kSlotsPerBucket;
+  s.tail = s.slots + nslots;
   s.head = s.tail + nbuckets;
   s.avail = s.head + nbuckets;
   s.gcnt = s.avail + nbuckets;
@@ -108,9 +109,8 @@ struct ServeDev {
 struct KParams {
   const Task* tasks;
   const Seg* segs;
-  const int32_t* succ_off;  // successors in schedule order
-  const int32_t* succ;
-  const int32_t* bcap;  // parts per bucket
+  const int32_t* succ;  // successors in schedule order
+  const int32_t* soff;  // first slot of each bucket (nbuckets + 1)
   int ntasks;
   int nbuckets;
   int ucap;             // urgent queue capacity

@@ -110,28 +110,62 @@ __device__ void check_fail(const KParams& p, int what, long long t, int q) {
   } while (0)
 #endif
 
-// Push a ready task into the bucket of its queue position: one slot per part
-// (value 4 t + part), so that the parts run on different CTAs. The slots are
-// reserved (tail), stored, and only then counted as available.
-__device__ void serve_push(const KParams& p, int t);
+// Order of the scheduler's memory operations. A part's writes are released by
+// one fence of the finishing warp (its block barrier made them that warp's
+// past), after which relaxed atomics count it off; whoever brings a counter to
+// zero fences again (it takes on the other finishers' writes) and publishes
+// queue slots with relaxed stores. A worker takes a slot with an acquire load,
+// and its block barrier passes that on to the other warps.
+__device__ __forceinline__ void fence_dev() { cuda::atomic_thread_fence(cuda::memory_order_acq_rel, cuda::thread_scope_device); }
 
-__device__ __forceinline__ void push_task(const KParams& p, int t) {
+__device__ __forceinline__ void store_relaxed_i(int* a, int v) {
+  cuda::atomic_ref<int, cuda::thread_scope_device>(*a).store(v, cuda::memory_order_relaxed);
+}
+
+__device__ __forceinline__ int add_relaxed_i(int* a, int v) {
+  return cuda::atomic_ref<int, cuda::thread_scope_device>(*a).fetch_add(v, cuda::memory_order_relaxed);
+}
+
+// The word of a task row that a releaser needs (op, flags, parts, pmode).
+struct TaskWord {
+  uint32_t w;
+  __device__ __forceinline__ int op() const { return (int)(w & 0xffu); }
+  __device__ __forceinline__ int flags() const { return (int)((w >> 8) & 0xffu); }
+  __device__ __forceinline__ int parts() const { return (int)((w >> 16) & 0xffu); }
+};
+static_assert(offsetof(Task, flags) == offsetof(Task, op) + 1 && offsetof(Task, parts) == offsetof(Task, op) + 2,
+              "task word");
+
+// Plain load, as load_task (a request server's rows are ordered by the
+// acquire of the slot that delivered a task of the same request).
+__device__ __forceinline__ TaskWord load_task_word(const KParams& p, int t) {
+  return {*reinterpret_cast<const uint32_t*>(&p.tasks[t].op)};
+}
+
+__device__ void serve_push(const KParams& p, int t, TaskWord tw, int q0);
+
+// Push parts q0 .. of a ready task (one slot per part, value kMaxParts t +
+// part, so that the parts run on different CTAs): urgent tasks into their
+// FIFO, the others into the bucket of their queue position. The slots are
+// reserved (tail), stored, and only then counted as available. The caller has
+// fenced.
+__device__ __forceinline__ void push_task(const KParams& p, int t, TaskWord tw, int q0) {
   if (p.serve) {
-    serve_push(p, t);
+    serve_push(p, t, tw, q0);
     return;
   }
-  const Task tk = load_task(p, t);
-  const int parts = tk.parts;
+  const int parts = tw.parts() - q0;
+  if (parts <= 0) return;
   // The queue capacities are checked in every build (one compare on an
   // atomic path): a table that would overflow a queue stops the launch with
   // a check failure instead of writing past the slots.
-  if (tk.flags & TF_URGENT) {
-    const int pos = atomicAdd(p.q.lo + 8, parts);
+  if (tw.flags() & TF_URGENT) {
+    const int pos = add_relaxed_i(p.q.lo + 8, parts);
     if (pos + parts > p.ucap) {
       check_fail(p, 1, t, 0);
       return;
     }
-    for (int q = 0; q < parts; ++q) store_release_i(p.q.uslots + pos + q, 4 * t + q);
+    for (int q = 0; q < parts; ++q) store_relaxed_i(p.q.uslots + pos + q, kMaxParts * t + q0 + q);
     atomicAdd(p.q.lo + 24, parts);
     return;
   }
@@ -140,12 +174,13 @@ __device__ __forceinline__ void push_task(const KParams& p, int t) {
     check_fail(p, 2, t, 0);
     return;
   }
-  const int pos = atomicAdd(p.q.tail + b, parts);
-  if (pos + parts > p.bcap[b]) {
+  const int s0 = p.soff[b], cap = p.soff[b + 1] - s0;
+  const int pos = add_relaxed_i(p.q.tail + b, parts);
+  if (pos + parts > cap) {
     check_fail(p, 3, t, 0);
     return;
   }
-  for (int q = 0; q < parts; ++q) store_release_i(p.q.slots + (size_t)b * kSlotsPerBucket + pos + q, 4 * t + q);
+  for (int q = 0; q < parts; ++q) store_relaxed_i(p.q.slots + s0 + pos + q, kMaxParts * t + q0 + q);
   atomicAdd(p.q.avail + b, parts);
   atomicAdd(p.q.gcnt + (b >> 5), parts);
   atomicAdd(p.q.scnt + (b >> 10), parts);
@@ -170,10 +205,10 @@ __device__ int wait_slot(const KParams& p, int* slot, unsigned long long start) 
 
 // Lane 0: claim one available part of a queue (avail / head pair) without a
 // compare-and-swap retry loop: many idle workers contending for the same
-// bucket each cost two fetch-and-adds, not a round trip per lost race.
-// Returns the claimed slot index, or -1 if nothing was available.
+// bucket each cost two fetch-and-adds, not a round trip per lost race. The
+// caller has just read avail > 0. Returns the claimed slot index, or -1 if
+// nothing was available.
 __device__ __forceinline__ int claim(int* avail, int* head) {
-  if (load_relaxed_flag(avail) <= 0) return -1;
   if (atomicSub(avail, 1) <= 0) {
     atomicAdd(avail, 1);
     return -1;
@@ -181,15 +216,21 @@ __device__ __forceinline__ int claim(int* avail, int* head) {
   return atomicAdd(head, 1);
 }
 
+// Pause of a worker that found nothing. The first half of the grid (one CTA
+// per SM) looks again at once, the second half after a longer pause: with few
+// ready parts they go to different SMs, whose FP64 pipes they then do not
+// share, and fewer workers contend for them.
+__device__ __forceinline__ void idle_pause() { __nanosleep(blockIdx.x * 2 < gridDim.x ? 20 : 600); }
+
 // ---- request server: three FIFO rings (urgent, other factor tasks, rest) ---
 // Ring entries are reserved (tail), stored, then counted available, like the
 // buckets; a popped entry is reset to -1 so the ring can wrap (its capacity
 // exceeds the parts that can be ready at once).
-__device__ void serve_push(const KParams& p, int t) {
-  const Task tk = load_task(p, t);
-  const int parts = tk.parts;
-  const bool factor = tk.op == OP_UPD || tk.op == OP_POTRF || tk.op == OP_TRSM_RLT || tk.op == OP_PREP;
-  const ServeRing& R = p.sv.ring[(tk.flags & TF_URGENT) ? 0 : factor ? 1 : 2];
+__device__ void serve_push(const KParams& p, int t, TaskWord tw, int q0) {
+  const int parts = tw.parts() - q0, op = tw.op();
+  if (parts <= 0) return;
+  const bool factor = op == OP_UPD || op == OP_POTRF || op == OP_TRSM_RLT || op == OP_PREP;
+  const ServeRing& R = p.sv.ring[(tw.flags() & TF_URGENT) ? 0 : factor ? 1 : 2];
   const unsigned pos = (unsigned)atomicAdd(R.ctr, parts);
   for (int q = 0; q < parts; ++q) {
     int* slot = R.slots + ((pos + q) & R.mask);
@@ -202,36 +243,9 @@ __device__ void serve_push(const KParams& p, int t) {
       }
       __nanosleep(64);
     }
-    store_release_i(slot, 4 * t + q);
+    store_release_i(slot, kMaxParts * t + q0 + q);
   }
   atomicAdd(R.ctr + 16, parts);
-}
-
-// Lane 0 of an idle worker: a ready part of the highest non-empty ring
-// (>= 0), a new request to activate (-4 - record index), -1 to stop, or -3.
-__device__ int serve_try_lane0(const KParams& p, unsigned long long deadline) {
-  if (load_relaxed_flag(&p.st->abort)) return -1;
-  for (int r = 0; r < 3; ++r) {
-    const ServeRing& R = p.sv.ring[r];
-    const int h = claim(R.ctr + 16, R.ctr + 8);
-    if (h >= 0) {
-      int* slot = R.slots + ((unsigned)h & R.mask);
-      const int v = wait_slot(p, slot, gtimer());
-      if (v >= 0) cuda::atomic_ref<int, cuda::thread_scope_device>(*slot).store(-1, cuda::memory_order_relaxed);
-      return v;
-    }
-  }
-  const int seen = load_relaxed_flag(p.sv.inbox_seen);
-  if (seen < load_acquire_sys(&p.sv.ctl->inbox_count)) {
-    if (atomicCAS(p.sv.inbox_seen, seen, seen + 1) == seen) return -4 - seen;
-    return -3;
-  }
-  if (load_acquire_sys(&p.sv.ctl->stop)) return -1;
-  if (gtimer() > deadline) {
-    raise_timeout(p, -2);
-    return -1;
-  }
-  return -3;
 }
 
 // Warp 0: activate inbox record `idx`: its value parameters, then its root
@@ -253,142 +267,234 @@ __device__ void serve_activate(const KParams& p, int idx) {
   root0 = __shfl_sync(0xffffffffu, root0, 0);
   nroots = __shfl_sync(0xffffffffu, nroots, 0);
   __syncwarp();
-  for (int i = lane; i < nroots; i += 32) push_task(p, __ldcg(p.sv.roots + root0 + i));
+  for (int i = lane; i < nroots; i += 32) {
+    const int t = __ldcg(p.sv.roots + root0 + i);
+    push_task(p, t, load_task_word(p, t), 0);
+  }
 }
 
+// Idle worker of a request server: a ready part of the highest non-empty
+// ring, or -1 to stop. One round of loads per look (the abort flag and the
+// three rings' counts, one lane each); the host-mapped words (inbox, stop),
+// whose reads cross the host link, are looked at by a few workers on every
+// round and by the others on every eighth.
 __device__ int serve_pop(const KParams& p, unsigned long long deadline) {
   const unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
-  for (;;) {
-    int r = -3;
-    if (lane == 0) r = serve_try_lane0(p, deadline);
-    r = __shfl_sync(FULL, r, 0);
-    if (r >= -1) return r;
-    if (r <= -4) {
-      serve_activate(p, -4 - r);
-      continue;
-    }
-    __nanosleep(400);
-  }
-}
-
-// Lane 0: abort / budget check, then one attempt on the urgent queue.
-// Returns an item (>= 0), -1 to stop, or -3 when no urgent part is ready.
-__device__ int pop_urgent_lane0(const KParams& p, unsigned long long start) {
-  if (load_relaxed_flag(&p.st->abort)) return -1;
-  if (gtimer() - start > (unsigned long long)p.budget_ns) {
-    raise_timeout(p, (long long)load_relaxed_flag(p.q.lo) * kTasksPerBucket);
-    return -1;
-  }
-  if (p.ucap <= 0) return -3;
-  const int uh = claim(p.q.lo + 24, p.q.lo + 16);
-  if (uh < 0) return -3;
-  if (uh >= p.ucap) {  // claimed past the urgent queue (checked in every build)
-    check_fail(p, 4, uh, 0);
-    return -1;
-  }
-  return wait_slot(p, p.q.uslots + uh, start);
-}
-
-// Warp 0 pops a ready task part: the urgent queue first, then the earliest
-// bucket (queue order) with an available part. Lane 0 takes every decision
-// and broadcasts it, the other lanes only help to scan 32 super-groups /
-// groups / buckets per load round, so the warp stays uniform. Returns
-// 4 * task + part, or -1 when every part has been popped, the launch was
-// aborted, or the wait budget of this call expired (TIMEOUT; checked on
-// every pass of the loop).
-__device__ int pop_task(const KParams& p, unsigned long long deadline) {
-  if (p.serve) return serve_pop(p, deadline);
-  const unsigned FULL = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
-  const int nb = p.nbuckets, ngroups = (nb + 31) / 32, nsuper = (ngroups + 31) / 32;
-  const unsigned long long start = lane == 0 ? gtimer() : 0ull;
-  for (;;) {
-    int r = -3;
-    if (lane == 0) r = pop_urgent_lane0(p, start);
-    r = __shfl_sync(FULL, r, 0);
-    if (r != -3) return r;
-    int l = 0;
-    if (lane == 0) l = load_relaxed_flag(p.q.lo);
-    l = __shfl_sync(FULL, l, 0);
-    // scan from lo: super-groups of 32 groups, groups of 32 buckets, buckets
-    int got = -3;  // -3: nothing found, -1: stop, >= 0: item
-    const int g_lo = l >> 5;
-    for (int sbase = l >> 10; sbase < nsuper && got == -3; sbase += 32) {
-      const int sg = sbase + lane;
-      unsigned sm = __ballot_sync(FULL, sg < nsuper && load_relaxed_flag(p.q.scnt + sg) > 0);
-      while (sm && got == -3) {
-        const int si = sbase + __ffs(sm) - 1;
-        sm &= sm - 1;
-        const int g = si * 32 + lane;
-        unsigned gm = __ballot_sync(FULL, g < ngroups && g >= g_lo && load_relaxed_flag(p.q.gcnt + g) > 0);
-        while (gm && got == -3) {
-          const int gi = si * 32 + __ffs(gm) - 1;
-          gm &= gm - 1;
-          const int b = gi * 32 + lane;
-          unsigned rm = __ballot_sync(FULL, b < nb && b >= l && load_relaxed_flag(p.q.avail + b) > 0);
-          while (rm && got == -3) {  // try the ready buckets in order
-            const int bb = gi * 32 + __ffs(rm) - 1;
-            rm &= rm - 1;
-            if (lane == 0) {
-              const int h = claim(p.q.avail + bb, p.q.head + bb);
-              if (h >= 0) {
-                atomicSub(p.q.gcnt + gi, 1);
-                atomicSub(p.q.scnt + (gi >> 5), 1);
-                if (h >= p.bcap[bb]) {  // claimed past the bucket (checked in every build)
-                  check_fail(p, 5, bb, 0);
-                  got = -1;
-                } else {
-                  got = wait_slot(p, p.q.slots + (size_t)bb * kSlotsPerBucket + h, start);
-                }
-              }
-            }
-            got = __shfl_sync(FULL, got, 0);
-          }
+  const bool watcher = blockIdx.x < 8;
+  for (unsigned round = 0;; ++round) {
+    int* word = lane == 0 ? &p.st->abort : p.sv.ring[min(max(lane - 1, 0), 2)].ctr + 16;
+    const int v = lane < 4 ? load_relaxed_flag(word) : 0;
+    if (__shfl_sync(FULL, v, 0)) return -1;
+    unsigned ready = __ballot_sync(FULL, lane >= 1 && lane < 4 && v > 0);
+    while (ready) {
+      const int r = __ffs(ready) - 2;
+      ready &= ready - 1;
+      int got = -3;
+      if (lane == 0) {
+        const ServeRing& R = p.sv.ring[r];
+        const int h = claim(R.ctr + 16, R.ctr + 8);
+        if (h >= 0) {
+          int* slot = R.slots + ((unsigned)h & R.mask);
+          got = wait_slot(p, slot, gtimer());
+          if (got >= 0) store_relaxed_i(slot, -1);
         }
       }
+      got = __shfl_sync(FULL, got, 0);
+      if (got != -3) return got;
     }
-    if (got != -3) return got;
-    // nothing claimed: move lo past finished buckets (finished is permanent,
-    // so atomicMax is safe), stop once every part was popped, else back off
-    if (l >= nb) {
-      int done = 0;
-      if (lane == 0) done = load_relaxed_flag(p.q.lo + 16) >= p.ucap;
-      if (__shfl_sync(FULL, done, 0)) return -1;
-    } else {
-      const int b = l + lane;
-      const bool fin = b >= nb || load_relaxed_flag(p.q.head + b) >= p.bcap[b];
-      const unsigned unf = __ballot_sync(FULL, !fin);
-      const int nfin = unf ? __ffs(unf) - 1 : 32;
-      if (nfin > 0) {
-        if (lane == 0) atomicMax(p.q.lo, l + nfin);
+    if (watcher || (round & 7) == 1) {
+      int rec = -3;
+      if (lane == 0) {
+        const int seen = load_relaxed_flag(p.sv.inbox_seen);
+        if (seen < load_acquire_sys(&p.sv.ctl->inbox_count)) {
+          if (atomicCAS(p.sv.inbox_seen, seen, seen + 1) == seen) rec = seen;
+        } else if (load_acquire_sys(&p.sv.ctl->stop)) {
+          rec = -1;
+        } else if (gtimer() > deadline) {
+          raise_timeout(p, -2);
+          rec = -1;
+        }
+      }
+      rec = __shfl_sync(FULL, rec, 0);
+      if (rec == -1) return -1;
+      if (rec >= 0) {
+        serve_activate(p, rec);
         continue;
       }
     }
-    __nanosleep(200);
+    __nanosleep(watcher ? 20 : 300);
   }
 }
 
-// Warp 0, after task t finished and its writes were fenced: release the
-// successors whose last predecessor this was.
-__device__ void complete_task(const KParams& p, int t) {
+// Warp 0 pops a ready task part: the urgent queue first, then the earliest
+// bucket (queue order) with an available part. Lane 0 claims and broadcasts,
+// so the warp stays uniform. One look costs one round of loads, each lane its
+// own word: the abort flag, the urgent queue's count, lo, the first 29
+// top-level counts (the buckets' own in a plan of at most 29, else the groups'
+// or super-groups'), and the heads of the 32 buckets from lo on (to move lo).
+// Returns kMaxParts * task + part, or -1 when every part has been popped, the
+// launch was aborted, or the wait budget of this call expired (TIMEOUT;
+// checked on every pass of the loop).
+__device__ int pop_task(const KParams& p, unsigned long long deadline) {
+  if (p.serve) return serve_pop(p, deadline);
+  const unsigned FULL = 0xffffffffu;
+  constexpr int kTop = 29;
   const int lane = threadIdx.x & 31;
-  const int s0 = __ldcg(p.succ_off + t), s1 = __ldcg(p.succ_off + t + 1);
-  for (int q = s0 + lane; q < s1; q += 32) {
-    const int s = __ldcg(p.succ + q);
-    STILES_CHECK(s >= 0 && s < p.ntasks, 6, t, 0);
-    const int left = cuda::atomic_ref<int, cuda::thread_scope_device>(p.q.rem[s]).fetch_sub(1, cuda::memory_order_acq_rel);
-    if (left == 1) push_task(p, s);
+  const int nb = p.nbuckets, ngroups = (nb + 31) / 32, nsuper = (ngroups + 31) / 32;
+  const int level = nb <= kTop ? 0 : ngroups <= kTop ? 1 : 2;  // counts looked at first
+  int* const top = level == 0 ? p.q.avail : level == 1 ? p.q.gcnt : p.q.scnt;
+  const int ntop = level == 0 ? nb : level == 1 ? ngroups : nsuper;
+  const unsigned long long start = lane == 0 ? gtimer() : 0ull;
+  int l = 0;
+  for (;;) {
+    int* word = lane == 0 ? &p.st->abort : lane == 1 ? p.q.lo + 24 : lane == 2 ? p.q.lo : top + min(lane - 3, ntop - 1);
+    const bool used = lane < 3 || lane - 3 < ntop;
+    const int hb = l + lane;
+    const int v = used ? load_relaxed_flag(word) : 0;
+    const int head = hb < nb ? load_relaxed_flag(p.q.head + hb) : 0;
+    if (__shfl_sync(FULL, v, 0)) return -1;
+    if (__shfl_sync(FULL, v, 1) > 0) {  // urgent parts
+      int got = -3;
+      if (lane == 0) {
+        const int uh = claim(p.q.lo + 24, p.q.lo + 16);
+        if (uh >= p.ucap) {  // claimed past the urgent queue (checked in every build)
+          check_fail(p, 4, uh, 0);
+          got = -1;
+        } else if (uh >= 0) {
+          got = wait_slot(p, p.q.uslots + uh, start);
+        }
+      }
+      got = __shfl_sync(FULL, got, 0);
+      if (got != -3) return got;
+    }
+    int got = -3;  // -3: nothing found, -1: stop, >= 0: item
+    // claim from the ready buckets of a 32-bucket group, in order
+    auto try_buckets = [&](unsigned rm, int base) {
+      while (rm && got == -3) {
+        const int bb = base + __ffs(rm) - 1;
+        rm &= rm - 1;
+        if (lane == 0) {
+          const int h = claim(p.q.avail + bb, p.q.head + bb);
+          if (h >= 0) {
+            atomicSub(p.q.gcnt + (bb >> 5), 1);
+            atomicSub(p.q.scnt + (bb >> 10), 1);
+            const int s0 = p.soff[bb];
+            if (h >= p.soff[bb + 1] - s0) {  // claimed past the bucket (checked in every build)
+              check_fail(p, 5, bb, 0);
+              got = -1;
+            } else {
+              got = wait_slot(p, p.q.slots + s0 + h, start);
+            }
+          }
+        }
+        got = __shfl_sync(FULL, got, 0);
+      }
+    };
+    auto try_groups = [&](unsigned gm, int base) {  // groups in order, the buckets of each
+      while (gm && got == -3) {
+        const int gi = base + __ffs(gm) - 1;
+        gm &= gm - 1;
+        const int b = gi * 32 + lane;
+        try_buckets(__ballot_sync(FULL, b < nb && load_relaxed_flag(p.q.avail + b) > 0), gi * 32);
+      }
+    };
+    auto try_supers = [&](unsigned sm, int base) {  // super-groups in order, the groups of each
+      while (sm && got == -3) {
+        const int si = base + __ffs(sm) - 1;
+        sm &= sm - 1;
+        const int g = si * 32 + lane;
+        try_groups(__ballot_sync(FULL, g < ngroups && load_relaxed_flag(p.q.gcnt + g) > 0), si * 32);
+      }
+    };
+    const unsigned tm = __ballot_sync(FULL, lane >= 3 && v > 0) >> 3;
+    if (level == 0) try_buckets(tm, 0);
+    else if (level == 1) try_groups(tm, 0);
+    else try_supers(tm, 0);
+    if (level == 2)
+      for (int sbase = kTop; sbase < nsuper && got == -3; sbase += 32) {
+        const int sg = sbase + lane;
+        try_supers(__ballot_sync(FULL, sg < nsuper && load_relaxed_flag(p.q.scnt + sg) > 0), sbase);
+      }
+    if (got != -3) return got;
+    // nothing claimed: move lo past finished buckets (finished is permanent,
+    // so atomicMax is safe), stop once every part was popped, else back off
+    const bool fin = hb >= nb || head >= p.soff[hb + 1] - p.soff[hb];
+    const unsigned unf = __ballot_sync(FULL, !fin);
+    const int nfin = unf ? __ffs(unf) - 1 : 32;
+    const int seen = __shfl_sync(FULL, v, 2);
+    if (nfin > 0 && l < nb && lane == 0 && l + nfin > seen) atomicMax(p.q.lo, l + nfin);
+    const int next = max(seen, l < nb ? min(l + nfin, nb) : l);
+    if (next >= nb) {  // every bucket popped: the urgent parts too?
+      const int u = lane < 2 ? load_relaxed_flag(p.q.lo + 16 + 4 * lane) : 0;
+      if (__shfl_sync(FULL, u, 0) + __shfl_sync(FULL, u, 1) >= p.ucap) return -1;
+    }
+    int stop = 0;
+    if (lane == 0 && gtimer() - start > (unsigned long long)p.budget_ns) {
+      raise_timeout(p, (long long)seen * kTasksPerBucket);
+      stop = 1;
+    }
+    if (__shfl_sync(FULL, stop, 0)) return -1;
+    if (next != l) {
+      l = next;
+      continue;
+    }
+    idle_pause();
   }
-  if (p.serve) {  // request accounting: the last task of a request signals the host
-    __syncwarp();
-    if (lane == 0) {
-      const int slot = __ldcg(p.sv.treq + t);
-      if (atomicSub(p.sv.req_left + slot, 1) == 1) {
-        __threadfence_system();
-        store_release_sys(&p.sv.ctl->done_seq[slot], __ldcg(p.sv.req_seq + slot));
+}
+
+// Warp 0, after a part (of a task that counts parts) or the last part of a task
+// finished and its writes were fenced: count it off every successor and queue
+// those that became ready. `first` / `word`: this lane's successor (-1: none) and its
+// task word, read ahead while the part ran. Of the urgent tasks released, one
+// part is kept for this worker (a one-part task, the block POTRF, before any
+// other): it starts without a trip through the queue. Returns that part or -1.
+__device__ int release_successors(const KParams& p, const Task& tk, int first, TaskWord word) {
+  const unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  int keep = -1;
+  const int aborted = load_relaxed_flag(&p.st->abort);  // looked at below, after the counts' round trip
+  int next = 32 + lane < tk.nsucc ? __ldcg(p.succ + tk.succ0 + 32 + lane) : -1;
+  for (int q = lane; q - lane < tk.nsucc; q += 32) {
+    int s = first;
+    TaskWord tw = word;
+    if (q >= 32) {
+      s = next;
+      if (s >= 0) tw = load_task_word(p, s);  // in flight with the count below
+      next = q + 32 < tk.nsucc ? __ldcg(p.succ + tk.succ0 + q + 32) : -1;
+    }
+    STILES_CHECK(s < p.ntasks, 6, s, 0);
+    bool ready = false;
+    if (s >= 0) ready = add_relaxed_i(p.q.rem + s, -1) == 1;
+    const bool urgent = ready && (tw.flags() & TF_URGENT);
+    int q0 = 0;
+    if (keep < 0) {
+      const unsigned one = __ballot_sync(FULL, urgent && tw.parts() == 1), any = __ballot_sync(FULL, urgent);
+      const int who = one ? __ffs(one) - 1 : any ? __ffs(any) - 1 : -1;
+      if (who >= 0) {
+        keep = kMaxParts * __shfl_sync(FULL, s, who);
+        q0 = lane == who;
+        if (lane == 0 && !p.serve) atomicAdd(p.q.lo + 20, 1);
       }
     }
+    if (ready) {
+      fence_dev();
+      push_task(p, s, tw, q0);
+    }
+  }
+  __syncwarp();
+  return aborted ? -1 : keep;
+}
+
+// Lane 0 of warp 0, once a task's last part is complete in every respect:
+// count it; the last task of a served request signals the host.
+__device__ void account_task(const KParams& p, int t) {
+  atomicAdd(&p.st->done, 1ull);
+  if (!p.serve) return;
+  const int slot = __ldcg(p.sv.treq + t);
+  if (atomicSub(p.sv.req_left + slot, 1) == 1) {
+    __threadfence_system();
+    store_release_sys(&p.sv.ctl->done_seq[slot], __ldcg(p.sv.req_seq + slot));
   }
 }
 
@@ -421,40 +527,6 @@ __device__ void run_prep(const KParams& p, const Task& tk, int t) {
   for (int64_t e = threadIdx.x; e < (int64_t)a * b; e += NTHREADS) O[arrow0 + e] = __ldg(B + arrow0 + e);
 }
 
-// Sub-tile of a task's output block computed by one part (rows r0 .. r0+rm,
-// columns c0 .. c0+cn; rm or cn <= 0: nothing to do for this part).
-struct Sub {
-  int r0, c0, rm, cn;
-};
-
-__device__ __forceinline__ Sub sub_of(const Task& tk, int q) {
-  Sub sb{0, 0, tk.m, tk.n};
-  switch (tk.pmode) {
-    case PM_ROWS2: sb.r0 = 32 * q; sb.rm = min(32, tk.m - sb.r0); break;
-    case PM_ROWS4: sb.r0 = 16 * q; sb.rm = min(16, tk.m - sb.r0); break;
-    case PM_QUAD4: sb.r0 = 32 * (q & 1); sb.c0 = 32 * (q >> 1); break;
-    case PM_TRI3: sb.r0 = q == 0 ? 0 : 32; sb.c0 = q == 2 ? 32 : 0; break;
-    case PM_TILE32: {
-      const int pr = tk.m > 32 ? 2 : 1;
-      sb.r0 = 32 * (q % pr);
-      sb.c0 = 32 * (q / pr);
-      break;
-    }
-    case PM_ROWS8: sb.r0 = 8 * q; sb.rm = min(8, tk.m - sb.r0); break;
-    case PM_TRI16: sb.r0 = q == 0 ? 0 : 16; sb.c0 = q == 2 ? 16 : 0; break;
-    case PM_QUAD16: sb.r0 = 16 * (q >> 1); sb.c0 = 16 * (q & 1); break;
-    default: break;
-  }
-  if (tk.pmode == PM_QUAD4 || tk.pmode == PM_TRI3 || tk.pmode == PM_TILE32) {
-    sb.rm = min(32, tk.m - sb.r0);
-    sb.cn = min(32, tk.n - sb.c0);
-  } else if (tk.pmode == PM_TRI16 || tk.pmode == PM_QUAD16) {
-    sb.rm = min(16, tk.m - sb.r0);
-    sb.cn = min(16, tk.n - sb.c0);
-  }
-  return sb;
-}
-
 // acc[i][j] += sum over the task's segments of op(A)[r0 + tx + 16 i, :] op(B)[:, c0 + ty + 8 j]
 // with 128 threads as a 16 x 8 grid (tx = tid % 16, ty = tid / 16): a
 // (16 TM) x (8 TN) sub-tile, staged KC columns of K at a time in shared
@@ -464,6 +536,8 @@ __device__ __forceinline__ void accumulate(const KParams& p, const Task& tk, con
                                            double* As, double* Bs) {
   constexpr int RM = 16 * TM, CN = 8 * TN;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  const int ntm = (sb.rm + 15) / 16, ntn = (sb.cn + 7) / 8;
+  const bool full = ntm == TM && ntn == TN;
 #pragma unroll
   for (int i = 0; i < TM; ++i)
 #pragma unroll
@@ -520,17 +594,39 @@ __device__ __forceinline__ void accumulate(const KParams& p, const Task& tk, con
         }
       }
       __syncthreads();
-#pragma unroll 8
-      for (int kk = 0; kk < KC; ++kk) {
-        double a[TM], b[TN];
+      // (every FP64 instruction holds the pipe for 64 cycles: the rows, columns
+      // and K steps that pad a ragged part are left out)
+      if (full) {
+#pragma unroll 1
+        for (int k1 = 0; k1 < kc; k1 += 8)
 #pragma unroll
-        for (int i = 0; i < TM; ++i) a[i] = As[kk * LDS + tx + 16 * i];
+          for (int kk = k1; kk < k1 + 8; ++kk) {
+            double a[TM], b[TN];
 #pragma unroll
-        for (int j = 0; j < TN; ++j) b[j] = Bs[kk * LDS + ty + 8 * j];
+            for (int i = 0; i < TM; ++i) a[i] = As[kk * LDS + tx + 16 * i];
 #pragma unroll
-        for (int i = 0; i < TM; ++i)
+            for (int j = 0; j < TN; ++j) b[j] = Bs[kk * LDS + ty + 8 * j];
 #pragma unroll
-          for (int j = 0; j < TN; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+            for (int i = 0; i < TM; ++i)
+#pragma unroll
+              for (int j = 0; j < TN; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+          }
+      } else {
+#pragma unroll 1
+        for (int kk = 0; kk < kc; ++kk) {
+          double a[TM], b[TN];
+#pragma unroll
+          for (int i = 0; i < TM; ++i) a[i] = As[kk * LDS + tx + 16 * i];
+#pragma unroll
+          for (int j = 0; j < TN; ++j) b[j] = Bs[kk * LDS + ty + 8 * j];
+#pragma unroll
+          for (int i = 0; i < TM; ++i)
+            if (i < ntm) {
+#pragma unroll
+              for (int j = 0; j < TN; ++j)
+                if (j < ntn) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+            }
+        }
       }
       __syncthreads();
     }
@@ -1063,7 +1159,8 @@ __device__ __forceinline__ void acc_to_smem(const KParams& p, const Task& tk, co
     for (int j = 0; j < TN; ++j) {
       const int r = tx + 16 * i, c = ty + 8 * j;
       const bool in = sub_cin && r < sb.rm && c < sb.cn;
-      X[r * LDS + c] = in ? v[i][j] - acc[i][j] : sign * acc[i][j];
+      if (tk.nseg == 0) X[r * LDS + c] = v[i][j];  // no product to subtract (an FP64 instruction saved)
+      else X[r * LDS + c] = in ? v[i][j] - acc[i][j] : sign * acc[i][j];
     }
 }
 
@@ -1103,25 +1200,6 @@ __device__ __forceinline__ void store_sub(const KParams& p, const Task& tk, cons
 // FP64 runs at 1/64 of the FP32 rate on GB300, so these avoid block-wide
 // barriers in their inner loops: independent rows (or columns) are owned by
 // one warp and stepped with __syncwarp only.
-
-// X (m x n) <- X T^{-T}, T lower n x n, rcp[j*LDS] = 1 / T[j][j].
-// Rows are independent: warp w owns rows RPW w .. RPW w + RPW - 1 (RPW = 16,
-// 8 when m <= 32, 4 when m <= 16), its lanes split the columns of each step.
-__device__ __forceinline__ void trsm_rows_lt(double* X, const double* T, const double* rcp, int m, int n) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int rpw = m > 32 ? 16 : m > 16 ? 8 : 4, phases = 32 / rpw;
-  const int r = warp * rpw + lane % rpw, ph = lane / rpw;
-  const bool own = r < m;
-  for (int j = 0; j < n; ++j) {
-    if (own && ph == 0) X[r * LDS + j] *= rcp[j * LDS];
-    __syncwarp();
-    if (own) {
-      const double xj = X[r * LDS + j];
-      for (int c = j + 1 + ph; c < n; c += phases) X[r * LDS + c] -= xj * T[c * LDS + j];
-    }
-    __syncwarp();
-  }
-}
 
 // X (m x n, m <= 16) <- X T^{-T} with the row values in registers: T lower
 // n x n with its strict lower part already divided by the pivot of its column
@@ -1209,124 +1287,246 @@ __device__ __forceinline__ void trsm_cols_ln(double* X, const double* T, const d
   }
 }
 
-// Trailing rank-1 update of the block POTRF, one batch of B elements per
-// thread: element e of the packed lower triangle (width w, row pairs
-// (a, w-1-a) of w+1 elements) maps to X[c0+a][c0+b] and is updated by column
-// k. fetch() loads a batch (indices past ne are marked -1) and advances the
-// (i, kk) walk; apply() writes it.
-struct Rank1Walk {
-  int c0, w, w1, k, ne, nt, di, dk, i, kk;
-};
-template <int B>
-__device__ __forceinline__ void rank1_fetch(const double* X, Rank1Walk& s, int e, int (&id)[B], double (&xr)[B],
-                                            double (&lr)[B], double (&lc)[B]) {
-#pragma unroll
-  for (int u = 0; u < B; ++u) {
-    const int a = s.kk <= s.i ? s.i : s.w - 1 - s.i, b = s.kk <= s.i ? s.kk : s.kk - s.i - 1;
-    id[u] = e + u * s.nt < s.ne ? (s.c0 + a) * LDS + s.c0 + b : -1;
-    if (id[u] >= 0) {
-      xr[u] = X[id[u]];
-      lr[u] = X[(s.c0 + a) * LDS + s.k];
-      lc[u] = X[(s.c0 + b) * LDS + s.k];
-    }
-    s.kk += s.dk;
-    s.i += s.di;
-    if (s.kk >= s.w1) {
-      s.kk -= s.w1;
-      ++s.i;
-    }
+// ---- block POTRF ---------------------------------------------------------
+// In-place lower Cholesky of the n x n block X (n <= FB, padded with the
+// identity to a multiple of 4) in panels of 4 columns, as L = M D^1/2: a pivot
+// d_j gives the multipliers m_ij = a_ij / d_j, the later columns take
+// a_ik -= m_ij a_kj, and the columns are scaled by d_j^-1/2 only when they are
+// stored. What bounds it: an FP64 warp instruction holds its sub-partition's
+// pipe for 64 cycles whatever its active lanes, so the pivot chain is counted
+// in the FP64 instructions of the warp that runs it, and the trailing update
+// (43.7k multiply-adds: 22k cycles over the four pipes) in packed elements.
+// Hence
+//   * 1 / d is formed in integers (recip_fixed, ~145 cycles, an rsqrt takes
+//     380), beside the FP64 pipe; a pivot then costs a multiply and a
+//     multiply-add on the chain;
+//   * a panel runs in registers, a row per lane (its 4 pivot rows in lanes
+//     0-3 of every warp that takes part, so no warp waits for another); four
+//     columns keep the multiply-adds inside the panel (6) off the chain, eight
+//     (28) took 2.5 times as long per panel;
+//   * the trailing update takes a panel at a time; the next panel's columns
+//     first, so that the next panel runs while the other warps, and then its
+//     own, apply the rest (batches of 32 2 x 2 elements of the packed lower
+//     triangle, shared out by their FP64 time; single elements claimed from a
+//     counter, their rows found by a division, took three times as long).
+
+constexpr int PNB = 4;           // panel width
+constexpr int PROWS = 32 - PNB;  // rows below the panel's own per warp
+constexpr int PMS = PNB + 1;     // row length of a multiplier buffer
+// shared memory beside X (doubles from the start of the dynamic region)
+constexpr int PT_M = 0;                       // two multiplier buffers, FB x PMS
+constexpr int PT_PIV = PT_M + 2 * FB * PMS;   // pivots d_j
+constexpr int PT_RS = PT_PIV + FB;            // scale of column j
+constexpr int PT_DIAG = PT_RS + FB;           // L_jj
+static_assert(PT_DIAG + FB <= 2 * KC * LDS, "fits in the staging region");
+// a panel's time in batches of the trailing update (16 multiply-adds of 64 cycles)
+constexpr int PBATCH = 1;
+
+// ceil(2^20 / w): e / w = (e * kInv20[w]) >> 20 for the e < 1600 walked here
+struct Inv20 {
+  uint32_t v[FB + 1];
+  constexpr Inv20() : v{} {
+    for (int w = 1; w <= FB; ++w) v[w] = ((1u << 20) + w - 1) / w;
   }
-}
-template <int B>
-__device__ __forceinline__ void rank1_apply(double* X, const int (&id)[B], const double (&xr)[B],
-                                            const double (&lr)[B], const double (&lc)[B]) {
-#pragma unroll
-  for (int u = 0; u < B; ++u)
-    if (id[u] >= 0) X[id[u]] = fma(-lr[u], lc[u], xr[u]);
+};
+__constant__ const Inv20 kInv20{};
+
+// 1 / |d| of a normal d with biased exponent in [1, 2043], correctly rounded
+// but for rare cases (error below 0.51 ulp). Newton's iteration in fixed point
+// from a single-precision estimate q / 2^24 of 1 / m, d = m 2^e, m in [1, 2):
+// with M = 2^52 m the residual e1 = 1 - m q / 2^24 = (2^76 - M q) / 2^76 is
+// below 2^-21 and exact in 64 bits; 1 / m = q / 2^24 (1 + e1 + e1^2) to 2^-63.
+__device__ __forceinline__ double recip_fixed(double d) {
+  const unsigned long long bits = (unsigned long long)__double_as_longlong(d);
+  const int e = (int)((bits >> 52) & 0x7ff);
+  const unsigned long long M = (bits & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+  const float f = __uint_as_float(0x3f800000u | (uint32_t)((bits >> 29) & 0x7fffffu));
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(f));
+  r = fminf(r, 0.99999994f);  // below 1, so that its exponent is that of [1/2, 1)
+  const uint32_t q = (__float_as_uint(r) & 0x7fffffu) | 0x800000u;
+  const long long E = (long long)(0ull - M * (unsigned long long)q);
+  const int Eh = (int)(E >> 24);
+  const long long S = E + (((long long)Eh * Eh) >> 28);
+  const long long Y = ((long long)q << 39) + (((S >> 16) * (long long)q) >> 21);
+  return __longlong_as_double(((long long)(2044 - e) << 52) + ((Y + 512) >> 10));
 }
 
-// In-place lower Cholesky of the n x n block X (n <= FB), one column per
-// step with a two-column lookahead, so that a step has one block barrier:
-//   warp 0, step j: pivot d = X[j][j], r = rsqrt(d) (one dependent FP64
-//     chain instead of sqrt then a divide), column j scaled by r, then
-//     column j+1 updated by columns j-1 and j (it is pivot j+1 next); the
-//     column j-1 term does not depend on r and is applied while r is formed,
-//     lane 0's scaled row j+1 is broadcast by a shuffle;
-//   warps 1-3, step j: columns j+2 .. n-1 (lower part) updated by column j-1,
-//     walking the lower triangle of width w as w/2 row pairs (a, w-1-a) of
-//     w+1 elements each (no lane idles), in batches of six.
-// Every column thus receives the updates of the columns before it in
-// ascending order, and only warp 0's pivot chain is on the critical path.
-// X[j][j] keeps the pivot d until the end (nothing reads it after step j);
-// r is kept in the row's padding slot X[j][FB], and L_jj = d r and the pivot
-// check are done for all columns at once after the loop.
-// Returns the first column (0-based) whose pivot was not positive, or -1.
-__device__ int potrf_smem(double* X, int n) {
-  static_assert(FB <= 64 && LDS > FB, "two rows per lane of warp 0; a padding column per row");
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  __shared__ int s_bad;
-  if (tid == 0) s_bad = n;
-  for (int j = 0; j < n; ++j) {
-    if (warp == 0) {
-      const int j1 = j + 1;
-      const double d = X[j * LDS + j];
-      const double l0 = j > 0 && j1 < n ? X[j1 * LDS + j - 1] : 0.0;
-      double xj[2] = {0.0, 0.0}, x1[2] = {0.0, 0.0}, lj[2] = {0.0, 0.0};
+__device__ __forceinline__ bool recip_range(double d) {  // recip_fixed's range
+  const unsigned e = (unsigned)((__double_as_longlong(d) >> 52) & 0x7ff);
+  return e - 1u <= 2042u;
+}
+
+// Panel j0 .. j0 + 3 in registers: lanes 0-3 hold the panel's own rows, the
+// others rows j0 + 28 cw + lane of warp cw. Writes the (unscaled) panel columns
+// back to X, the multipliers to M and the pivots. A pivot whose reciprocal
+// leaves the normal range (zero, subnormal, above 2^1020, not finite) has its
+// column scaled by d^-1/2 at once (m = l), and a 1 left in its scale slot: the
+// panel is then done again that way, from the columns still in X.
+__device__ __forceinline__ void potrf_panel(double* X, double* M, double* piv, double* rs, int j0, int n, int cw) {
+  const unsigned FULL = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  const int row = j0 + (lane < PNB ? lane : PROWS * cw + lane);
+  const bool own = row < n;
+  double a[PNB], m[PNB], d[PNB], fin[PNB];
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const int r = j1 + lane + 32 * u;
-        if (r < n) {
-          xj[u] = X[r * LDS + j];
-          x1[u] = X[r * LDS + j1];
-          if (j > 0) x1[u] = fma(-X[r * LDS + j - 1], l0, x1[u]);
-        }
-      }
-      const double rr = rsqrt(d);
-      if (lane == 0) X[j * LDS + FB] = rr;
+  for (int k = 0; k < PNB; ++k) a[k] = own ? X[row * LDS + j0 + k] : 0.0;
+  bool range = true;
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const int r = j1 + lane + 32 * u;
-        if (r < n) {
-          lj[u] = xj[u] * rr;
-          X[r * LDS + j] = lj[u];
-        }
-      }
-      const double l1 = __shfl_sync(0xffffffffu, lj[0], 0);  // L[j+1][j], row j+1 is lane 0's
+  for (int j = 0; j < PNB; ++j) {
+    fin[j] = 0.0;
+    d[j] = __shfl_sync(FULL, a[j], j);
+    double u[PNB];
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        const int r = j1 + lane + 32 * u;
-        if (r < n) X[r * LDS + j1] = fma(-lj[u], l1, x1[u]);
-      }
-    } else if (j > 0 && j + 2 < n) {
-      Rank1Walk s;
-      s.c0 = j + 2;
-      s.w = n - s.c0;
-      s.w1 = s.w + 1;
-      s.k = j - 1;
-      s.ne = s.w * s.w1 / 2;
-      s.nt = NTHREADS - 32;
-      s.di = s.nt / s.w1;
-      s.dk = s.nt % s.w1;
-      const int t = tid - 32;
-      s.i = t / s.w1;
-      s.kk = t % s.w1;
-      constexpr int B = 6;  // elements per batch: their loads are issued before their stores
-      int id[B];
-      double xr[B], lr[B], lc[B];
-      for (int e = t; e < s.ne; e += B * s.nt) {
-        rank1_fetch<B>(X, s, e, id, xr, lr, lc);
-        rank1_apply<B>(X, id, xr, lr, lc);
+    for (int k = j + 1; k < PNB; ++k) u[k] = __shfl_sync(FULL, a[j], k);
+    m[j] = a[j] * recip_fixed(d[j]);
+    range = range && recip_range(d[j]);
+#pragma unroll
+    for (int k = j + 1; k < PNB; ++k) a[k] = fma(-m[j], u[k], a[k]);
+  }
+  if (!range) {
+#pragma unroll
+    for (int k = 0; k < PNB; ++k) a[k] = own ? X[row * LDS + j0 + k] : 0.0;
+#pragma unroll
+    for (int j = 0; j < PNB; ++j) {
+      d[j] = __shfl_sync(FULL, a[j], j);
+      const bool in = recip_range(d[j]);
+      fin[j] = in ? 0.0 : 1.0;
+      if (!in) a[j] *= rsqrt(d[j]);
+      m[j] = in ? a[j] * recip_fixed(d[j]) : a[j];
+#pragma unroll
+      for (int k = j + 1; k < PNB; ++k) a[k] = fma(-m[j], __shfl_sync(FULL, a[j], k), a[k]);
+    }
+  }
+  if (own && lane >= PNB) {
+#pragma unroll
+    for (int k = 0; k < PNB; ++k) {
+      M[row * PMS + k] = m[k];
+      X[row * LDS + j0 + k] = a[k];
+    }
+  } else if (cw == 0 && lane < PNB) {
+#pragma unroll
+    for (int k = 0; k < PNB; ++k)
+      if (k <= lane) X[row * LDS + j0 + k] = a[k];
+    if (lane == 0) {
+#pragma unroll
+      for (int k = 0; k < PNB; ++k) {
+        piv[j0 + k] = d[k];
+        rs[j0 + k] = fin[k];
       }
     }
-    __syncthreads();
   }
-  if (tid < n) {
-    const double d = X[tid * LDS + tid];
-    if (!(d > 0.0)) atomicMin(&s_bad, tid);
-    X[tid * LDS + tid] = d * X[tid * LDS + FB];
+}
+
+// 2 x TC elements (rows r, r + 1; columns c ..) of a trailing update by the
+// panel at j0: X[r][c] -= sum_k M[r][k] X[c][j0 + k]. Elements above the
+// diagonal are computed and not stored.
+template <int TC>
+__device__ __forceinline__ void potrf_update(double* X, const double* M, int j0, int r, int c) {
+  double x[2][TC], m[2][PNB], u[TC][PNB];
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+#pragma unroll
+    for (int t = 0; t < TC; ++t) x[i][t] = X[(r + i) * LDS + c + t];
+#pragma unroll
+    for (int k = 0; k < PNB; ++k) m[i][k] = M[(r + i) * PMS + k];
+  }
+#pragma unroll
+  for (int t = 0; t < TC; ++t)
+#pragma unroll
+    for (int k = 0; k < PNB; ++k) u[t][k] = X[(c + t) * LDS + j0 + k];
+#pragma unroll
+  for (int k = 0; k < PNB; ++k)
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+      for (int t = 0; t < TC; ++t) x[i][t] = fma(-m[i][k], u[t][k], x[i][t]);
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int t = 0; t < TC; ++t)
+      if (r + i >= c + t) X[(r + i) * LDS + c + t] = x[i][t];
+}
+
+// The factorization of X; `S` is the staging region. On return (after a block
+// barrier) L = X diag(scale): column j times S[PT_RS + j], whose diagonal
+// entry is S[PT_DIAG + j].
+__device__ void potrf_smem(double* X, double* S, int n) {
+  static_assert(FB % PNB == 0 && FB - PNB <= 3 * PROWS, "panels; three warps hold a panel's rows");
+  static_assert(FB * PNB <= 2 * NTHREADS, "a panel's columns are two elements per thread");
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  double *piv = S + PT_PIV, *rs = S + PT_RS;
+  const int np = (n + PNB - 1) / PNB * PNB;
+  for (int e = tid; e < (np - n) * np; e += NTHREADS) {  // identity rows up to a whole panel
+    const int r = n + e / np, c = e % np;
+    X[r * LDS + c] = r == c ? 1.0 : 0.0;
   }
   __syncthreads();
-  return s_bad < n ? s_bad : -1;
+  if (warp == 0 || (warp < 3 && PNB + PROWS * warp < np)) potrf_panel(X, S + PT_M, piv, rs, 0, np, warp);
+  for (int j0 = 0; j0 + PNB < np; j0 += PNB) {
+    const int j1 = j0 + PNB, j2 = j1 + PNB, pb = j0 / PNB;
+    const double* M = S + PT_M + (pb & 1) * FB * PMS;
+    double* Mn = S + PT_M + ((pb & 1) ^ 1) * FB * PMS;
+    __syncthreads();
+    {  // the next panel's columns
+      const int r = j1 + 2 * (tid / PNB), c = j1 + tid % PNB;
+      if (r < np && r + 1 >= c) potrf_update<1>(X, M, j0, r, c);
+    }
+    __syncthreads();
+    // warps 0 .. npw - 1 hold the panel's rows
+    const int npw = 1 + (j1 + PNB + PROWS < np) + (j1 + PNB + 2 * PROWS < np);
+    if (warp < npw) potrf_panel(X, Mn, piv, rs, j1, np, warp);
+    // columns j2 .. np - 1: the lower triangle in 2 x 2 elements, h of them
+    // wide (even), line a (a + 1 of them) folded with line h - 1 - a; every
+    // warp gets the same time, the panel's warps less by the panel
+    const int h = (np - j2) / 2, w1 = h + 1, ne = h / 2 * w1, nbatch = (ne + 31) / 32;
+    const int mine = max(0, (nbatch + PBATCH * npw) / 4 - PBATCH), others = nbatch - npw * mine;
+    const int each = npw == 1 ? (others + 2) / 3 : npw == 2 ? (others + 1) / 2 : others;
+    int b = warp < npw ? others + mine * warp : each * (warp - npw);
+    const int b1 = warp < npw ? b + mine : min(others, b + each);
+    const uint32_t inv = kInv20.v[w1];
+#pragma unroll 1
+    for (; b < b1; ++b) {
+      const int e = 32 * b + lane, i = (int)((e * inv) >> 20), kk = e - i * w1;
+      const bool low = kk <= i;
+      const int r = j2 + 2 * (low ? i : h - 1 - i), c = j2 + 2 * (low ? kk : kk - i - 1);
+      if (e < ne) potrf_update<2>(X, M, j0, r, c);
+    }
+  }
+  __syncthreads();
+  if (tid < n) {
+    const double d = piv[tid];
+    const double r = rsqrt(d);
+    S[PT_DIAG + tid] = d * r;
+    rs[tid] = rs[tid] == 0.0 ? r : 1.0;
+  }
+  __syncthreads();
+}
+
+// After a block POTRF has released its successors: its log-diagonal partial
+// sum (in a fixed tree order) and its first pivot that is not positive.
+__device__ void finish_potrf(const KParams& p, const Task& tk, const double* S) {
+  const int tid = threadIdx.x;
+  __shared__ double s_lg[2];
+  __shared__ int s_bad;
+  if (tid == 0) s_bad = FB;
+  __syncthreads();
+  if (tid < FB) {
+    double lg = tid < tk.n ? log(S[PT_DIAG + tid]) : 0.0;
+    if (tid < tk.n && !(S[PT_PIV + tid] > 0.0)) atomicMin(&s_bad, tid);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) lg += __shfl_down_sync(0xffffffffu, lg, o);
+    if ((tid & 31) == 0) s_lg[tid >> 5] = lg;
+  }
+  __syncthreads();
+  if (tid == 0) {
+    p.logdet_part[tk.diag] = s_lg[0] + s_lg[1];
+    if (s_bad < FB) {
+      atomicCAS(&p.st->code, 0, STILES_DEV_NOT_SPD);
+      atomicMin(&p.st->spd_col, (unsigned long long)tk.gcol + (unsigned long long)s_bad);
+      if (p.badpiv) p.badpiv[tk.diag] = s_bad;
+    }
+  }
 }
 
 template <bool TC, int TM, int TN>
@@ -1416,16 +1616,13 @@ __device__ void run_sub(const KParams& p, const Task& tk, const Sub& sb, double*
       double* rcp = T + FB;  // column FB of T's padded rows is free: rcp[j * LDS]
       if (tid < n) rcp[tid * LDS] = 1.0 / T[tid * LDS + tid];
       __syncthreads();
-      if (sb.rm <= 16) {  // every part of a row-split block
-        const int warp = tid >> 5, lane = tid & 31;
-        for (int c = warp + 1; c < n; c += NTHREADS / 32)
-          for (int j = lane; j < c; j += 32) T[c * LDS + j] *= rcp[j * LDS];
-        __syncthreads();
-        if (sb.rm <= 8) trsm_rows_lt8(X, T, rcp, sb.rm, n);
-        else trsm_rows_lt16(X, T, rcp, sb.rm, n);
-      } else {
-        trsm_rows_lt(X, T, rcp, sb.rm, n);
-      }
+      // (parts have at most 16 rows; the strict lower part divided by its pivots)
+      const int warp = tid >> 5, lane = tid & 31;
+      for (int c = warp + 1; c < n; c += NTHREADS / 32)
+        for (int j = lane; j < c; j += 32) T[c * LDS + j] *= rcp[j * LDS];
+      __syncthreads();
+      if (sb.rm <= 8) trsm_rows_lt8(X, T, rcp, sb.rm, n);
+      else trsm_rows_lt16(X, T, rcp, sb.rm, n);
       __syncthreads();
       store_sub(p, tk, sb, X, false);
       break;
@@ -1434,24 +1631,15 @@ __device__ void run_sub(const KParams& p, const Task& tk, const Sub& sb, double*
       if constexpr (TM == 4 && TN == 8) {
         switch (tk.op) {
           case OP_POTRF: {
+            // (finish_potrf does the rest, once the successors are released)
             acc_to_smem<TM, TN>(p, tk, sb, acc, X, true, 1.0);
             __syncthreads();
-            const int bad = potrf_smem(X, n);
-            store_sub(p, tk, sb, X, true);
-            // log of the pivots, summed in a fixed tree order
-            double lg = tid < n ? log(X[tid * LDS + tid]) : 0.0;
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) lg += __shfl_down_sync(0xffffffffu, lg, o);
-            __shared__ double s_lg[NTHREADS / 32];
-            if ((tid & 31) == 0) s_lg[tid >> 5] = lg;
-            __syncthreads();
-            if (tid == 0) {
-              p.logdet_part[tk.diag] = (s_lg[0] + s_lg[1]) + (s_lg[2] + s_lg[3]);
-              if (bad >= 0) {
-                atomicCAS(&p.st->code, 0, STILES_DEV_NOT_SPD);
-                atomicMin(&p.st->spd_col, (unsigned long long)tk.gcol + (unsigned long long)bad);
-                if (p.badpiv) p.badpiv[tk.diag] = bad;
-              }
+            potrf_smem(X, smem, n);
+            double* O = resolve(p, tk.out);
+            for (int e = tid; e < FB * FB; e += NTHREADS) {
+              const int r = e % FB, c = e / FB;
+              if (r < n && c < n)
+                O[r + (int64_t)c * tk.ldo] = r < c ? 0.0 : r == c ? smem[PT_DIAG + c] : X[r * LDS + c] * smem[PT_RS + c];
             }
             break;
           }
@@ -1548,7 +1736,7 @@ __device__ void run_task(const KParams& p, const Task& tk, int t, int q, double*
     return;
   }
   if (tk.op == OP_JOIN) return;  // a dependency point only
-  const Sub sb = sub_of(tk, q);
+  const Sub sb = part_sub(tk.pmode, tk.m, tk.n, q);
   if (sb.rm <= 0 || sb.cn <= 0) return;
 #ifdef STILES_CHECKED
   if (!task_part_ok(p, tk, sb)) {
@@ -1561,7 +1749,7 @@ __device__ void run_task(const KParams& p, const Task& tk, int t, int q, double*
     case PM_ROWS4:
     case PM_ROWS8: run_sub<TC, 1, 8>(p, tk, sb, smem, ts); break;
     case PM_TRI16:
-    case PM_QUAD16: run_sub<TC, 1, 2>(p, tk, sb, smem, ts); break;
+    case PM_GRID16: run_sub<TC, 1, 2>(p, tk, sb, smem, ts); break;
     case PM_QUAD4:
     case PM_TRI3:
     case PM_TILE32: run_sub<TC, 2, 4>(p, tk, sb, smem, ts); break;
@@ -1592,7 +1780,7 @@ __device__ __forceinline__ TcShared* tc_shared() {
 template <bool TC>
 __global__ void __launch_bounds__(NTHREADS, 2) persistent_kernel(KParams p) {
   extern __shared__ __align__(16) double smem[];
-  __shared__ int s_item, s_last;
+  __shared__ int s_item;
   TcShared* ts = tc_shared<TC>();
   // plans with reduced-precision products hold TC_COLS TMEM columns and two
   // completion barriers for the kernel's lifetime (two CTAs per SM: 512)
@@ -1610,17 +1798,18 @@ __global__ void __launch_bounds__(NTHREADS, 2) persistent_kernel(KParams p) {
   }
   // request server: idle workers give up this long after the kernel started
   const unsigned long long deadline = p.serve ? gtimer() + p.sv.deadline : 0ull;
+  int kept = -1;  // warp 0: a part released to this worker by its last task
   for (;;) {
     unsigned long long t_claim = 0;
     if (threadIdx.x < 32) {
       if (p.trace && threadIdx.x == 0) t_claim = gtimer();
-      const int v = pop_task(p, deadline);
+      const int v = kept >= 0 ? kept : pop_task(p, deadline);
       if (threadIdx.x == 0) s_item = v;
     }
     __syncthreads();
     const int v = s_item;
     if (v < 0) break;
-    const int t = v >> 2, q = v & 3;
+    const int t = v / kMaxParts, q = v % kMaxParts;
 #ifdef STILES_CHECKED
     if (t >= p.ntasks || q >= load_task(p, t).parts) {
       if (threadIdx.x == 0) check_fail(p, 8, t, q);
@@ -1629,29 +1818,41 @@ __global__ void __launch_bounds__(NTHREADS, 2) persistent_kernel(KParams p) {
 #endif
     unsigned long long t_ready = 0;
     if (p.trace && threadIdx.x == 0) t_ready = gtimer();
-    __threadfence();
     const Task tk = load_task(p, t);
+    // the first 32 successors, read ahead (in flight while the part runs)
+    int succ = -1;
+    if (threadIdx.x < 32 && (int)threadIdx.x < tk.nsucc) succ = __ldcg(p.succ + tk.succ0 + threadIdx.x);
     run_task<TC>(p, tk, t, q, smem, ts);
-    __threadfence();
+    TaskWord word{0u};
+    if (threadIdx.x < 32 && succ >= 0) word = load_task_word(p, succ);
     __syncthreads();
+    int last = tk.parts <= 1;
     if (threadIdx.x < 32) {
-      if (threadIdx.x == 0) {
-        s_last = tk.parts <= 1 ||
-                 cuda::atomic_ref<int, cuda::thread_scope_device>(p.q.pdone[t]).fetch_add(1, cuda::memory_order_acq_rel) ==
-                     tk.parts - 1;
+      fence_dev();
+      const bool by_part = counts_parts(tk);
+      if (!by_part && !last) {
+        if (threadIdx.x == 0) last = add_relaxed_i(p.q.pdone + t, 1) == tk.parts - 1;
+        last = __shfl_sync(0xffffffffu, last, 0);
+        if (last) fence_dev();
       }
-      __syncwarp();
-      if (s_last) {
-        complete_task(p, t);
-        if (threadIdx.x == 0) atomicAdd(&p.st->done, 1ull);
+      kept = -1;
+      if (by_part || last) kept = release_successors(p, tk, succ, word);
+      if (by_part && !last && threadIdx.x == 0) {
+        last = add_relaxed_i(p.q.pdone + t, 1) == tk.parts - 1;
+        if (last) fence_dev();
       }
-      if (p.trace && threadIdx.x == 0) {  // one record per task part
-        unsigned long long* tr = p.trace + 4 * (4 * (size_t)t + q);
+    }
+    if (tk.op == OP_POTRF) finish_potrf(p, tk, smem);  // what no successor waits for
+    if (threadIdx.x == 0) {
+      if (tk.op == OP_POTRF) fence_dev();
+      if (last) account_task(p, t);
+      if (p.trace) {  // one record per task part (parts 4 apart share one)
+        unsigned long long* tr = p.trace + 4 * (4 * (size_t)t + (q & 3));
         tr[0] = t_claim;
         tr[1] = t_ready;
         tr[2] = gtimer();
         tr[3] = ((unsigned long long)smid() << 32) | ((unsigned long long)blockIdx.x << 12) |
-                ((unsigned long long)tk.prec << 10) | ((unsigned long long)s_last << 9) |
+                ((unsigned long long)tk.prec << 10) | ((unsigned long long)last << 9) |
                 ((unsigned long long)(tk.flags & TF_URGENT) << 7) | tk.op;
       }
     }

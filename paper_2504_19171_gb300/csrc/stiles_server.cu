@@ -124,7 +124,7 @@ struct stiles_server {
   double* data = nullptr;
   int64_t data_doubles = 0;
   Task* tasks = nullptr;
-  int32_t *succ_off = nullptr, *rem = nullptr, *pdone = nullptr, *treq = nullptr;
+  int32_t *rem = nullptr, *pdone = nullptr, *treq = nullptr;
   int64_t task_cap = 0;
   Seg* segs = nullptr;
   int64_t seg_cap = 0;
@@ -164,7 +164,6 @@ static void free_server(stiles_server* h) {
   cudaFree(h->base);
   cudaFree(h->data);
   cudaFree(h->tasks);
-  cudaFree(h->succ_off);
   cudaFree(h->rem);
   cudaFree(h->pdone);
   cudaFree(h->treq);
@@ -199,7 +198,7 @@ extern "C" int stiles_server_create(int nshapes, const int* nt, const int* b, co
   if (!h) return STILES_ERR_OOM;
   h->prec = precision;
   h->max_req = max_requests;
-  int64_t max_tasks = 0, max_segs = 0, max_succ = 0, max_diag = 0, max_roots = 0;
+  int64_t max_tasks = 0, max_segs = 0, max_succ = 0, max_diag = 0, max_roots = 0, max_parts = 0;
   for (int m = 0; m < nshapes; ++m) {
     const int tune = tuning ? tuning[m] : 0;
     if (nt[m] < 1 || b[m] < 1 || band[m] < 0 || arrow[m] < 0 || !tune_valid(tune)) {
@@ -215,8 +214,12 @@ extern "C" int stiles_server_create(int nshapes, const int* nt, const int* b, co
     }
     T.doubles = Layout(T.s).doubles();
     T.n = (int64_t)nt[m] * b[m] + arrow[m];
-    for (size_t t = 0; t < T.plan.tasks.size(); ++t)
+    int64_t parts = 0;
+    for (size_t t = 0; t < T.plan.tasks.size(); ++t) {
       if (T.plan.indeg[t] == 0) T.roots.push_back((int32_t)t);
+      parts += T.plan.tasks[t].parts;
+    }
+    max_parts = std::max(max_parts, parts);
     T.base_off = h->base_doubles;
     h->base_doubles += (T.doubles + 2 * T.n + 31) / 32 * 32;
     max_tasks = std::max<int64_t>(max_tasks, (int64_t)T.plan.tasks.size() + 1);
@@ -234,20 +237,19 @@ extern "C" int stiles_server_create(int nshapes, const int* nt, const int* b, co
   h->grid = h->sms * kCtasPerSm;
   // table arenas: room for max_requests of the largest shape, capped by 4 of them at least
   const int64_t k = std::max(4, max_requests);
-  h->task_cap = std::min<int64_t>(k * max_tasks, (int64_t)1 << 28);
+  h->task_cap = std::min<int64_t>(k * max_tasks, kMaxTasks);
   h->seg_cap = k * std::max<int64_t>(max_segs, 1);
   h->succ_cap = k * std::max<int64_t>(max_succ, 1);
   h->diag_cap = k * std::max<int64_t>(max_diag, 1);
   h->root_cap = k * std::max<int64_t>(max_roots, 1);
   h->data_doubles = (int64_t)(data_bytes / sizeof(double));
   unsigned ring = 1;
-  while ((int64_t)ring < 4 * h->task_cap && ring < (1u << 30)) ring <<= 1;
+  while ((int64_t)ring < k * max_parts && ring < (1u << 30)) ring <<= 1;
   h->ring_mask = ring - 1;
   int rc = 0;
   if (!rc) rc = dmalloc(&h->base, h->base_doubles);
   if (!rc) rc = dmalloc(&h->data, h->data_doubles);
   if (!rc) rc = dmalloc(&h->tasks, h->task_cap);
-  if (!rc) rc = dmalloc(&h->succ_off, h->task_cap);
   if (!rc) rc = dmalloc(&h->rem, h->task_cap);
   if (!rc) rc = dmalloc(&h->pdone, h->task_cap);
   if (!rc) rc = dmalloc(&h->treq, h->task_cap);
@@ -333,7 +335,6 @@ extern "C" int stiles_server_start(stiles_server_t h, double window_s) {
   h->posted = 0;
   KParams p{};
   p.tasks = h->tasks;
-  p.succ_off = h->succ_off;
   p.succ = h->succ;
   p.segs = h->segs;
   p.ntasks = (int)h->task_cap;
@@ -440,8 +441,6 @@ static int submit_impl(stiles_server_t h, int shape, double tau, double rho, con
   st += sizeof(Task) * n;
   Seg* sg = (Seg*)st;
   st += sizeof(Seg) * R.ng;
-  int32_t* so = (int32_t*)st;
-  st += sizeof(int32_t) * (n + 1);
   int32_t* sc = (int32_t*)st;
   st += sizeof(int32_t) * R.ns;
   int32_t* rm = (int32_t*)st;
@@ -480,12 +479,11 @@ static int submit_impl(stiles_server_t h, int shape, double tau, double rho, con
       if (x.diag >= 0) x.diag += (int32_t)R.d0;
     }
     x.seg0 += (int32_t)R.g0;
+    x.succ0 += (int32_t)R.s0;
     tk[t] = x;
-    so[t] = P.succ_off[t] + (int32_t)R.s0;
-    rm[t] = P.indeg[t];
+    rm[t] = P.rem0[t];
     tq[t] = slot;
   }
-  so[n] = P.succ_off[n] + (int32_t)R.s0;
   for (int64_t g = 0; g < R.ng; ++g) {
     Seg x = P.segs[g];
     auto fix = [&](int64_t ref) {
@@ -507,7 +505,6 @@ static int submit_impl(stiles_server_t h, int shape, double tau, double rho, con
   bool cok = cudaSetDevice(h->device) == cudaSuccess;
   cok = cok && cudaMemcpyAsync(h->tasks + R.t0, tk, sizeof(Task) * n, cudaMemcpyHostToDevice, cs) == cudaSuccess;
   if (R.ng) cok = cok && cudaMemcpyAsync(h->segs + R.g0, sg, sizeof(Seg) * R.ng, cudaMemcpyHostToDevice, cs) == cudaSuccess;
-  cok = cok && cudaMemcpyAsync(h->succ_off + R.t0, so, sizeof(int32_t) * (n + 1), cudaMemcpyHostToDevice, cs) == cudaSuccess;
   if (R.ns) cok = cok && cudaMemcpyAsync(h->succ + R.s0, sc, sizeof(int32_t) * R.ns, cudaMemcpyHostToDevice, cs) == cudaSuccess;
   cok = cok && cudaMemcpyAsync(h->rem + R.t0, rm, sizeof(int32_t) * n, cudaMemcpyHostToDevice, cs) == cudaSuccess;
   // copy-engine transfers only: a memset may run as a kernel, which would
