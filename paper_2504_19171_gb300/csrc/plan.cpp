@@ -1,6 +1,6 @@
 // Host planner: expands the tile DAG of the tiled Cholesky and of the
 // two-phase selected inversion into fine-block tasks, then orders them by a
-// critical-path-first list schedule.
+// critical-path-first order.
 //
 // Tile-level method (sTiles selected inversion, arXiv 2504.19171):
 //   factor  (Sec. III)       for k: L_kk = POTRF(A_kk); L_ik = A_ik L_kk^{-T};
@@ -37,12 +37,13 @@
 namespace stiles {
 namespace {
 
-// Cost model for the list schedule: one SM of a GB300 at about 1.9 GHz with
+// Cost model for that order: one SM of a GB300 at about 1.9 GHz with
 // 2 FP64 FMA per clock does ~7.6 flop/ns, shared by the kCtasPerSm workers
 // that run on it; plus a per-task overhead.
 constexpr double kFlopPerNs = 7.6 / kCtasPerSm;
 constexpr double kTaskOverheadNs = 2500.0;
 constexpr int kGpuSms = 152;  // of a GB300
+constexpr int kPlanesMinB = 128;
 constexpr double kSweepStepNs = 120.0;  // one step of an in-shared-memory triangular sweep
 
 struct Builder {
@@ -87,6 +88,7 @@ struct Builder {
     if (t.pmode == PM_TRI16) f *= 0.625;
     if (t.prec == PREC_EMU64) f /= 10.0;   // order of the emulated-FP64 speed-up per block
     if (t.prec == PREC_FP32X) f /= 25.0;
+    if (t.flags & TF_PLANES) f /= 4.0;
     int id = (int)tasks.size();
     tasks.push_back(t);
     // parts run side by side on different CTAs
@@ -167,23 +169,12 @@ struct Builder {
     else if (mode == 1) split(t, PM_ROWS2);
   }
 
-  // Mark a bulk product task with the plan's reduced precision. The tensor-
-  // core digit products work on sub-tiles of at most 32 x 32 (four digit
-  // planes of 32 rows fill the 128 rows of one MMA): blocks that are not
-  // already split that way run as a grid of such tiles.
+  // Mark a bulk product task with the plan's reduced precision: parts of 64 x 32.
   void lower_precision(Task& t) const {
     if (s.prec == PREC_FP64) return;
     t.prec = (uint8_t)s.prec;
-    if (t.pmode == PM_TRI16) {  // its FP64 parts are smaller
-      t.pmode = PM_FULL;
-      t.parts = 1;
-      split(t, PM_TRI3);
-    }
-    if (t.pmode != PM_QUAD4 && t.pmode != PM_TRI3) {
-      const int pr = t.m > 32 ? 2 : 1, pc = t.n > 32 ? 2 : 1;
-      t.pmode = PM_TILE32;
-      t.parts = (uint8_t)(pr * pc);
-    }
+    t.pmode = PM_COLS2;
+    t.parts = t.n > 32 ? 2 : 1;
   }
 
   static Seg seg(int64_t a, int lda, int64_t b, int ldb, int k, bool ta, bool tb) {
@@ -318,7 +309,7 @@ struct Builder {
     // the TRSMs of the kUrgentReach blocks below a diagonal block, and the
     // updates from block column c into blocks whose row is within
     // kUrgentReach of c. Work further below has slack of one block step or
-    // more and runs in list-schedule order, so the urgent queue stays short.
+    // more and runs in queue order, so the urgent queue stays short.
     constexpr int64_t kUrgentReach = 3;
     const int64_t dist = grow(i, r) - grow(kq, cq);
     const int32_t me = lctr[lidx(i, kq, r, cq)];
@@ -463,9 +454,9 @@ struct Builder {
   }
 
   // ------------------------------------------------------------ selinv ----
-  // Counters: Linv column panels (chain), Sigma^0 blocks (chain), U column
+  // Counters: Linv column and row panels, Sigma^0 blocks (chain), U column
   // panels, Sigma row / column panels (diagonal tiles: lower blocks only).
-  std::vector<int32_t> linv_col;   // [i][c]
+  std::vector<int32_t> linv_col;   // [i][columns, then rows]
   std::vector<int64_t> linv_base;
   std::vector<int32_t> s0_ctr;     // [i][r][c] lower
   std::vector<int64_t> s0_base;
@@ -486,7 +477,7 @@ struct Builder {
     for (int i = 0; i < cols; ++i) {
       const int R = L.nblk(i);
       linv_base[i] = linv_col.size();
-      for (int c = 0; c < R; ++c) linv_col.push_back(newctr(true));
+      for (int c = 0; c < 2 * R; ++c) linv_col.push_back(newctr(false));
       s0_base[i] = s0_ctr.size();
       for (int r = 0; r < R; ++r)
         for (int c = 0; c <= r; ++c) s0_ctr.push_back(newctr(true));
@@ -518,11 +509,14 @@ struct Builder {
         emit(blank(OP_JOIN, 0, 0), {}, {{colfinal[i], colblocks[i]}}, {coljoin[i]}, 0.0);
       }
     }
+    if (s.planes) alloc_planes(cols);
     for (int i = s.sel0; i < cols; ++i) emit_phase1(i);
     for (int i = cols - 1; i >= s.sel0; --i) emit_phase2(i);
   }
 
+  // blocks of a column / row of Linv, in the order they are emitted
   int32_t linv_ctr(int i, int c) const { return linv_col[linv_base[i] + c]; }
+  int32_t linv_row(int i, int r) const { return linv_col[linv_base[i] + L.nblk(i) + r]; }
   int32_t s0(int i, int r, int c) const { return s0_ctr[s0_base[i] + (int64_t)r * (r + 1) / 2 + c]; }
   int32_t ucol(int k, int i, int c) const { return u_col[ut_base[slot_index(k, i)] + c]; }
   int32_t srow(int j, int i, int r) const { return s_row[st_rbase[slot_index(j, i)] + r]; }
@@ -535,32 +529,70 @@ struct Builder {
   void emit_phase1(int i) {
     const int R = L.nblk(i), ld = L.rows(i);
     std::vector<int> st;
-    // TRTRI of the diagonal tile, block column by block column
-    for (int c = 0; c < R; ++c) {
-      for (int r = c; r < R; ++r) {
-        const int m = L.bdim(i, r), n = L.bdim(i, c);
-        std::vector<Wait> w;
-        add_fused_wait(i, w);
-        if (r == c) {
-          Task t = blank(OP_TRTRI, m, n);
-          t.out = mkref(BUF_W, L.blk(i, i, r, c));
-          t.ldo = ld;
-          t.aux = mkref(BUF_L, L.blk(i, i, r, r));
-          t.ldx = ld;
-          emit(t, {}, w, {linv_ctr(i, c)}, 2.0 * m * kSweepStepNs);
-        } else {
-          // Linv[r,c] = -L[r,r]^{-1} sum_{q=c}^{r-1} L[r,q] Linv[q,c]
-          Task t = blank(OP_TRSM_LLN, m, n);
-          t.out = mkref(BUF_W, L.blk(i, i, r, c));
-          t.ldo = ld;
-          t.aux = mkref(BUF_L, L.blk(i, i, r, r));
-          t.ldx = ld;
-          w.push_back({linv_ctr(i, c), r - c});
-          Seg g = seg(mkref(BUF_L, L.blk(i, i, r, c)), ld, mkref(BUF_W, L.blk(i, i, c, c)), ld, (r - c) * FB, false,
-                      false);
-          emit(t, {g}, w, {linv_ctr(i, c)}, 2.0 * m * kSweepStepNs);
+    // TRTRI of the diagonal tile: its 64 x 64 diagonal blocks, then by doubling:
+    // with the inverses of two neighbouring groups of h block columns known,
+    //   Linv[r,c] = -Linv_22 (L_21 Linv_11)
+    // for the rows r of the second and the columns c of the first. Two products
+    // per level (log2 of the blocks), each of h^2 independent blocks; the
+    // column-by-column substitution before was a chain of R tasks that each
+    // solved a triangle (9-12 ms of waiting at the end of a b = 1024
+    // factorization, for its last tile). The inner product, negated, is kept
+    // transposed in the tile's upper part, which nothing else uses.
+    // (phase 1 of the last columns is waited for, that of the others runs beside
+    // each other's and the factorization)
+    const int columns = i >= s.nt - 1 ? 1 : L.last() + 1 - s.sel0;
+    for (int r = 0; r < R; ++r) {
+      const int m = L.bdim(i, r);
+      std::vector<Wait> w;
+      add_fused_wait(i, w);
+      Task t = blank(OP_TRTRI, m, m);
+      t.out = mkref(BUF_W, L.blk(i, i, r, r));
+      t.ldo = ld;
+      t.aux = mkref(BUF_L, L.blk(i, i, r, r));
+      t.ldx = ld;
+      emit(t, {}, w, {linv_ctr(i, r), linv_row(i, r)}, 2.0 * m * kSweepStepNs);
+    }
+    for (int h = 1; h < R; h *= 2) {
+      const uint8_t mode = fine_mode((long long)h * ((R + 1) / 2) * columns, PM_QUAD4);
+      for (int g = 0; g + h < R; g += 2 * h) {
+        const int mid = g + h, end = std::min(g + 2 * h, R);
+        for (int c = g; c < mid; ++c) {
+          const int n = L.bdim(i, c);
+          const int32_t tctr = newctr(false);
+          for (int r = mid; r < end; ++r) {  // (c, r) <- -(L[r, c .. mid) Linv[c .. mid, c])^T
+            Task t = blank(OP_STORE, n, L.bdim(i, r));
+            t.flags = TF_NEG;
+            split_fp64(t, mode, false);
+            t.out = mkref(BUF_W, L.blk(i, i, c, r));
+            t.ldo = ld;
+            std::vector<Wait> w;
+            add_fused_wait(i, w);
+            w.push_back({linv_ctr(i, c), mid - c});
+            emit(t, {seg(mkref(BUF_W, L.blk(i, i, c, c)), ld, mkref(BUF_L, L.blk(i, i, r, c)), ld, (mid - c) * FB, true, true)},
+                 w, {tctr}, 0.0);
+          }
+          for (int r = mid; r < end; ++r) {  // Linv[r,c] = Linv[r, mid .. r] (that, transposed back)
+            Task t = blank(OP_STORE, L.bdim(i, r), n);
+            split_fp64(t, mode, false);
+            t.out = mkref(BUF_W, L.blk(i, i, r, c));
+            t.ldo = ld;
+            std::vector<Wait> w{{linv_row(i, r), r - mid + 1}, {tctr, r - mid + 1}};
+            emit(t, {seg(mkref(BUF_W, L.blk(i, i, r, mid)), ld, mkref(BUF_W, L.blk(i, i, c, mid)), ld,
+                         (r - mid) * FB + L.bdim(i, r), false, true)},
+                 w, {linv_ctr(i, c), linv_row(i, r)}, 0.0);
+          }
         }
       }
+    }
+    // a block column's many readers wait for one join of its blocks (few blocks:
+    // for the blocks themselves)
+    std::vector<Wait> col(R);
+    for (int c = 0; c < R; ++c) {
+      col[c] = {linv_ctr(i, c), R - c};
+      if (R < 8) continue;
+      const int32_t j = newctr(true);
+      emit(blank(OP_JOIN, 0, 0), {}, {col[c]}, {j}, 0.0);
+      col[c] = {j, 1};
     }
     // LAUUM: Sigma^0[r,c] = sum_{q>=r} Linv[q,r]^T Linv[q,c], r >= c
     for (int r = 0; r < R; ++r)
@@ -568,10 +600,10 @@ struct Builder {
         const int m = L.bdim(i, r), n = L.bdim(i, c);
         Task t = blank(OP_STORE, m, n);
         // only the lower part of a diagonal block is used
-        split_fp64(t, 2LL * R * (R + 1) * crowd <= kGpuSms ? PM_GRID16 : PM_FULL, r == c);
+        split_fp64(t, 2LL * R * (R + 1) * crowd * columns <= kGpuSms ? PM_GRID16 : PM_FULL, r == c);
         t.out = mkref(BUF_S, L.blk(i, i, r, c));
         t.ldo = ld;
-        std::vector<Wait> w{{linv_ctr(i, r), R - r}, {linv_ctr(i, c), R - c}};
+        std::vector<Wait> w{col[r], col[c]};
         Seg g = seg(mkref(BUF_W, L.blk(i, i, r, r)), ld, mkref(BUF_W, L.blk(i, i, r, c)), ld, ld - r * FB, true,
                     false);
         emit(t, {g}, w, {s0(i, r, c)}, 0.0);
@@ -584,12 +616,12 @@ struct Builder {
         for (int r = 0; r < L.nblk(k); ++r) {
           const int m = L.bdim(k, r), n = L.bdim(i, c);
           Task t = blank(OP_STORE, m, n);
-          split_fp64(t, fine_mode((col_blocks(i) - R) * R, PM_FULL), false);
+          split_fp64(t, fine_mode((col_blocks(i) - R) * R * columns, PM_FULL), false);
           t.out = mkref(BUF_W, L.blk(k, i, r, c));
           t.ldo = ldk;
           std::vector<Wait> w;
           add_fused_wait(i, w);
-          w.push_back({linv_ctr(i, c), R - c});
+          w.push_back(col[c]);
           Seg g = seg(mkref(BUF_L, L.blk(k, i, r, c)), ldk, mkref(BUF_W, L.blk(i, i, c, c)), ld, ld - c * FB, false,
                       false);
           lower_precision(t);
@@ -598,10 +630,116 @@ struct Builder {
     }
   }
 
+  // ---- planes (see plan.h). Tile column i's planes live in ring slots: those of
+  // Sigma (the diagonal tile by rows; each tile below it by columns, and by rows
+  // where an earlier column needs them so) in slot i mod (w + 2), read by the
+  // columns i - w .. i; those of U in slot i mod 2, read by column i; the arrow
+  // corner has a slot of its own. `p2join[i]`: the products of column i are done,
+  // so the planes that only it and later columns read may be overwritten.
+  std::vector<int32_t> p2join;
+  std::vector<int32_t> pl_d, pl_c, pl_r, pl_u;  // counters per vector group: diagonal rows; tile columns / rows; U
+  std::vector<int64_t> pl_dbase, pl_cbase, pl_rbase, pl_ubase;
+  int64_t pu_sigma = 0, pu_u = 0, pu_corner = 0;  // units of a Sigma slot, a U slot, the corner's
+  int64_t sig_slots() const { return s.w + 2; }
+  // offset of a tile's planes inside its column's Sigma or U slot
+  enum PlaneSet { PS_DIAG, PS_COL, PS_ROW, PS_U };
+  int64_t plane_off(PlaneSet set, int k, int i) const {
+    const int R = L.nblk(i);
+    if (i == s.nt) return 2 * pu_u + sig_slots() * pu_sigma;
+    const int64_t gb = plane_group(s.prec, s.b), ga = s.a > 0 ? plane_group(s.prec, s.a) : 0;
+    if (set == PS_U) return (int64_t)(i % 2) * pu_u + (k == s.nt ? (int64_t)s.w * R * gb : (int64_t)(k - i - 1) * R * gb);
+    const int64_t slot = 2 * pu_u + (int64_t)(i % sig_slots()) * pu_sigma;
+    if (set == PS_DIAG) return slot;
+    if (set == PS_COL) return slot + (int64_t)R * gb * (k == s.nt ? 1 + s.w : k - i);
+    const int64_t rows0 = slot + (int64_t)R * gb * (1 + s.w) + (int64_t)R * ga;
+    return rows0 + (k == s.nt ? (int64_t)s.w * R * gb : (int64_t)(k - i - 1) * R * gb);
+  }
+  int64_t plane_ref(PlaneSet set, int k, int i, int g) const {  // group g of the tile's planes
+    const int kk = set == PS_DIAG || set == PS_ROW ? L.rows(i) : L.rows(k);
+    return mkref(BUF_P, plane_off(set, k, i) + (int64_t)g * plane_group(s.prec, kk));
+  }
+  void alloc_planes(int cols) {
+    const int R = L.nblk(0), ra = s.a > 0 ? L.nblk(s.nt) : 0;
+    const int64_t gb = plane_group(s.prec, s.b), ga = s.a > 0 ? plane_group(s.prec, s.a) : 0;
+    pu_u = (int64_t)s.w * R * gb + (int64_t)R * ga;
+    pu_sigma = (int64_t)R * gb * (1 + 2 * s.w) + (int64_t)R * ga + (int64_t)ra * gb;
+    pu_corner = (int64_t)ra * ga;
+    if (out) out->plane_units = 2 * pu_u + sig_slots() * pu_sigma + pu_corner;
+    p2join.assign(cols, -1);
+    pl_dbase.assign(cols, 0);
+    for (auto* v : {&pl_cbase, &pl_rbase, &pl_ubase}) v->assign((size_t)cols * (s.w + 2), -1);
+  }
+  // counters of the groups of one split tile, in `ctr` from `base`
+  void split_tile(PlaneSet set, int k, int i, std::vector<int32_t>& ctr, int64_t& base) {
+    const bool rows = set == PS_DIAG || set == PS_ROW;  // vectors are the tile's rows
+    const int nv = rows ? L.rows(k) : L.rows(i), kk = rows ? L.rows(i) : L.rows(k);
+    base = (int64_t)ctr.size();
+    for (int g = 0; g < (nv + FB - 1) / FB; ++g) {
+      ctr.push_back(newctr(false));
+      std::vector<Wait> w;
+      if (set == PS_U) w.push_back({ucol(k, i, g), L.nblk(k)});
+      else if (set == PS_DIAG) {
+        w.push_back({srow(i, i, g), g + 1});
+        w.push_back({scol(i, i, g), L.nblk(i) - g});
+      } else if (set == PS_COL) w.push_back({scol(k, i, g), L.nblk(k)});
+      else w.push_back({srow(k, i, g), L.nblk(i)});
+      if (i < s.nt && i + 2 < (int)p2join.size() && p2join[i + 2] >= 0) w.push_back({p2join[i + 2], 1});
+      // at most 4 chunks of K (16 parts) per task
+      for (int c0 = 0; c0 < (int)plane_chunks(kk); c0 += 4) {
+        const int k0 = c0 * kPlaneChunk;
+        Task t = blank(OP_SPLIT, std::min(FB, nv - g * FB), 1);
+        t.prec = (uint8_t)s.prec;
+        t.out = plane_ref(set, k, i, g);
+        t.cin = set == PS_U ? mkref(BUF_W, L.tile(k, i)) : mkref(BUF_S, L.tile(k, i));
+        const int ld = L.rows(k);
+        t.cin += rows ? (int64_t)g * FB + (int64_t)k0 * ld : (int64_t)g * FB * ld + k0;
+        t.ldc = ld;
+        t.zrows = kk;   // whole K (layout of the group)
+        t.gcol = k0;    // this task's first K
+        if (!rows) t.flags |= TF_KCONT;
+        if (set == PS_U) t.flags |= TF_BSIDE;
+        t.pmode = PM_SPLIT;
+        t.parts = (uint8_t)(4 * std::min<int64_t>(4, plane_chunks(kk) - c0));
+        emit(t, {}, w, {ctr.back()}, 6000.0);
+      }
+    }
+  }
+  int split_tasks(int kk) const { return (int)((plane_chunks(kk) + 3) / 4); }  // per vector group
+  // Does a column before i need tile (k, i) by rows (S_ki with k > i)?
+  bool need_rows(int k, int i) const { return i > s.sel0 && s.w > 0 && i < s.nt && (k == s.nt || k - i < s.w); }
+  // segment of A = S_jk (group r) and B = U_ki (group c), and what it waits for
+  void plane_seg(int j, int k, int r, int i, int c, std::vector<Seg>& segs, std::vector<Wait>& w) {
+    int64_t a;
+    if (j == k) {
+      a = plane_ref(PS_DIAG, j, j, r);
+      w.push_back({pl_d[pl_dbase[j] + r], split_tasks(L.rows(j))});
+    } else if (j > k) {
+      a = plane_ref(PS_ROW, j, k, r);
+      w.push_back({pl_r[pl_rbase[slot_index(j, k)] + r], split_tasks(L.rows(k))});
+    } else {
+      a = plane_ref(PS_COL, k, j, r);
+      w.push_back({pl_c[pl_cbase[slot_index(k, j)] + r], split_tasks(L.rows(k))});
+    }
+    w.push_back({pl_u[pl_ubase[slot_index(k, i)] + c], split_tasks(L.rows(k))});
+    segs.push_back(seg(a, 0, plane_ref(PS_U, k, i, c), 0, L.rows(k), false, false));
+  }
+  void plane_product(Task& t) const {
+    t.prec = (uint8_t)s.prec;
+    t.flags |= TF_PLANES;
+    t.pmode = PM_COLS2;
+    t.parts = t.n > 32 ? 2 : 1;
+  }
+
   void emit_phase2(int i) {
     const int R = L.nblk(i), ld = L.rows(i);
     std::vector<int> st;
     L.structure(i, st);
+    std::vector<int32_t> done{};
+    if (s.planes) {
+      for (int k : st) split_tile(PS_U, k, i, pl_u, pl_ubase[slot_index(k, i)]);
+      done.push_back(newctr(false));  // signalled by every product of this column
+    }
+    int nprod = 0;
     // off-diagonal tiles, j from the last down (Algorithm 3's j loop)
     for (int tj = (int)st.size() - 1; tj >= 0; --tj) {
       const int j = st[tj], ldj = L.rows(j);
@@ -609,13 +747,16 @@ struct Builder {
         for (int r = 0; r < L.nblk(j); ++r) {
           const int m = L.bdim(j, r), n = L.bdim(i, c);
           Task t = blank(OP_NEG, m, n);
-          split_p2(t, (col_blocks(i) - R) * R);  // phase 2 is a chain of joins: shorter tasks, shorter steps
           t.out = mkref(BUF_S, L.blk(j, i, r, c));
           t.ldo = ldj;
           std::vector<Seg> segs;
           std::vector<Wait> w;
           for (int k : st) {
             const int ldk = L.rows(k);
+            if (s.planes) {
+              plane_seg(j, k, r, i, c, segs, w);
+              continue;
+            }
             if (j == k) {
               segs.push_back(seg(mkref(BUF_S, L.blk(j, j, r, 0)), ldj, mkref(BUF_W, L.blk(k, i, 0, c)), ldk, ldk,
                                  false, false));
@@ -632,19 +773,28 @@ struct Builder {
             }
             w.push_back({ucol(k, i, c), L.nblk(k)});
           }
-          lower_precision(t);
-          emit(t, segs, w, {srow(j, i, r), scol(j, i, c)}, 0.0);
+          if (s.planes) plane_product(t);
+          else {
+            split_p2(t, (col_blocks(i) - R) * R);  // phase 2 is a chain of joins: shorter tasks, shorter steps
+            lower_precision(t);
+          }
+          std::vector<int32_t> sig{srow(j, i, r), scol(j, i, c)};
+          sig.insert(sig.end(), done.begin(), done.end());
+          emit(t, segs, w, sig, 0.0);
+          ++nprod;
         }
       tile_gemms += (long long)st.size();
     }
+    if (s.planes)
+      for (int k : st) {
+        split_tile(PS_COL, k, i, pl_c, pl_cbase[slot_index(k, i)]);
+        if (need_rows(k, i)) split_tile(PS_ROW, k, i, pl_r, pl_rbase[slot_index(k, i)]);
+      }
     // diagonal tile: Sigma_ii = Sigma^0 - sum_k Sigma_ki^T U_ki (lower blocks, mirrored)
     for (int r = 0; r < R; ++r)
       for (int c = 0; c <= r; ++c) {
         const int m = L.bdim(i, r), n = L.bdim(i, c);
         Task t = blank(OP_SYMUPD, m, n);
-        const long long blocks = (long long)R * (R + 1) / 2;
-        if (r == c) split_fp64(t, fine_mode(blocks, PM_QUAD4), true);
-        else split_p2(t, blocks);
         t.out = mkref(BUF_S, L.blk(i, i, r, c));
         t.ldo = ld;
         t.cin = t.out;
@@ -659,16 +809,37 @@ struct Builder {
         std::vector<Wait> w{{s0(i, r, c), 1}};
         for (int k : st) {
           const int ldk = L.rows(k);
+          if (s.planes) {
+            segs.push_back(seg(plane_ref(PS_COL, k, i, r), 0, plane_ref(PS_U, k, i, c), 0, ldk, false, false));
+            w.push_back({pl_c[pl_cbase[slot_index(k, i)] + r], split_tasks(ldk)});
+            w.push_back({pl_u[pl_ubase[slot_index(k, i)] + c], split_tasks(ldk)});
+            continue;
+          }
           segs.push_back(seg(mkref(BUF_S, L.blk(k, i, 0, r)), ldk, mkref(BUF_W, L.blk(k, i, 0, c)), ldk, ldk, true,
                              false));
           w.push_back({scol(k, i, r), L.nblk(k)});
           w.push_back({ucol(k, i, c), L.nblk(k)});
         }
-        if (!segs.empty()) lower_precision(t);  // the products; the assembly (cin - acc, mirror) stays FP64
+        if (s.planes && !segs.empty()) {
+          plane_product(t);
+        } else {
+          const long long blocks = (long long)R * (R + 1) / 2;
+          if (r == c) split_fp64(t, fine_mode(blocks, PM_QUAD4), true);
+          else split_p2(t, blocks);
+          if (!segs.empty()) lower_precision(t);  // the products; the assembly (cin - acc, mirror) stays FP64
+        }
         sym_block = r == c;
-        emit(t, segs, w, {srow(i, i, r), scol(i, i, c)}, 0.0);
+        std::vector<int32_t> sig{srow(i, i, r), scol(i, i, c)};
+        sig.insert(sig.end(), done.begin(), done.end());
+        emit(t, segs, w, sig, 0.0);
+        ++nprod;
       }
     tile_gemms += (long long)st.size();
+    if (s.planes) {
+      if (i > s.sel0 && (s.w > 0 || i == s.nt)) split_tile(PS_DIAG, i, i, pl_d, pl_dbase[i]);
+      p2join[i] = newctr(true);
+      emit(blank(OP_JOIN, 0, 0), {}, {{done[0], nprod}}, {p2join[i]}, 0.0);
+    }
   }
 
   // ---------------------------------------------------------- schedule ----
@@ -739,48 +910,40 @@ struct Builder {
       blevel[t] = cost[t] + best;
       cp = std::max(cp, blevel[t]);
     }
-    // list schedule: free workers take the ready task with the largest bottom level
-    using RItem = std::pair<double, int32_t>;
-    using EItem = std::pair<double, int32_t>;  // (finish time, task)
-    std::vector<RItem> rbuf;
-    rbuf.reserve(nt_);
-    std::priority_queue<RItem> ready(std::less<RItem>(), std::move(rbuf));
-    std::vector<EItem> ebuf;
-    ebuf.reserve((size_t)std::max(1, workers) + 1);
-    std::priority_queue<EItem, std::vector<EItem>, std::greater<EItem>> running(std::greater<EItem>(), std::move(ebuf));
-    for (int t = 0; t < nt_; ++t)
-      if (indeg[t] == 0) ready.push({blevel[t], t});
-    std::vector<int32_t> order;
-    order.reserve(nt_);
+    // device queue order: by bottom level, the longest way to the end first (a
+    // topological order: every task costs time). Workers take the first ready
+    // task of it, so the factorization goes before the phase 1 of finished
+    // columns, which fills the gaps. In the order of simulated start times, as
+    // before, phase-1 tasks of early columns went before factor tasks that the
+    // simulation saw later: 322 against 300 ms (n = 122,944 in emulated FP64).
+    std::vector<int32_t> order(nt_);
+    for (int t = 0; t < nt_; ++t) order[t] = t;
+    std::stable_sort(order.begin(), order.end(), [&](int32_t a, int32_t b) { return blevel[a] > blevel[b]; });
     double now = 0;
-    int free_workers = std::max(1, workers);
-    auto release = [&](int32_t t) {
-      for (int64_t e = soff[t]; e < soff[t + 1]; ++e)
-        if (--indeg[succ[e]] == 0) ready.push({blevel[succ[e]], succ[e]});
-    };
-    while ((int)order.size() < nt_) {
-      while (free_workers > 0 && !ready.empty()) {
-        int32_t t = ready.top().second;
-        ready.pop();
-        order.push_back(t);
-        running.push({now + cost[t], t});
-        --free_workers;
-      }
-      if (running.empty()) return STILES_ERR_PLAN;  // cycle
-      EItem e = running.top();
-      running.pop();
-      now = e.first;
-      ++free_workers;
-      release(e.second);
-      while (!running.empty() && running.top().first <= now) {
-        EItem e2 = running.top();
+    if (workers > 0) {
+      // makespan of a list schedule in that order (plan statistics)
+      using RItem = std::pair<double, int32_t>;
+      using EItem = std::pair<double, int32_t>;  // (finish time, task)
+      std::priority_queue<RItem> ready;
+      std::priority_queue<EItem, std::vector<EItem>, std::greater<EItem>> running;
+      for (int t = 0; t < nt_; ++t)
+        if (indeg[t] == 0) ready.push({blevel[t], t});
+      int free_workers = workers;
+      while (!ready.empty() || !running.empty()) {
+        while (free_workers > 0 && !ready.empty()) {
+          running.push({now + cost[ready.top().second], ready.top().second});
+          ready.pop();
+          --free_workers;
+        }
+        const EItem e = running.top();
         running.pop();
+        now = e.first;
         ++free_workers;
-        release(e2.second);
+        for (int64_t x = soff[e.second]; x < soff[e.second + 1]; ++x)
+          if (--indeg[succ[x]] == 0) ready.push({blevel[succ[x]], succ[x]});
       }
     }
-    while (!running.empty()) { now = std::max(now, running.top().first); running.pop(); }
-    // write the plan in list-schedule order (the device queue order)
+    // write the plan in that order
     Plan& p = *out;
     p.tasks.clear(); p.segs.clear(); p.waits.clear(); p.sigs.clear();
     p.wait_off.assign(1, 0); p.sig_off.assign(1, 0);
@@ -893,6 +1056,10 @@ static double task_estimate(const Shape& s) {
   return (double)s.nt * (s.w + 2) * nb * (nb + na) * ((s.w + 2) * nb + 8);
 }
 
+// Products from planes need the split of every Sigma and U tile as two more
+// steps of phase 2's chain, which short products do not pay back.
+bool use_planes(const Shape& s) { return s.prec != PREC_FP64 && s.b >= kPlanesMinB && tune_p2_split(s.tune) == 0; }
+
 static bool shape_ok(const Shape& s) {
   return s.nt >= 1 && s.b >= 1 && s.w >= 0 && s.a >= 0 && s.w <= s.nt - 1 && tune_valid(s.tune) && s.sel0 >= 0 &&
          s.sel0 <= (s.a > 0 ? s.nt : s.nt - 1);
@@ -901,6 +1068,7 @@ static bool shape_ok(const Shape& s) {
 int build_plan(const Shape& s, PlanKind kind, int workers, Plan* out) {
   if (!shape_ok(s)) return STILES_ERR_INVALID_ARG;
   if (task_estimate(s) > 4.0e8) return STILES_ERR_INVALID_ARG;
+  out->plane_units = 0;
   Builder B(s, kind, out);
   if (kind == PLAN_FACTOR || kind == PLAN_FUSED) B.build_factor();
   if (kind == PLAN_SELINV || kind == PLAN_FUSED) B.build_selinv();
@@ -913,6 +1081,7 @@ int build_plan(const Shape& s, PlanKind kind, int workers, Plan* out) {
 int build_serve_template(const Shape& s, int workers, Plan* out) {
   if (!shape_ok(s)) return STILES_ERR_INVALID_ARG;
   if (task_estimate(s) > 4.0e8) return STILES_ERR_INVALID_ARG;
+  out->plane_units = 0;
   Builder B(s, PLAN_FUSED, out);
   B.serve = true;
   B.crowd = 2;  // requests run side by side
@@ -934,15 +1103,18 @@ int build_batch_plan(const std::vector<Shape>& shapes, const std::vector<int64_t
   }
   if (est > 4.0e8) return STILES_ERR_INVALID_ARG;
   Builder M(shapes[0], PLAN_FUSED, out);
+  out->plane_units = 0;
   diag_base->assign(shapes.size() + 1, 0);
   for (size_t m = 0; m < shapes.size(); ++m) {
-    Builder B(shapes[m], PLAN_FUSED, nullptr);
+    Plan one;  // its plane units only
+    Builder B(shapes[m], PLAN_FUSED, &one);
+    const int64_t poff = out->plane_units;
     B.crowd = (int)shapes.size();
     B.build_factor();
     B.build_selinv();
     const int32_t coff = (int32_t)M.chain.size(), doff = M.ndiag;
     const int64_t off = base[m];
-    auto shift = [off](int64_t ref) { return ref < 0 ? ref : ref + off; };
+    auto shift = [off, poff](int64_t ref) { return ref < 0 ? ref : ref + ((ref >> BUF_SHIFT) == BUF_P ? poff : off); };
     for (size_t t = 0; t < B.tasks.size(); ++t) {
       Task tk = B.tasks[t];
       tk.out = shift(tk.out);
@@ -973,6 +1145,7 @@ int build_batch_plan(const std::vector<Shape>& shapes, const std::vector<int64_t
     M.flops += tile_flops(shapes[m], PLAN_FUSED);
     M.flops_lowered += B.flops_lowered;
     (*diag_base)[m + 1] = M.ndiag;
+    out->plane_units += one.plane_units;
   }
   const int rc = M.finish(workers);
   if (rc) return rc;
@@ -987,8 +1160,8 @@ int check_plan(const Plan& p) {
     const Task& tk = p.tasks[t];
     if (tk.seg0 < 0 || tk.nseg < 0 || (int64_t)tk.seg0 + tk.nseg > (int64_t)p.segs.size()) return STILES_ERR_PLAN;
     if (tk.succ0 < 0 || tk.nsucc < 0 || (int64_t)tk.succ0 + tk.nsucc > (int64_t)p.succ.size()) return STILES_ERR_PLAN;
-    if (tk.m < 0 || tk.n < 0 || tk.m > FB || tk.n > FB || tk.op > OP_JOIN) return STILES_ERR_PLAN;
-    if (tk.parts < 1 || tk.parts > kMaxParts || tk.pmode > PM_TRI16 || tk.prec > PREC_FP32X) return STILES_ERR_PLAN;
+    if (tk.m < 0 || tk.n < 0 || tk.m > FB || tk.n > FB || tk.op > OP_SPLIT) return STILES_ERR_PLAN;
+    if (tk.parts < 1 || tk.parts > kMaxParts || tk.pmode > PM_SPLIT || tk.prec > PREC_FP32X) return STILES_ERR_PLAN;
     for (int64_t q = p.wait_off[t]; q < p.wait_off[t + 1]; ++q) {
       const Wait& w = p.waits[q];
       if (w.ctr < 0 || w.ctr >= p.nctr) return STILES_ERR_PLAN;
@@ -1048,6 +1221,20 @@ int validate_plan_len(const Plan& p, int64_t lim, int kind) {
       if (tk.parts != 1 || tk.nseg != 0) return bad("join with work", t);
       continue;
     }
+    // units [ref, ref + len) of BUF_P
+    auto in_planes = [&](int64_t ref, int64_t len) {
+      return ref >= 0 && (ref >> BUF_SHIFT) == BUF_P && (ref & OFF_MASK) + len <= p.plane_units;
+    };
+    if (tk.op == OP_SPLIT) {
+      const int64_t kc = std::min<int64_t>(tk.zrows - tk.gcol, kPlaneChunk * (int64_t)(tk.parts / 4));
+      const bool kcont = tk.flags & TF_KCONT;
+      if (tk.m < 1 || tk.parts % 4 || tk.gcol % kPlaneChunk || kc < 1 || tk.prec == PREC_FP64 ||
+          (tk.parts / 4 - 1) * kPlaneChunk >= tk.zrows - tk.gcol ||
+          !in(tk.cin, 0, kcont ? (tk.m - 1) * (int64_t)tk.ldc + kc - 1 : tk.m - 1 + (kc - 1) * (int64_t)tk.ldc) ||
+          !in_planes(tk.out, plane_group(tk.prec, tk.zrows)))
+        return bad("split out of bounds", t);
+      continue;
+    }
     if (tk.op == OP_ZERO) {  // zrows x n above the block
       if (tk.parts != 1 || tk.nseg != 0 || tk.zrows < 1 || tk.n < 1 ||
           !in(tk.out, -(int64_t)tk.zrows, -1 + (int64_t)(tk.n - 1) * tk.ldo))
@@ -1060,7 +1247,7 @@ int validate_plan_len(const Plan& p, int64_t lim, int kind) {
       if ((tk.pmode == PM_TRI16 || tk.pmode == PM_TRI3) && tk.m != tk.n) return bad("triangle parts on a block that is not square", t);
       if ((tk.pmode == PM_TRI16 || tk.pmode == PM_GRID16) && tk.prec != PREC_FP64)
         return bad("16 x 16 parts on a reduced-precision task", t);
-      if (tk.prec == PREC_EMU64 && (rm > 32 || cn > 32)) return bad("emulated task part larger than 32 x 32", t);
+      if (tk.prec != PREC_FP64 && (tk.pmode != PM_COLS2 || cn > 32)) return bad("reduced-precision part larger than 64 x 32", t);
       if (tk.prec != PREC_FP64 && tk.op != OP_UPD && tk.op != OP_NEG && tk.op != OP_STORE && tk.op != OP_SYMUPD)
         return bad("reduced precision on a triangular task", t);
       if (rm <= 0 || cn <= 0) continue;
@@ -1068,6 +1255,11 @@ int validate_plan_len(const Plan& p, int64_t lim, int kind) {
       for (int g = tk.seg0; g < tk.seg0 + tk.nseg; ++g) {
         const Seg& sg = p.segs[g];
         if (sg.k <= 0) return bad("empty segment", t);
+        if (tk.flags & TF_PLANES) {
+          if (!in_planes(sg.a, plane_group(tk.prec, sg.k)) || !in_planes(sg.b, plane_group(tk.prec, sg.k)))
+            return bad("planes out of bounds", t);
+          continue;
+        }
         const int64_t amax = (sg.trans & 1) ? (sg.k - 1) + (int64_t)r1 * sg.lda : r1 + (int64_t)(sg.k - 1) * sg.lda;
         const int64_t amin = (sg.trans & 1) ? (int64_t)r0 * sg.lda : r0;
         const int64_t bmax = (sg.trans & 2) ? c1 + (int64_t)(sg.k - 1) * sg.ldb : (sg.k - 1) + (int64_t)c1 * sg.ldb;
@@ -1079,7 +1271,7 @@ int validate_plan_len(const Plan& p, int64_t lim, int kind) {
       const bool uses_cin = tk.op == OP_UPD || tk.op == OP_POTRF || tk.op == OP_TRSM_RLT || tk.op == OP_SYMUPD;
       if (uses_cin && !in(tk.cin, r0 + (int64_t)c0 * tk.ldc, r1 + (int64_t)c1 * tk.ldc)) return bad("input out of bounds", t);
       if (tk.op == OP_TRSM_RLT && !in(tk.aux, 0, (tk.n - 1) + (int64_t)(tk.n - 1) * tk.ldx)) return bad("T out of bounds", t);
-      if ((tk.op == OP_TRSM_LLN || tk.op == OP_TRTRI) && !in(tk.aux, 0, (tk.m - 1) + (int64_t)(tk.m - 1) * tk.ldx))
+      if (tk.op == OP_TRTRI && !in(tk.aux, 0, (tk.m - 1) + (int64_t)(tk.m - 1) * tk.ldx))
         return bad("T out of bounds", t);
       if (tk.op == OP_SYMUPD && !(tk.flags & TF_SYM_DIAG) &&
           !in(tk.aux, c0 + (int64_t)r0 * tk.ldx, c1 + (int64_t)r1 * tk.ldx))
@@ -1155,17 +1347,18 @@ class RaceCheck {
         for (int w = 0; w < words_; ++w) a[w] |= b[w];
         a[q >> 6] |= 1ull << (q & 63);
       }
-    for (int b = 0; b < 4; ++b) {
-      lw_[b].assign(lim, -1);
-      head_[b].assign(lim, -1);
+    for (int b = 0; b < 5; ++b) {  // planes: one cell per kPlaneCell units
+      lw_[b].assign(b == BUF_P ? p.plane_units / kPlaneCell + 1 : lim, -1);
+      head_[b].assign(lw_[b].size(), -1);
     }
   }
+  static constexpr int kPlaneCell = 16;  // units: divides every group's head and stages
   bool before(int a, int b) const { return (anc_[(size_t)b * words_ + (a >> 6)] >> (a & 63)) & 1; }
 
   // one access of part `id` (kMaxParts task + part) to element `off` of buffer `buf`
   bool access(int buf, int64_t off, int id, bool write) {
     if (serve_ && buf == BUF_A) buf = BUF_L;  // a served request's A is built in place in L
-    if (buf < 0 || buf > 3 || off < 0 || off >= lim_) return fail("access outside the buffers", id, -1, buf, off);
+    if (buf < 0 || buf > 4 || off < 0 || off >= (int64_t)lw_[buf].size()) return fail("access outside the buffers", id, -1, buf, off);
     const int t = id / kMaxParts;
     const int w = lw_[buf][off];
     if (w >= 0 && w != id && !before(w / kMaxParts, t)) return fail(write ? "unordered writes" : "read not ordered after the write", w, id, buf, off);
@@ -1201,6 +1394,13 @@ class RaceCheck {
           if (!access(buf, base + r + (int64_t)c * ld, id, write)) return false;
     return true;
   }
+  // the cells of units [u0, u0 + len) of a plane group
+  bool planes(int64_t ref, int64_t u0, int64_t len, int id, bool write) {
+    const int64_t base = (ref & OFF_MASK) + u0;
+    for (int64_t c = base / kPlaneCell; c <= (base + len - 1) / kPlaneCell; ++c)
+      if (!access(BUF_P, c, id, write)) return false;
+    return true;
+  }
   bool task_part(int t, int q) {
     const Task& tk = p_.tasks[t];
     const int id = kMaxParts * t + q;
@@ -1211,9 +1411,28 @@ class RaceCheck {
       const int64_t len = (tk.flags & TF_CORNER) ? a * a : (1 + (int64_t)tk.zrows) * b * b + a * b;
       return len > 0 ? rect(tk.out, (int)len, 0, (int)len, 0, 1, id, true) : true;
     }
+    if (tk.op == OP_SPLIT) {
+      // 16 vectors x one chunk of K read; the chunk's stages written (the four
+      // vector parts of a chunk write disjoint slices: recorded once)
+      const int v0 = 16 * (q & 3), nv = std::min(16, tk.m - v0), k0 = kPlaneChunk * (q >> 2);
+      const int kc = std::min(kPlaneChunk, tk.zrows - tk.gcol - k0);
+      const bool kcont = tk.flags & TF_KCONT;
+      if (nv > 0 && (kcont ? !rect(tk.cin, tk.ldc, k0, kc, v0, nv, id, false) : !rect(tk.cin, tk.ldc, v0, nv, k0, kc, id, false)))
+        return false;
+      if (q & 3) return true;
+      const int64_t st = 128 * plane_count(tk.prec);
+      return planes(tk.out, plane_head(tk.prec, tk.zrows) + st * ((tk.gcol + k0) / kPlaneK), st * plane_stages(kc), id, true);
+    }
     const Sub x = part_sub(tk.pmode, tk.m, tk.n, q);
     if (x.rm <= 0 || x.cn <= 0) return true;
-    for (int g = tk.seg0; g < tk.seg0 + tk.nseg; ++g) {
+    if (tk.flags & TF_PLANES) {
+      for (int g = tk.seg0; g < tk.seg0 + tk.nseg; ++g) {
+        const Seg& sg = p_.segs[g];
+        const int64_t hd = plane_head(tk.prec, sg.k), len = plane_group(tk.prec, sg.k) - hd;
+        if (!planes(sg.a, hd, len, id, false) || !planes(sg.b, hd, len, id, false)) return false;
+      }
+    }
+    for (int g = tk.flags & TF_PLANES ? tk.seg0 + tk.nseg : tk.seg0; g < tk.seg0 + tk.nseg; ++g) {
       const Seg& sg = p_.segs[g];
       const bool ta = sg.trans & 1, tb = sg.trans & 2;
       // op(A) rows r0 .. r0+rm-1, op(B) columns c0 .. c0+cn-1, K = 0 .. k-1
@@ -1222,10 +1441,15 @@ class RaceCheck {
       if (tb ? !rect(sg.b, sg.ldb, x.c0, x.cn, 0, sg.k, id, false) : !rect(sg.b, sg.ldb, 0, sg.k, x.c0, x.cn, id, false))
         return false;
     }
+    if (tk.prec != PREC_FP64 && (tk.flags & TF_SYM_DIAG)) {  // columns c0 .. from the diagonal down, and their transpose
+      const int len = tk.m - x.c0;
+      return rect(tk.cin, tk.ldc, x.c0, len, x.c0, x.cn, id, false) && rect(tk.out, tk.ldo, x.c0, len, x.c0, x.cn, id, true) &&
+             rect(tk.out, tk.ldo, x.c0, x.cn, x.c0, len, id, true);
+    }
     const bool cin = tk.op == OP_UPD || tk.op == OP_POTRF || tk.op == OP_TRSM_RLT || tk.op == OP_SYMUPD;
     if (cin && !rect(tk.cin, tk.ldc, x.r0, x.rm, x.c0, x.cn, id, false)) return false;
     if (tk.op == OP_TRSM_RLT && !rect(tk.aux, tk.ldx, 0, tk.n, 0, tk.n, id, false, true)) return false;
-    if ((tk.op == OP_TRSM_LLN || tk.op == OP_TRTRI) && !rect(tk.aux, tk.ldx, 0, tk.m, 0, tk.m, id, false, true))
+    if (tk.op == OP_TRTRI && !rect(tk.aux, tk.ldx, 0, tk.m, 0, tk.m, id, false, true))
       return false;
     if (!rect(tk.out, tk.ldo, x.r0, x.rm, x.c0, x.cn, id, true)) return false;
     if (tk.op == OP_SYMUPD && !((tk.flags & TF_SYM_DIAG) && x.r0 == x.c0)) {
@@ -1249,7 +1473,7 @@ class RaceCheck {
   int n_, words_;
   bool serve_;
   std::vector<uint64_t> anc_;
-  std::vector<int> lw_[4], head_[4];
+  std::vector<int> lw_[5], head_[5];
   std::vector<std::pair<int, int>> pool_;
 };
 

@@ -23,7 +23,7 @@ constexpr int FB = 64;  // fine block order (rows and columns of one task's outp
 constexpr int kCtasPerSm = 2;  // persistent CTAs (workers) per SM
 
 // Buffer ids, stored in the top bits of a 64-bit element offset.
-enum Buf : int { BUF_A = 0, BUF_L = 1, BUF_S = 2, BUF_W = 3 };
+enum Buf : int { BUF_A = 0, BUF_L = 1, BUF_S = 2, BUF_W = 3, BUF_P = 4 };
 constexpr int BUF_SHIFT = 60;
 constexpr int64_t OFF_MASK = (int64_t(1) << BUF_SHIFT) - 1;
 inline int64_t mkref(int buf, int64_t off) { return (int64_t(buf) << BUF_SHIFT) | off; }
@@ -33,8 +33,7 @@ enum Op : uint8_t {
   OP_POTRF = 1,     // out = chol(cin - acc)           (square, lower; zero above the diagonal)
   OP_TRSM_RLT = 2,  // out = (cin - acc) * T^{-T}      (T = aux, lower n x n)
   OP_TRTRI = 3,     // out = T^{-1}                    (T = aux, lower m x m; zero above)
-  OP_TRSM_LLN = 4,  // out = -T^{-1} * acc             (T = aux, lower m x m)
-  OP_STORE = 5,     // out = acc
+  OP_STORE = 5,     // out = acc, or -acc (TF_NEG)
   OP_NEG = 6,       // out = -acc
   OP_SYMUPD = 7,    // out = cin - acc and its transpose into the mirror block (aux)
   OP_PREP = 8,      // served requests: one tile column of A from the shape's base values and the
@@ -42,6 +41,7 @@ enum Op : uint8_t {
                     // diagonal tau + rho rb[i] + ra[i] (rb / ra = band / arrow absolute row sums)
   OP_ZERO = 9,      // the zrows x n block above out (L's strict upper part in a diagonal tile's
                     // block column) set to zero; off the factorization's critical path
+  OP_SPLIT = 11,    // digit / piece planes of one vector group of a tile (see "Planes" below)
   OP_JOIN = 10,     // no work: one dependency point for many waiters (a tile column of L final)
 };
 
@@ -56,6 +56,8 @@ enum PartMode : uint8_t {
   PM_TILE32 = 5, // a grid of at most 2 x 2 sub-tiles of at most 32 x 32 (parts = row tiles x column tiles)
   PM_ROWS8 = 6,  // rows [0,8), [8,16), ..
   PM_GRID16 = 7, // a grid of at most 4 x 4 sub-tiles of at most 16 x 16 (parts = row tiles x column tiles)
+  PM_COLS2 = 9,  // columns [0,32) and [32,64) (products from planes)
+  PM_SPLIT = 10, // OP_SPLIT: 16 vectors x 512 of K
   PM_TRI16 = 8,  // the sub-tiles of that grid on or below the diagonal of a square block, row by row
 };
 
@@ -73,7 +75,33 @@ enum TaskFlag : uint8_t {
   TF_SYM_DIAG = 1,  // OP_SYMUPD on a diagonal block (mirror inside the block)
   TF_URGENT = 2,    // on the critical path: queued ahead of the buckets
   TF_CORNER = 4,    // OP_PREP of the arrow corner column
+  TF_PLANES = 8,    // products from planes: the segments' operands are BUF_P refs
+  TF_KCONT = 16,    // OP_SPLIT: K is the contiguous dimension of the source tile
+  TF_BSIDE = 32,    // OP_SPLIT: planes of a right-hand operand
+  TF_NEG = 64,      // OP_STORE: out = -acc
 };
+
+// Planes. The reduced-precision products of phase 2 read their operands as bf16
+// planes (8 digits for emulated FP64, 3 pieces for the FP32-class mode) that
+// OP_SPLIT tasks have written once, in the layout the tensor core reads, so a
+// product part is bulk copies and MMAs with no conversion. A plane group holds
+// 64 vectors (rows of a left-hand operand, columns of a right-hand one) and the
+// whole K of one tile, K padded to stages of 16:
+//   emulated FP64: int32 exponent of vector v in K chunk ch (512 of K) at
+//   [64 ch + v], then the stages; FP32-class: the stages alone.
+// A stage is NP planes x 64 vectors x 16 K of bf16 in core matrices of 8 x 8;
+// left-hand: plane order of the MMA's row stacks, 64 vectors each; right-hand:
+// two halves of 32 vectors, planes in order.
+// Offsets in BUF_P count units of 16 bytes.
+constexpr int kPlaneChunk = 512;  // K per exponent (the most that cells sum exactly)
+constexpr int kPlaneK = 16;       // K per stage
+inline int plane_count(int prec) { return prec == PREC_EMU64 ? 8 : 3; }
+inline int64_t plane_stages(int k) { return (k + kPlaneK - 1) / kPlaneK; }
+inline int64_t plane_chunks(int k) { return (k + kPlaneChunk - 1) / kPlaneChunk; }
+inline int64_t plane_head(int prec, int k) { return prec == PREC_EMU64 ? 16 * plane_chunks(k) : 0; }
+inline int64_t plane_group(int prec, int k) {  // units of one group
+  return plane_head(prec, k) + plane_stages(k) * 128 * plane_count(prec);
+}
 
 // Sub-tile of part q of an m x n block (rm or cn <= 0: nothing to do).
 struct Sub {
@@ -90,6 +118,7 @@ inline Sub part_sub(int pmode, int m, int n, int q) {
     case PM_ROWS2: s.r0 = 32 * q; s.rm = 32; break;
     case PM_ROWS4: s.r0 = 16 * q; s.rm = 16; break;
     case PM_ROWS8: s.r0 = 8 * q; s.rm = 8; break;
+    case PM_COLS2: s.c0 = 32 * q; s.cn = 32; break;
     case PM_QUAD4: dim = 32; s.r0 = 32 * (q & 1); s.c0 = 32 * (q >> 1); break;
     case PM_TRI3: dim = 32; s.r0 = q == 0 ? 0 : 32; s.c0 = q == 2 ? 32 : 0; break;
     case PM_TILE32: {
@@ -187,7 +216,12 @@ struct Shape {
   int prec = PREC_FP64;  // precision of the off-diagonal bulk products (Precision)
   int tune = 0;          // tuning code (see above)
   int sel0 = 0;          // selected inversion of tile columns >= sel0 only (their phase 1 and 2)
+  bool planes = false;   // reduced precisions: phase-2 products from planes
 };
+
+// Phase-2 products of reduced-precision plans read planes from this tile order
+// on (a rule on b: see use_planes in plan.cpp).
+bool use_planes(const Shape& s);
 
 // A task with few successors is counted off them by each of its parts as it
 // finishes (one atomic per successor and part, no join of the parts on the
@@ -200,15 +234,16 @@ inline bool counts_parts(const Task& t) { return t.nsucc <= kPartSucc; }
 
 // Dynamic schedule: a task becomes ready when the last part of its last
 // predecessor finishes (device counter rem[t], initialised to rem0[t]) and is
-// pushed into the bucket of its expected start time in the list schedule;
+// pushed into the bucket of its queue position (by bottom level);
 // workers pop from the earliest non-empty bucket. Buckets hold kTasksPerBucket
-// consecutive tasks of the list-schedule order.
+// consecutive tasks of that order.
 constexpr int kTasksPerBucket = 64;
 constexpr int kMaxParts = 16;  // parts of one task; a queue entry is kMaxParts * task + part
 constexpr int kMaxTasks = (1 << 27) - 1;  // entries stay positive 32-bit integers
 
 struct Plan {
-  std::vector<Task> tasks;  // in list-schedule order
+  int64_t plane_units = 0;  // BUF_P: units of 16 bytes (0: no product reads planes)
+  std::vector<Task> tasks;  // in queue order
   std::vector<Seg> segs;
   std::vector<Wait> waits;  // counter form of the dependencies (host checks)
   std::vector<int32_t> sigs;
@@ -260,8 +295,9 @@ struct Layout {
   }
 };
 
-// Build the task table of one plan kind, ordered by a list schedule on
-// `workers` persistent workers. Returns 0 or a negative stiles status code.
+// Build the task table of one plan kind, ordered by bottom level; workers > 0:
+// also the makespan of its list schedule on so many workers (statistics).
+// Returns 0 or a negative stiles status code.
 int build_plan(const Shape& s, PlanKind kind, int workers, Plan* out);
 
 // Consistency check of a task table: every wait names an existing counter

@@ -85,9 +85,8 @@ struct stiles_handle {
   DevStatus* dstatus = nullptr;  // one block per plan kind
   double* dlogdet = nullptr;
   int ndiag = 0;
-  size_t state_ints_max = 0;
   size_t w_bytes = 0;        // scratch: L^{-1} and U tiles (packed layout)
-  size_t ctr_offset = 0;     // scratch: scheduler state start (bytes)
+  size_t ctr_offset = 0;     // scratch: planes (if any) from w_bytes on, scheduler state from here on
   size_t scratch_bytes = 0;
   unsigned long long* dtrace = nullptr;  // optional per-task trace (STILES_OPT_TRACE)
   size_t trace_tasks = 0;
@@ -144,6 +143,25 @@ extern "C" int stiles_create_selected(int nt, int b, int band, int arrow, int pr
   return create_handle(nt, b, band, arrow, precision, 0, first_column, out);
 }
 
+// The three plans of a handle's shape and the scratch layout they need: L^-1 and
+// U tiles, planes, scheduler state.
+static int build_handle_plans(stiles_handle* h) {
+  size_t state = 0;
+  int64_t units = 0;
+  for (int k = 0; k < 3; ++k) {
+    Plan& p = h->plans[k];
+    const int rc = build_plan(h->s, (PlanKind)k, 0, &p);
+    if (rc) return rc;
+    const size_t ints = sched_state_ints((int)p.tasks.size(), p.nbuckets, (int)p.slots0.size(), p.urgent_parts);
+    state = ints > state ? ints : state;
+    units = p.plane_units > units ? p.plane_units : units;
+  }
+  h->w_bytes = align_up((size_t)Layout(h->s).doubles() * sizeof(double), 256);
+  h->ctr_offset = align_up(h->w_bytes + 16 * (size_t)units, 256);
+  h->scratch_bytes = align_up(h->ctr_offset + sizeof(int) * state, 256);
+  return 0;
+}
+
 static int create_handle(int nt, int b, int band, int arrow, int precision, int tuning, int first_column,
                          stiles_t* out) {
   if (!out) return STILES_ERR_INVALID_ARG;
@@ -160,12 +178,21 @@ static int create_handle(int nt, int b, int band, int arrow, int precision, int 
     return STILES_ERR_CUDA;
   }
   h->grid = h->sms * kCtasPerSm;
-  for (int k = 0; k < 3; ++k) {
-    int rc = build_plan(h->s, (PlanKind)k, h->grid, &h->plans[k]);
-    if (rc) {
-      delete h;
-      return rc;
+  h->s.planes = use_planes(h->s);
+  int brc = build_handle_plans(h);
+  // Planes may not push a shape out of the fixed no-allocation scratch: one
+  // that fits it without them keeps the products without.
+  if (!brc && h->s.planes && h->scratch_bytes > STILES_NOALLOC_SCRATCH_BYTES && h->w_bytes <= STILES_NOALLOC_SCRATCH_BYTES) {
+    h->s.planes = false;
+    brc = build_handle_plans(h);
+    if (!brc && h->scratch_bytes > STILES_NOALLOC_SCRATCH_BYTES) {
+      h->s.planes = true;
+      brc = build_handle_plans(h);
     }
+  }
+  if (brc) {
+    delete h;
+    return brc;
   }
   int rc = 0;
   for (int k = 0; k < 3 && !rc; ++k) {
@@ -181,7 +208,6 @@ static int create_handle(int nt, int b, int band, int arrow, int precision, int 
     h->dev[k].nbuckets = p.nbuckets;
     h->dev[k].nslots = (int)p.slots0.size();
     h->dev[k].ucap = p.urgent_parts;
-    if (img.size() > h->state_ints_max) h->state_ints_max = img.size();
     if (p.ndiag > h->ndiag) h->ndiag = p.ndiag;
   }
   if (!rc) rc = dev_malloc((void**)&h->dstatus, 3 * sizeof(DevStatus));
@@ -191,10 +217,6 @@ static int create_handle(int nt, int b, int band, int arrow, int precision, int 
     return rc;
   }
   h->mirror_ok = sigma_writes_in_sigma(h->plans[PLAN_FUSED]);
-  Layout L(h->s);
-  h->w_bytes = align_up((size_t)L.doubles() * sizeof(double), 256);
-  h->ctr_offset = h->w_bytes;
-  h->scratch_bytes = align_up(h->ctr_offset + sizeof(int) * h->state_ints_max, 256);
   *out = h;
   return STILES_OK;
 }
@@ -244,6 +266,7 @@ static int launch(stiles_t h, int kind, const double* A, double* L, double* S, v
   p.buf[BUF_L] = L;
   p.buf[BUF_S] = S;
   p.buf[BUF_W] = (double*)scr;
+  p.planes = (uint8_t*)scr + h->w_bytes;
   p.smirror = smirror;
   p.budget_ns = h->budget_ns;
   p.use_tc = h->s.prec != PREC_FP64;
@@ -446,8 +469,9 @@ extern "C" int stiles_plan_stats(int nt, int b, int band, int arrow, int which, 
     return STILES_ERR_INVALID_ARG;
   if (nt < 1 || b < 1 || band < 0 || arrow < 0) return STILES_ERR_INVALID_ARG;
   Plan p;
-  int rc = build_plan(Shape{nt, b, band < nt - 1 ? band : nt - 1, arrow, prec, tune, sel0}, (PlanKind)kind, workers,
-                      &p);
+  Shape sh{nt, b, band < nt - 1 ? band : nt - 1, arrow, prec, tune, sel0};
+  sh.planes = use_planes(sh);
+  int rc = build_plan(sh, (PlanKind)kind, workers, &p);
   if (rc) return rc;
   stats[0] = (long long)p.tasks.size();
   stats[1] = (long long)p.segs.size();
@@ -471,9 +495,10 @@ extern "C" int stiles_debug_validate(int nt, int b, int band, int arrow, int whi
   const int kind = which & 15, prec = (which >> 4) & 15, tune = (which >> 8) & 255, sel0 = which >> 16;
   if (kind < 0 || kind > 2 || prec > PREC_FP32X || !tune_valid(tune) || nt < 1 || b < 1 || band < 0 || arrow < 0)
     return STILES_ERR_INVALID_ARG;
-  const Shape sh{nt, b, band < nt - 1 ? band : nt - 1, arrow, prec, tune, sel0};
+  Shape sh{nt, b, band < nt - 1 ? band : nt - 1, arrow, prec, tune, sel0};
+  sh.planes = use_planes(sh);
   Plan p;
-  int rc = build_plan(sh, (PlanKind)kind, 304, &p);
+  int rc = build_plan(sh, (PlanKind)kind, 0, &p);
   return rc ? rc : validate_plan(p, sh, kind);
 }
 
@@ -506,9 +531,10 @@ extern "C" int stiles_debug_race_check(int nt, int b, int band, int arrow, int w
   if (kind < 0 || kind > 2 || prec > PREC_FP32X || !tune_valid(tune) || nt < 1 || b < 1 || band < 0 || arrow < 0 ||
       plant < 0 || plant > 2)
     return STILES_ERR_INVALID_ARG;
-  const Shape sh{nt, b, band < nt - 1 ? band : nt - 1, arrow, prec, tune, sel0};
+  Shape sh{nt, b, band < nt - 1 ? band : nt - 1, arrow, prec, tune, sel0};
+  sh.planes = use_planes(sh);
   Plan p;
-  const int rc = build_plan(sh, (PlanKind)kind, 304, &p);
+  const int rc = build_plan(sh, (PlanKind)kind, 0, &p);
   if (rc) return rc;
   if (plant == 2) {
     if (!plant_unjoined_column(p)) return STILES_ERR_INVALID_ARG;
@@ -523,7 +549,7 @@ extern "C" int stiles_debug_race_check_serve(int nt, int b, int band, int arrow,
     return STILES_ERR_INVALID_ARG;
   const Shape sh{nt, b, band < nt - 1 ? band : nt - 1, arrow, precision, tuning};
   Plan p;
-  const int rc = build_serve_template(sh, 304, &p);
+  const int rc = build_serve_template(sh, 0, &p);
   return rc ? rc : race_check_plan(p, Layout(sh).doubles(), plant, true);
 }
 
@@ -536,10 +562,9 @@ extern "C" int stiles_debug_check_corrupted(int nt, int b, int band, int arrow, 
   switch (mode) {
     case 1: p.waits.back().ctr = p.nctr; break;
     case 2: p.waits.back().need += 1000000; break;
-    case 3: {  // make the first task that waits depend on the last task's signal
-      const size_t nt_ = p.tasks.size();
-      if (p.sig_off[nt_] <= p.sig_off[nt_ - 1]) return STILES_ERR_INVALID_ARG;
-      p.waits.front() = Wait{p.sigs[p.sig_off[nt_ - 1]], 1 << 20};
+    case 3: {  // make the first task that waits depend on the last signal of the table
+      if (p.sigs.empty()) return STILES_ERR_INVALID_ARG;
+      p.waits.front() = Wait{p.sigs.back(), 1 << 20};
       break;
     }
     default: return STILES_ERR_INVALID_ARG;
@@ -663,7 +688,8 @@ extern "C" int stiles_batch_create(int count, const int* nt, const int* b, const
       delete h;
       return STILES_ERR_INVALID_ARG;
     }
-    const Shape s{nt[m], b[m], band[m] < nt[m] - 1 ? band[m] : nt[m] - 1, arrow[m], precision, tune};
+    Shape s{nt[m], b[m], band[m] < nt[m] - 1 ? band[m] : nt[m] - 1, arrow[m], precision, tune};
+    s.planes = use_planes(s);
     h->shapes.push_back(s);
     h->off[m + 1] = (int64_t)align_up((size_t)(h->off[m] + Layout(s).doubles()), 32);
   }
@@ -674,7 +700,7 @@ extern "C" int stiles_batch_create(int count, const int* nt, const int* b, const
   }
   h->grid = h->sms * kCtasPerSm;
   std::vector<int64_t> base(h->off.begin(), h->off.end() - 1);
-  int rc = build_batch_plan(h->shapes, base, h->grid, &h->plan, &h->diag_base);
+  int rc = build_batch_plan(h->shapes, base, 0, &h->plan, &h->diag_base);
   if (rc) {
     delete h;
     return rc;
@@ -716,7 +742,7 @@ extern "C" int stiles_batch_create(int count, const int* nt, const int* b, const
   p.succ_off.clear(); p.succ_off.shrink_to_fit();
   p.slots0.clear(); p.slots0.shrink_to_fit();
   h->w_bytes = align_up((size_t)h->off[count] * sizeof(double), 256);
-  h->ctr_offset = h->w_bytes;
+  h->ctr_offset = align_up(h->w_bytes + 16 * (size_t)p.plane_units, 256);
   h->scratch_bytes = align_up(h->ctr_offset + sizeof(int) * h->dev.image_ints, 256);
   *out = h;
   return STILES_OK;
@@ -762,6 +788,7 @@ static int build_batch_graph(stiles_batch* h, const double* A, double* L, double
   p.buf[BUF_L] = L;
   p.buf[BUF_S] = S;
   p.buf[BUF_W] = (double*)scr;
+  p.planes = (uint8_t*)scr + h->w_bytes;
   p.budget_ns = h->budget_ns;
   p.use_tc = h->prec != PREC_FP64;
   p.trace = nullptr;
@@ -963,12 +990,13 @@ extern "C" int stiles_debug_validate_batch(int count, const int* nt, const int* 
     const int tune = tuning ? tuning[m] : 0;
     if (nt[m] < 1 || b[m] < 1 || band[m] < 0 || arrow[m] < 0 || !tune_valid(tune)) return STILES_ERR_INVALID_ARG;
     shapes.push_back(Shape{nt[m], b[m], band[m] < nt[m] - 1 ? band[m] : nt[m] - 1, arrow[m], precision, tune});
+    shapes.back().planes = use_planes(shapes.back());
     base.push_back(off);
     off = (int64_t)align_up((size_t)(off + Layout(shapes.back()).doubles()), 32);
   }
   Plan p;
   std::vector<int32_t> diag_base;
-  const int rc = build_batch_plan(shapes, base, 304, &p, &diag_base);
+  const int rc = build_batch_plan(shapes, base, 0, &p, &diag_base);
   return rc ? rc : validate_plan_len(p, off, PLAN_FUSED);
 }
 
@@ -983,12 +1011,13 @@ extern "C" int stiles_debug_race_check_batch(int count, const int* nt, const int
     const int tune = tuning ? tuning[m] : 0;
     if (nt[m] < 1 || b[m] < 1 || band[m] < 0 || arrow[m] < 0 || !tune_valid(tune)) return STILES_ERR_INVALID_ARG;
     shapes.push_back(Shape{nt[m], b[m], band[m] < nt[m] - 1 ? band[m] : nt[m] - 1, arrow[m], precision, tune});
+    shapes.back().planes = use_planes(shapes.back());
     base.push_back(off);
     off = (int64_t)align_up((size_t)(off + Layout(shapes.back()).doubles()), 32);
   }
   Plan p;
   std::vector<int32_t> diag_base;
-  const int rc = build_batch_plan(shapes, base, 304, &p, &diag_base);
+  const int rc = build_batch_plan(shapes, base, 0, &p, &diag_base);
   return rc ? rc : race_check_plan(p, off, plant);
 }
 
@@ -997,7 +1026,7 @@ extern "C" int stiles_debug_validate_serve(int nt, int b, int band, int arrow, i
     return STILES_ERR_INVALID_ARG;
   const Shape sh{nt, b, band < nt - 1 ? band : nt - 1, arrow, precision, tuning};
   Plan p;
-  const int rc = build_serve_template(sh, 304, &p);
+  const int rc = build_serve_template(sh, 0, &p);
   if (rc) return rc;
   int roots_prep = 0, roots = 0;
   for (size_t t = 0; t < p.tasks.size(); ++t)

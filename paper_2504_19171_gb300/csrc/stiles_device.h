@@ -118,6 +118,7 @@ struct KParams {
   DevStatus* st;        // status block (reset before the launch)
   double* logdet_part;  // one partial sum of log diag(L) per POTRF task
   double* buf[4];       // BUF_A, BUF_L, BUF_S, BUF_W base pointers
+  uint8_t* planes;      // BUF_P base pointer (units of 16 bytes), or null
   double* smirror;      // optional: second copy of every final Sigma write, same layout as buf[BUF_S]
                         // (a host buffer mapped into the device's address space), or null
   long long budget_ns;  // bound of one dependency wait

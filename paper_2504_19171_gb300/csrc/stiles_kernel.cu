@@ -7,7 +7,7 @@
 // device form of Algorithm 3's "WaitForTile / SignalTileReady" flags); the
 // finisher pushes its parts into a queue, and idle workers claim parts with
 // fetch-and-add on availability counters. Static plans queue parts in
-// buckets of the host's list-schedule order behind an urgent FIFO for the
+// buckets of the host's critical-path order behind an urgent FIFO for the
 // factorization's frontier; the request server (serve mode) uses three FIFO
 // rings and activates new requests from a host-mapped inbox while it runs.
 // Every wait is bounded by %globaltimer and ends the launch with a TIMEOUT
@@ -26,6 +26,7 @@
 // load each block) and every final Sigma write is repeated into a host
 // buffer, so the transfers overlap the computation.
 #include <cuda/atomic>
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -635,159 +636,88 @@ __device__ __forceinline__ void accumulate(const KParams& p, const Task& tk, con
 
 // ---- split-precision block products on the tensor cores (tcgen05) -------
 //
-// Error-free splitting in the manner of Ozaki, Ogita, Oishi and Rump. For one
-// task part (at most 32 x 32 outputs) every row i of op(A) gets the biased
-// exponent E_i of its largest entry over all the task's segments and every
-// column j of op(B) the exponent F_j. Each entry becomes a signed fixed-point
-// integer X relative to that exponent, |X| < 2^(DB S - 2) (the largest entry
-// of the row keeps its 53-bit significand in the emulated-FP64 mode; the
-// others are rounded to the same unit), written as S balanced base-2^DB
-// digits d_t in [-2^(DB-1), 2^(DB-1)), X = sum_t d_t 2^(DB (S-1-t)), which
-// bf16 holds exactly. A digit product is an integer of magnitude at most
-// 2^(2 DB - 2); products of levels L = t + u <= S - 1 are kept. Emulated FP64
-// uses S = 8 digits of DB = 8 bits (|X| < 2^62: entries down to 2^-9 of their
-// row maximum keep all 53 bits, the dropped levels weigh below 2^-56 of the
-// leading product). The FP32-class mode uses no shared exponent: every entry
-// becomes its FP32 value (rounded to nearest) written as three bf16 pieces
-// that keep their own exponents (piece_pairs), in the same four-plane layout
-// with a zero fourth plane; its cells hold ordinary FP32 sums.
+// Error-free splitting in the manner of Ozaki, Ogita, Oishi and Rump. Emulated
+// FP64: every vector (row of op(A), column of op(B)) gets, per stretch of K, the
+// biased exponent of its largest entry; each entry becomes a signed fixed-point
+// integer X relative to that exponent, |X| < 2^62 (the largest entry keeps its
+// 53-bit significand, and so does every entry down to 2^-9 of it), written as 8
+// balanced base-2^8 digits d_t in [-128, 128), X = sum_t d_t 2^(8 (7 - t)), which
+// fp16 holds exactly. Digit products of levels t + u <= 7 are kept (36 of 64; the
+// dropped levels weigh below 2^-56 of the leading product). FP32-class: no shared
+// exponent; every entry becomes its FP32 value (rounded to nearest) written as
+// three bf16 pieces that keep their own exponents (piece_pairs), the 8 products
+// of levels <= 3 accumulate in FP32.
 //
-// Tensor-core layout. D has M = 128 rows, made from a 32-row part by
-// stacking four digit planes of A: stack g (g < G = S / 4) holds plane
-// g + G p in rows 32 p + i (p = 0..3). The B planes are concatenated along
-// N ([B_0 | B_1 | ... | B_{S-1}], 32 columns each). Stack g is multiplied by
-// the first 32 (S - g) columns of that concatenation into TMEM columns from
-// 32 g on, so TMEM cell (lane block p, column block c) collects the plane
-// pairs (g + G p, c - g), all of one level L = G p + c. A cell receives at
-// most G pairs per K step: in the emulated-FP64 mode its FP32 sums are
-// integers of magnitude at most 2^24, hence exact, for up to
-// 2^24 / (G 2^14) = 512 of K.
-// Before that much K has been accumulated (or at the end of the task) the
-// cells of levels <= S - 1 are read -- warp p reads lane block p -- and
-// combined per output: exactly in two 64-bit halves for emulated FP64, then
-// scaled by 2^(E_i + F_j - bias); summed in FP32 for the FP32-class mode. The
-// result is added to the part's FP64 value.
+// A part is 64 x 32 outputs. Its MMAs have M = 128: two planes of A (64 rows)
+// stacked. Emulated FP64: stack g (planes g, g + 4 in rows 0-63, 64-127) times
+// the first 32 (8 - g) columns of [B_0 | .. | B_7] into TMEM columns from 32 g:
+// cell (p, c) collects the pairs of level 4 p + c, at most 4 per K, so its FP32
+// sum is an integer of magnitude at most 2^24, exact, for 256 of K. 8 levels of
+// 32 columns are the 256 TMEM columns of each of two CTAs per SM. FP32-class:
+// planes 0, 1 stacked times [B_0 | B_1 | B_2] into columns 0-95, plane 2 times
+// [B_0 | B_1] into 96-159: every plane pair sums in a cell of its own, over up to
+// 4096 of K. Then the cells are drained: read, combined per output (exactly, for
+// emulated FP64) and added to the part's FP64 result in registers.
 // Non-finite operands make their row or column NaN (emulated FP64: biased
-// exponent 0x7ff; FP32-class: NaN pieces, also for values beyond the FP32
-// range).
-
-constexpr int TC_KS = 32;           // K per staging buffer (two MMA K steps)
-constexpr uint32_t TC_COLS = 256;   // TMEM columns per CTA (two CTAs per SM share 512)
-constexpr int TC_STAGE_BYTES_MAX = 2 * 32 * 8 * TC_KS * 2;  // A and B digit planes of S = 8
-// shared memory of a tensor part: two staging buffers, the row / column
-// exponents, then the part's FP64 result (32 x 33 doubles)
-constexpr int TC_EXP_OFF = 2 * TC_STAGE_BYTES_MAX;
-constexpr int TC_RES_OFF = TC_EXP_OFF + 64 * 4;
-constexpr int TC_SMEM_BYTES = TC_RES_OFF + 32 * 33 * 8;
-
-// Per-CTA state of the tensor path (static shared memory of the kernel).
-struct TcShared {
-  uint64_t mbar[2];      // completion barriers of the two staging buffers
-  uint32_t ncommit[2];   // commits issued to each barrier so far (this launch)
-  uint32_t tmem;         // TMEM base address of this CTA's TC_COLS columns
-};
+// exponent 0x7ff; FP32-class: NaN pieces, also beyond the FP32 range).
+//
+// Operands reach shared memory in one of two ways, in the same layout:
+//   * run_planes: phase 2's operands, each read by many products, are split once
+//     into planes in global memory (OP_SPLIT) and copied in whole stages;
+//   * run_tc: a part loads its operands 64 of K at a time into registers, takes
+//     the exponents there and writes the digits itself (factor updates, TRMM).
 
 __device__ __forceinline__ int biased_exp(double v) {
   return (int)((__double_as_longlong(v) >> 52) & 0x7ff);
 }
 
-// out[i] = max(out[i], largest biased exponent over k < K of element (i, k))
-// of a panel of n <= 32 vectors: element (i, k) sits at P[i + k ld] when
-// `along_i` (the vectors' index is the contiguous one), else at P[k + i ld].
-// Loads follow the contiguous dimension, 16 independent ones in flight per
-// thread. Ends with a block barrier.
-__device__ __forceinline__ void max_exp_into(const double* P, int ld, bool along_i, int n, int K, int* out) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  constexpr int U = 16;
-  if (along_i) {  // lanes over i, warps over k (k = warp + 4 u)
-    int mx = 0;
-    if (lane < n)
-      for (int k0 = warp; k0 < K; k0 += 4 * U) {
-        double v[U];
-#pragma unroll
-        for (int u = 0; u < U; ++u) v[u] = k0 + 4 * u < K ? __ldcg(P + lane + (int64_t)(k0 + 4 * u) * ld) : 0.0;
-#pragma unroll
-        for (int u = 0; u < U; ++u) mx = max(mx, biased_exp(v[u]));
-      }
-    __shared__ int part[4][32];
-    part[warp][lane] = mx;
-    __syncthreads();
-    if (warp == 0) out[lane] = max(out[lane], max(max(part[0][lane], part[1][lane]), max(part[2][lane], part[3][lane])));
-  } else {  // lanes over k; warp w takes vectors w, w + 4, ..., w + 28 at once (two k per lane)
-    int mx[8];
-#pragma unroll
-    for (int v = 0; v < 8; ++v) mx[v] = 0;
-    for (int k0 = lane; k0 < K; k0 += 64) {
-      double x[8][2];
-#pragma unroll
-      for (int v = 0; v < 8; ++v) {
-        const int i = warp + 4 * v;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int k = k0 + 32 * h;
-          x[v][h] = (i < n && k < K) ? __ldcg(P + k + (int64_t)i * ld) : 0.0;
-        }
-      }
-#pragma unroll
-      for (int v = 0; v < 8; ++v) mx[v] = max(mx[v], max(biased_exp(x[v][0]), biased_exp(x[v][1])));
-    }
-#pragma unroll
-    for (int v = 0; v < 8; ++v) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) mx[v] = max(mx[v], __shfl_xor_sync(0xffffffffu, mx[v], o));
-      if (lane == 0) out[warp + 4 * v] = max(out[warp + 4 * v], mx[v]);
-    }
-  }
-  __syncthreads();
-}
+constexpr uint32_t TC_COLS = 256;   // TMEM columns per CTA (two CTAs per SM share 512)
 
-// Signed fixed-point value of v relative to the biased exponent emax of its
-// row or column (emax >= its own), rounded to nearest: the row maximum maps
-// to [2^(BITS-1), 2^BITS).
-template <int BITS>
-__device__ __forceinline__ long long fixed_point(double v, int emax) {
+// Per-CTA state of the tensor path (static shared memory of the kernel).
+constexpr int PL_SLOTS = 8;         // staging slots of a product from planes, at most
+struct TcShared {
+  uint64_t pfull[PL_SLOTS];   // products from planes: a slot's copies have landed
+  uint64_t pempty[PL_SLOTS];  // ... its MMAs are done
+  uint64_t pdone;             // every MMA issued before is done
+  uint32_t pstage;       // stages this CTA has run so far: stage g is slot g % NST, phase g / NST
+  uint32_t pdone_n;      // phases of pdone
+  uint32_t tmem;         // TMEM base address of this CTA's TC_COLS columns
+};
+
+
+// Signed fixed-point value of v relative to the biased exponent emax of its row
+// or column (emax >= its own), rounded to nearest: the row maximum maps to
+// [2^61, 2^62).
+__device__ __forceinline__ unsigned long long fixed_point(double v, int emax) {
   const unsigned long long bits = (unsigned long long)__double_as_longlong(v);
   const int e = (int)((bits >> 52) & 0x7ff);
-  const long long m = (long long)((bits & 0xFFFFFFFFFFFFFull) | (e ? (1ull << 52) : 0ull));
-  const int sh = max(emax, 1) - max(e, 1) + 53 - BITS;  // >= 53 - BITS
-  long long X;
-  if (sh < 0) X = m << -sh;
-  else if (sh == 0) X = m;
-  else if (sh < 63) X = (m + (1ll << (sh - 1))) >> sh;
-  else X = 0;
-  return (bits >> 63) ? -X : X;
+  const int d = max(emax, 1) - max(e, 1);
+  const unsigned long long m = d > 62 ? 0ull : (bits & 0xFFFFFFFFFFFFFull) | ((unsigned long long)(e != 0) << 52);
+  const unsigned long long X = (((m << 11) >> (1 + min(d, 62))) + 1) >> 1;
+  const unsigned long long s = 0ull - (bits >> 63);  // all ones for a negative value
+  return (X ^ s) - s;
 }
 
-// C = sum_{t < S} 2^(DB-1) 2^(DB t): X + C has base-2^DB digits d_t + 2^(DB-1).
-template <int S, int DB>
-__host__ __device__ constexpr unsigned long long digit_bias() {
-  unsigned long long c = 0;
-  for (int t = 0; t < S; ++t) c |= 1ull << (DB * t + DB - 1);
-  return c;
-}
-
-// The S digits (DB bits each, balanced) of a pair of K-adjacent values (v0
-// at k, v1 at k + 1) as packed bf16 pairs: w[t] = bf16(d_t(v0)) | bf16(d_t(v1)) << 16.
-template <int S, int DB>
-__device__ __forceinline__ void digit_pairs(double v0, double v1, int emax, uint32_t (&w)[S]) {
-  constexpr int BITS = DB * S - 2;
-  constexpr unsigned long long C = digit_bias<S, DB>();
-  constexpr float kMagic = 8388608.0f + (float)(1 << (DB - 1));  // 2^23 + 2^(DB-1)
-  // in unsigned arithmetic: with DB S = 64 the bias C is above 2^63
-  const unsigned long long y0 = (unsigned long long)fixed_point<BITS>(v0, emax) + C;
-  const unsigned long long y1 = (unsigned long long)fixed_point<BITS>(v1, emax) + C;
-  static_assert(DB == 8 && S <= 8, "byte digits of a 64-bit value");
-  // digit t is byte S - 1 - t of y: one byte permute puts it under the
-  // exponent of 2^23 (bytes 0x00, 0x00, 0x4B above it); the float minus
-  // 2^23 + 2^(DB-1) is the digit exactly, and its bf16 is its upper half
+// The 8 digits (balanced, base 2^8) of a pair of K-adjacent values (v0 at k, v1
+// at k + 1) as packed fp16 pairs: w[t] = d_t(v0) | d_t(v1) << 16. With 128 added
+// to every digit they are the bytes of the fixed-point value plus the bias C, top
+// byte first; a byte under 0x64 is the fp16 value 1024 + byte, and one packed
+// subtraction of 1152 leaves the digits exactly (two permutes and one subtraction
+// per pair and digit; through FP32 and bf16 it took five instructions).
+__device__ __forceinline__ void digit_pairs(double v0, double v1, int emax, uint32_t (&w)[8]) {
+  constexpr unsigned long long C = 0x8080808080808080ull;
+  const unsigned long long y0 = fixed_point(v0, emax) + C, y1 = fixed_point(v1, emax) + C;
   const uint32_t h0[2] = {(uint32_t)y0, (uint32_t)(y0 >> 32)}, h1[2] = {(uint32_t)y1, (uint32_t)(y1 >> 32)};
+  const __half2 bias = __halves2half2(__ushort_as_half(0x6480), __ushort_as_half(0x6480));  // 1152
 #pragma unroll
-  for (int t = 0; t < S; ++t) {
-    const int bi = S - 1 - t;
-    const uint32_t sel = 0x7540u | (uint32_t)(bi & 3);
-    const float f0 = __uint_as_float(__byte_perm(h0[bi >> 2], 0x4B000000u, sel)) - kMagic;
-    const float f1 = __uint_as_float(__byte_perm(h1[bi >> 2], 0x4B000000u, sel)) - kMagic;
-    w[t] = __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);
+  for (int h = 0; h < 2; ++h) {
+    const uint32_t lo = __byte_perm(h0[h], h1[h], 0x5140), hi = __byte_perm(h0[h], h1[h], 0x7362);  // byte pairs 0, 1; 2, 3
+#pragma unroll
+    for (int b = 0; b < 4; ++b) {
+      const uint32_t u = __byte_perm(b < 2 ? lo : hi, 0x64646464u, b & 1 ? 0x4342 : 0x4140);
+      const __half2 f = __hsub2(*reinterpret_cast<const __half2*>(&u), bias);
+      w[7 - (4 * h + b)] = *reinterpret_cast<const uint32_t*>(&f);  // digit t is byte 7 - t
+    }
   }
 }
 
@@ -826,28 +756,6 @@ __device__ __forceinline__ void piece_pairs(double v0, double v1, uint32_t (&w)[
   w[3] = 0u;
 }
 
-// Byte offset of element (row, k) (k even: a packed pair) in a staging
-// operand of canonical K-major core matrices: 8 rows x 8 K per 128 bytes,
-// TC_KS / 8 core matrices along K per 8-row group.
-__device__ __forceinline__ uint32_t tc_off(int row, int k) {
-  return (uint32_t)((((row >> 3) * (TC_KS / 8) + (k >> 3)) << 7) + ((row & 7) << 4) + ((k & 7) << 1));
-}
-constexpr uint32_t TC_LBO = 128;                 // K-adjacent core matrices
-constexpr uint32_t TC_SBO = (TC_KS / 8) * 128;   // 8-row groups
-
-// Panel element owned by slot q (0..3) of this thread, for a stage of 32
-// vectors x TC_KS: vector index `vi` and the even K offset `kk` of its pair.
-// Warp w takes the 8-vector group w, slot q the K core matrix q, and lane
-// (r, kp) = (lane % 8, lane / 8) the vector 8 w + r and K pair kp of it: the
-// warp's 32 packed-pair stores then fill the 32 words of one core matrix
-// (no shared-memory bank conflict), and its loads read 8 x 64 contiguous
-// bytes whichever dimension of the operand is the contiguous one.
-__device__ __forceinline__ void tc_slot(int q, int& vi, int& kk) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  vi = 8 * warp + (lane & 7);
-  kk = 8 * q + 2 * (lane >> 3);
-}
-
 // Bounded wait for phase `parity` of a staging barrier (all threads).
 __device__ bool tc_wait(const KParams& p, uint32_t mbar, uint32_t parity) {
   if (tc::mbar_test(mbar, parity)) return true;
@@ -861,279 +769,580 @@ __device__ bool tc_wait(const KParams& p, uint32_t mbar, uint32_t parity) {
   return true;
 }
 
-// Raw values of one stage (TC_KS of K from k0) of the part's operands, as
-// this thread's four K-adjacent pairs of op(A) and of op(B) (zero outside
-// the part or the segment).
-__device__ __forceinline__ void tc_load(const double* A, const double* B, const Seg& gs, const Sub& sb, int k0,
-                                        double (&va)[8], double (&vb)[8]) {
-  const bool ta = gs.trans & 1, tb = gs.trans & 2;
-  const int kc = min(TC_KS, gs.k - k0);
+template <int S>
+struct PlaneFmt {
+  static constexpr int NP = S == 8 ? 8 : 3;              // planes
+  static constexpr int A_BYTES = 64 * kPlaneK * 2 * NP;  // a stage of a left-hand group
+  static constexpr int B_BYTES = A_BYTES / 2;            // half a stage of a right-hand group
+  static constexpr int STAGE = A_BYTES + B_BYTES;
+  static constexpr int NST = S == 8 ? 4 : 8;             // staging slots
+  // K that cells sum: exactly (emulated FP64), or with FP32 rounding
+  static constexpr int KMAX = S == 8 ? 256 : 4096;
+  static_assert(NST <= PL_SLOTS, "slots");
+};
+constexpr int PL_STAGE_BYTES = 4 * PlaneFmt<8>::STAGE;
+static_assert(8 * PlaneFmt<4>::STAGE + 4096 <= PL_STAGE_BYTES, "an MMA of plane 2 reads one plane beyond its stage");
+constexpr int PL_XCH_OFF = PL_STAGE_BYTES;            // exchange between the warps of two lane blocks
+constexpr int PL_XCH_BYTES = 64 * 8 * 3 * 8;          // 64 rows x 8 columns x (high, low; low)
+constexpr int PL_EXP_OFF = PL_XCH_OFF + PL_XCH_BYTES;  // exponents: 32 columns; run_tc's partial ones
+constexpr int PL_SMEM_BYTES = PL_EXP_OFF + (32 + 4 * 96) * 4;
+constexpr uint32_t PL_LBO = 128, PL_SBO = 256;        // K- and row-adjacent core matrices of a stage
+
+// One thread: the MMAs of one stage (16 of K) at shared address a0, adding to the
+// cells or (acc = false) starting them.
+template <int S>
+__device__ __forceinline__ void stage_mmas(uint32_t tmem, uint32_t a0, bool acc) {
+  const uint64_t bd = tc::smem_desc(a0 + PlaneFmt<S>::A_BYTES, PL_LBO, PL_SBO);
+  if constexpr (S == 8) {
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    int i, kk;
-    tc_slot(q, i, kk);
-    const double* P = ta ? A + (int64_t)(k0 + kk) + (int64_t)i * gs.lda : A + (int64_t)i + (int64_t)(k0 + kk) * gs.lda;
-    const int64_t step = ta ? 1 : gs.lda;
-    va[2 * q] = (i < sb.rm && kk < kc) ? __ldcg(P) : 0.0;
-    va[2 * q + 1] = (i < sb.rm && kk + 1 < kc) ? __ldcg(P + step) : 0.0;
-  }
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    int j, kk;
-    tc_slot(q, j, kk);
-    const double* P = tb ? B + (int64_t)j + (int64_t)(k0 + kk) * gs.ldb : B + (int64_t)(k0 + kk) + (int64_t)j * gs.ldb;
-    const int64_t step = tb ? gs.ldb : 1;
-    vb[2 * q] = (j < sb.cn && kk < kc) ? __ldcg(P) : 0.0;
-    vb[2 * q + 1] = (j < sb.cn && kk + 1 < kc) ? __ldcg(P + step) : 0.0;
+    for (int g = 0; g < 4; ++g)
+      tc::mma_f16(tmem + 32 * g, tc::smem_desc(a0 + g * 4096, PL_LBO, PL_SBO), bd, tc::idesc_f16_f32(128, 32 * (8 - g)),
+                   g > 0 || acc ? 1u : 0u);
+  } else {
+    tc::mma_f16(tmem, tc::smem_desc(a0, PL_LBO, PL_SBO), bd, tc::idesc_bf16_f32(128, 96), acc ? 1u : 0u);
+    tc::mma_f16(tmem + 96, tc::smem_desc(a0 + 4096, PL_LBO, PL_SBO), bd, tc::idesc_bf16_f32(128, 64), acc ? 1u : 0u);
   }
 }
 
-// acc (accumulate<2,4> thread mapping: rows tx + 16 i, columns ty + 8 jj) =
-// sum over the task's segments of op(A) op(B) for the sub-tile sb (<= 32 x
-// 32), through S-digit products on the tensor cores (see above). The next
-// stage's operands are loaded while the current one is split into digits.
-template <int S, int DB>
-__device__ void accumulate_tc(const KParams& p, const Task& tk, const Sub& sb, double (&acc)[2][4], double* smem,
-                              TcShared& ts) {
-  // FP32-class parts (S = 4) take per-element FP32 pieces (piece_pairs): no
-  // shared exponents, so no exponent pre-pass and no scaling at the drain
-  constexpr bool FLT = S == 4;
-  constexpr int G = S / 4;                 // stacks of four A planes
-  constexpr int BITS = DB * S - 2;
-  // K accumulated in a TMEM cell before it is read: exactly (integers of
-  // magnitude at most 2^24, at most G products of 2^(2 DB - 2) per K step)
-  // for emulated FP64;
-  // the FP32-class mode only needs FP32 accumulation
-  constexpr int KMAX = S == 8 ? (1 << 24) / (G << (2 * DB - 2)) : 4096;
-  constexpr int ROWS = 32 * S;             // rows of the A stacks and of the B concatenation
-  constexpr uint32_t OPB = ROWS * TC_KS * 2;  // bytes of one operand in a stage
-  // k2 = E_i + F_j - kScale: X_a X_b summed over the kept levels is
-  // 2^(DB (S - 1)) V with V = sum_L S_L 2^(DB (S - 1 - L))
-  constexpr int kScale = 2044 + 2 * BITS - DB * (S - 1);
-  static_assert((S == 8 || S == 4) && DB == 8, "digit formats of the two modes");
-  static_assert(S == 4 || KMAX >= TC_KS, "exact chunk");
-  static_assert(32 * 4 * 32 * 16 <= 2 * TC_STAGE_BYTES_MAX, "drain buffer fits the staging region");
-  uint8_t* stage = reinterpret_cast<uint8_t*>(smem);
-  int* rexp = reinterpret_cast<int*>(stage + TC_EXP_OFF);
-  int* cexp = rexp + 32;
-  // the part's result, row lane, column 4 js + warp owned by thread (warp, lane)
-  double* R = reinterpret_cast<double*>(stage + TC_RES_OFF);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  // A part whose whole K is two stages (one segment of at most 2 TC_KS: the
-  // factor's one-block-column updates) takes the exact row / column exponents
-  // from the two stages' values in registers (in the segment loop below),
-  // read back to back, instead of a pass of its own.
-  bool small = false;
-  if constexpr (!FLT) small = tk.nseg == 1 && load_seg(p, tk.seg0).k <= 2 * TC_KS;
-  if constexpr (!FLT) if (!small) {
-    if (tid < 64) rexp[tid] = 0;
-    __syncthreads();
-    for (int s = 0; s < tk.nseg; ++s) {
-      const Seg gs = load_seg(p, tk.seg0 + s);
-      const bool ta = gs.trans & 1, tb = gs.trans & 2;
-      const double* A = resolve(p, gs.a) + (ta ? (int64_t)sb.r0 * gs.lda : (int64_t)sb.r0);
-      const double* B = resolve(p, gs.b) + (tb ? (int64_t)sb.c0 : (int64_t)sb.c0 * gs.ldb);
-      max_exp_into(A, gs.lda, !ta, sb.rm, gs.k, rexp);
-      max_exp_into(B, gs.ldb, tb, sb.cn, gs.k, cexp);
-    }
-  }
-#pragma unroll
-  for (int js = 0; js < 8; ++js) R[lane * 33 + 4 * js + warp] = 0.0;
-  int nstage = 0, kacc = 0;
-  const uint32_t mb0 = tc::smem_addr(&ts.mbar[0]), mb1 = tc::smem_addr(&ts.mbar[1]);
-  for (int s = 0; s < tk.nseg; ++s) {
-    const Seg gs = load_seg(p, tk.seg0 + s);
-    const bool ta = gs.trans & 1, tb = gs.trans & 2;
-    const double* A = resolve(p, gs.a) + (ta ? (int64_t)sb.r0 * gs.lda : (int64_t)sb.r0);
-    const double* B = resolve(p, gs.b) + (tb ? (int64_t)sb.c0 : (int64_t)sb.c0 * gs.ldb);
-    double na[8], nb[8];  // the next stage's values, in flight
-    tc_load(A, B, gs, sb, 0, na, nb);
-    if (small) {
-      // this thread holds row 8 warp + lane % 8 of op(A) and column 8 warp +
-      // lane % 8 of op(B) at 8 of each stage's K; lanes lane % 8 + 8 m hold the
-      // rest. The second stage is read here for its exponents only (the loop
-      // reads it again as its prefetch, from L2).
-      int ea = 0, eb = 0;
-      if (gs.k > TC_KS) {
-        double xa[8], xb[8];
-        tc_load(A, B, gs, sb, TC_KS, xa, xb);
-#pragma unroll
-        for (int x = 0; x < 8; ++x) {
-          ea = max(ea, biased_exp(xa[x]));
-          eb = max(eb, biased_exp(xb[x]));
-        }
-      }
-#pragma unroll
-      for (int x = 0; x < 8; ++x) {
-        ea = max(ea, biased_exp(na[x]));
-        eb = max(eb, biased_exp(nb[x]));
-      }
-#pragma unroll
-      for (int o = 8; o < 32; o <<= 1) {
-        ea = max(ea, __shfl_xor_sync(0xffffffffu, ea, o));
-        eb = max(eb, __shfl_xor_sync(0xffffffffu, eb, o));
-      }
-      if (lane < 8) {
-        rexp[8 * warp + lane] = ea;
-        cexp[8 * warp + lane] = eb;
-      }
-      __syncthreads();
-    }
-    for (int k0 = 0; k0 < gs.k; k0 += TC_KS) {
-      double ca[8], cb[8];
-#pragma unroll
-      for (int x = 0; x < 8; ++x) {
-        ca[x] = na[x];
-        cb[x] = nb[x];
-      }
-      if (k0 + TC_KS < gs.k) tc_load(A, B, gs, sb, k0 + TC_KS, na, nb);
-      const int buf = nstage & 1;
-      uint8_t* sa = stage + buf * TC_STAGE_BYTES_MAX;
-      uint8_t* sbuf = sa + OPB;
-      // the MMAs that last read this buffer (two stages ago) must be done
-      // (a wait that runs out of budget ends the part on every thread at the barrier below)
-      const bool ok = nstage < 2 || tc_wait(p, buf ? mb1 : mb0, (ts.ncommit[buf] - 1) & 1);
-      if (ok) {
-        // op(A) rows: digit t of row i goes to stack row 128 (t % G) + 32 (t / G) + i
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          int i, kk;
-          tc_slot(q, i, kk);
-          uint32_t w[S];
-          if constexpr (FLT) piece_pairs(ca[2 * q], ca[2 * q + 1], w);
-          else digit_pairs<S, DB>(ca[2 * q], ca[2 * q + 1], rexp[i], w);
-#pragma unroll
-          for (int t = 0; t < S; ++t)
-            *reinterpret_cast<uint32_t*>(sa + tc_off(128 * (t % G) + 32 * (t / G) + i, kk)) = w[t];
-        }
-        // op(B) columns: digit u of column j goes to row 32 u + j
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          int j, kk;
-          tc_slot(q, j, kk);
-          uint32_t w[S];
-          if constexpr (FLT) piece_pairs(cb[2 * q], cb[2 * q + 1], w);
-          else digit_pairs<S, DB>(cb[2 * q], cb[2 * q + 1], cexp[j], w);
-#pragma unroll
-          for (int t = 0; t < S; ++t) *reinterpret_cast<uint32_t*>(sbuf + tc_off(32 * t + j, kk)) = w[t];
-        }
-      }
-      tc::fence_smem_to_async();
-      if (__syncthreads_or(!ok)) return;
-      if (tid == 0) {
-        tc::fence_after_sync();
-        const uint32_t a0 = tc::smem_addr(sa), b0 = tc::smem_addr(sbuf);
-#pragma unroll
-        for (int ks = 0; ks < TC_KS / 16; ++ks)
-#pragma unroll
-          for (int g = 0; g < G; ++g) {
-            const uint64_t ad = tc::smem_desc(a0 + g * (128 / 8) * TC_SBO + ks * 2 * TC_LBO, TC_LBO, TC_SBO);
-            const uint64_t bd = tc::smem_desc(b0 + ks * 2 * TC_LBO, TC_LBO, TC_SBO);
-            tc::mma_bf16(ts.tmem + 32 * g, ad, bd, tc::idesc_bf16_f32(128, 32 * (S - g)),
-                         (kacc == 0 && ks == 0 && g == 0) ? 0u : 1u);
-          }
-        tc::commit(buf ? mb1 : mb0);
-        ts.ncommit[buf] += 1;
-      }
-      ++nstage;
-      kacc += TC_KS;
-      const bool last = (s == tk.nseg - 1) && (k0 + TC_KS >= gs.k);
-      if (!last && kacc + TC_KS <= KMAX) continue;
-      // ---- drain: every MMA done, cells -> exact sums -> FP64
-      __syncthreads();  // ncommit of the last stage visible
-      const bool done = (ts.ncommit[0] == 0 || tc_wait(p, mb0, (ts.ncommit[0] - 1) & 1)) &&
-                        (ts.ncommit[1] == 0 || tc_wait(p, mb1, (ts.ncommit[1] - 1) & 1));
-      if (__syncthreads_or(!done)) return;
-      tc::fence_after_sync();
-      kacc = 0;
-      // lane block p (= warp) reads its cells, four columns at a time, and
-      // leaves its partial sums for every (column, row) in the staging region
-      long long* part = reinterpret_cast<long long*>(stage);  // [32 j][4 p][32 i] x (hi, lo)
-      float* partf = reinterpret_cast<float*>(stage);          // [32 j][4 p][32 i]
-      const uint32_t trow = ts.tmem + ((uint32_t)(32 * warp) << 16);
+// (H 2^32 + Lo) 2^k2 as a double, without an FP64 instruction (a conversion holds
+// the pipe like a multiply-add, and the drains would keep it from the block
+// POTRFs). |H 2^32 + Lo| < 2^76: its low 16 bits are rounded off first, 2^-58 or
+// less of the largest entries' product, a quarter of what the dropped digit
+// levels weigh.
+__device__ __forceinline__ double scaled_sum(long long H, long long Lo, int k2) {
+  const long long T = (H << 16) + ((Lo + (1ll << 15)) >> 16);
+  if (T == 0) return 0.0;
+  const unsigned long long sign = (unsigned long long)T & 0x8000000000000000ull;
+  const unsigned long long mag = sign ? 0ull - (unsigned long long)T : (unsigned long long)T;
+  const int lz = __clzll((long long)mag);
+  const unsigned long long norm = mag << lz;                             // top bit set
+  const unsigned long long mant = (norm >> 11) + ((norm >> 10) & 1ull);  // 2^52 .. 2^53
+  const int e = (63 - lz) + 16 + k2 + 1023;                              // biased exponent
+  if (e >= 1 && e < 0x7fe) return __longlong_as_double((long long)((((unsigned long long)(e - 1) << 52) + mant) | sign));
+  return ldexp((double)T, k2 + 16);  // subnormal or beyond the range
+}
+
+// acc += cell 2^sh for an integer-valued FP32 cell. SMALL (at most 64 of K, so
+// |cell| <= 2^22): adding 3 2^22 leaves the integer in the low mantissa bits, so
+// the sum runs on the bit patterns (a conversion runs at a quarter of the rate)
+// and kCellBias takes the patterns' constant part back out of four levels.
+constexpr long long kCellBias = 0x4B400000ll * ((1ll << 24) + (1ll << 16) + (1ll << 8) + 1);
+template <bool SMALL>
+__device__ __forceinline__ void add_cell(long long& acc, uint32_t cell, int sh) {
+  const float f = __uint_as_float(cell);
+  const int v = SMALL ? __float_as_int(f + 12582912.0f) : __float2int_rn(f);
+  asm("mad.wide.s32 %0, %1, %2, %0;" : "+l"(acc) : "r"(v), "r"(1 << sh));
+}
+
+// Read the cells and add the part's sums of this stretch of K to r16. er: the
+// biased exponent of the thread's row, cexp: of the 32 columns (shared memory;
+// emulated FP64). SMALL: at most 64 of K in the cells.
+// Each warp reads the cells of all 32 columns in its lane block (warps 0, 1: the
+// low levels / planes 0 and 2; warps 2, 3: the high levels / plane 1), 4 columns
+// of the other side's, handed over through shared memory, and 4 of its own at a
+// time. The loop is not unrolled (r16 is rotated instead, back in place after its
+// four steps): straight-line code of this size ran at the instruction cache's
+// rate, 13k cycles a drain.
+template <int S, bool SMALL>
+__device__ __forceinline__ void drain_cells(uint32_t tmem, uint8_t* xch, int er, const int* cexp, double (&r16)[16]) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int side = warp >> 1, row = 32 * (warp & 1) + lane;
+  const uint32_t trow = tmem + ((uint32_t)(32 * warp) << 16);
 #pragma unroll 1
-      for (int js = 0; js < 8; ++js) {
-        uint32_t cell[S][4];  // every column block is read; blocks of levels >= S are not used
-        tc::ld_cells(trow + 4 * js, cell);
-        if constexpr (S == 8) {
-          long long hi[4], lo[4];
+  for (int i = 0; i < 4; ++i) {
+    uint8_t* buf = xch + (i & 1) * (PL_XCH_BYTES / 2);  // free since the barrier of the step before
+    if constexpr (S == 8) {
+      constexpr int kScale = 2044 + 2 * 62 - 8 * 7;
+      long long* xhl = reinterpret_cast<long long*>(buf);  // [4 c][64 r] x (hi, lo) for side 1
+      long long* xlo = xhl + 2 * 4 * 64;                    // [4 c][64 r] lo for side 0
+      // level sums of 4 columns from col: hi (levels 0-3), lo (levels 4-7)
+      auto sums = [&](int col, long long (&hi)[4], long long (&lo)[4]) {
 #pragma unroll
-          for (int x = 0; x < 4; ++x) hi[x] = lo[x] = 0;
+        for (int x = 0; x < 4; ++x) hi[x] = lo[x] = SMALL ? -kCellBias : 0;
+        if (side == 0) {
+          uint32_t cell[8][4];
+          tc::ld_cells(trow + col, cell);
 #pragma unroll
-          for (int c = 0; c < S; ++c) {
-            const int L = G * warp + c;
-            if (L <= S - 1) {
+          for (int c = 0; c < 8; ++c)
 #pragma unroll
-              for (int x = 0; x < 4; ++x) {
-                const long long v = (long long)__float2int_rn(__uint_as_float(cell[c][x]));
-                if (L <= 3) hi[x] += v << (DB * (3 - L));
-                else lo[x] += v << (DB * (7 - L));
-              }
+            for (int x = 0; x < 4; ++x) {
+              if (c <= 3) add_cell<SMALL>(hi[x], cell[c][x], 8 * (3 - c));
+              else add_cell<SMALL>(lo[x], cell[c][x], 8 * (7 - c));
             }
-          }
-#pragma unroll
-          for (int x = 0; x < 4; ++x) {
-            const int e = ((4 * js + x) * 4 + warp) * 32 + lane;
-            part[2 * e] = hi[x];
-            part[2 * e + 1] = lo[x];
-          }
         } else {
+          uint32_t cell[4][4];
+          tc::ld_cells(trow + col, cell);
 #pragma unroll
-          for (int x = 0; x < 4; ++x) {
-            float v = 0.0f;
+          for (int c = 0; c < 4; ++c)
 #pragma unroll
-            for (int c = 0; c < S; ++c) {
-              const int L = G * warp + c;
-              if (L <= S - 1) v = FLT ? v + __uint_as_float(cell[c][x]) : fmaf(__uint_as_float(cell[c][x]), (float)(1 << (DB * (3 - L))), v);
-            }
-            partf[((4 * js + x) * 4 + warp) * 32 + lane] = v;
-          }
+            for (int x = 0; x < 4; ++x) add_cell<SMALL>(lo[x], cell[c][x], 8 * (3 - c));
+        }
+      };
+      long long hi[4], lo[4];
+      sums(16 * (1 - side) + 4 * i, hi, lo);
+#pragma unroll
+      for (int x = 0; x < 4; ++x) {
+        const int e = x * 64 + row;
+        if (side == 0) {
+          xhl[2 * e] = hi[x];
+          xhl[2 * e + 1] = lo[x];
+        } else {
+          xlo[e] = lo[x];
         }
       }
       __syncthreads();
-      // thread (warp, lane): outputs (row lane, column 4 js + warp)
-#pragma unroll 2
-      for (int js = 0; js < 8; ++js) {
-        const int j = 4 * js + warp;
-        double V;
-        if constexpr (S == 8) {
-          long long H = 0, Lo = 0;
+      sums(16 * side + 4 * i, hi, lo);
 #pragma unroll
-          for (int pb = 0; pb < 4; ++pb) {
-            const int e = (j * 4 + pb) * 32 + lane;
-            H += part[2 * e];
-            Lo += part[2 * e + 1];
-          }
-          V = fma((double)H, (double)(1ll << (4 * DB)), (double)Lo);  // H 2^(4 DB) + Lo, one rounding
-        } else {
-          float f = 0.0f;
+      for (int x = 0; x < 4; ++x) {
+        const int e = x * 64 + row, ec = cexp[16 * side + 4 * i + x];
+        const long long H = side == 0 ? hi[x] : xhl[2 * e], Lo = lo[x] + (side == 0 ? xlo[e] : xhl[2 * e + 1]);
+        r16[x] = (er == 0x7ff || ec == 0x7ff) ? __longlong_as_double(0x7ff8000000000000ll)
+                                              : r16[x] + scaled_sum(H, Lo, max(er, 1) + max(ec, 1) - kScale);
+      }
+    } else {
+      float* x0 = reinterpret_cast<float*>(buf);  // [4 c][64 r] plane 0, then plane 2, for side 1
+      float* x1 = x0 + 2 * 4 * 64;                // [4 c][64 r] plane 1, for side 0
+      auto pieces = [&](int col, float (&v)[4], float (&v2)[4]) {  // lane block's sums of 4 columns
+        uint32_t cell[8][4];
+        tc::ld_cells(trow + col, cell);
 #pragma unroll
-          for (int pb = 0; pb < 4; ++pb) f += partf[(j * 4 + pb) * 32 + lane];
-          V = (double)f;
+        for (int x = 0; x < 4; ++x) {
+          v[x] = ((0.0f + __uint_as_float(cell[0][x])) + __uint_as_float(cell[1][x])) + __uint_as_float(cell[2][x]);
+          v2[x] = (0.0f + __uint_as_float(cell[3][x])) + __uint_as_float(cell[4][x]);
         }
-        double& r = R[lane * 33 + j];
-        if constexpr (FLT) {
-          r += V;
+      };
+      float v[4], v2[4];
+      pieces(16 * (1 - side) + 4 * i, v, v2);
+#pragma unroll
+      for (int x = 0; x < 4; ++x) {
+        const int e = x * 64 + row;
+        if (side == 0) {
+          x0[e] = v[x];
+          x0[4 * 64 + e] = v2[x];
         } else {
-          const int er = rexp[lane], ec = cexp[j];
-          const int k2 = max(er, 1) + max(ec, 1) - kScale;
-          const double sc =
-              (k2 >= -1022 && k2 <= 1023) ? __longlong_as_double((long long)(k2 + 1023) << 52) : ldexp(1.0, k2);
-          r = (er == 0x7ff || ec == 0x7ff) ? __longlong_as_double(0x7ff8000000000000ll) : fma(V, sc, r);
+          x1[e] = v[x];
         }
       }
-      tc::fence_before_sync();
-      __syncthreads();  // TMEM reads done before the next MMAs; staging free again
+      __syncthreads();
+      pieces(16 * side + 4 * i, v, v2);
+#pragma unroll
+      for (int x = 0; x < 4; ++x) {
+        const int e = x * 64 + row;
+        const float p0 = side == 0 ? v[x] : x0[e], p1 = side == 0 ? x1[e] : v[x], p2 = side == 0 ? v2[x] : x0[4 * 64 + e];
+        r16[x] += (double)(((0.0f + p0) + p1) + p2);
+      }
+    }
+    double t[4];
+#pragma unroll
+    for (int x = 0; x < 4; ++x) t[x] = r16[x];
+#pragma unroll
+    for (int x = 0; x < 12; ++x) r16[x] = r16[x + 4];
+#pragma unroll
+    for (int x = 0; x < 4; ++x) r16[12 + x] = t[x];
+  }
+}
+
+// Epilogue of a 64 x 32 part from its result in registers (the thread mapping of
+// run_planes); smem: the staging region, free.
+__device__ __forceinline__ void store_part(const KParams& p, const Task& tk, int q, double* smem, double (&r16)[16]) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int side = warp >> 1, row = 32 * (warp & 1) + lane;
+  const int c0 = 32 * q + 16 * side;
+  const int m = tk.m, n = tk.n;
+  double* O = resolve(p, tk.out);
+  if (tk.op != OP_SYMUPD) {  // OP_UPD, OP_STORE, OP_NEG
+    double* Om = tk.op == OP_NEG && p.smirror ? p.smirror + (O - p.buf[BUF_S]) : nullptr;
+    if (tk.op == OP_UPD) {
+      const double* C = resolve(p, tk.cin);
+      double v[16];
+#pragma unroll
+      for (int x = 0; x < 16; ++x)
+        v[x] = row < m && c0 + x < n ? __ldcg(C + row + (int64_t)(c0 + x) * tk.ldc) : 0.0;
+#pragma unroll
+      for (int x = 0; x < 16; ++x) r16[x] = v[x] - r16[x];
+    }
+#pragma unroll
+    for (int x = 0; x < 16; ++x)
+      if (row < m && c0 + x < n) {
+        const double v = tk.op == OP_NEG ? -r16[x] : r16[x];
+        O[row + (int64_t)(c0 + x) * tk.ldo] = v;
+        if (Om) Om[row + (int64_t)(c0 + x) * tk.ldo] = v;
+      }
+    return;
+  }
+  // OP_SYMUPD: cin - acc, and its transpose into the mirror position (inside the
+  // block for a diagonal one, whose part above the diagonal is left out)
+  const double* C = resolve(p, tk.cin);
+  const bool dblk = tk.flags & TF_SYM_DIAG;
+  double* M = dblk ? O : resolve(p, tk.aux);
+  const int ldm = dblk ? tk.ldo : tk.ldx;
+  double* Om = p.smirror ? p.smirror + (O - p.buf[BUF_S]) : nullptr;
+  double* Mm = p.smirror ? p.smirror + (M - p.buf[BUF_S]) : nullptr;
+  double v[16];
+#pragma unroll
+  for (int x = 0; x < 16; ++x) {
+    const bool in = row < m && c0 + x < n && (!dblk || row >= c0 + x);
+    v[x] = in ? __ldcg(C + row + (int64_t)(c0 + x) * tk.ldc) - r16[x] : 0.0;
+  }
+  double* X = smem;  // [64 rows][33]: the staging region, every copy of which has been used
+#pragma unroll
+  for (int x = 0; x < 16; ++x) {
+    X[row * 33 + 16 * side + x] = v[x];
+    if (row < m && c0 + x < n && (!dblk || row >= c0 + x)) {
+      O[row + (int64_t)(c0 + x) * tk.ldo] = v[x];
+      if (Om) Om[row + (int64_t)(c0 + x) * tk.ldo] = v[x];
     }
   }
-  // to the accumulate<2,4> mapping
   __syncthreads();
-  const int tx = tid & 15, ty = tid >> 4;
+  for (int e = tid; e < 64 * 32; e += NTHREADS) {
+    const int c = e % 32, r = e / 32, cc = 32 * q + c;
+    if (r < m && cc < n && (!dblk || r > cc)) {
+      M[cc + (int64_t)r * ldm] = X[r * 33 + c];
+      if (Mm) Mm[cc + (int64_t)r * ldm] = X[r * 33 + c];
+    }
+  }
+}
+
+// The 64 x 32 sub-tile (columns 32 q ..) of a product task from planes, and its
+// epilogue. Thread (warp, lane) owns row 32 (warp & 1) + lane, columns
+// 16 (warp >> 1) + 0..15 of it. Thread 32 copies, thread 0 multiplies: one
+// thread doing both waits for the MMAs of the stage before in between.
+template <int S>
+__device__ __noinline__ void run_planes(const KParams& p, const Task& tk, int q, double* smem, TcShared& ts) {
+  using F = PlaneFmt<S>;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int side = warp >> 1, row = 32 * (warp & 1) + lane;
+  uint8_t* stage = reinterpret_cast<uint8_t*>(smem);
+  const uint32_t stage_a = tc::smem_addr(stage);
+  double r16[16];
 #pragma unroll
-  for (int i = 0; i < 2; ++i)
-#pragma unroll
-    for (int jj = 0; jj < 4; ++jj) acc[i][jj] = R[(tx + 16 * i) * 33 + ty + 8 * jj];
+  for (int x = 0; x < 16; ++x) r16[x] = 0.0;
+  int* cexp = reinterpret_cast<int*>(stage + PL_EXP_OFF);
+  const uint32_t base = ts.pstage;  // this part's stages are base, base + 1, ..
+  const bool copier = tid == 32;
+  // copies: a cursor over the stages of all segments
+  int ls = 0, lk = 0;
+  uint32_t issued = 0, used = 0;  // stages copied / multiplied by this part
+  Seg lseg = load_seg(p, tk.seg0);
+  auto issue = [&]() {  // the next stage into its slot, once the MMAs that last read it are done
+    const uint32_t g = base + issued, slot = g % F::NST;
+    if (g >= F::NST && !tc_wait(p, tc::smem_addr(&ts.pempty[slot]), (g / F::NST - 1) & 1)) return false;
+    const int nst = (lseg.k + kPlaneK - 1) / kPlaneK, nch = (lseg.k + kPlaneChunk - 1) / kPlaneChunk;
+    const int64_t head = S == 8 ? 256 * (int64_t)nch : 0;
+    const uint8_t* A = p.planes + 16 * (lseg.a & OFF_MASK) + head + (int64_t)lk * F::A_BYTES;
+    const uint8_t* B = p.planes + 16 * (lseg.b & OFF_MASK) + head + (int64_t)lk * F::A_BYTES + q * F::B_BYTES;
+    const uint32_t bar = tc::smem_addr(&ts.pfull[slot]), dst = stage_a + slot * F::STAGE;
+    tc::expect_tx(bar, F::STAGE);
+    tc::bulk_load(dst, A, F::A_BYTES, bar);
+    tc::bulk_load(dst + F::A_BYTES, B, F::B_BYTES, bar);
+    ++issued;
+    if (++lk == nst) {
+      lk = 0;
+      if (++ls < tk.nseg) lseg = load_seg(p, tk.seg0 + ls);
+    }
+    return true;
+  };
+  tc::fence_smem_to_async();  // earlier tasks' shared-memory accesses before the copies' writes
   __syncthreads();
+  if (copier) {
+    tc::fence_global_async();  // the planes' writes (this task was released after them)
+    for (int x = 0; x < F::NST && ls < tk.nseg; ++x)
+      if (!issue()) break;
+  }
+  uint32_t ndone = ts.pdone_n;
+  int kacc = 0;
+  bool ok = true;
+  for (int s = 0; s < tk.nseg && ok; ++s) {
+    const Seg gs = load_seg(p, tk.seg0 + s);
+    const int nst = (gs.k + kPlaneK - 1) / kPlaneK;
+    const int* ea = reinterpret_cast<const int*>(p.planes + 16 * (gs.a & OFF_MASK));
+    const int* eb = reinterpret_cast<const int*>(p.planes + 16 * (gs.b & OFF_MASK));
+    // runs of stages between drains: K chunks of one exponent cut where the
+    // cells' exact range ends; FP32-class: 4096 of K, counted in steps of 32
+    for (int st0 = 0; st0 < nst && ok;) {
+      int st1;
+      bool drain, fresh = true;
+      if constexpr (S == 8) {
+        st1 = min(nst, st0 + F::KMAX / kPlaneK);
+        drain = true;
+      } else {
+        const int room = (F::KMAX - kacc) / 32;
+        fresh = kacc == 0;
+        st1 = min(nst, st0 + 2 * room);
+        kacc += (st1 - st0 + 1) / 2 * 32;
+        drain = (s == tk.nseg - 1 && st1 == nst) || kacc + 32 > F::KMAX;
+      }
+      const uint32_t end = used + (uint32_t)(st1 - st0);
+      if (copier)  // up to the slots that the run's last MMAs free (those after the drain's wait)
+        while (ls < tk.nseg && issued + 1 < end + F::NST && issue()) {}
+      if (tid == 0) {
+        bool go = true;
+        for (uint32_t x = used; x < end; ++x) {
+          const uint32_t g = base + x, slot = g % F::NST;
+          if (!tc_wait(p, tc::smem_addr(&ts.pfull[slot]), (g / F::NST) & 1)) {
+            go = false;  // pdone is not committed: every thread's wait for it runs out too
+            break;
+          }
+          tc::fence_after_sync();
+          stage_mmas<S>(ts.tmem, stage_a + slot * F::STAGE, !(fresh && x == used));
+          tc::commit(tc::smem_addr(&ts.pempty[slot]));
+        }
+        if (drain && go) tc::commit(tc::smem_addr(&ts.pdone));
+      }
+      used = end;
+      const int first = st0;
+      st0 = st1;
+      if (!drain) continue;
+      kacc = 0;
+      int er = 0;
+      if constexpr (S == 8) {  // this chunk's exponents, in flight while the MMAs finish
+        const int ch = first / (kPlaneChunk / kPlaneK);
+        er = __ldcg(ea + 64 * ch + row);
+        if (warp == 3) cexp[lane] = __ldcg(eb + 64 * ch + 32 * q + lane);  // (read after the barrier below)
+      }
+      __syncwarp();
+      ok = tc_wait(p, tc::smem_addr(&ts.pdone), ndone & 1);
+      ++ndone;
+      ok = !__syncthreads_or(!ok);
+      if (!ok) break;
+      tc::fence_after_sync();
+      if (copier)  // every slot is free: the next stages load while the cells are read
+        while (ls < tk.nseg && issued < end + F::NST && issue()) {}
+      drain_cells<S, false>(ts.tmem, stage + PL_XCH_OFF, er, cexp, r16);
+      tc::fence_before_sync();
+      __syncthreads();  // TMEM and exchange reads done before the next MMAs
+    }
+  }
+  if (!ok) {  // timed out: the copies in flight must land before the part ends (again bounded waits)
+    if (copier)
+      for (uint32_t g = base + (issued > F::NST ? issued - F::NST : 0); g != base + issued; ++g)
+        tc_wait(p, tc::smem_addr(&ts.pfull[g % F::NST]), (g / F::NST) & 1);
+    __syncthreads();
+    return;
+  }
+  if (tid == 0) {  // (read again only after the next part's first barrier)
+    ts.pstage = base + used;
+    ts.pdone_n = ndone;
+  }
+  store_part(p, tk, q, smem, r16);
+}
+
+// A 64 x 32 part (columns 32 q ..) that splits its own operands: 64 of K at a
+// time. Thread (warp, lane) loads the K octets warp and warp + 4 of the vectors
+// lane and lane + 32 of op(A) and lane of op(B) (48 values, the next 64 of K in
+// flight while the MMAs of these run), takes the exponents from them (emulated
+// FP64: one per vector and 64 of K) and writes the planes of four stages. What
+// bounds it: the splits (about 35 instructions per operand value, 48 values per
+// thread for 1664 cycles of MMAs) and, for the factor's updates with an inner
+// length of 64, the fixed cost of a task. The 32 x 32 parts before split each
+// operand twice as often and scanned the whole K for exponents first.
+// (x[0 .. 3]: op(A), x[4], x[5]: op(B))
+__device__ __forceinline__ void tc_load(const KParams& p, const Task& tk, const Seg& g, int k0, int kc, int q,
+                                        double (&x)[6][8]) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const bool ta = g.trans & 1, tb = g.trans & 2;
+  const int64_t sa = ta ? 1 : g.lda, sb = tb ? g.ldb : 1;
+  const double* A = resolve(p, g.a) + (int64_t)k0 * sa;
+  const double* B = resolve(p, g.b) + (int64_t)k0 * sb + (int64_t)(32 * q) * (tb ? 1 : g.ldb);
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    const int v = lane + 32 * (u & 1), k = 8 * (warp + 4 * (u >> 1));
+    const double* P = A + (int64_t)v * (ta ? g.lda : 1) + (int64_t)k * sa;
+#pragma unroll
+    for (int y = 0; y < 8; ++y) x[u][y] = v < tk.m && k + y < kc ? __ldcg(P + (int64_t)y * sa) : 0.0;
+  }
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int k = 8 * (warp + 4 * u);
+    const double* P = B + (int64_t)lane * (tb ? 1 : g.ldb) + (int64_t)k * sb;
+#pragma unroll
+    for (int y = 0; y < 8; ++y) x[4 + u][y] = 32 * q + lane < tk.n && k + y < kc ? __ldcg(P + (int64_t)y * sb) : 0.0;
+  }
+}
+
+// The planes of 8 K-adjacent values, 16 bytes each: plane t at dst + (t % 4) s1 + (t / 4) s2.
+template <int S, bool GLOBAL>
+__device__ __forceinline__ void store_planes(const double (&x)[8], int emax, uint8_t* dst, int s1, int s2) {
+  uint32_t w[4][S];
+#pragma unroll
+  for (int y = 0; y < 4; ++y) {
+    if constexpr (S == 8) digit_pairs(x[2 * y], x[2 * y + 1], emax, w[y]);
+    else piece_pairs(x[2 * y], x[2 * y + 1], w[y]);
+  }
+#pragma unroll
+  for (int t = 0; t < PlaneFmt<S>::NP; ++t) {
+    uint4* d = reinterpret_cast<uint4*>(dst + (t % 4) * s1 + (t / 4) * s2);
+    const uint4 v = make_uint4(w[0][t], w[1][t], w[2][t], w[3][t]);
+    if constexpr (GLOBAL) __stcg(d, v);
+    else *d = v;
+  }
+}
+// s1, s2 of a stage's left- / right-hand planes (64 / 32 vectors)
+template <int S>
+struct PlaneStep {
+  static constexpr int A1 = S == 8 ? 4096 : 2048, A2 = 2048, B1 = 1024, B2 = 4096;
+};
+
+template <int S>
+__device__ __noinline__ void run_tc(const KParams& p, const Task& tk, int q, double* smem, TcShared& ts) {
+  using F = PlaneFmt<S>;
+  static_assert(4 * F::STAGE <= PL_STAGE_BYTES, "64 of K in the staging region");
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int side = warp >> 1;
+  uint8_t* stage = reinterpret_cast<uint8_t*>(smem);
+  const uint32_t stage_a = tc::smem_addr(stage);
+  // column exponents, partial exponents [4 warps][64 rows, then 32 columns]
+  int* cexp = reinterpret_cast<int*>(stage + PL_EXP_OFF);
+  int* pexp = cexp + 32;
+  if (tk.op == OP_UPD) {  // the input block into L2, one line per thread
+    const int col = 32 * q + (tid >> 2), r = 16 * (tid & 3);
+    if (col < tk.n && r < tk.m)
+      asm volatile("prefetch.global.L2 [%0];" ::"l"(resolve(p, tk.cin) + r + (int64_t)col * tk.ldc));
+  }
+  double r16[16];
+#pragma unroll
+  for (int x = 0; x < 16; ++x) r16[x] = 0.0;
+  uint32_t ndone = ts.pdone_n;
+  int kacc = 0;
+  double x[6][8];
+  Seg g = load_seg(p, tk.seg0);
+  int kc = min(64, g.k);
+  tc_load(p, tk, g, 0, kc, q, x);
+  for (int s = 0, k0 = 0; s < tk.nseg;) {
+    int er = 0, ea[2] = {0, 0}, eb = 0;
+    if constexpr (S == 8) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+#pragma unroll
+        for (int y = 0; y < 8; ++y) ea[u & 1] = max(ea[u & 1], biased_exp(x[u][y]));
+#pragma unroll
+      for (int u = 4; u < 6; ++u)
+#pragma unroll
+        for (int y = 0; y < 8; ++y) eb = max(eb, biased_exp(x[u][y]));
+      int* mine = pexp + 96 * warp;
+      mine[lane] = ea[0];
+      mine[32 + lane] = ea[1];
+      mine[64 + lane] = eb;
+      __syncthreads();
+      ea[0] = ea[1] = eb = 0;
+#pragma unroll
+      for (int w = 0; w < 4; ++w) {
+        ea[0] = max(ea[0], pexp[96 * w + lane]);
+        ea[1] = max(ea[1], pexp[96 * w + 32 + lane]);
+        eb = max(eb, pexp[96 * w + 64 + lane]);
+      }
+      er = warp & 1 ? ea[1] : ea[0];
+      if (warp == 0) cexp[lane] = eb;
+    }
+    // octet o of the chunk: stage o / 2, half o % 2 (a loop over the six octets,
+    // their values rotated through x[0], for the instruction cache)
+    const int nst = (kc + kPlaneK - 1) / kPlaneK;
+#pragma unroll 1
+    for (int u = 0; u < 6; ++u) {
+      const bool isa = u < 4;
+      const int v = isa ? lane + 32 * (u & 1) : lane, o = warp + 4 * (isa ? u >> 1 : u - 4);
+      if (o < 2 * nst)
+        store_planes<S, false>(x[0], !isa ? eb : u & 1 ? ea[1] : ea[0],
+                               stage + (o >> 1) * F::STAGE + (isa ? 0 : F::A_BYTES) + (o & 1) * 128 + (v >> 3) * 256 + (v & 7) * 16,
+                               isa ? PlaneStep<S>::A1 : PlaneStep<S>::B1, isa ? PlaneStep<S>::A2 : PlaneStep<S>::B2);
+#pragma unroll
+      for (int w = 0; w < 5; ++w)
+#pragma unroll
+        for (int y = 0; y < 8; ++y) x[w][y] = x[w + 1][y];
+    }
+    // the next stretch of K
+    const bool fresh = S == 8 || kacc == 0;
+    kacc += (kc + 31) / 32 * 32;
+    k0 += kc;
+    if (k0 >= g.k) {
+      k0 = 0;
+      if (++s < tk.nseg) g = load_seg(p, tk.seg0 + s);
+    }
+    const bool last = s >= tk.nseg;
+    const bool drain = S == 8 || last || kacc + 32 > F::KMAX;
+    tc::fence_smem_to_async();
+    __syncthreads();
+    if (tid == 0) {
+      tc::fence_after_sync();
+      for (int st = 0; st < nst; ++st) stage_mmas<S>(ts.tmem, stage_a + st * F::STAGE, !(fresh && st == 0));
+      tc::commit(tc::smem_addr(&ts.pdone));
+    }
+    __syncwarp();
+    if (drain) kacc = 0;
+    if (!last) {
+      kc = min(64, g.k - k0);
+      if constexpr (S == 4) kc = min(kc, F::KMAX - kacc);
+      tc_load(p, tk, g, k0, kc, q, x);
+    }
+    bool ok = tc_wait(p, tc::smem_addr(&ts.pdone), ndone & 1);
+    ++ndone;
+    ok = !__syncthreads_or(!ok);
+    if (!ok) return;
+    if (!drain) continue;
+    tc::fence_after_sync();
+    drain_cells<S, true>(ts.tmem, stage + PL_XCH_OFF, er, cexp, r16);
+    tc::fence_before_sync();
+    __syncthreads();  // TMEM and exchange reads done before the next MMAs
+  }
+  if (tid == 0) ts.pdone_n = ndone;  // (read again only after the next part's first barrier)
+  store_part(p, tk, q, smem, r16);
+}
+
+// OP_SPLIT, part (vectors 16 (q & 3) .., K chunk q >> 2): the chunk's planes of
+// 16 vectors, and their exponents (emulated FP64). Lane l of warp w holds vector
+// l % 16 and the K octets 2 w + l / 16 + 8 u (u < 8) of the chunk in registers,
+// read once: exponents first, then the digits, stored 16 bytes (one core-matrix
+// row) at a time. Vectors beyond the tile and the padding of K are zeros.
+template <int S>
+__device__ __noinline__ void run_split(const KParams& p, const Task& tk, int q, double* smem) {
+  using F = PlaneFmt<S>;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int v = 16 * (q & 3) + (lane & 15), oct0 = 2 * warp + (lane >> 4);
+  const int k0 = tk.gcol + kPlaneChunk * (q >> 2), kc = min(kPlaneChunk, tk.zrows - k0);
+  const int noct = (kc + kPlaneK - 1) / kPlaneK * 2;
+  const bool kcont = tk.flags & TF_KCONT, bside = tk.flags & TF_BSIDE;
+  const double* A = resolve(p, tk.cin);
+  A += kcont ? (int64_t)v * tk.ldc + (k0 - tk.gcol) : v + (int64_t)(k0 - tk.gcol) * tk.ldc;
+  const int64_t step = kcont ? 1 : tk.ldc;
+  double x[8][8];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const int k = 8 * (oct0 + 8 * u);
+#pragma unroll
+    for (int y = 0; y < 8; ++y) x[u][y] = v < tk.m && k + y < kc ? __ldcg(A + (int64_t)(k + y) * step) : 0.0;
+  }
+  int emax = 0;
+  const int nch = (tk.zrows + kPlaneChunk - 1) / kPlaneChunk;
+  uint8_t* out = p.planes + 16 * (tk.out & OFF_MASK);
+  if constexpr (S == 8) {
+    int* part = reinterpret_cast<int*>(smem);
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+#pragma unroll
+      for (int y = 0; y < 8; ++y) emax = max(emax, biased_exp(x[u][y]));
+    emax = max(emax, __shfl_xor_sync(0xffffffffu, emax, 16));
+    part[warp * 16 + (lane & 15)] = emax;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < 4; ++w) emax = max(emax, part[16 * w + (lane & 15)]);
+    if (tid < 16) __stcg(reinterpret_cast<int*>(out) + 64 * (k0 / kPlaneChunk) + v, emax);
+    out += 256 * (int64_t)nch;
+  }
+  out += (int64_t)(k0 / kPlaneK) * F::A_BYTES;
+  const int vg = bside ? (v & 31) : v;  // vector inside its plane
+  out += (bside ? (v >> 5) * F::B_BYTES : 0) + (vg >> 3) * 256 + (vg & 7) * 16;
+#pragma unroll 1
+  for (int u = 0; u < 8; ++u) {  // (rotated through x[0], as in run_tc)
+    const int o = oct0 + 8 * u;
+    if (o < noct)
+      store_planes<S, true>(x[0], emax, out + (int64_t)(o >> 1) * F::A_BYTES + (o & 1) * 128,
+                            bside ? PlaneStep<S>::B1 : PlaneStep<S>::A1, bside ? PlaneStep<S>::B2 : PlaneStep<S>::A2);
+#pragma unroll
+    for (int w = 0; w < 7; ++w)
+#pragma unroll
+      for (int y = 0; y < 8; ++y) x[w][y] = x[w + 1][y];
+  }
+  tc::fence_global_async();
 }
 
 // X[rl][cl] = sign * acc (or cin - acc) over the whole (16 TM) x (8 TN) sub-tile
@@ -1529,8 +1738,8 @@ __device__ void finish_potrf(const KParams& p, const Task& tk, const double* S) 
   }
 }
 
-template <bool TC, int TM, int TN>
-__device__ void run_sub(const KParams& p, const Task& tk, const Sub& sb, double* smem, TcShared* ts) {
+template <int TM, int TN>
+__device__ void run_sub(const KParams& p, const Task& tk, const Sub& sb, double* smem) {
   double* As = smem;             // KC x LDS
   double* Bs = smem + KC * LDS;  // KC x LDS
   double* T = smem;              // FB x LDS, reuses As/Bs after the K-loop
@@ -1539,13 +1748,7 @@ __device__ void run_sub(const KParams& p, const Task& tk, const Sub& sb, double*
   const int m = tk.m, n = tk.n;
   double acc[TM][TN];
   if (tk.op != OP_TRTRI) {
-    if constexpr (TC && TM == 2 && TN == 4) {  // reduced-precision parts are <= 32 x 32 sub-tiles
-      if (tk.prec == PREC_EMU64) accumulate_tc<8, 8>(p, tk, sb, acc, smem, *ts);
-      else if (tk.prec == PREC_FP32X) accumulate_tc<4, 8>(p, tk, sb, acc, smem, *ts);
-      else accumulate<TM, TN>(p, tk, sb, acc, As, Bs);
-    } else {
-      accumulate<TM, TN>(p, tk, sb, acc, As, Bs);
-    }
+    accumulate<TM, TN>(p, tk, sb, acc, As, Bs);
   }
 
   switch (tk.op) {
@@ -1566,7 +1769,7 @@ __device__ void run_sub(const KParams& p, const Task& tk, const Sub& sb, double*
           if (r < sb.rm && c < sb.cn) {
             double v = acc[i][j];
             if (tk.op == OP_UPD) v = __ldcg(C + r + (int64_t)c * tk.ldc) - v;
-            else if (tk.op == OP_NEG) v = -v;
+            else if (tk.op == OP_NEG || (tk.flags & TF_NEG)) v = -v;
             O[r + (int64_t)c * tk.ldo] = v;
             if (Om) Om[r + (int64_t)c * tk.ldo] = v;
           }
@@ -1643,18 +1846,6 @@ __device__ void run_sub(const KParams& p, const Task& tk, const Sub& sb, double*
             }
             break;
           }
-          case OP_TRSM_LLN: {  // X = -T^{-1} acc, T lower m x m: columns are independent
-            acc_to_smem<TM, TN>(p, tk, sb, acc, X, false, -1.0);
-            load_tri(p, tk, m, T);
-            __syncthreads();
-            double* rcp = T + FB;
-            if (tid < m) rcp[tid * LDS] = 1.0 / T[tid * LDS + tid];
-            __syncthreads();
-            trsm_cols_ln(X, T, rcp, m, n, false);
-            __syncthreads();
-            store_sub(p, tk, sb, X, false);
-            break;
-          }
           case OP_TRTRI: {  // X = T^{-1}, T lower m x m: solve T X = I column by column
             load_tri(p, tk, m, T);
             for (int e = tid; e < FB * FB; e += NTHREADS) {
@@ -1704,7 +1895,7 @@ __device__ bool task_part_ok(const KParams& p, const Task& tk, const Sub& sb) {
   const bool cin = tk.op == OP_UPD || tk.op == OP_POTRF || tk.op == OP_TRSM_RLT || tk.op == OP_SYMUPD;
   if (cin && !ref_ok(p, tk.cin, r0 + (int64_t)c0 * tk.ldc, r1 + (int64_t)c1 * tk.ldc)) return false;
   if (tk.op == OP_TRSM_RLT && !ref_ok(p, tk.aux, 0, (tk.n - 1) + (int64_t)(tk.n - 1) * tk.ldx)) return false;
-  if ((tk.op == OP_TRSM_LLN || tk.op == OP_TRTRI) && !ref_ok(p, tk.aux, 0, (tk.m - 1) + (int64_t)(tk.m - 1) * tk.ldx))
+  if (tk.op == OP_TRTRI && !ref_ok(p, tk.aux, 0, (tk.m - 1) + (int64_t)(tk.m - 1) * tk.ldx))
     return false;
   if (tk.op == OP_SYMUPD && !(tk.flags & TF_SYM_DIAG) && !ref_ok(p, tk.aux, c0 + (int64_t)r0 * tk.ldx, c1 + (int64_t)r1 * tk.ldx))
     return false;
@@ -1736,6 +1927,29 @@ __device__ void run_task(const KParams& p, const Task& tk, int t, int q, double*
     return;
   }
   if (tk.op == OP_JOIN) return;  // a dependency point only
+  if constexpr (TC) {
+    if (tk.op == OP_SPLIT) {
+      if (tk.prec == PREC_EMU64) run_split<8>(p, tk, q, smem);
+      else run_split<4>(p, tk, q, smem);
+      return;
+    }
+    if (tk.flags & TF_PLANES) {
+      if (tk.prec == PREC_EMU64) run_planes<8>(p, tk, q, smem, *ts);
+      else run_planes<4>(p, tk, q, smem, *ts);
+      return;
+    }
+    if (tk.prec != PREC_FP64) {
+#ifdef STILES_CHECKED
+      if (!task_part_ok(p, tk, part_sub(tk.pmode, tk.m, tk.n, q))) {
+        if (threadIdx.x == 0) check_fail(p, 7, t, q);
+        return;
+      }
+#endif
+      if (tk.prec == PREC_EMU64) run_tc<8>(p, tk, q, smem, *ts);
+      else run_tc<4>(p, tk, q, smem, *ts);
+      return;
+    }
+  }
   const Sub sb = part_sub(tk.pmode, tk.m, tk.n, q);
   if (sb.rm <= 0 || sb.cn <= 0) return;
 #ifdef STILES_CHECKED
@@ -1745,15 +1959,15 @@ __device__ void run_task(const KParams& p, const Task& tk, int t, int q, double*
   }
 #endif
   switch (tk.pmode) {
-    case PM_ROWS2: run_sub<TC, 2, 8>(p, tk, sb, smem, ts); break;
+    case PM_ROWS2: run_sub<2, 8>(p, tk, sb, smem); break;
     case PM_ROWS4:
-    case PM_ROWS8: run_sub<TC, 1, 8>(p, tk, sb, smem, ts); break;
+    case PM_ROWS8: run_sub<1, 8>(p, tk, sb, smem); break;
     case PM_TRI16:
-    case PM_GRID16: run_sub<TC, 1, 2>(p, tk, sb, smem, ts); break;
+    case PM_GRID16: run_sub<1, 2>(p, tk, sb, smem); break;
     case PM_QUAD4:
     case PM_TRI3:
-    case PM_TILE32: run_sub<TC, 2, 4>(p, tk, sb, smem, ts); break;
-    default: run_sub<TC, 4, 8>(p, tk, sb, smem, ts); break;
+    case PM_TILE32: run_sub<2, 4>(p, tk, sb, smem); break;
+    default: run_sub<4, 8>(p, tk, sb, smem); break;
   }
 }
 
@@ -1778,7 +1992,7 @@ __device__ __forceinline__ TcShared* tc_shared() {
 // Two instances: TC = false for plans whose products are all FP64 (no
 // tensor-core code at all), TC = true for plans with reduced-precision parts.
 template <bool TC>
-__global__ void __launch_bounds__(NTHREADS, 2) persistent_kernel(KParams p) {
+__global__ void __launch_bounds__(NTHREADS, 2) persistent_kernel(const __grid_constant__ KParams p) {
   extern __shared__ __align__(16) double smem[];
   __shared__ int s_item;
   TcShared* ts = tc_shared<TC>();
@@ -1787,10 +2001,13 @@ __global__ void __launch_bounds__(NTHREADS, 2) persistent_kernel(KParams p) {
   if constexpr (TC) {
     if (threadIdx.x < 32) tc::tmem_alloc<TC_COLS>(&ts->tmem);
     if (threadIdx.x == 0) {
-      tc::mbar_init(tc::smem_addr(&ts->mbar[0]), 1);
-      tc::mbar_init(tc::smem_addr(&ts->mbar[1]), 1);
+      for (int x = 0; x < PL_SLOTS; ++x) {
+        tc::mbar_init(tc::smem_addr(&ts->pfull[x]), 1);
+        tc::mbar_init(tc::smem_addr(&ts->pempty[x]), 1);
+      }
+      tc::mbar_init(tc::smem_addr(&ts->pdone), 1);
+      ts->pdone_n = ts->pstage = 0;
       tc::fence_mbar_init();
-      ts->ncommit[0] = ts->ncommit[1] = 0;
     }
     tc::fence_before_sync();
     __syncthreads();
@@ -1865,8 +2082,11 @@ __global__ void __launch_bounds__(NTHREADS, 2) persistent_kernel(KParams p) {
       tc::tmem_dealloc<TC_COLS>(ts->tmem);
     }
     if (threadIdx.x == 0) {
-      tc::mbar_inval(tc::smem_addr(&ts->mbar[0]));
-      tc::mbar_inval(tc::smem_addr(&ts->mbar[1]));
+      for (int x = 0; x < PL_SLOTS; ++x) {
+        tc::mbar_inval(tc::smem_addr(&ts->pfull[x]));
+        tc::mbar_inval(tc::smem_addr(&ts->pempty[x]));
+      }
+      tc::mbar_inval(tc::smem_addr(&ts->pdone));
     }
   }
 }
@@ -1875,7 +2095,7 @@ __global__ void __launch_bounds__(NTHREADS, 2) persistent_kernel(KParams p) {
 // regions, or more when the plan has tensor-core parts.
 size_t kernel_smem_bytes(bool use_tc) {
   const size_t fp64 = sizeof(double) * (size_t)(2 * KC * LDS + FB * LDS);
-  return use_tc && (size_t)TC_SMEM_BYTES > fp64 ? (size_t)TC_SMEM_BYTES : fp64;
+  return use_tc && (size_t)PL_SMEM_BYTES > fp64 ? (size_t)PL_SMEM_BYTES : fp64;
 }
 
 int kernel_threads() { return NTHREADS; }

@@ -207,7 +207,7 @@ extern "C" int stiles_server_create(int nshapes, const int* nt, const int* b, co
     }
     ShapeT T;
     T.s = Shape{nt[m], b[m], band[m] < nt[m] - 1 ? band[m] : nt[m] - 1, arrow[m], precision, tune};
-    int rc = build_serve_template(T.s, 304, &T.plan);
+    int rc = build_serve_template(T.s, 0, &T.plan);
     if (rc) {
       delete h;
       return rc;

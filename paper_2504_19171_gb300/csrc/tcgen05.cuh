@@ -3,7 +3,7 @@
 // asynchronous MMA with its completion barrier, and tensor-memory loads.
 //
 // Conventions used here (checked on GB300 by a layout probe before use):
-//  * Operands are bf16 in shared memory, K-major, without swizzle: a "core
+//  * Operands are bf16 (or both fp16) in shared memory, K-major, without swizzle: a "core
 //    matrix" is 8 rows x 16 bytes (8 bf16 of K) stored as 128 contiguous
 //    bytes. The descriptor's leading-dimension offset is the byte distance
 //    between core matrices adjacent in K, the stride-dimension offset the
@@ -29,6 +29,9 @@ __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint
 // Instruction descriptor of kind::f16 with bf16 A and B, FP32 D, both
 // operands K-major, dense: D format bits 4-5, A / B formats bits 7-9 / 10-12,
 // N / 8 in bits 17-22, M / 16 in bits 24-28.
+__host__ __device__ constexpr uint32_t idesc_f16_f32(int M, int N) {  // the same with fp16 A and B
+  return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+}
 __host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
@@ -52,7 +55,7 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t base) {
 }
 
 // One thread: D (+)= A * B^T, M x N x 16 (accumulate when acc != 0).
-__device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
+__device__ __forceinline__ void mma_f16(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                          uint32_t acc) {
   asm volatile(
       "{\n .reg .pred p;\n setp.ne.u32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
@@ -71,6 +74,24 @@ __device__ __forceinline__ void fence_before_sync() { asm volatile("tcgen05.fenc
 __device__ __forceinline__ void fence_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 // Generic-proxy shared-memory writes become visible to the tensor core (async proxy).
 __device__ __forceinline__ void fence_smem_to_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+
+// Generic-proxy global writes become visible to bulk copies (async proxy), and
+// the other way round.
+__device__ __forceinline__ void fence_global_async() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
+
+// One thread: the barrier's current phase expects `bytes` of bulk copies (and
+// counts this thread's arrival).
+__device__ __forceinline__ void expect_tx(uint32_t mbar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mbar), "r"(bytes) : "memory");
+}
+
+// One thread: copy `bytes` (a multiple of 16, both addresses 16-byte aligned)
+// from global to shared memory, counted off the barrier's expected bytes.
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint32_t mbar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(mbar)
+               : "memory");
+}
 
 __device__ __forceinline__ void mbar_init(uint32_t mbar, uint32_t count) {
   asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(mbar), "r"(count) : "memory");
