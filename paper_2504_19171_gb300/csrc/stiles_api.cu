@@ -547,7 +547,8 @@ extern "C" int stiles_debug_race_check_serve(int nt, int b, int band, int arrow,
   if (nt < 1 || b < 1 || band < 0 || arrow < 0 || precision < 0 || precision > PREC_FP32X || !tune_valid(tuning) ||
       plant < 0 || plant > 1)
     return STILES_ERR_INVALID_ARG;
-  const Shape sh{nt, b, band < nt - 1 ? band : nt - 1, arrow, precision, tuning};
+  Shape sh{nt, b, band < nt - 1 ? band : nt - 1, arrow, precision, tuning};
+  sh.planes = use_planes(sh);
   Plan p;
   const int rc = build_serve_template(sh, 0, &p);
   return rc ? rc : race_check_plan(p, Layout(sh).doubles(), plant, true);
@@ -1024,7 +1025,8 @@ extern "C" int stiles_debug_race_check_batch(int count, const int* nt, const int
 extern "C" int stiles_debug_validate_serve(int nt, int b, int band, int arrow, int precision, int tuning) {
   if (nt < 1 || b < 1 || band < 0 || arrow < 0 || precision < 0 || precision > PREC_FP32X || !tune_valid(tuning))
     return STILES_ERR_INVALID_ARG;
-  const Shape sh{nt, b, band < nt - 1 ? band : nt - 1, arrow, precision, tuning};
+  Shape sh{nt, b, band < nt - 1 ? band : nt - 1, arrow, precision, tuning};
+  sh.planes = use_planes(sh);
   Plan p;
   const int rc = build_serve_template(sh, 0, &p);
   if (rc) return rc;

@@ -809,17 +809,22 @@ __device__ __forceinline__ void stage_mmas(uint32_t tmem, uint32_t a0, bool acc)
 // POTRFs). |H 2^32 + Lo| < 2^76: its low 16 bits are rounded off first, 2^-58 or
 // less of the largest entries' product, a quarter of what the dropped digit
 // levels weigh.
-__device__ __forceinline__ double scaled_sum(long long H, long long Lo, int k2) {
-  const long long T = (H << 16) + ((Lo + (1ll << 15)) >> 16);
-  if (T == 0) return 0.0;
-  const unsigned long long sign = (unsigned long long)T & 0x8000000000000000ull;
-  const unsigned long long mag = sign ? 0ull - (unsigned long long)T : (unsigned long long)T;
+// `slow` is set when the result leaves the normal range (scaled_sum_any then).
+__device__ __forceinline__ long long rounded_sum(long long H, long long Lo) { return (H << 16) + ((Lo + (1ll << 15)) >> 16); }
+__device__ __forceinline__ double scaled_sum(long long H, long long Lo, int k2, bool& slow) {
+  const long long T = rounded_sum(H, Lo);
+  const unsigned long long sign = (unsigned long long)(T >> 63);  // all ones for a negative sum
+  const unsigned long long mag = ((unsigned long long)T ^ sign) - sign;
   const int lz = __clzll((long long)mag);
-  const unsigned long long norm = mag << lz;                             // top bit set
+  const unsigned long long norm = mag << (lz & 63);                      // top bit set
   const unsigned long long mant = (norm >> 11) + ((norm >> 10) & 1ull);  // 2^52 .. 2^53
   const int e = (63 - lz) + 16 + k2 + 1023;                              // biased exponent
-  if (e >= 1 && e < 0x7fe) return __longlong_as_double((long long)((((unsigned long long)(e - 1) << 52) + mant) | sign));
-  return ldexp((double)T, k2 + 16);  // subnormal or beyond the range
+  slow = slow || (T != 0 && (unsigned)(e - 1) >= 0x7fdu);
+  const unsigned long long bits = (((unsigned long long)(unsigned)(e - 1) << 52) + mant) | (sign << 63);
+  return T == 0 ? 0.0 : __longlong_as_double((long long)bits);
+}
+__device__ __noinline__ double scaled_sum_any(long long H, long long Lo, int k2) {
+  return ldexp((double)rounded_sum(H, Lo), k2 + 16);
 }
 
 // acc += cell 2^sh for an integer-valued FP32 cell. SMALL (at most 64 of K, so
@@ -892,13 +897,25 @@ __device__ __forceinline__ void drain_cells(uint32_t tmem, uint8_t* xch, int er,
       }
       __syncthreads();
       sums(16 * side + 4 * i, hi, lo);
+      bool slow = false;
+      double v[4];
+      int k2[4];
 #pragma unroll
       for (int x = 0; x < 4; ++x) {
         const int e = x * 64 + row, ec = cexp[16 * side + 4 * i + x];
-        const long long H = side == 0 ? hi[x] : xhl[2 * e], Lo = lo[x] + (side == 0 ? xlo[e] : xhl[2 * e + 1]);
-        r16[x] = (er == 0x7ff || ec == 0x7ff) ? __longlong_as_double(0x7ff8000000000000ll)
-                                              : r16[x] + scaled_sum(H, Lo, max(er, 1) + max(ec, 1) - kScale);
+        hi[x] = side == 0 ? hi[x] : xhl[2 * e];
+        lo[x] += side == 0 ? xlo[e] : xhl[2 * e + 1];
+        k2[x] = max(er, 1) + max(ec, 1) - kScale;
+        v[x] = scaled_sum(hi[x], lo[x], k2[x], slow);
+        if (er == 0x7ff || ec == 0x7ff) v[x] = __longlong_as_double(0x7ff8000000000000ll);
       }
+      if (slow) {
+#pragma unroll
+        for (int x = 0; x < 4; ++x)
+          if (v[x] == v[x]) v[x] = scaled_sum_any(hi[x], lo[x], k2[x]);
+      }
+#pragma unroll
+      for (int x = 0; x < 4; ++x) r16[x] += v[x];
     } else {
       float* x0 = reinterpret_cast<float*>(buf);  // [4 c][64 r] plane 0, then plane 2, for side 1
       float* x1 = x0 + 2 * 4 * 64;                // [4 c][64 r] plane 1, for side 0
@@ -1136,6 +1153,24 @@ __device__ __noinline__ void run_planes(const KParams& p, const Task& tk, int q,
 // thread for 1664 cycles of MMAs) and, for the factor's updates with an inner
 // length of 64, the fixed cost of a task. The 32 x 32 parts before split each
 // operand twice as often and scanned the whole K for exponents first.
+// 8 K-adjacent values of one vector from P (`step` apart), zero from the n-th on.
+// Contiguous ones are read in pairs where `pairs` says that P is 16-byte aligned
+// (single 8-byte loads fetch each 32-byte sector four times: a lane per vector).
+__device__ __forceinline__ void load_octet(const double* P, int64_t step, bool pairs, int n, double (&x)[8]) {
+  if (pairs && n >= 8) {
+#pragma unroll
+    for (int y = 0; y < 4; ++y) {
+      const double2 v = __ldcg(reinterpret_cast<const double2*>(P) + y);
+      x[2 * y] = v.x;
+      x[2 * y + 1] = v.y;
+    }
+  } else {
+#pragma unroll
+    for (int y = 0; y < 8; ++y) x[y] = y < n ? __ldcg(P + (int64_t)y * step) : 0.0;
+  }
+}
+__device__ __forceinline__ bool pairs_ok(const double* P, int ld) { return ((((uintptr_t)P) & 15) | (ld & 1)) == 0; }
+
 // (x[0 .. 3]: op(A), x[4], x[5]: op(B))
 __device__ __forceinline__ void tc_load(const KParams& p, const Task& tk, const Seg& g, int k0, int kc, int q,
                                         double (&x)[6][8]) {
@@ -1144,19 +1179,18 @@ __device__ __forceinline__ void tc_load(const KParams& p, const Task& tk, const 
   const int64_t sa = ta ? 1 : g.lda, sb = tb ? g.ldb : 1;
   const double* A = resolve(p, g.a) + (int64_t)k0 * sa;
   const double* B = resolve(p, g.b) + (int64_t)k0 * sb + (int64_t)(32 * q) * (tb ? 1 : g.ldb);
+  const bool va = ta && pairs_ok(A, g.lda), vb = !tb && pairs_ok(B, g.ldb);
 #pragma unroll
   for (int u = 0; u < 4; ++u) {
     const int v = lane + 32 * (u & 1), k = 8 * (warp + 4 * (u >> 1));
     const double* P = A + (int64_t)v * (ta ? g.lda : 1) + (int64_t)k * sa;
-#pragma unroll
-    for (int y = 0; y < 8; ++y) x[u][y] = v < tk.m && k + y < kc ? __ldcg(P + (int64_t)y * sa) : 0.0;
+    load_octet(P, sa, va, v < tk.m ? kc - k : 0, x[u]);
   }
 #pragma unroll
   for (int u = 0; u < 2; ++u) {
     const int k = 8 * (warp + 4 * u);
     const double* P = B + (int64_t)lane * (tb ? 1 : g.ldb) + (int64_t)k * sb;
-#pragma unroll
-    for (int y = 0; y < 8; ++y) x[4 + u][y] = 32 * q + lane < tk.n && k + y < kc ? __ldcg(P + (int64_t)y * sb) : 0.0;
+    load_octet(P, sb, vb, 32 * q + lane < tk.n ? kc - k : 0, x[4 + u]);
   }
 }
 
@@ -1304,12 +1338,12 @@ __device__ __noinline__ void run_split(const KParams& p, const Task& tk, int q, 
   const double* A = resolve(p, tk.cin);
   A += kcont ? (int64_t)v * tk.ldc + (k0 - tk.gcol) : v + (int64_t)(k0 - tk.gcol) * tk.ldc;
   const int64_t step = kcont ? 1 : tk.ldc;
+  const bool pairs = kcont && pairs_ok(A, tk.ldc);
   double x[8][8];
 #pragma unroll
   for (int u = 0; u < 8; ++u) {
     const int k = 8 * (oct0 + 8 * u);
-#pragma unroll
-    for (int y = 0; y < 8; ++y) x[u][y] = v < tk.m && k + y < kc ? __ldcg(A + (int64_t)(k + y) * step) : 0.0;
+    load_octet(A + (int64_t)k * step, step, pairs, v < tk.m ? kc - k : 0, x[u]);
   }
   int emax = 0;
   const int nch = (tk.zrows + kPlaneChunk - 1) / kPlaneChunk;

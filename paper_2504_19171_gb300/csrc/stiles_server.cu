@@ -123,6 +123,8 @@ struct stiles_server {
   int64_t base_doubles = 0;
   double* data = nullptr;
   int64_t data_doubles = 0;
+  uint8_t* planes = nullptr;  // plane_units units of 16 bytes per request slot, or none
+  int64_t plane_units = 0;
   Task* tasks = nullptr;
   int32_t *rem = nullptr, *pdone = nullptr, *treq = nullptr;
   int64_t task_cap = 0;
@@ -163,6 +165,7 @@ static void free_server(stiles_server* h) {
   if (!h) return;
   cudaFree(h->base);
   cudaFree(h->data);
+  cudaFree(h->planes);
   cudaFree(h->tasks);
   cudaFree(h->rem);
   cudaFree(h->pdone);
@@ -186,11 +189,10 @@ static void free_server(stiles_server* h) {
   delete h;
 }
 
-extern "C" int stiles_server_create(int nshapes, const int* nt, const int* b, const int* band, const int* arrow,
-                                    int precision, const int* tuning, size_t data_bytes, int max_requests,
-                                    stiles_server_t* out) {
-  if (!out) return STILES_ERR_INVALID_ARG;
-  *out = nullptr;
+// `planes`: phase-2 products from planes, whose memory is beside the data arena
+// (one set per request slot) and at most a quarter of it.
+static int create_server(int nshapes, const int* nt, const int* b, const int* band, const int* arrow, int precision,
+                         const int* tuning, size_t data_bytes, int max_requests, bool planes, stiles_server_t* out) {
   if (nshapes < 1 || !nt || !b || !band || !arrow || max_requests < 1 || max_requests > kServeMaxReq)
     return STILES_ERR_INVALID_ARG;
   if (precision != STILES_FP64 && precision != STILES_EMU64 && precision != STILES_FP32X) return STILES_ERR_UNSUPPORTED;
@@ -207,6 +209,7 @@ extern "C" int stiles_server_create(int nshapes, const int* nt, const int* b, co
     }
     ShapeT T;
     T.s = Shape{nt[m], b[m], band[m] < nt[m] - 1 ? band[m] : nt[m] - 1, arrow[m], precision, tune};
+    T.s.planes = planes && use_planes(T.s);
     int rc = build_serve_template(T.s, 0, &T.plan);
     if (rc) {
       delete h;
@@ -220,6 +223,7 @@ extern "C" int stiles_server_create(int nshapes, const int* nt, const int* b, co
       parts += T.plan.tasks[t].parts;
     }
     max_parts = std::max(max_parts, parts);
+    h->plane_units = std::max(h->plane_units, T.plan.plane_units);
     T.base_off = h->base_doubles;
     h->base_doubles += (T.doubles + 2 * T.n + 31) / 32 * 32;
     max_tasks = std::max<int64_t>(max_tasks, (int64_t)T.plan.tasks.size() + 1);
@@ -228,6 +232,11 @@ extern "C" int stiles_server_create(int nshapes, const int* nt, const int* b, co
     max_diag = std::max<int64_t>(max_diag, (int64_t)T.plan.ndiag);
     max_roots = std::max<int64_t>(max_roots, (int64_t)T.roots.size());
     h->shapes.push_back(std::move(T));
+  }
+  h->plane_units = (h->plane_units + 15) / 16 * 16;
+  if (16 * h->plane_units * max_requests > (int64_t)(data_bytes / 4)) {
+    delete h;
+    return create_server(nshapes, nt, b, band, arrow, precision, tuning, data_bytes, max_requests, false, out);
   }
   if (cudaGetDevice(&h->device) != cudaSuccess ||
       cudaDeviceGetAttribute(&h->sms, cudaDevAttrMultiProcessorCount, h->device) != cudaSuccess) {
@@ -246,9 +255,9 @@ extern "C" int stiles_server_create(int nshapes, const int* nt, const int* b, co
   unsigned ring = 1;
   while ((int64_t)ring < k * max_parts && ring < (1u << 30)) ring <<= 1;
   h->ring_mask = ring - 1;
-  int rc = 0;
-  if (!rc) rc = dmalloc(&h->base, h->base_doubles);
+  int rc = dmalloc(&h->base, h->base_doubles);
   if (!rc) rc = dmalloc(&h->data, h->data_doubles);
+  if (!rc && h->plane_units) rc = dmalloc(&h->planes, 16 * h->plane_units * max_requests);
   if (!rc) rc = dmalloc(&h->tasks, h->task_cap);
   if (!rc) rc = dmalloc(&h->rem, h->task_cap);
   if (!rc) rc = dmalloc(&h->pdone, h->task_cap);
@@ -292,6 +301,17 @@ extern "C" int stiles_server_create(int nshapes, const int* nt, const int* b, co
   for (int q = max_requests - 1; q >= 0; --q) h->free_slots.push_back(q);
   *out = h;
   return STILES_OK;
+}
+
+extern "C" int stiles_server_create(int nshapes, const int* nt, const int* b, const int* band, const int* arrow,
+                                    int precision, const int* tuning, size_t data_bytes, int max_requests,
+                                    stiles_server_t* out) {
+  if (!out) return STILES_ERR_INVALID_ARG;
+  *out = nullptr;
+  int rc = create_server(nshapes, nt, b, band, arrow, precision, tuning, data_bytes, max_requests, true, out);
+  if (rc == STILES_ERR_OOM && precision != STILES_FP64)  // memory is tight: do without planes
+    rc = create_server(nshapes, nt, b, band, arrow, precision, tuning, data_bytes, max_requests, false, out);
+  return rc;
 }
 
 extern "C" int stiles_server_shape_doubles(stiles_server_t h, int shape, size_t* doubles, size_t* n) {
@@ -347,6 +367,7 @@ extern "C" int stiles_server_start(stiles_server_t h, double window_s) {
   p.buf[BUF_L] = h->data;
   p.buf[BUF_S] = h->data;
   p.buf[BUF_W] = h->data;
+  p.planes = h->planes;
   p.budget_ns = h->budget_ns;
   p.buf_len = h->data_doubles;
   p.serve = 1;
@@ -457,6 +478,7 @@ static int submit_impl(stiles_server_t h, int shape, double tau, double rho, con
   memset(zero, 0, sizeof(int32_t) * n);
   for (int64_t q = 0; q < R.nd; ++q) minus1[q] = -1;
   const int64_t base = T.base_off;
+  const int64_t p0 = h->plane_units * slot;  // this slot's planes
   for (int64_t t = 0; t < n; ++t) {
     Task x = P.tasks[t];
     if (x.op == OP_PREP) {
@@ -470,6 +492,7 @@ static int submit_impl(stiles_server_t h, int shape, double tau, double rho, con
           case BUF_A: return rebuf(ref, BUF_L, R.dL);  // A is built in place in L
           case BUF_L: return reloc(ref, R.dL);
           case BUF_S: return reloc(ref, R.dS);
+          case BUF_P: return reloc(ref, p0);
           default: return reloc(ref, R.dW);
         }
       };
@@ -491,6 +514,7 @@ static int submit_impl(stiles_server_t h, int shape, double tau, double rho, con
         case BUF_A: return rebuf(ref, BUF_L, R.dL);
         case BUF_L: return reloc(ref, R.dL);
         case BUF_S: return reloc(ref, R.dS);
+        case BUF_P: return reloc(ref, p0);
         default: return reloc(ref, R.dW);
       }
     };
