@@ -93,7 +93,7 @@ struct Builder {
     tasks.push_back(t);
     // parts run side by side on different CTAs
     cost.push_back(kTaskOverheadNs + f / kFlopPerNs / t.parts +
-                   epi_ns / (t.pmode == PM_ROWS2 || t.pmode == PM_ROWS4 || t.pmode == PM_ROWS8 ? t.parts : 1));
+                   epi_ns / (t.pmode == PM_ROWS2 || t.pmode == PM_ROWS4 || t.pmode == PM_ROWS8 || t.pmode == PM_ROWS4F ? t.parts : 1));
     fsegs.insert(fsegs.end(), segs.begin(), segs.end());
     seg_off.push_back((int64_t)fsegs.size());
     fwaits.insert(fwaits.end(), waits.begin(), waits.end());
@@ -123,6 +123,7 @@ struct Builder {
     else if (mode == PM_ROWS4 && t.m > 16) { t.pmode = PM_ROWS4; t.parts = (uint8_t)((t.m + 15) / 16); }
     else if (mode == PM_QUAD4 && t.m > 32 && t.n > 32) { t.pmode = PM_QUAD4; t.parts = 4; }
     else if (mode == PM_TRI3 && t.m > 32 && t.m == t.n) { t.pmode = PM_TRI3; t.parts = 3; }
+    else if (mode == PM_ROWS4F && t.m > 4) { t.pmode = PM_ROWS4F; t.parts = (uint8_t)((t.m + 3) / 4); }
     else if (mode == PM_ROWS8 && t.m > 8) { t.pmode = PM_ROWS8; t.parts = (uint8_t)((t.m + 7) / 8); }
     else if (mode == PM_GRID16 && (t.m > 16 || t.n > 16)) {
       t.pmode = PM_GRID16;
@@ -375,7 +376,7 @@ struct Builder {
     // The critical path's links run as small parts on more CTAs: the FP64
     // newest update of a diagonal block as the 16 x 16 parts of its lower
     // triangle, the final TRSM of the block right below a diagonal block in
-    // parts of 8 rows.
+    // parts of 4 rows.
     const int total_writers = (int)terms.size() + 1;
     lfinal[lidx(i, kq, r, cq)] = total_writers;
     // blocks updated by one source block column: the lower triangle over the
@@ -417,12 +418,16 @@ struct Builder {
     if (nwritten > 0) w.push_back({me, nwritten});
     if (!written && serve) w.push_back({prep_ctr[kq], 1});
     Task tk = blank(diag ? OP_POTRF : OP_TRSM_RLT, m, n);
-    if (!diag) split(tk, dist == 1 || W * crowd <= 2 * kUrgentReach ? PM_ROWS8 : PM_ROWS4);
+    if (!diag) split(tk, dist == 1 ? PM_ROWS4F : W * crowd <= 2 * kUrgentReach ? PM_ROWS8 : PM_ROWS4);
     if (diag || dist <= kUrgentReach) tk.flags |= TF_URGENT;
     tk.out = outref;
     tk.ldo = ld_i;
     tk.cin = written ? outref : mkref(BUF_A, L.blk(i, kq, r, cq));
     tk.ldc = ld_i;
+    // the multipliers of a diagonal block, for the solves with it: in its place in
+    // the scratch tiles, which phase 1 overwrites once the column is final
+    tk.aux = mkref(BUF_W, L.blk(kq, kq, cq, cq));
+    tk.ldx = L.rows(kq);
     std::vector<int32_t> sig{me};
     double epi;
     if (diag) {
@@ -432,8 +437,6 @@ struct Builder {
     } else {
       const int32_t dctr = lctr[lidx(kq, kq, cq, cq)];
       w.push_back({dctr, lfinal[lidx(kq, kq, cq, cq)]});
-      tk.aux = mkref(BUF_L, L.blk(kq, kq, cq, cq));
-      tk.ldx = L.rows(kq);
       epi = 2.0 * n * kSweepStepNs;
     }
     if (kind == PLAN_FUSED) sig.push_back(colfinal[kq]);
@@ -1161,7 +1164,7 @@ int check_plan(const Plan& p) {
     if (tk.seg0 < 0 || tk.nseg < 0 || (int64_t)tk.seg0 + tk.nseg > (int64_t)p.segs.size()) return STILES_ERR_PLAN;
     if (tk.succ0 < 0 || tk.nsucc < 0 || (int64_t)tk.succ0 + tk.nsucc > (int64_t)p.succ.size()) return STILES_ERR_PLAN;
     if (tk.m < 0 || tk.n < 0 || tk.m > FB || tk.n > FB || tk.op > OP_SPLIT) return STILES_ERR_PLAN;
-    if (tk.parts < 1 || tk.parts > kMaxParts || tk.pmode > PM_SPLIT || tk.prec > PREC_FP32X) return STILES_ERR_PLAN;
+    if (tk.parts < 1 || tk.parts > kMaxParts || tk.pmode > PM_ROWS4F || tk.prec > PREC_FP32X) return STILES_ERR_PLAN;
     for (int64_t q = p.wait_off[t]; q < p.wait_off[t + 1]; ++q) {
       const Wait& w = p.waits[q];
       if (w.ctr < 0 || w.ctr >= p.nctr) return STILES_ERR_PLAN;
@@ -1270,7 +1273,7 @@ int validate_plan_len(const Plan& p, int64_t lim, int kind) {
       if (!in(tk.out, r0 + (int64_t)c0 * tk.ldo, r1 + (int64_t)c1 * tk.ldo)) return bad("output out of bounds", t);
       const bool uses_cin = tk.op == OP_UPD || tk.op == OP_POTRF || tk.op == OP_TRSM_RLT || tk.op == OP_SYMUPD;
       if (uses_cin && !in(tk.cin, r0 + (int64_t)c0 * tk.ldc, r1 + (int64_t)c1 * tk.ldc)) return bad("input out of bounds", t);
-      if (tk.op == OP_TRSM_RLT && !in(tk.aux, 0, (tk.n - 1) + (int64_t)(tk.n - 1) * tk.ldx)) return bad("T out of bounds", t);
+      if ((tk.op == OP_TRSM_RLT || tk.op == OP_POTRF) && !in(tk.aux, 0, (tk.n - 1) + (int64_t)(tk.n - 1) * tk.ldx)) return bad("T out of bounds", t);
       if (tk.op == OP_TRTRI && !in(tk.aux, 0, (tk.m - 1) + (int64_t)(tk.m - 1) * tk.ldx))
         return bad("T out of bounds", t);
       if (tk.op == OP_SYMUPD && !(tk.flags & TF_SYM_DIAG) &&
@@ -1452,6 +1455,7 @@ class RaceCheck {
     if (tk.op == OP_TRTRI && !rect(tk.aux, tk.ldx, 0, tk.m, 0, tk.m, id, false, true))
       return false;
     if (!rect(tk.out, tk.ldo, x.r0, x.rm, x.c0, x.cn, id, true)) return false;
+    if (tk.op == OP_POTRF && !rect(tk.aux, tk.ldx, 0, tk.n, 0, tk.n, id, true, true)) return false;
     if (tk.op == OP_SYMUPD && !((tk.flags & TF_SYM_DIAG) && x.r0 == x.c0)) {
       // the transpose of the sub-block: inside the same block, or the mirror block
       const bool dblk = tk.flags & TF_SYM_DIAG;

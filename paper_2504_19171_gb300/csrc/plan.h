@@ -30,8 +30,9 @@ inline int64_t mkref(int buf, int64_t off) { return (int64_t(buf) << BUF_SHIFT) 
 
 enum Op : uint8_t {
   OP_UPD = 0,       // out = cin - acc
-  OP_POTRF = 1,     // out = chol(cin - acc)           (square, lower; zero above the diagonal)
-  OP_TRSM_RLT = 2,  // out = (cin - acc) * T^{-T}      (T = aux, lower n x n)
+  OP_POTRF = 1,     // out = chol(cin - acc)           (square, lower; zero above the diagonal); aux = its
+                    // columns divided by their pivots (below the diagonal) and 1 / L_jj (on it)
+  OP_TRSM_RLT = 2,  // out = (cin - acc) * T^{-T}      (T lower n x n, given by aux as OP_POTRF leaves it)
   OP_TRTRI = 3,     // out = T^{-1}                    (T = aux, lower m x m; zero above)
   OP_STORE = 5,     // out = acc, or -acc (TF_NEG)
   OP_NEG = 6,       // out = -acc
@@ -55,6 +56,7 @@ enum PartMode : uint8_t {
   PM_ROWS4 = 4,  // rows [0,16), [16,32), ..
   PM_TILE32 = 5, // a grid of at most 2 x 2 sub-tiles of at most 32 x 32 (parts = row tiles x column tiles)
   PM_ROWS8 = 6,  // rows [0,8), [8,16), ..
+  PM_ROWS4F = 11, // rows [0,4), [4,8), ..
   PM_GRID16 = 7, // a grid of at most 4 x 4 sub-tiles of at most 16 x 16 (parts = row tiles x column tiles)
   PM_COLS2 = 9,  // columns [0,32) and [32,64) (products from planes)
   PM_SPLIT = 10, // OP_SPLIT: 16 vectors x 512 of K
@@ -118,6 +120,7 @@ inline Sub part_sub(int pmode, int m, int n, int q) {
     case PM_ROWS2: s.r0 = 32 * q; s.rm = 32; break;
     case PM_ROWS4: s.r0 = 16 * q; s.rm = 16; break;
     case PM_ROWS8: s.r0 = 8 * q; s.rm = 8; break;
+    case PM_ROWS4F: s.r0 = 4 * q; s.rm = 4; break;
     case PM_COLS2: s.c0 = 32 * q; s.cn = 32; break;
     case PM_QUAD4: dim = 32; s.r0 = 32 * (q & 1); s.c0 = 32 * (q >> 1); break;
     case PM_TRI3: dim = 32; s.r0 = q == 0 ? 0 : 32; s.c0 = q == 2 ? 32 : 0; break;

@@ -532,10 +532,14 @@ __device__ void run_prep(const KParams& p, const Task& tk, int t) {
 // with 128 threads as a 16 x 8 grid (tx = tid % 16, ty = tid / 16): a
 // (16 TM) x (8 TN) sub-tile, staged KC columns of K at a time in shared
 // memory through L2-only loads.
+// (the 16 x 16 parts of critical paths: 64 at a time, every load of a stage in
+// flight at once, in rows of 17 values).
 template <int TM, int TN>
 __device__ __forceinline__ void accumulate(const KParams& p, const Task& tk, const Sub& sb, double (&acc)[TM][TN],
                                            double* As, double* Bs) {
   constexpr int RM = 16 * TM, CN = 8 * TN;
+  constexpr bool SMALL = TM == 1 && TN == 2;
+  constexpr int KC = SMALL ? 64 : stiles::KC, LDS = SMALL ? 17 : stiles::LDS;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const int ntm = (sb.rm + 15) / 16, ntn = (sb.cn + 7) / 8;
   const bool full = ntm == TM && ntn == TN;
@@ -1407,25 +1411,23 @@ __device__ __forceinline__ void acc_to_smem(const KParams& p, const Task& tk, co
     }
 }
 
-// T[r][c] = lower triangle of the dim x dim block at tk.aux (zero above):
-// thread t reads rows t % 64 of columns t / 64, +2, +4, ... in batches of 8
-// loads in flight before their shared-memory stores.
+// T[r][c] = lower triangle of the dim x dim block at tk.aux (zero above): thread
+// t reads rows t % 64 of columns t / 64, +2, +4, ..., every load in flight before
+// the first shared-memory store (one round trip to L2).
 __device__ __forceinline__ void load_tri(const KParams& p, const Task& tk, int dim, double* T) {
   const double* S = resolve(p, tk.aux);
   const int r = threadIdx.x & (FB - 1), c0 = threadIdx.x / FB;
-  constexpr int kStep = NTHREADS / FB, kBatch = 8;
-  for (int cb = c0; cb < FB; cb += kStep * kBatch) {
-    double v[kBatch];
+  constexpr int kStep = NTHREADS / FB, kBatch = FB / kStep;
+  double v[kBatch];
 #pragma unroll
-    for (int u = 0; u < kBatch; ++u) {
-      const int c = cb + u * kStep;
-      v[u] = (r < dim && c < dim && r >= c) ? __ldcg(S + r + (int64_t)c * tk.ldx) : 0.0;
-    }
+  for (int u = 0; u < kBatch; ++u) {
+    const int c = c0 + u * kStep;
+    v[u] = (r < dim && c < dim && r >= c) ? __ldcg(S + r + (int64_t)c * tk.ldx) : 0.0;
+  }
 #pragma unroll
-    for (int u = 0; u < kBatch; ++u) {
-      const int c = cb + u * kStep;
-      if (r < dim && c < dim) T[r * LDS + c] = v[u];
-    }
+  for (int u = 0; u < kBatch; ++u) {
+    const int c = c0 + u * kStep;
+    if (r < dim && c < dim) T[r * LDS + c] = v[u];
   }
 }
 
@@ -1444,70 +1446,40 @@ __device__ __forceinline__ void store_sub(const KParams& p, const Task& tk, cons
 // barriers in their inner loops: independent rows (or columns) are owned by
 // one warp and stepped with __syncwarp only.
 
-// X (m x n, m <= 16) <- X T^{-T} with the row values in registers: T lower
-// n x n with its strict lower part already divided by the pivot of its column
-// (Tn[c][j] = T[c][j] / T[j][j]), rcp[j*LDS] = 1 / T[j][j]. Warp w owns rows
-// 4w .. 4w+3; the 8 lanes of a row hold its columns ph, ph+8, ... (ph = lane /
-// 4). Step j takes the finished (not yet scaled) value y_j of each row from
-// the lane that holds it (a shuffle) and subtracts y_j Tn[c][j] from the
-// columns c > j; x = y / diag(T) at the end. No shared-memory round trip and
-// no one-lane scaling between two steps.
-__device__ __forceinline__ void trsm_rows_lt16(double* X, const double* Tn, const double* rcp, int m, int n) {
-  static_assert(FB == 64, "8 lanes x 8 columns per row");
+// X (m x n, m <= 128 / LANES) <- X T^{-T} with the row values in registers. Tn: the
+// block POTRF's multipliers T[c][j] / T[j][j] below the diagonal, 1 / T[j][j] on
+// it. The LANES lanes of a row hold its columns ph, ph + LANES, ...; step j takes
+// the finished (not yet scaled) value y_j of each row from the lane that holds it
+// (a shuffle) and subtracts y_j Tn[c][j] from the columns c > j; x = y / diag(T)
+// at the end. No shared-memory round trip, division or scaling between two steps.
+// LANES = 8, 16, 32 for parts of 16, 8, 4 rows: at most 64 / LANES multiply-adds
+// per step and lane (10k and 6k cycles of the FP64 pipe for 8 and 4 rows).
+template <int LANES>
+__device__ __forceinline__ void trsm_rows(double* X, const double* Tn, int m, int n) {
+  constexpr int R = 32 / LANES, Q = FB / LANES;  // rows per warp, columns per lane
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int r = warp * 4 + (lane & 3), ph = lane >> 2;
+  const int r = warp * R + lane % R, ph = lane / R;
   const bool own = r < m;
-  double y[8];
+  double y[Q];
 #pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    const int c = ph + 8 * q;
+  for (int q = 0; q < Q; ++q) {
+    const int c = ph + LANES * q;
     y[q] = own && c < n ? X[r * LDS + c] : 0.0;
   }
 #pragma unroll
   for (int j = 0; j < FB; ++j) {
     if (j >= n) break;
-    const double yj = __shfl_sync(0xffffffffu, y[j >> 3], (lane & 3) + 4 * (j & 7));
+    const double yj = __shfl_sync(0xffffffffu, y[j / LANES], lane % R + R * (j % LANES));
 #pragma unroll
-    for (int q = j >> 3; q < 8; ++q) {
-      const int c = ph + 8 * q;
+    for (int q = j / LANES; q < Q; ++q) {
+      const int c = ph + LANES * q;
       if (c > j) y[q] = fma(-yj, Tn[c * LDS + j], y[q]);
     }
   }
 #pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    const int c = ph + 8 * q;
-    if (own && c < n) X[r * LDS + c] = y[q] * rcp[c * LDS];
-  }
-}
-
-// The same for m <= 8 (the parts of a row-split block on the factorization's
-// critical path): two rows per warp, 16 lanes per row, so that a lane applies
-// at most four columns per step.
-__device__ __forceinline__ void trsm_rows_lt8(double* X, const double* Tn, const double* rcp, int m, int n) {
-  static_assert(FB == 64, "16 lanes x 4 columns per row");
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int r = warp * 2 + (lane & 1), ph = lane >> 1;
-  const bool own = r < m;
-  double y[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int c = ph + 16 * q;
-    y[q] = own && c < n ? X[r * LDS + c] : 0.0;
-  }
-#pragma unroll
-  for (int j = 0; j < FB; ++j) {
-    if (j >= n) break;
-    const double yj = __shfl_sync(0xffffffffu, y[j >> 4], (lane & 1) + 2 * (j & 15));
-#pragma unroll
-    for (int q = j >> 4; q < 4; ++q) {
-      const int c = ph + 16 * q;
-      if (c > j) y[q] = fma(-yj, Tn[c * LDS + j], y[q]);
-    }
-  }
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int c = ph + 16 * q;
-    if (own && c < n) X[r * LDS + c] = y[q] * rcp[c * LDS];
+  for (int q = 0; q < Q; ++q) {
+    const int c = ph + LANES * q;
+    if (own && c < n) X[r * LDS + c] = y[q] * Tn[c * LDS + c];
   }
 }
 
@@ -1561,7 +1533,8 @@ constexpr int PT_M = 0;                       // two multiplier buffers, FB x PM
 constexpr int PT_PIV = PT_M + 2 * FB * PMS;   // pivots d_j
 constexpr int PT_RS = PT_PIV + FB;            // scale of column j
 constexpr int PT_DIAG = PT_RS + FB;           // L_jj
-static_assert(PT_DIAG + FB <= 2 * KC * LDS, "fits in the staging region");
+constexpr int PT_RCP = PT_DIAG + FB;          // 1 / L_jj
+static_assert(PT_RCP + FB <= 2 * KC * LDS, "fits in the staging region");
 // a panel's time in batches of the trailing update (16 multiply-adds of 64 cycles)
 constexpr int PBATCH = 1;
 
@@ -1693,7 +1666,7 @@ __device__ __forceinline__ void potrf_update(double* X, const double* M, int j0,
 
 // The factorization of X; `S` is the staging region. On return (after a block
 // barrier) L = X diag(scale): column j times S[PT_RS + j], whose diagonal
-// entry is S[PT_DIAG + j].
+// entry is S[PT_DIAG + j] and its reciprocal S[PT_RCP + j].
 __device__ void potrf_smem(double* X, double* S, int n) {
   static_assert(FB % PNB == 0 && FB - PNB <= 3 * PROWS, "panels; three warps hold a panel's rows");
   static_assert(FB * PNB <= 2 * NTHREADS, "a panel's columns are two elements per thread");
@@ -1741,6 +1714,7 @@ __device__ void potrf_smem(double* X, double* S, int n) {
     const double d = piv[tid];
     const double r = rsqrt(d);
     S[PT_DIAG + tid] = d * r;
+    S[PT_RCP + tid] = r;
     rs[tid] = rs[tid] == 0.0 ? r : 1.0;
   }
   __syncthreads();
@@ -1781,9 +1755,20 @@ __device__ void run_sub(const KParams& p, const Task& tk, const Sub& sb, double*
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   const int m = tk.m, n = tk.n;
   double acc[TM][TN];
-  if (tk.op != OP_TRTRI) {
-    accumulate<TM, TN>(p, tk, sb, acc, As, Bs);
+  // the small parts of critical paths have their input block in flight meanwhile
+  constexpr bool EARLY = TM == 1 && TN == 2;
+  double cin[TM][TN];
+  if constexpr (EARLY) {
+    const double* C = tk.op == OP_UPD ? resolve(p, tk.cin) + sb.r0 + (int64_t)sb.c0 * tk.ldc : nullptr;
+#pragma unroll
+    for (int i = 0; i < TM; ++i)
+#pragma unroll
+      for (int j = 0; j < TN; ++j) {
+        const int r = tx + 16 * i, c = ty + 8 * j;
+        cin[i][j] = C && r < sb.rm && c < sb.cn ? __ldcg(C + r + (int64_t)c * tk.ldc) : 0.0;
+      }
   }
+  if (tk.op != OP_TRTRI) accumulate<TM, TN>(p, tk, sb, acc, As, Bs);
 
   switch (tk.op) {
     case OP_UPD:
@@ -1802,7 +1787,7 @@ __device__ void run_sub(const KParams& p, const Task& tk, const Sub& sb, double*
           const int r = tx + 16 * i, c = ty + 8 * j;
           if (r < sb.rm && c < sb.cn) {
             double v = acc[i][j];
-            if (tk.op == OP_UPD) v = __ldcg(C + r + (int64_t)c * tk.ldc) - v;
+            if (tk.op == OP_UPD) v = (EARLY ? cin[i][j] : __ldcg(C + r + (int64_t)c * tk.ldc)) - v;
             else if (tk.op == OP_NEG || (tk.flags & TF_NEG)) v = -v;
             O[r + (int64_t)c * tk.ldo] = v;
             if (Om) Om[r + (int64_t)c * tk.ldo] = v;
@@ -1847,19 +1832,12 @@ __device__ void run_sub(const KParams& p, const Task& tk, const Sub& sb, double*
       break;
     }
     case OP_TRSM_RLT: {  // X = (C - acc) T^{-T}, T lower n x n: rows are independent
-      acc_to_smem<TM, TN>(p, tk, sb, acc, X, true, 1.0);
       load_tri(p, tk, n, T);
+      acc_to_smem<TM, TN>(p, tk, sb, acc, X, true, 1.0);
       __syncthreads();
-      double* rcp = T + FB;  // column FB of T's padded rows is free: rcp[j * LDS]
-      if (tid < n) rcp[tid * LDS] = 1.0 / T[tid * LDS + tid];
-      __syncthreads();
-      // (parts have at most 16 rows; the strict lower part divided by its pivots)
-      const int warp = tid >> 5, lane = tid & 31;
-      for (int c = warp + 1; c < n; c += NTHREADS / 32)
-        for (int j = lane; j < c; j += 32) T[c * LDS + j] *= rcp[j * LDS];
-      __syncthreads();
-      if (sb.rm <= 8) trsm_rows_lt8(X, T, rcp, sb.rm, n);
-      else trsm_rows_lt16(X, T, rcp, sb.rm, n);
+      if (sb.rm <= 4) trsm_rows<32>(X, T, sb.rm, n);
+      else if (sb.rm <= 8) trsm_rows<16>(X, T, sb.rm, n);
+      else trsm_rows<8>(X, T, sb.rm, n);  // parts have at most 16 rows
       __syncthreads();
       store_sub(p, tk, sb, X, false);
       break;
@@ -1873,10 +1851,14 @@ __device__ void run_sub(const KParams& p, const Task& tk, const Sub& sb, double*
             __syncthreads();
             potrf_smem(X, smem, n);
             double* O = resolve(p, tk.out);
+            double* Mo = resolve(p, tk.aux);  // multipliers and 1 / L_jj for the solves with this block
             for (int e = tid; e < FB * FB; e += NTHREADS) {
               const int r = e % FB, c = e / FB;
-              if (r < n && c < n)
-                O[r + (int64_t)c * tk.ldo] = r < c ? 0.0 : r == c ? smem[PT_DIAG + c] : X[r * LDS + c] * smem[PT_RS + c];
+              if (r < n && c < n) {
+                const double l = r < c ? 0.0 : r == c ? smem[PT_DIAG + c] : X[r * LDS + c] * smem[PT_RS + c];
+                O[r + (int64_t)c * tk.ldo] = l;
+                if (r >= c) Mo[r + (int64_t)c * tk.ldx] = r == c ? smem[PT_RCP + c] : l * smem[PT_RCP + c];
+              }
             }
             break;
           }
@@ -1928,7 +1910,8 @@ __device__ bool task_part_ok(const KParams& p, const Task& tk, const Sub& sb) {
   if (!ref_ok(p, tk.out, r0 + (int64_t)c0 * tk.ldo, r1 + (int64_t)c1 * tk.ldo)) return false;
   const bool cin = tk.op == OP_UPD || tk.op == OP_POTRF || tk.op == OP_TRSM_RLT || tk.op == OP_SYMUPD;
   if (cin && !ref_ok(p, tk.cin, r0 + (int64_t)c0 * tk.ldc, r1 + (int64_t)c1 * tk.ldc)) return false;
-  if (tk.op == OP_TRSM_RLT && !ref_ok(p, tk.aux, 0, (tk.n - 1) + (int64_t)(tk.n - 1) * tk.ldx)) return false;
+  if ((tk.op == OP_TRSM_RLT || tk.op == OP_POTRF) && !ref_ok(p, tk.aux, 0, (tk.n - 1) + (int64_t)(tk.n - 1) * tk.ldx))
+    return false;
   if (tk.op == OP_TRTRI && !ref_ok(p, tk.aux, 0, (tk.m - 1) + (int64_t)(tk.m - 1) * tk.ldx))
     return false;
   if (tk.op == OP_SYMUPD && !(tk.flags & TF_SYM_DIAG) && !ref_ok(p, tk.aux, c0 + (int64_t)r0 * tk.ldx, c1 + (int64_t)r1 * tk.ldx))
@@ -1995,7 +1978,8 @@ __device__ void run_task(const KParams& p, const Task& tk, int t, int q, double*
   switch (tk.pmode) {
     case PM_ROWS2: run_sub<2, 8>(p, tk, sb, smem); break;
     case PM_ROWS4:
-    case PM_ROWS8: run_sub<1, 8>(p, tk, sb, smem); break;
+    case PM_ROWS8:
+    case PM_ROWS4F: run_sub<1, 8>(p, tk, sb, smem); break;
     case PM_TRI16:
     case PM_GRID16: run_sub<1, 2>(p, tk, sb, smem); break;
     case PM_QUAD4:
