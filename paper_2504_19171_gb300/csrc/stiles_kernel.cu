@@ -1519,11 +1519,12 @@ __device__ __forceinline__ void trsm_cols_ln(double* X, const double* T, const d
 //     0-3 of every warp that takes part, so no warp waits for another); four
 //     columns keep the multiply-adds inside the panel (6) off the chain, eight
 //     (28) took 2.5 times as long per panel;
-//   * the trailing update takes a panel at a time; the next panel's columns
-//     first, so that the next panel runs while the other warps, and then its
-//     own, apply the rest (batches of 32 2 x 2 elements of the packed lower
-//     triangle, shared out by their FP64 time; single elements claimed from a
-//     counter, their rows found by a division, took three times as long).
+//   * the trailing update takes a panel at a time; the next panel's own columns
+//     take it in the next panel's registers, so that one barrier a panel is
+//     enough and the next panel runs while the other warps, and then its own,
+//     apply the rest (batches of 32 2 x 2 elements of the packed lower triangle,
+//     shared out by their FP64 time; single elements claimed from a counter,
+//     their rows found by a division, took three times as long).
 
 constexpr int PNB = 4;           // panel width
 constexpr int PROWS = 32 - PNB;  // rows below the panel's own per warp
@@ -1536,7 +1537,7 @@ constexpr int PT_DIAG = PT_RS + FB;           // L_jj
 constexpr int PT_RCP = PT_DIAG + FB;          // 1 / L_jj
 static_assert(PT_RCP + FB <= 2 * KC * LDS, "fits in the staging region");
 // a panel's time in batches of the trailing update (16 multiply-adds of 64 cycles)
-constexpr int PBATCH = 1;
+constexpr int PBATCH = 2;
 
 // ceil(2^20 / w): e / w = (e * kInv20[w]) >> 20 for the e < 1600 walked here
 struct Inv20 {
@@ -1578,15 +1579,33 @@ __device__ __forceinline__ bool recip_range(double d) {  // recip_fixed's range
 // back to X, the multipliers to M and the pivots. A pivot whose reciprocal
 // leaves the normal range (zero, subnormal, above 2^1020, not finite) has its
 // column scaled by d^-1/2 at once (m = l), and a 1 left in its scale slot: the
-// panel is then done again that way, from the columns still in X.
-__device__ __forceinline__ void potrf_panel(double* X, double* M, double* piv, double* rs, int j0, int n, int cw) {
+// panel is then done again that way.
+// The panel before (its multipliers Mp, columns j0 - 4 ..) has updated every column
+// but this panel's: that update is applied here first (16 multiply-adds a row).
+__device__ __forceinline__ void potrf_panel(double* X, double* M, const double* Mp, double* piv, double* rs, int j0, int n,
+                                            int cw) {
   const unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
   const int row = j0 + (lane < PNB ? lane : PROWS * cw + lane);
   const bool own = row < n;
-  double a[PNB], m[PNB], d[PNB], fin[PNB];
+  double a[PNB], a0[PNB], m[PNB], d[PNB], fin[PNB];
 #pragma unroll
   for (int k = 0; k < PNB; ++k) a[k] = own ? X[row * LDS + j0 + k] : 0.0;
+  if (j0 > 0) {
+    double mr[PNB], u[PNB][PNB];
+#pragma unroll
+    for (int k = 0; k < PNB; ++k) mr[k] = own ? Mp[row * PMS + k] : 0.0;
+#pragma unroll
+    for (int c = 0; c < PNB; ++c)
+#pragma unroll
+      for (int k = 0; k < PNB; ++k) u[c][k] = X[(j0 + c) * LDS + j0 - PNB + k];
+#pragma unroll
+    for (int c = 0; c < PNB; ++c)
+#pragma unroll
+      for (int k = 0; k < PNB; ++k) a[c] = fma(-mr[k], u[c][k], a[c]);
+  }
+#pragma unroll
+  for (int k = 0; k < PNB; ++k) a0[k] = a[k];
   bool range = true;
 #pragma unroll
   for (int j = 0; j < PNB; ++j) {
@@ -1602,7 +1621,7 @@ __device__ __forceinline__ void potrf_panel(double* X, double* M, double* piv, d
   }
   if (!range) {
 #pragma unroll
-    for (int k = 0; k < PNB; ++k) a[k] = own ? X[row * LDS + j0 + k] : 0.0;
+    for (int k = 0; k < PNB; ++k) a[k] = a0[k];
 #pragma unroll
     for (int j = 0; j < PNB; ++j) {
       d[j] = __shfl_sync(FULL, a[j], j);
@@ -1634,42 +1653,49 @@ __device__ __forceinline__ void potrf_panel(double* X, double* M, double* piv, d
   }
 }
 
-// 2 x TC elements (rows r, r + 1; columns c ..) of a trailing update by the
+// 2 x 2 elements (rows r, r + 1; columns c, c + 1) of a trailing update by the
 // panel at j0: X[r][c] -= sum_k M[r][k] X[c][j0 + k]. Elements above the
-// diagonal are computed and not stored.
-template <int TC>
-__device__ __forceinline__ void potrf_update(double* X, const double* M, int j0, int r, int c) {
-  double x[2][TC], m[2][PNB], u[TC][PNB];
+// diagonal are computed and not stored. load / apply: the operands of the next
+// batch are read while the pipe works on this one.
+struct PotrfTile {
+  double x[2][2], m[2][PNB], u[2][PNB];
+  int at;  // of (r, c); -1: none
+  bool diag;
+  __device__ __forceinline__ void load(const double* X, const double* M, int j0, int r, int c, bool own) {
+    at = own ? r * LDS + c : -1;
+    diag = r == c;
+    const double *Xr = X + (own ? r * LDS + c : 0), *Mr = M + (own ? r * PMS : 0), *Xc = X + (own ? c * LDS : 0) + j0;
 #pragma unroll
-  for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < 2; ++i) {
 #pragma unroll
-    for (int t = 0; t < TC; ++t) x[i][t] = X[(r + i) * LDS + c + t];
+      for (int t = 0; t < 2; ++t) x[i][t] = Xr[i * LDS + t];
 #pragma unroll
-    for (int k = 0; k < PNB; ++k) m[i][k] = M[(r + i) * PMS + k];
+      for (int k = 0; k < PNB; ++k) m[i][k] = Mr[i * PMS + k];
+#pragma unroll
+      for (int k = 0; k < PNB; ++k) u[i][k] = Xc[i * LDS + k];
+    }
   }
+  __device__ __forceinline__ void apply(double* X) {
 #pragma unroll
-  for (int t = 0; t < TC; ++t)
+    for (int k = 0; k < PNB; ++k)
 #pragma unroll
-    for (int k = 0; k < PNB; ++k) u[t][k] = X[(c + t) * LDS + j0 + k];
+      for (int i = 0; i < 2; ++i)
 #pragma unroll
-  for (int k = 0; k < PNB; ++k)
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-      for (int t = 0; t < TC; ++t) x[i][t] = fma(-m[i][k], u[t][k], x[i][t]);
-#pragma unroll
-  for (int i = 0; i < 2; ++i)
-#pragma unroll
-    for (int t = 0; t < TC; ++t)
-      if (r + i >= c + t) X[(r + i) * LDS + c + t] = x[i][t];
-}
+        for (int t = 0; t < 2; ++t) x[i][t] = fma(-m[i][k], u[t][k], x[i][t]);
+    if (at >= 0) {
+      X[at] = x[0][0];
+      if (!diag) X[at + 1] = x[0][1];
+      X[at + LDS] = x[1][0];
+      X[at + LDS + 1] = x[1][1];
+    }
+  }
+};
 
 // The factorization of X; `S` is the staging region. On return (after a block
 // barrier) L = X diag(scale): column j times S[PT_RS + j], whose diagonal
 // entry is S[PT_DIAG + j] and its reciprocal S[PT_RCP + j].
-__device__ void potrf_smem(double* X, double* S, int n) {
+__device__ __noinline__ void potrf_smem(double* X, double* S, int n) {
   static_assert(FB % PNB == 0 && FB - PNB <= 3 * PROWS, "panels; three warps hold a panel's rows");
-  static_assert(FB * PNB <= 2 * NTHREADS, "a panel's columns are two elements per thread");
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   double *piv = S + PT_PIV, *rs = S + PT_RS;
   const int np = (n + PNB - 1) / PNB * PNB;
@@ -1678,20 +1704,15 @@ __device__ void potrf_smem(double* X, double* S, int n) {
     X[r * LDS + c] = r == c ? 1.0 : 0.0;
   }
   __syncthreads();
-  if (warp == 0 || (warp < 3 && PNB + PROWS * warp < np)) potrf_panel(X, S + PT_M, piv, rs, 0, np, warp);
+  if (warp == 0 || (warp < 3 && PNB + PROWS * warp < np)) potrf_panel(X, S + PT_M, nullptr, piv, rs, 0, np, warp);
   for (int j0 = 0; j0 + PNB < np; j0 += PNB) {
     const int j1 = j0 + PNB, j2 = j1 + PNB, pb = j0 / PNB;
     const double* M = S + PT_M + (pb & 1) * FB * PMS;
     double* Mn = S + PT_M + ((pb & 1) ^ 1) * FB * PMS;
     __syncthreads();
-    {  // the next panel's columns
-      const int r = j1 + 2 * (tid / PNB), c = j1 + tid % PNB;
-      if (r < np && r + 1 >= c) potrf_update<1>(X, M, j0, r, c);
-    }
-    __syncthreads();
     // warps 0 .. npw - 1 hold the panel's rows
     const int npw = 1 + (j1 + PNB + PROWS < np) + (j1 + PNB + 2 * PROWS < np);
-    if (warp < npw) potrf_panel(X, Mn, piv, rs, j1, np, warp);
+    if (warp < npw) potrf_panel(X, Mn, M, piv, rs, j1, np, warp);
     // columns j2 .. np - 1: the lower triangle in 2 x 2 elements, h of them
     // wide (even), line a (a + 1 of them) folded with line h - 1 - a; every
     // warp gets the same time, the panel's warps less by the panel
@@ -1701,12 +1722,23 @@ __device__ void potrf_smem(double* X, double* S, int n) {
     int b = warp < npw ? others + mine * warp : each * (warp - npw);
     const int b1 = warp < npw ? b + mine : min(others, b + each);
     const uint32_t inv = kInv20.v[w1];
-#pragma unroll 1
-    for (; b < b1; ++b) {
-      const int e = 32 * b + lane, i = (int)((e * inv) >> 20), kk = e - i * w1;
+    auto load_batch = [&](PotrfTile& t, int bb) {
+      const int e = 32 * bb + lane, i = (int)((e * inv) >> 20), kk = e - i * w1;
       const bool low = kk <= i;
-      const int r = j2 + 2 * (low ? i : h - 1 - i), c = j2 + 2 * (low ? kk : kk - i - 1);
-      if (e < ne) potrf_update<2>(X, M, j0, r, c);
+      t.load(X, M, j0, j2 + 2 * (low ? i : h - 1 - i), j2 + 2 * (low ? kk : kk - i - 1), e < ne);
+    };
+    if (b < b1) {
+      PotrfTile t0, t1;
+      load_batch(t0, b);
+#pragma unroll 1
+      for (;;) {
+        load_batch(t1, min(b + 1, b1 - 1));
+        t0.apply(X);
+        if (++b >= b1) break;
+        load_batch(t0, min(b + 1, b1 - 1));
+        t1.apply(X);
+        if (++b >= b1) break;
+      }
     }
   }
   __syncthreads();
@@ -1852,12 +1884,17 @@ __device__ void run_sub(const KParams& p, const Task& tk, const Sub& sb, double*
             potrf_smem(X, smem, n);
             double* O = resolve(p, tk.out);
             double* Mo = resolve(p, tk.aux);  // multipliers and 1 / L_jj for the solves with this block
-            for (int e = tid; e < FB * FB; e += NTHREADS) {
-              const int r = e % FB, c = e / FB;
-              if (r < n && c < n) {
-                const double l = r < c ? 0.0 : r == c ? smem[PT_DIAG + c] : X[r * LDS + c] * smem[PT_RS + c];
-                O[r + (int64_t)c * tk.ldo] = l;
-                if (r >= c) Mo[r + (int64_t)c * tk.ldx] = r == c ? smem[PT_RCP + c] : l * smem[PT_RCP + c];
+            for (int c = tid >> 5; c < n; c += NTHREADS / 32) {  // a warp per column
+              const double rs = smem[PT_RS + c], rcp = smem[PT_RCP + c];
+#pragma unroll
+              for (int h = 0; h < FB / 32; ++h) {
+                const int r = 32 * h + (tid & 31);
+                double l = 0.0;
+                if (32 * h + 31 >= c) {  // not all above the diagonal: no FP64 instruction for those
+                  if (r >= c) l = r == c ? smem[PT_DIAG + c] : X[r * LDS + c] * rs;
+                  if (r >= c && r < n) Mo[r + (int64_t)c * tk.ldx] = r == c ? rcp : l * rcp;
+                }
+                if (r < n) O[r + (int64_t)c * tk.ldo] = l;
               }
             }
             break;
