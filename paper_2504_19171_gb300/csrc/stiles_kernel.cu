@@ -20,9 +20,9 @@
 // from a stale L1 line) and accumulates up to a 64 x 64 block in registers
 // (4 x 8 per thread). The reduced-precision modes replace the products of
 // the bulk tasks by split-precision digit products on the tensor cores
-// (tcgen05 MMAs from shared memory into tensor memory): 8 digits per operand
-// for emulated FP64, 4 for the FP32-class mode. In the end-to-end call the matrix may live in
-// page-locked host memory (read over the host link by the tasks that first
+// (tcgen05 MMAs from shared memory into tensor memory): 8 fixed-point digits
+// per operand for emulated FP64, 3 bf16 pieces for the FP32-class mode. In the
+// end-to-end call the matrix may live in page-locked host memory (read over the host link by the tasks that first
 // load each block) and every final Sigma write is repeated into a host
 // buffer, so the transfers overlap the computation.
 #include <cuda/atomic>
@@ -1591,31 +1591,34 @@ __device__ __forceinline__ void potrf_panel(double* X, double* M, const double* 
   double a[PNB], a0[PNB], m[PNB], d[PNB], fin[PNB];
 #pragma unroll
   for (int k = 0; k < PNB; ++k) a[k] = own ? X[row * LDS + j0 + k] : 0.0;
-  if (j0 > 0) {
-    double mr[PNB], u[PNB][PNB];
+  double mr[PNB], up[PNB][PNB];
 #pragma unroll
-    for (int k = 0; k < PNB; ++k) mr[k] = own ? Mp[row * PMS + k] : 0.0;
+  for (int k = 0; k < PNB; ++k) mr[k] = j0 > 0 && own ? Mp[row * PMS + k] : 0.0;
 #pragma unroll
-    for (int c = 0; c < PNB; ++c)
+  for (int c = 0; c < PNB; ++c)
 #pragma unroll
-      for (int k = 0; k < PNB; ++k) u[c][k] = X[(j0 + c) * LDS + j0 - PNB + k];
+    for (int k = 0; k < PNB; ++k) up[c][k] = j0 > 0 ? X[(j0 + c) * LDS + j0 - PNB + k] : 0.0;
 #pragma unroll
-    for (int c = 0; c < PNB; ++c)
-#pragma unroll
-      for (int k = 0; k < PNB; ++k) a[c] = fma(-mr[k], u[c][k], a[c]);
-  }
-#pragma unroll
-  for (int k = 0; k < PNB; ++k) a0[k] = a[k];
+  for (int k = 0; k < PNB; ++k) a[0] = fma(-mr[k], up[0][k], a[0]);
   bool range = true;
 #pragma unroll
   for (int j = 0; j < PNB; ++j) {
     fin[j] = 0.0;
     d[j] = __shfl_sync(FULL, a[j], j);
+    const double rd = recip_fixed(d[j]);
+    range = range && recip_range(d[j]);
+    if (j == 0) {  // the other columns' update runs on the FP64 pipe beside the first reciprocal
+#pragma unroll
+      for (int c = 1; c < PNB; ++c)
+#pragma unroll
+        for (int k = 0; k < PNB; ++k) a[c] = fma(-mr[k], up[c][k], a[c]);
+#pragma unroll
+      for (int k = 0; k < PNB; ++k) a0[k] = a[k];
+    }
     double u[PNB];
 #pragma unroll
     for (int k = j + 1; k < PNB; ++k) u[k] = __shfl_sync(FULL, a[j], k);
-    m[j] = a[j] * recip_fixed(d[j]);
-    range = range && recip_range(d[j]);
+    m[j] = a[j] * rd;
 #pragma unroll
     for (int k = j + 1; k < PNB; ++k) a[k] = fma(-m[j], u[k], a[k]);
   }
