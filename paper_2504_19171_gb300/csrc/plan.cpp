@@ -46,6 +46,20 @@ constexpr int kGpuSms = 152;  // of a GB300
 constexpr int kPlanesMinB = 128;
 constexpr double kSweepStepNs = 120.0;  // one step of an in-shared-memory triangular sweep
 
+// Units (16 bytes) of a tile column's planes of Sigma and of U, and of the corner's.
+struct PlaneUnits {
+  int64_t u, sigma, corner;
+  explicit PlaneUnits(const Shape& s) {
+    const Layout L(s);
+    const int R = L.nblk(0), ra = s.a > 0 ? L.nblk(s.nt) : 0;
+    const int64_t gb = plane_group(s.prec, s.b), ga = s.a > 0 ? plane_group(s.prec, s.a) : 0;
+    u = (int64_t)s.w * R * gb + (int64_t)R * ga;
+    sigma = (int64_t)R * gb * (1 + 2 * s.w) + (int64_t)R * ga + (int64_t)ra * gb;
+    corner = (int64_t)ra * ga;
+  }
+  int64_t total(const Shape& s) const { return 2 * u + (s.w + 2) * sigma + corner; }
+};
+
 struct Builder {
   Shape s;
   Layout L;
@@ -642,7 +656,7 @@ struct Builder {
   std::vector<int32_t> p2join;
   std::vector<int32_t> pl_d, pl_c, pl_r, pl_u;  // counters per vector group: diagonal rows; tile columns / rows; U
   std::vector<int64_t> pl_dbase, pl_cbase, pl_rbase, pl_ubase;
-  int64_t pu_sigma = 0, pu_u = 0, pu_corner = 0;  // units of a Sigma slot, a U slot, the corner's
+  int64_t pu_sigma = 0, pu_u = 0;  // units of a Sigma slot, a U slot
   int64_t sig_slots() const { return s.w + 2; }
   // offset of a tile's planes inside its column's Sigma or U slot
   enum PlaneSet { PS_DIAG, PS_COL, PS_ROW, PS_U };
@@ -662,12 +676,10 @@ struct Builder {
     return mkref(BUF_P, plane_off(set, k, i) + (int64_t)g * plane_group(s.prec, kk));
   }
   void alloc_planes(int cols) {
-    const int R = L.nblk(0), ra = s.a > 0 ? L.nblk(s.nt) : 0;
-    const int64_t gb = plane_group(s.prec, s.b), ga = s.a > 0 ? plane_group(s.prec, s.a) : 0;
-    pu_u = (int64_t)s.w * R * gb + (int64_t)R * ga;
-    pu_sigma = (int64_t)R * gb * (1 + 2 * s.w) + (int64_t)R * ga + (int64_t)ra * gb;
-    pu_corner = (int64_t)ra * ga;
-    if (out) out->plane_units = 2 * pu_u + sig_slots() * pu_sigma + pu_corner;
+    const PlaneUnits u(s);
+    pu_u = u.u;
+    pu_sigma = u.sigma;
+    if (out) out->plane_units = u.total(s);
     p2join.assign(cols, -1);
     pl_dbase.assign(cols, 0);
     for (auto* v : {&pl_cbase, &pl_rbase, &pl_ubase}) v->assign((size_t)cols * (s.w + 2), -1);
@@ -1060,8 +1072,17 @@ static double task_estimate(const Shape& s) {
 }
 
 // Products from planes need the split of every Sigma and U tile as two more
-// steps of phase 2's chain, which short products do not pay back.
-bool use_planes(const Shape& s) { return s.prec != PREC_FP64 && s.b >= kPlanesMinB && tune_p2_split(s.tune) == 0; }
+// steps of phase 2's chain, which short products do not pay back. Planes are
+// scratch, and may not push a shape out of the fixed scratch of
+// stiles_factor_selinv_noalloc: one whose tiles fit that array has planes only if
+// both leave a sixteenth of it (4 MiB) to the scheduler's state, which takes below
+// 1 MiB at that size. (A rule on the shape alone, so that a matrix gets the same
+// arithmetic in every form of call.)
+bool use_planes(const Shape& s) {
+  if (s.prec == PREC_FP64 || s.b < kPlanesMinB) return false;
+  const int64_t tiles = 8 * Layout(s).doubles(), fixed = (int64_t)STILES_NOALLOC_SCRATCH_BYTES;
+  return tiles > fixed || tiles + 16 * PlaneUnits(s).total(s) <= fixed / 16 * 15;
+}
 
 static bool shape_ok(const Shape& s) {
   return s.nt >= 1 && s.b >= 1 && s.w >= 0 && s.a >= 0 && s.w <= s.nt - 1 && tune_valid(s.tune) && s.sel0 >= 0 &&

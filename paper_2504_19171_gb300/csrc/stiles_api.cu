@@ -179,17 +179,7 @@ static int create_handle(int nt, int b, int band, int arrow, int precision, int 
   }
   h->grid = h->sms * kCtasPerSm;
   h->s.planes = use_planes(h->s);
-  int brc = build_handle_plans(h);
-  // Planes may not push a shape out of the fixed no-allocation scratch: one
-  // that fits it without them keeps the products without.
-  if (!brc && h->s.planes && h->scratch_bytes > STILES_NOALLOC_SCRATCH_BYTES && h->w_bytes <= STILES_NOALLOC_SCRATCH_BYTES) {
-    h->s.planes = false;
-    brc = build_handle_plans(h);
-    if (!brc && h->scratch_bytes > STILES_NOALLOC_SCRATCH_BYTES) {
-      h->s.planes = true;
-      brc = build_handle_plans(h);
-    }
-  }
+  const int brc = build_handle_plans(h);
   if (brc) {
     delete h;
     return brc;
