@@ -83,16 +83,16 @@ enum stiles_status_code {
  * POTRF, TRSM, TRTRI, LAUUM and the Sigma_ii assembly (subtract, mirror)
  * always run in FP64.
  *   STILES_FP64   IEEE binary64 on the FP64 pipe.
- *   STILES_EMU64  emulated FP64: every operand is split, per row / column of
- *                 its panel, into seven 8-bit integer digits (56-bit fixed
- *                 point, the entry's sign on each) held exactly in bf16;
- *                 digit products run on the tensor cores with exact FP32
- *                 accumulation per K chunk, move into int32 level sums and
- *                 are recombined exactly in 128-bit integers, then rounded to
- *                 FP64 (split-precision scheme of Ozaki, Ogita, Oishi and
- *                 Rump). Error of a product term about 8 x 2^-56 of
- *                 (max |row| x max |column|).
- *   STILES_FP32X  FP32-class: operands rounded to FP32, FP32 FMA accumulation. */
+ *   STILES_EMU64  emulated FP64: every operand is split, per row / column and
+ *                 stretch of its inner length, into eight balanced 8-bit
+ *                 integer digits (62-bit fixed point relative to the largest
+ *                 entry) held exactly in fp16; digit products run on the
+ *                 tensor cores with exact FP32 accumulation and are recombined
+ *                 exactly in integers, then rounded to FP64 (split-precision
+ *                 scheme of Ozaki, Ogita, Oishi and Rump). Error of a product
+ *                 term about 8 x 2^-56 of (max |row| x max |column|).
+ *   STILES_FP32X  FP32-class: operands rounded to FP32 and written as three bf16
+ *                 pieces, piece products on the tensor cores, FP32 accumulation. */
 enum stiles_precision { STILES_FP64 = 0, STILES_EMU64 = 1, STILES_FP32X = 2 };
 
 /* Create a handle for one matrix shape.
@@ -100,7 +100,7 @@ enum stiles_precision { STILES_FP64 = 0, STILES_EMU64 = 1, STILES_FP32X = 2 };
  *   bandwidth (clipped to nt-1), arrow = a >= 0 arrow width,
  *   precision = STILES_FP64, STILES_EMU64 or STILES_FP32X.
  * Builds the task DAG of the factorization, of the selected inversion and of
- * both fused (host, C++), orders each by a critical-path list schedule, and
+ * both fused (host, C++), orders each by its critical path, and
  * uploads the tables. Returns STILES_ERR_INVALID_ARG for a bad shape,
  * STILES_ERR_UNSUPPORTED for another precision, STILES_ERR_OOM /
  * STILES_ERR_CUDA if the tables cannot be placed on the current device.
@@ -115,10 +115,12 @@ int stiles_create(int nt, int b, int band, int arrow, int precision, stiles_t *o
  * changes which products a reduced-precision handle lowers:
  *   bits 0-1  factor: source block columns per update task for tile columns
  *             older than k-1 (0: 8, 1: 4, 2: 16, 3: 32)
- *   bits 2-3  phase 2: parts of an off-diagonal Sigma block task
- *             (0: four 32 x 32 quadrants, 1: two 32-row halves, 2: whole)
- *   bits 4-5  factor: parts of the newest update of an off-diagonal block
- *             (0: four quadrants, 1: whole)
+ *   bits 2-3  phase 2: parts of an off-diagonal FP64 Sigma block task
+ *             (0: four 32 x 32 quadrants, or 16 x 16 parts while a step offers
+ *             fewer blocks than SMs; 1: two 32-row halves; 2: whole)
+ *   bits 4-5  factor: parts of the newest FP64 update of an off-diagonal block
+ *             (0: as for bits 2-3; 1: whole)
+ *             (reduced-precision tasks always run in 64 x 32 parts)
  *   bit 6     STILES_EMU64 / STILES_FP32X: also lower the block updates inside
  *             each diagonal tile (its POTRF's own SYRK / GEMM steps); with 0
  *             the whole diagonal-tile POTRF runs in true FP64
@@ -147,9 +149,10 @@ int stiles_layout_doubles(stiles_t h, size_t *doubles);
 
 /* Bytes the caller must provide: L and Sigma buffers (equal to the packed
  * size * 8) and a scratch buffer (device, 256-byte aligned) that holds
- * L_ii^{-1}, the scaled off-diagonal tiles L_ki L_ii^{-1} and the device
- * scheduler's state (dependency counters and ready queues). Any pointer may
- * be NULL to skip it. */
+ * L_ii^{-1}, the scaled off-diagonal tiles L_ki L_ii^{-1}, for the reduced
+ * precisions a ring of a few tile columns' operands split for the tensor cores,
+ * and the device scheduler's state (dependency counters and ready queues). Any
+ * pointer may be NULL to skip it. */
 int stiles_workspace_bytes(stiles_t h, size_t *L_bytes, size_t *sigma_bytes, size_t *scratch_bytes);
 
 /* Tiled Cholesky (Sec. III): reads A_tiles (device, packed layout), writes
@@ -259,9 +262,9 @@ int stiles_set_option(stiles_t h, int option, long long value);
 /* Per-part trace of the last launch (tracing must be on). Waits for the
  * launch. *n_tasks receives the task count of that launch; if out_host is not
  * NULL it must hold capacity >= 16 * n_tasks words and receives 4 records of
- * 4 words per task (one per possible part, in list-schedule order; records of
- * parts a task does not have are zero): time the worker started looking for
- * work, time it got this part, end time (ns of the GPU's global timer), and
+ * 4 words per task (in queue order; record r holds the last to finish of the
+ * parts r, r + 4, ..; records of parts a task does not have are zero): time the
+ * worker started looking for work, time it got this part, end time (ns of the GPU's global timer), and
  * (sm << 32 | cta << 12 | precision << 10 | last part << 9 | urgent << 8 | op). */
 int stiles_trace(stiles_t h, unsigned long long *out_host, size_t capacity, size_t *n_tasks);
 
@@ -353,8 +356,8 @@ int stiles_destroy(stiles_t h);
 /* ---------------------------------------------------------------- batch --
  * Many independent matrices of different shapes factored and inverted in ONE
  * persistent launch (no counterpart in the paper, which treats one matrix at
- * a time). Their task tables are merged into one table and ordered by one
- * critical-path list schedule, so the small matrices fill the GPU beside the
+ * a time). Their task tables are merged into one table and ordered by the
+ * longest way to the end, so the small matrices fill the GPU beside the
  * sequential factorization chains of the large ones.
  *
  * Layout. Matrix m occupies doubles [off[m], off[m] + stiles_layout_doubles
@@ -429,8 +432,10 @@ int stiles_batch_stats(stiles_batch_t h, long long stats[9]);
  * every shape, a data arena of data_bytes from which each request takes its
  * L, Sigma and scratch (3 x stiles_layout_doubles of its shape, rounded up to
  * 32 doubles; stiles_server_request_bytes), task-table arenas for
- * max(4, max_requests) copies of the largest shape, ready rings and a pinned,
- * host-mapped control block. stiles_server_submit returns STILES_ERR_BUSY if
+ * max(4, max_requests) copies of the largest shape, for the reduced precisions
+ * room for split operands beside the arena (per request slot; at most a quarter of
+ * data_bytes, none when it cannot be had), ready rings and a pinned, host-mapped
+ * control block. stiles_server_submit returns STILES_ERR_BUSY if
  * the request does not fit now (admission by HBM footprint): retry after a
  * stiles_server_release.
  *
