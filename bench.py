@@ -47,7 +47,7 @@ FP32_SIMT_PEAK_TFLOPS = 2 * 128 * 152 * 2.070e9 / 1e12
 # operand the levels t + u <= s - 1 are kept, s (s + 1) / 2 products), and the
 # pipe that runs them. EMU64: 8 fixed-point digits; FP32X: 3 bf16 pieces of
 # the FP32 value, levels t + u <= 3.
-VARIANT_PRODUCTS = {"emu64": {"pipe": "fp16 tensor (tcgen05)", "digits": 8, "products": 36},
+VARIANT_PRODUCTS = {"emu64": {"pipe": "bf16 tensor (tcgen05)", "digits": 8, "products": 36},
                     "fp32x": {"pipe": "bf16 tensor (tcgen05)", "digits": 3, "products": 8}}
 
 # DRAM traffic of the persistent kernel per launch, from ncu captures of the

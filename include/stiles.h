@@ -212,8 +212,10 @@ int stiles_factor_selinv_host(stiles_t h, const double *A_host, double *Sigma_ho
  * GPU that loads the library holds it until the process exits). The call
  * allocates nothing. The handle must already exist (stiles_create allocates
  * its task tables when it is created, not here).
- *   - Shapes whose scratch (stiles_workspace_bytes) exceeds the array return
- *     STILES_ERR_TOO_LARGE and launch nothing.
+ *   - Shapes whose scratch exceeds the array return STILES_ERR_TOO_LARGE and
+ *     launch nothing. A reduced-precision shape whose scratch
+ *     (stiles_workspace_bytes) exceeds it only by the operands split for the
+ *     tensor cores runs without those: the same results up to rounding, slower.
  *   - A call whose stream is not capturing looks up the array's device
  *     address (cudaGetSymbolAddress, with the handle's device current) and
  *     remembers it; a call made during stream capture uses the address the

@@ -43,7 +43,7 @@ namespace {
 constexpr double kFlopPerNs = 7.6 / kCtasPerSm;
 constexpr double kTaskOverheadNs = 2500.0;
 constexpr int kGpuSms = 152;  // of a GB300
-constexpr int kPlanesMinB = 128;
+constexpr int kPlanesMinB = 64, kPlanesMinK = 112;
 constexpr double kSweepStepNs = 120.0;  // one step of an in-shared-memory triangular sweep
 
 // Units (16 bytes) of a tile column's planes of Sigma and of U, and of the corner's.
@@ -157,7 +157,10 @@ struct Builder {
   // reach the SMs, and no further (a fuller step is bound by the FP64 pipes, and
   // smaller parts then only add their fixed cost and operand traffic).
   // `blocks`: 64 x 64 blocks that are ready at a time; `crowd`: matrices that
-  // share the GPU. Tasks whose products are lowered keep their 32 x 32 parts.
+  // share the GPU. With the 16 x 16 parts and the cheaper hand-over between tasks
+  // n = 1040 (16, 64, 1, 16) went from 4018 to 1696 us, (40, 100, 2, 37) from
+  // 24,016 to 8,235; 16 x 16 parts in full steps too cost n = 204,864 1,416 for
+  // 1,401 ms. Tasks whose products are lowered are cut by lower_precision.
   int crowd = 1;
   uint8_t fine_mode(long long blocks, uint8_t coarse) const {
     blocks *= crowd;
@@ -553,10 +556,11 @@ struct Builder {
     // per level (log2 of the blocks), each of h^2 independent blocks; the
     // column-by-column substitution before was a chain of R tasks that each
     // solved a triangle (9-12 ms of waiting at the end of a b = 1024
-    // factorization, for its last tile). The inner product, negated, is kept
+    // factorization, for its last tile; about 3 now). The inner product, negated, is kept
     // transposed in the tile's upper part, which nothing else uses.
     // (phase 1 of the last columns is waited for, that of the others runs beside
-    // each other's and the factorization)
+    // each other's and the factorization: 16 x 16 parts for all of them took
+    // n = 204,864 from 1,400 to 1,408 ms)
     const int columns = i >= s.nt - 1 ? 1 : L.last() + 1 - s.sel0;
     for (int r = 0; r < R; ++r) {
       const int m = L.bdim(i, r);
@@ -1072,16 +1076,16 @@ static double task_estimate(const Shape& s) {
 }
 
 // Products from planes need the split of every Sigma and U tile as two more
-// steps of phase 2's chain, which short products do not pay back. Planes are
-// scratch, and may not push a shape out of the fixed scratch of
-// stiles_factor_selinv_noalloc: one whose tiles fit that array has planes only if
-// both leave a sixteenth of it (4 MiB) to the scheduler's state, which takes below
-// 1 MiB at that size. (A rule on the shape alone, so that a matrix gets the same
-// arithmetic in every form of call.)
+// steps of phase 2's chain, which short products do not pay back. us per pass
+// (emulated FP64, factor + selected inversion, 60 tile columns, w / arrow after the
+// tile order), without -> with planes: 48 (1/20) 6333 -> 6638, 64 (1/16) 7262 ->
+// 7446, 112 (1/20) 11897 -> 11274, 96 (1/64) 11389 -> 10517, 80 (2/33) 14692 ->
+// 12465, 64 (4/64) 11161 -> 10229, 128 (4/64) 20963 -> 15753; FP32-class products
+// gain from 48 (1/20) on: 5760 -> 5631. So the line lies at an inner length
+// (w b + arrow) of 112, between 80 and 132. (A rule on the shape alone, so that a
+// matrix gets the same arithmetic in every form of call.)
 bool use_planes(const Shape& s) {
-  if (s.prec == PREC_FP64 || s.b < kPlanesMinB) return false;
-  const int64_t tiles = 8 * Layout(s).doubles(), fixed = (int64_t)STILES_NOALLOC_SCRATCH_BYTES;
-  return tiles > fixed || tiles + 16 * PlaneUnits(s).total(s) <= fixed / 16 * 15;
+  return s.prec != PREC_FP64 && s.b >= kPlanesMinB && (int64_t)s.w * s.b + s.a >= kPlanesMinK;
 }
 
 static bool shape_ok(const Shape& s) {

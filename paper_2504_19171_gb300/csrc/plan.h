@@ -83,15 +83,15 @@ enum TaskFlag : uint8_t {
   TF_NEG = 64,      // OP_STORE: out = -acc
 };
 
-// Planes. The reduced-precision products of phase 2 read their operands as bf16
-// planes (8 digits for emulated FP64, 3 pieces for the FP32-class mode) that
-// OP_SPLIT tasks have written once, in the layout the tensor core reads, so a
+// Planes. The reduced-precision products of phase 2 read their operands as 16-bit
+// planes (8 fp16 digits for emulated FP64, 3 bf16 pieces for the FP32-class mode)
+// that OP_SPLIT tasks have written once, in the layout the tensor core reads, so a
 // product part is bulk copies and MMAs with no conversion. A plane group holds
 // 64 vectors (rows of a left-hand operand, columns of a right-hand one) and the
 // whole K of one tile, K padded to stages of 16:
 //   emulated FP64: int32 exponent of vector v in K chunk ch (512 of K) at
 //   [64 ch + v], then the stages; FP32-class: the stages alone.
-// A stage is NP planes x 64 vectors x 16 K of bf16 in core matrices of 8 x 8;
+// A stage is NP planes x 64 vectors x 16 K in core matrices of 8 x 8;
 // left-hand: plane order of the MMA's row stacks, 64 vectors each; right-hand:
 // two halves of 32 vectors, planes in order.
 // Offsets in BUF_P count units of 16 bytes.
@@ -222,8 +222,8 @@ struct Shape {
   bool planes = false;   // reduced precisions: phase-2 products from planes
 };
 
-// Phase-2 products of reduced-precision plans read planes from this tile order
-// on (a rule on b: see use_planes in plan.cpp).
+// Whether the phase-2 products of a (reduced-precision) shape read planes: a rule
+// on its sizes, with its reasons at the definition.
 bool use_planes(const Shape& s);
 
 // A task with few successors is counted off them by each of its parts as it

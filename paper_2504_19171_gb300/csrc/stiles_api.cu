@@ -74,6 +74,10 @@ int upload(const std::vector<T>& v, T** out) {
 
 }  // namespace
 
+// Table of the fused plan without planes, for stiles_factor_selinv_noalloc where
+// the planes do not fit its fixed scratch.
+constexpr int kTableNoPlanes = 3;
+
 struct stiles_handle {
   Shape s;
   int device = 0;
@@ -81,18 +85,20 @@ struct stiles_handle {
   int grid = 0;
   long long budget_ns = 20LL * 1000 * 1000 * 1000;
   Plan plans[3];
-  DevPlan dev[3];
+  DevPlan dev[4];              // by plan kind; kTableNoPlanes
   DevStatus* dstatus = nullptr;  // one block per plan kind
   double* dlogdet = nullptr;
   int ndiag = 0;
   size_t w_bytes = 0;        // scratch: L^{-1} and U tiles (packed layout)
   size_t ctr_offset = 0;     // scratch: planes (if any) from w_bytes on, scheduler state from here on
   size_t scratch_bytes = 0;
+  size_t noalloc_ctr = 0;    // kTableNoPlanes: its scheduler state's offset
   unsigned long long* dtrace = nullptr;  // optional per-task trace (STILES_OPT_TRACE)
   size_t trace_tasks = 0;
   cudaStream_t last_stream = nullptr;
   bool launched = false;
   int last_kind = -1;         // plan kind of the last launch
+  int last_table = -1;        // and its table in dev
   int last_factor_kind = -1;  // plan kind of the last launch that factorized
   bool mirror_ok = false;     // fused plan: every final Sigma write (NEG, SYMUPD) lands in the Sigma buffer
 };
@@ -162,6 +168,37 @@ static int build_handle_plans(stiles_handle* h) {
   return 0;
 }
 
+static int upload_plan(const Plan& p, DevPlan* d) {
+  int rc = upload(p.tasks, &d->tasks);
+  if (!rc) rc = upload(p.segs, &d->segs);
+  if (!rc) rc = upload(p.succ, &d->succ);
+  if (!rc) rc = upload(p.soff, &d->soff);
+  const std::vector<int32_t> img = sched_image(p);
+  if (!rc) rc = upload(img, &d->image);
+  d->image_ints = img.size();
+  d->ntasks = (int)p.tasks.size();
+  d->nbuckets = p.nbuckets;
+  d->nslots = (int)p.slots0.size();
+  d->ucap = p.urgent_parts;
+  return rc;
+}
+
+// A shape that fits the no-allocation scratch only without its planes keeps a
+// second fused table for that call.
+static int add_noalloc_table(stiles_handle* h) {
+  if (!h->s.planes || h->scratch_bytes <= STILES_NOALLOC_SCRATCH_BYTES || h->w_bytes > STILES_NOALLOC_SCRATCH_BYTES)
+    return 0;
+  Shape s = h->s;
+  s.planes = false;
+  Plan p;
+  const int rc = build_plan(s, PLAN_FUSED, 0, &p);
+  if (rc) return rc;
+  const size_t ints = sched_state_ints((int)p.tasks.size(), p.nbuckets, (int)p.slots0.size(), p.urgent_parts);
+  if (h->w_bytes + sizeof(int) * ints > STILES_NOALLOC_SCRATCH_BYTES) return 0;
+  h->noalloc_ctr = h->w_bytes;
+  return upload_plan(p, &h->dev[kTableNoPlanes]);
+}
+
 static int create_handle(int nt, int b, int band, int arrow, int precision, int tuning, int first_column,
                          stiles_t* out) {
   if (!out) return STILES_ERR_INVALID_ARG;
@@ -186,20 +223,10 @@ static int create_handle(int nt, int b, int band, int arrow, int precision, int 
   }
   int rc = 0;
   for (int k = 0; k < 3 && !rc; ++k) {
-    Plan& p = h->plans[k];
-    rc = upload(p.tasks, &h->dev[k].tasks);
-    if (!rc) rc = upload(p.segs, &h->dev[k].segs);
-    if (!rc) rc = upload(p.succ, &h->dev[k].succ);
-    if (!rc) rc = upload(p.soff, &h->dev[k].soff);
-    std::vector<int32_t> img = sched_image(p);
-    if (!rc) rc = upload(img, &h->dev[k].image);
-    h->dev[k].image_ints = img.size();
-    h->dev[k].ntasks = (int)p.tasks.size();
-    h->dev[k].nbuckets = p.nbuckets;
-    h->dev[k].nslots = (int)p.slots0.size();
-    h->dev[k].ucap = p.urgent_parts;
-    if (p.ndiag > h->ndiag) h->ndiag = p.ndiag;
+    rc = upload_plan(h->plans[k], &h->dev[k]);
+    if (h->plans[k].ndiag > h->ndiag) h->ndiag = h->plans[k].ndiag;
   }
+  if (!rc) rc = add_noalloc_table(h);
   if (!rc) rc = dev_malloc((void**)&h->dstatus, 3 * sizeof(DevStatus));
   if (!rc) rc = dev_malloc((void**)&h->dlogdet, sizeof(double) * (h->ndiag > 0 ? h->ndiag : 1));
   if (rc) {
@@ -227,14 +254,15 @@ extern "C" int stiles_workspace_bytes(stiles_t h, size_t* L_bytes, size_t* sigma
 }
 
 static int launch(stiles_t h, int kind, const double* A, double* L, double* S, void* scratch, void* stream,
-                  double* smirror = nullptr) {
+                  double* smirror = nullptr, bool noalloc_table = false) {
   if (!h || !scratch) return STILES_ERR_INVALID_ARG;
   if (((uintptr_t)scratch) % 256 != 0) return STILES_ERR_INVALID_ARG;
   if (cudaSetDevice(h->device) != cudaSuccess) return STILES_ERR_CUDA;
   cudaStream_t st = (cudaStream_t)stream;
-  const DevPlan& d = h->dev[kind];
+  const int table = noalloc_table ? kTableNoPlanes : kind;
+  const DevPlan& d = h->dev[table];
   char* scr = (char*)scratch;
-  int* state = (int*)(scr + h->ctr_offset);
+  int* state = (int*)(scr + (noalloc_table ? h->noalloc_ctr : h->ctr_offset));
   if (d.image_ints &&
       cudaMemcpyAsync(state, d.image, sizeof(int) * d.image_ints, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
     return STILES_ERR_CUDA;
@@ -267,6 +295,7 @@ static int launch(stiles_t h, int kind, const double* A, double* L, double* S, v
   h->last_stream = st;
   h->launched = true;
   h->last_kind = kind;
+  h->last_table = table;
   if (kind != PLAN_SELINV) h->last_factor_kind = kind;
   if (d.ntasks == 0) return STILES_OK;
   if (launch_persistent(p, h->grid, st) != cudaSuccess) return STILES_ERR_CUDA;
@@ -363,12 +392,13 @@ int noalloc_scratch(int device, cudaStream_t stream, void** out) {
 
 extern "C" int stiles_factor_selinv_noalloc(stiles_t h, const double* A, double* L, double* S, void* stream) {
   if (!h || !A || !L || !S || S == L || (const double*)S == A) return STILES_ERR_INVALID_ARG;
-  if (h->scratch_bytes > STILES_NOALLOC_SCRATCH_BYTES) return STILES_ERR_TOO_LARGE;
+  const bool small = h->scratch_bytes > STILES_NOALLOC_SCRATCH_BYTES;  // only the table without planes fits
+  if (small && !h->dev[kTableNoPlanes].ntasks) return STILES_ERR_TOO_LARGE;
   if (cudaSetDevice(h->device) != cudaSuccess) return STILES_ERR_CUDA;
   void* scratch = nullptr;
   const int rc = noalloc_scratch(h->device, (cudaStream_t)stream, &scratch);
   if (rc) return rc;
-  return launch(h, PLAN_FUSED, A, L, S, scratch, stream);
+  return launch(h, PLAN_FUSED, A, L, S, scratch, stream, nullptr, small);
 }
 
 static int read_status(stiles_t h, int kind, DevStatus* ds) {
@@ -582,7 +612,7 @@ extern "C" int stiles_debug_break_plan(stiles_t h, int which) {
 extern "C" int stiles_trace(stiles_t h, unsigned long long* out_host, size_t capacity, size_t* n_tasks) {
   if (!h || !n_tasks) return STILES_ERR_INVALID_ARG;
   if (!h->dtrace || !h->launched) return STILES_ERR_INVALID_ARG;
-  const size_t n = (size_t)h->dev[h->last_kind].ntasks;
+  const size_t n = (size_t)h->dev[h->last_table].ntasks;
   *n_tasks = n;
   if (!out_host) return STILES_OK;
   if (capacity < 16 * n) return STILES_ERR_INVALID_ARG;

@@ -851,7 +851,8 @@ __device__ __forceinline__ void add_cell(long long& acc, uint32_t cell, int sh) 
 // of the other side's, handed over through shared memory, and 4 of its own at a
 // time. The loop is not unrolled (r16 is rotated instead, back in place after its
 // four steps): straight-line code of this size ran at the instruction cache's
-// rate, 13k cycles a drain.
+// rate, 13k cycles a drain (n = 122,944 in emulated FP64: 345 against 321 ms, with
+// the splits of run_tc, which had the same fault).
 template <int S, bool SMALL>
 __device__ __forceinline__ void drain_cells(uint32_t tmem, uint8_t* xch, int er, const int* cexp, double (&r16)[16]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1027,7 +1028,10 @@ __device__ __forceinline__ void store_part(const KParams& p, const Task& tk, int
 // The 64 x 32 sub-tile (columns 32 q ..) of a product task from planes, and its
 // epilogue. Thread (warp, lane) owns row 32 (warp & 1) + lane, columns
 // 16 (warp >> 1) + 0..15 of it. Thread 32 copies, thread 0 multiplies: one
-// thread doing both waits for the MMAs of the stage before in between.
+// thread doing both waits for the MMAs of the stage before in between. What bounds
+// it: the stages' way out of L2 (24 KB per 1055 cycles and SM, 7.1 TB/s in all). A
+// part of inner length 1088 takes 63 us in emulated FP64, 26 in the FP32-class mode;
+// 146 and 64 us for half the outputs when each part split its operands itself.
 template <int S>
 __device__ __noinline__ void run_planes(const KParams& p, const Task& tk, int q, double* smem, TcShared& ts) {
   using F = PlaneFmt<S>;
@@ -1148,15 +1152,6 @@ __device__ __noinline__ void run_planes(const KParams& p, const Task& tk, int q,
   store_part(p, tk, q, smem, r16);
 }
 
-// A 64 x 32 part (columns 32 q ..) that splits its own operands: 64 of K at a
-// time. Thread (warp, lane) loads the K octets warp and warp + 4 of the vectors
-// lane and lane + 32 of op(A) and lane of op(B) (48 values, the next 64 of K in
-// flight while the MMAs of these run), takes the exponents from them (emulated
-// FP64: one per vector and 64 of K) and writes the planes of four stages. What
-// bounds it: the splits (about 35 instructions per operand value, 48 values per
-// thread for 1664 cycles of MMAs) and, for the factor's updates with an inner
-// length of 64, the fixed cost of a task. The 32 x 32 parts before split each
-// operand twice as often and scanned the whole K for exponents first.
 // 8 K-adjacent values of one vector from P (`step` apart), zero from the n-th on.
 // Contiguous ones are read in pairs where `pairs` says that P is 16-byte aligned
 // (single 8-byte loads fetch each 32-byte sector four times: a lane per vector).
@@ -1221,6 +1216,17 @@ struct PlaneStep {
   static constexpr int A1 = S == 8 ? 4096 : 2048, A2 = 2048, B1 = 1024, B2 = 4096;
 };
 
+// A 64 x 32 part (columns 32 q ..) that splits its own operands: 64 of K at a
+// time. Thread (warp, lane) loads the K octets warp and warp + 4 of the vectors
+// lane and lane + 32 of op(A) and lane of op(B) (48 values, the next 64 of K in
+// flight while the MMAs of these run), takes the exponents from them (emulated
+// FP64: one per vector and 64 of K) and writes the planes of four stages. What
+// bounds it: the splits (about 35 instructions per operand value, 48 values per
+// thread for 1664 cycles of MMAs) and, for the factor's updates with an inner
+// length of 64, the fixed cost of a task. The 32 x 32 parts before split each
+// operand twice as often and scanned the whole K for exponents first: factor +
+// selected inversion of (28, 1024, 4, 64) in emulated FP64 464 ms then, 199 ms
+// with these parts and phase 2 from planes (454 ms with phase 2 in these parts).
 template <int S>
 __device__ __noinline__ void run_tc(const KParams& p, const Task& tk, int q, double* smem, TcShared& ts) {
   using F = PlaneFmt<S>;
@@ -1330,7 +1336,9 @@ __device__ __noinline__ void run_tc(const KParams& p, const Task& tk, int q, dou
 // 16 vectors, and their exponents (emulated FP64). Lane l of warp w holds vector
 // l % 16 and the K octets 2 w + l / 16 + 8 u (u < 8) of the chunk in registers,
 // read once: exponents first, then the digits, stored 16 bytes (one core-matrix
-// row) at a time. Vectors beyond the tile and the padding of K are zeros.
+// row) at a time. Vectors beyond the tile and the padding of K are zeros. Bound by
+// the latency of one round of loads and one of stores; a tile is split once for the
+// 2 (w + 1) products and more per 64 rows that read it.
 template <int S>
 __device__ __noinline__ void run_split(const KParams& p, const Task& tk, int q, double* smem) {
   using F = PlaneFmt<S>;
@@ -1453,7 +1461,9 @@ __device__ __forceinline__ void store_sub(const KParams& p, const Task& tk, cons
 // (a shuffle) and subtracts y_j Tn[c][j] from the columns c > j; x = y / diag(T)
 // at the end. No shared-memory round trip, division or scaling between two steps.
 // LANES = 8, 16, 32 for parts of 16, 8, 4 rows: at most 64 / LANES multiply-adds
-// per step and lane (10k and 6k cycles of the FP64 pipe for 8 and 4 rows).
+// per step and lane (10k and 6k cycles of the FP64 pipe for 8 and 4 rows). A part of
+// the block below the diagonal 13.7 -> 9.7 us, against a triangle loaded in four
+// round trips, scaled by the pivots in every part and 8-row parts.
 template <int LANES>
 __device__ __forceinline__ void trsm_rows(double* X, const double* Tn, int m, int n) {
   constexpr int R = 32 / LANES, Q = FB / LANES;  // rows per warp, columns per lane
@@ -1525,6 +1535,9 @@ __device__ __forceinline__ void trsm_cols_ln(double* X, const double* T, const d
 //     apply the rest (batches of 32 2 x 2 elements of the packed lower triangle,
 //     shared out by their FP64 time; single elements claimed from a counter,
 //     their rows found by a division, took three times as long).
+// A block POTRF task takes 42 us (51 with a column and a barrier per step); a panel
+// about 2.8k cycles, the early ones bound by the trailing update. Factor and logdet
+// of (60, 250, 2, 50): 36.6 ms before, 17.2 ms with the other links of the chain.
 
 constexpr int PNB = 4;           // panel width
 constexpr int PROWS = 32 - PNB;  // rows below the panel's own per warp

@@ -1,5 +1,5 @@
-"""Reduced-precision products from pre-split planes (phase 2, tile order 128 and
-up) and in self-splitting 64 x 32 parts, at the edges of their layout: vector
+"""Reduced-precision products from pre-split planes (phase 2, inner length 112
+and up) and in self-splitting 64 x 32 parts, at the edges of their layout: vector
 groups of 64, column halves of 32, stages of 16 and chunks of 512 of K (256 per
 drain), the ring of plane slots (more tile columns than bandwidth + 2), tiles by
 rows as well as by columns (bandwidth 2 and more), arrows of one and two groups.
@@ -43,3 +43,47 @@ def test_reduced_precisions(shape):
             assert abs(ld - ldr) < tol * max(1.0, abs(ldr))
             for i in range(M.nt + (1 if M.a else 0)):
                 assert np.array_equal(Sg[(i, i)], Sg[(i, i)].T)
+
+
+@pytest.mark.parametrize("shape", [(9, 64, 1, 47), (9, 64, 1, 48), (9, 63, 2, 64), (8, 65, 2, 1), (7, 100, 4, 9), (6, 112, 1, 0)])
+def test_small_tile_tables(shape):
+    """Host, both sides of the line between products with and without planes."""
+    for kind in (S.PLAN_SELINV, S.PLAN_FUSED):
+        assert S.stiles_debug_validate(*shape, kind, S.STILES_EMU64) == S.STILES_OK
+        assert S.stiles_debug_race_check(*shape, kind, S.STILES_EMU64) == S.STILES_OK
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("precision", [S.STILES_EMU64, S.STILES_FP32X])
+@pytest.mark.parametrize("nt", [20, 28])
+def test_noalloc_without_planes(nt, precision):
+    """Shapes whose tiles fit the fixed scratch but whose planes do not (but for
+    the FP32-class planes of the shorter one): the allocation-free call takes
+    products without planes. Both forms are within
+    the precision's bound of the exact result, so within twice of each other."""
+    need_gpu()
+    import torch
+    shape = (nt, 256, 3, 64)
+    st = S.Stiles(*shape, precision=precision)
+    try:
+        fits = nt == 20 and precision == S.STILES_FP32X
+        assert 8 * st.doubles <= S.NOALLOC_SCRATCH_BYTES
+        assert (S.stiles_workspace_bytes(st.h)[2] <= S.NOALLOC_SCRATCH_BYTES) == fits
+        st.A = torch.zeros(st.doubles, dtype=torch.float64, device="cuda")
+        W.random_arrowhead_packed(*shape, 5, st.A)
+        st.L.zero_()
+        st.S.zero_()
+        st.factor_selinv()
+        ref, ld = st.S.clone(), st.logdet()
+        L, Sg = torch.zeros_like(st.L), torch.zeros_like(st.S)
+        for _ in range(2):
+            S.stiles_factor_selinv_noalloc(st.h, st.A.data_ptr(), L.data_ptr(), Sg.data_ptr(), st.stream_ptr())
+        torch.cuda.synchronize()
+        assert st.status()[0] == S.STILES_OK
+        rc, ld2 = S.stiles_logdet(st.h)
+        tol = 2e-12 if precision == S.STILES_EMU64 else 2e-5
+        assert rc == S.STILES_OK and abs(ld2 - ld) <= tol * abs(ld)
+        assert (Sg - ref).abs().max() <= tol * ref.abs().max()
+        assert (L - st.L).abs().max() <= tol * st.L.abs().max()
+    finally:
+        st.close()
