@@ -808,27 +808,32 @@ __device__ __forceinline__ void stage_mmas(uint32_t tmem, uint32_t a0, bool acc)
   }
 }
 
-// (H 2^32 + Lo) 2^k2 as a double, without an FP64 instruction (a conversion holds
-// the pipe like a multiply-add, and the drains would keep it from the block
-// POTRFs). |H 2^32 + Lo| < 2^76: its low 16 bits are rounded off first, 2^-58 or
-// less of the largest entries' product, a quarter of what the dropped digit
-// levels weigh.
+// (H 2^32 + Lo) 2^k2 as a double, rounded once (|H 2^32 + Lo| < 2^76), without an
+// FP64 instruction (a conversion holds the pipe like a multiply-add, and the drains
+// would keep it from the block POTRFs). All 96 bits are kept up to the rounding:
+// with the low 16 rounded off first, half the integer work and 0.5 to 3 % of a
+// pass, the error of the n = 122,944 matrix was 3.3e-15 where one rounding gives
+// 1.4e-15.
 // `slow` is set when the result leaves the normal range (scaled_sum_any then).
-__device__ __forceinline__ long long rounded_sum(long long H, long long Lo) { return (H << 16) + ((Lo + (1ll << 15)) >> 16); }
 __device__ __forceinline__ double scaled_sum(long long H, long long Lo, int k2, bool& slow) {
-  const long long T = rounded_sum(H, Lo);
-  const unsigned long long sign = (unsigned long long)(T >> 63);  // all ones for a negative sum
-  const unsigned long long mag = ((unsigned long long)T ^ sign) - sign;
-  const int lz = __clzll((long long)mag);
-  const unsigned long long norm = mag << (lz & 63);                      // top bit set
+  const long long t = H + (Lo >> 32);  // the sum is t 2^32 + the low word of Lo
+  const unsigned long long sign = (unsigned long long)(t >> 63);  // all ones for a negative sum
+  const uint32_t mlo = ((uint32_t)Lo ^ (uint32_t)sign) - (uint32_t)sign;
+  const unsigned long long mhi = ((unsigned long long)t ^ sign) + (sign != 0 && mlo == 0 ? 1 : 0);
+  const bool far = mhi == 0;
+  const unsigned long long top = far ? mlo : mhi;
+  const uint32_t low = far ? 0u : mlo;
+  const int lz = __clzll((long long)top);
+  // top bit set (mhi < 2^45, so lz is 19 or more and the shift of low below 46)
+  const unsigned long long norm = (top << (lz & 63)) | (((unsigned long long)low << 32) >> ((64 - lz) & 63));
   const unsigned long long mant = (norm >> 11) + ((norm >> 10) & 1ull);  // 2^52 .. 2^53
-  const int e = (63 - lz) + 16 + k2 + 1023;                              // biased exponent
-  slow = slow || (T != 0 && (unsigned)(e - 1) >= 0x7fdu);
+  const int e = (63 - lz) + (far ? 0 : 32) + k2 + 1023;                  // biased exponent
+  slow = slow || (top != 0 && (unsigned)(e - 1) >= 0x7fdu);
   const unsigned long long bits = (((unsigned long long)(unsigned)(e - 1) << 52) + mant) | (sign << 63);
-  return T == 0 ? 0.0 : __longlong_as_double((long long)bits);
+  return top == 0 ? 0.0 : __longlong_as_double((long long)bits);
 }
 __device__ __noinline__ double scaled_sum_any(long long H, long long Lo, int k2) {
-  return ldexp((double)rounded_sum(H, Lo), k2 + 16);
+  return ldexp(fma((double)H, 4294967296.0, (double)Lo), k2);
 }
 
 // acc += cell 2^sh for an integer-valued FP32 cell. SMALL (at most 64 of K, so
@@ -1225,7 +1230,7 @@ struct PlaneStep {
 // thread for 1664 cycles of MMAs) and, for the factor's updates with an inner
 // length of 64, the fixed cost of a task. The 32 x 32 parts before split each
 // operand twice as often and scanned the whole K for exponents first: factor +
-// selected inversion of (28, 1024, 4, 64) in emulated FP64 464 ms then, 199 ms
+// selected inversion of (28, 1024, 4, 64) in emulated FP64 464 ms then, 205 ms
 // with these parts and phase 2 from planes (454 ms with phase 2 in these parts).
 template <int S>
 __device__ __noinline__ void run_tc(const KParams& p, const Task& tk, int q, double* smem, TcShared& ts) {
