@@ -62,7 +62,8 @@ struct Inv20 {
 __constant__ const Inv20 kInv20{};
 
 // 1 / |d| of a normal d with biased exponent in [1, 2043], correctly rounded
-// but for rare cases (error below 0.51 ulp). Newton's iteration in fixed point
+// but for rare cases (error below 0.51 ulp, from an estimate off by two units in its
+// last place too; exact for a power of two). Newton's iteration in fixed point
 // from a single-precision estimate q / 2^24 of 1 / m, d = m 2^e, m in [1, 2):
 // with M = 2^52 m the residual e1 = 1 - m q / 2^24 = (2^76 - M q) / 2^76 is
 // below 2^-21 and exact in 64 bits; 1 / m = q / 2^24 (1 + e1 + e1^2) to 2^-63.
@@ -78,14 +79,14 @@ __device__ __forceinline__ double recip_fixed(double d) {
   const int e = (int)((bits >> 52) & 0x7ff);
   const unsigned long long M = (bits & 0xFFFFFFFFFFFFFull) | (1ull << 52);
   const float f = __uint_as_float(0x3f800000u | (uint32_t)((bits >> 29) & 0x7fffffu));
-  float r = recip_estimate(f);
-  r = fminf(r, 0.99999994f);  // below 1, so that its exponent is that of [1/2, 1)
+  const float r = fminf(fmaxf(recip_estimate(f), 0.5f), 0.99999994f);  // the exponent of [1/2, 1)
   const uint32_t q = (__float_as_uint(r) & 0x7fffffu) | 0x800000u;
   const long long E = (long long)(0ull - M * (unsigned long long)q);
   const int Eh = (int)(E >> 24);
   const long long S = E + (((long long)Eh * Eh) >> 28);
-  const long long Y = ((long long)q << 39) + (((S >> 16) * (long long)q) >> 21);
-  return __longlong_as_double(((long long)(2044 - e) << 52) + ((Y + 512) >> 10));
+  // 2^63 / m, truncated: 2^63 - 1 for m = 1, so it is rounded without a sign
+  const unsigned long long Y = ((unsigned long long)q << 39) + (unsigned long long)(((S >> 16) * (long long)q) >> 21);
+  return __longlong_as_double(((long long)(2044 - e) << 52) + (long long)((Y + 512) >> 10));
 }
 
 __device__ __forceinline__ bool recip_range(double d) {  // recip_fixed's range
