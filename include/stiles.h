@@ -213,9 +213,11 @@ int stiles_factor_selinv_host(stiles_t h, const double *A_host, double *Sigma_ho
  * allocates nothing. The handle must already exist (stiles_create allocates
  * its task tables when it is created, not here).
  *   - Shapes whose scratch exceeds the array return STILES_ERR_TOO_LARGE and
- *     launch nothing. A reduced-precision shape whose scratch
- *     (stiles_workspace_bytes) exceeds it only by the operands split for the
- *     tensor cores runs without those: the same results up to rounding, slower.
+ *     launch nothing. A shape whose scratch (stiles_workspace_bytes) exceeds it
+ *     only by the scheduler's state of finely divided tasks runs in coarser ones:
+ *     the same results, slower. A reduced-precision shape that exceeds it only by
+ *     the operands split for the tensor cores runs without those: the same results
+ *     up to rounding, slower.
  *   - A call whose stream is not capturing looks up the array's device
  *     address (cudaGetSymbolAddress, with the handle's device current) and
  *     remembers it; a call made during stream capture uses the address the

@@ -164,6 +164,7 @@ struct Builder {
   int crowd = 1;
   uint8_t fine_mode(long long blocks, uint8_t coarse) const {
     blocks *= crowd;
+    if (s.coarse) return coarse;
     return 4 * blocks <= kGpuSms ? (uint8_t)PM_GRID16 : blocks <= kGpuSms ? (uint8_t)PM_QUAD4 : coarse;
   }
   // ... of a task, `tri`: only the lower triangle of its (square) block.
@@ -402,7 +403,7 @@ struct Builder {
     // FP64 share is small, as long as their own parts do).
     const long long W = col_blocks(kq) - cq, step = W * (W + 1) / 2;
     const uint8_t fine_old = fine_mode(step, PM_FULL);
-    const uint8_t fine_new = (s.prec == PREC_FP64 ? step : 4 * W) * crowd <= kGpuSms ? PM_GRID16 : PM_QUAD4;
+    const uint8_t fine_new = !s.coarse && (s.prec == PREC_FP64 ? step : 4 * W) * crowd <= kGpuSms ? PM_GRID16 : PM_QUAD4;
     bool written = false;  // the block already holds an update (read it from L, not A)
     for (size_t t = 0; t < terms.size(); ++t) {
       Task tk = blank(OP_UPD, m, n);
@@ -413,7 +414,7 @@ struct Builder {
       const bool newest = t + 1 == terms.size();
       // a diagonal block only needs its lower part; the newest update of a
       // block gates its TRSM / POTRF on the critical path
-      if (diag) split_fp64(tk, newest ? (uint8_t)PM_GRID16 : fine_old, true);
+      if (diag) split_fp64(tk, newest && !s.coarse ? (uint8_t)PM_GRID16 : fine_old, true);
       else if (!newest) split_fp64(tk, fine_old, false);
       else if (tune_upd_split(s.tune) == 0) split_fp64(tk, fine_new, false);
       if (grow(i, r) - grow(terms[t].k, terms[t].c1) <= kUrgentReach) tk.flags |= TF_URGENT;
@@ -435,7 +436,7 @@ struct Builder {
     if (nwritten > 0) w.push_back({me, nwritten});
     if (!written && serve) w.push_back({prep_ctr[kq], 1});
     Task tk = blank(diag ? OP_POTRF : OP_TRSM_RLT, m, n);
-    if (!diag) split(tk, dist == 1 ? PM_ROWS4F : W * crowd <= 2 * kUrgentReach ? PM_ROWS8 : PM_ROWS4);
+    if (!diag) split(tk, s.coarse ? PM_ROWS4 : dist == 1 ? PM_ROWS4F : W * crowd <= 2 * kUrgentReach ? PM_ROWS8 : PM_ROWS4);
     if (diag || dist <= kUrgentReach) tk.flags |= TF_URGENT;
     tk.out = outref;
     tk.ldo = ld_i;
@@ -621,7 +622,7 @@ struct Builder {
         const int m = L.bdim(i, r), n = L.bdim(i, c);
         Task t = blank(OP_STORE, m, n);
         // only the lower part of a diagonal block is used
-        split_fp64(t, 2LL * R * (R + 1) * crowd * columns <= kGpuSms ? PM_GRID16 : PM_FULL, r == c);
+        split_fp64(t, !s.coarse && 2LL * R * (R + 1) * crowd * columns <= kGpuSms ? PM_GRID16 : PM_FULL, r == c);
         t.out = mkref(BUF_S, L.blk(i, i, r, c));
         t.ldo = ld;
         std::vector<Wait> w{col[r], col[c]};
@@ -1104,6 +1105,17 @@ int build_plan(const Shape& s, PlanKind kind, int workers, Plan* out) {
   int rc = B.finish(workers);
   if (rc) return rc;
   return check_plan(*out);
+}
+
+int build_small_plan(Shape s, size_t w_bytes, size_t limit, Plan* out) {
+  for (int step = s.planes ? 0 : 1; step < 2; ++step) {
+    s.planes = false;
+    s.coarse = step == 1;
+    const int rc = build_plan(s, PLAN_FUSED, 0, out);
+    if (rc) return rc;
+    if (w_bytes + sizeof(int) * sched_state_ints(*out) <= limit) return 0;
+  }
+  return STILES_ERR_TOO_LARGE;
 }
 
 int build_serve_template(const Shape& s, int workers, Plan* out) {

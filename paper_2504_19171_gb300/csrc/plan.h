@@ -220,6 +220,7 @@ struct Shape {
   int tune = 0;          // tuning code (see above)
   int sel0 = 0;          // selected inversion of tile columns >= sel0 only (their phase 1 and 2)
   bool planes = false;   // reduced precisions: phase-2 products from planes
+  bool coarse = false;   // FP64 tasks in at most four parts (the same results, fewer queue slots)
 };
 
 // Whether the phase-2 products of a (reduced-precision) shape read planes: a rule
@@ -298,10 +299,25 @@ struct Layout {
   }
 };
 
+// 32-bit words of a launch's scheduler state (laid out in stiles_device.h).
+inline size_t sched_state_ints(int ntasks, int nbuckets, int nslots, int ucap) {
+  const int ngroups = (nbuckets + 31) / 32, nsuper = (ngroups + 31) / 32;
+  return 2 * (size_t)ntasks + (size_t)nslots + 3 * (size_t)nbuckets + (size_t)ngroups +
+         (size_t)nsuper + (size_t)(ucap > 0 ? ucap : 1) + 32;
+}
+inline size_t sched_state_ints(const Plan& p) {
+  return sched_state_ints((int)p.tasks.size(), p.nbuckets, (int)p.slots0.size(), p.urgent_parts);
+}
+
 // Build the task table of one plan kind, ordered by bottom level; workers > 0:
 // also the makespan of its list schedule on so many workers (statistics).
 // Returns 0 or a negative stiles status code.
 int build_plan(const Shape& s, PlanKind kind, int workers, Plan* out);
+
+// The fused table of a shape for a scratch of `limit` bytes that its ordinary table
+// exceeds: without planes, then with fewer parts as well. `w_bytes`: of the scratch
+// tiles, which the scheduler state follows. STILES_ERR_TOO_LARGE if none fits.
+int build_small_plan(Shape s, size_t w_bytes, size_t limit, Plan* out);
 
 // Consistency check of a task table: every wait names an existing counter
 // that enough tasks signal, and every such producer precedes the waiter in

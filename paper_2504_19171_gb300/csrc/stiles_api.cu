@@ -74,9 +74,9 @@ int upload(const std::vector<T>& v, T** out) {
 
 }  // namespace
 
-// Table of the fused plan without planes, for stiles_factor_selinv_noalloc where
-// the planes do not fit its fixed scratch.
-constexpr int kTableNoPlanes = 3;
+// Table of the fused plan with a smaller scratch (build_small_plan), for
+// stiles_factor_selinv_noalloc where the ordinary one does not fit its fixed array.
+constexpr int kTableSmall = 3;
 
 struct stiles_handle {
   Shape s;
@@ -85,14 +85,14 @@ struct stiles_handle {
   int grid = 0;
   long long budget_ns = 20LL * 1000 * 1000 * 1000;
   Plan plans[3];
-  DevPlan dev[4];              // by plan kind; kTableNoPlanes
+  DevPlan dev[4];              // by plan kind; kTableSmall
   DevStatus* dstatus = nullptr;  // one block per plan kind
   double* dlogdet = nullptr;
   int ndiag = 0;
   size_t w_bytes = 0;        // scratch: L^{-1} and U tiles (packed layout)
   size_t ctr_offset = 0;     // scratch: planes (if any) from w_bytes on, scheduler state from here on
   size_t scratch_bytes = 0;
-  size_t noalloc_ctr = 0;    // kTableNoPlanes: its scheduler state's offset
+  size_t noalloc_ctr = 0;    // kTableSmall: its scheduler state's offset
   unsigned long long* dtrace = nullptr;  // optional per-task trace (STILES_OPT_TRACE)
   size_t trace_tasks = 0;
   cudaStream_t last_stream = nullptr;
@@ -158,7 +158,7 @@ static int build_handle_plans(stiles_handle* h) {
     Plan& p = h->plans[k];
     const int rc = build_plan(h->s, (PlanKind)k, 0, &p);
     if (rc) return rc;
-    const size_t ints = sched_state_ints((int)p.tasks.size(), p.nbuckets, (int)p.slots0.size(), p.urgent_parts);
+    const size_t ints = sched_state_ints(p);
     state = ints > state ? ints : state;
     units = p.plane_units > units ? p.plane_units : units;
   }
@@ -183,20 +183,15 @@ static int upload_plan(const Plan& p, DevPlan* d) {
   return rc;
 }
 
-// A shape that fits the no-allocation scratch only without its planes keeps a
-// second fused table for that call.
+// A shape whose tiles fit the no-allocation scratch, but not with its planes or with
+// the queue slots of its finest parts, keeps a second fused table for that call.
 static int add_noalloc_table(stiles_handle* h) {
-  if (!h->s.planes || h->scratch_bytes <= STILES_NOALLOC_SCRATCH_BYTES || h->w_bytes > STILES_NOALLOC_SCRATCH_BYTES)
-    return 0;
-  Shape s = h->s;
-  s.planes = false;
+  if (h->scratch_bytes <= STILES_NOALLOC_SCRATCH_BYTES || h->w_bytes > STILES_NOALLOC_SCRATCH_BYTES) return 0;
   Plan p;
-  const int rc = build_plan(s, PLAN_FUSED, 0, &p);
-  if (rc) return rc;
-  const size_t ints = sched_state_ints((int)p.tasks.size(), p.nbuckets, (int)p.slots0.size(), p.urgent_parts);
-  if (h->w_bytes + sizeof(int) * ints > STILES_NOALLOC_SCRATCH_BYTES) return 0;
+  const int rc = build_small_plan(h->s, h->w_bytes, STILES_NOALLOC_SCRATCH_BYTES, &p);
+  if (rc) return rc == STILES_ERR_TOO_LARGE ? 0 : rc;
   h->noalloc_ctr = h->w_bytes;
-  return upload_plan(p, &h->dev[kTableNoPlanes]);
+  return upload_plan(p, &h->dev[kTableSmall]);
 }
 
 static int create_handle(int nt, int b, int band, int arrow, int precision, int tuning, int first_column,
@@ -259,7 +254,7 @@ static int launch(stiles_t h, int kind, const double* A, double* L, double* S, v
   if (((uintptr_t)scratch) % 256 != 0) return STILES_ERR_INVALID_ARG;
   if (cudaSetDevice(h->device) != cudaSuccess) return STILES_ERR_CUDA;
   cudaStream_t st = (cudaStream_t)stream;
-  const int table = noalloc_table ? kTableNoPlanes : kind;
+  const int table = noalloc_table ? kTableSmall : kind;
   const DevPlan& d = h->dev[table];
   char* scr = (char*)scratch;
   int* state = (int*)(scr + (noalloc_table ? h->noalloc_ctr : h->ctr_offset));
@@ -392,8 +387,8 @@ int noalloc_scratch(int device, cudaStream_t stream, void** out) {
 
 extern "C" int stiles_factor_selinv_noalloc(stiles_t h, const double* A, double* L, double* S, void* stream) {
   if (!h || !A || !L || !S || S == L || (const double*)S == A) return STILES_ERR_INVALID_ARG;
-  const bool small = h->scratch_bytes > STILES_NOALLOC_SCRATCH_BYTES;  // only the table without planes fits
-  if (small && !h->dev[kTableNoPlanes].ntasks) return STILES_ERR_TOO_LARGE;
+  const bool small = h->scratch_bytes > STILES_NOALLOC_SCRATCH_BYTES;  // only the smaller table fits
+  if (small && !h->dev[kTableSmall].ntasks) return STILES_ERR_TOO_LARGE;
   if (cudaSetDevice(h->device) != cudaSuccess) return STILES_ERR_CUDA;
   void* scratch = nullptr;
   const int rc = noalloc_scratch(h->device, (cudaStream_t)stream, &scratch);

@@ -20,7 +20,7 @@ struct DevStatus {
 };
 
 // Per-launch scheduler state, one contiguous int32 block in the caller's
-// scratch, reset before every launch from a device image built at create:
+// scratch (sched_state_ints of them), reset before every launch from a device image built at create:
 //   rem[ntasks]      predecessors, or their parts, not yet finished (image: rem0)
 //   pdone[ntasks]    parts of the task finished so far
 //   slots[nslots]    bucket b owns slots [soff[b], soff[b + 1])
@@ -46,12 +46,6 @@ struct SchedState {
   int* uslots;
   int* lo;
 };
-
-inline size_t sched_state_ints(int ntasks, int nbuckets, int nslots, int ucap) {
-  const int ngroups = (nbuckets + 31) / 32, nsuper = (ngroups + 31) / 32;
-  return 2 * (size_t)ntasks + (size_t)nslots + 3 * (size_t)nbuckets + (size_t)ngroups +
-         (size_t)nsuper + (size_t)(ucap > 0 ? ucap : 1) + 32;
-}
 
 inline SchedState sched_state_at(int* base, int ntasks, int nbuckets, int nslots, int ucap) {
   SchedState s;

@@ -1,0 +1,24 @@
+// Planner internals for host tests, built together with csrc/plan.cpp.
+#include "plan.h"
+
+using namespace stiles;
+
+static Shape shape(int nt, int b, int w, int a, int prec) {
+  Shape s{nt, b, w < nt - 1 ? w : nt - 1, a, prec, 0};
+  s.planes = use_planes(s);
+  return s;
+}
+
+// Scratch bytes of the fused plan that a fixed scratch of `limit` bytes takes
+// (tiles, planes, scheduler state), or -1 if none fits. most: the finest-cut
+// plan's bytes.
+extern "C" long long fixed_scratch(int nt, int b, int w, int a, int prec, long long limit, long long* most) {
+  const Shape s = shape(nt, b, w, a, prec);
+  const size_t w_bytes = ((size_t)Layout(s).doubles() * 8 + 255) / 256 * 256;
+  Plan p;
+  if (build_plan(s, PLAN_FUSED, 0, &p)) return -2;
+  *most = (long long)(w_bytes + 16 * (size_t)p.plane_units + 4 * sched_state_ints(p));
+  if (*most <= limit) return *most;
+  if (build_small_plan(s, w_bytes, (size_t)limit, &p)) return -1;
+  return validate_plan(p, s, PLAN_FUSED) ? -3 : (long long)(w_bytes + 4 * sched_state_ints(p));
+}
