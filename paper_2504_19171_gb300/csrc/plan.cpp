@@ -46,18 +46,25 @@ constexpr int kGpuSms = 152;  // of a GB300
 constexpr int kPlanesMinB = 64, kPlanesMinK = 112;
 constexpr double kSweepStepNs = 120.0;  // one step of an in-shared-memory triangular sweep
 
-// Units (16 bytes) of a tile column's planes of Sigma and of U, and of the corner's.
+// Units (16 bytes) of a tile column's planes of Sigma and of U, and of the corner's:
+// the tiles that products read. Of Sigma the diagonal tile by rows and the arrow and
+// band tiles by columns, and by rows those that an earlier column reads so (all but
+// the w-th band tile; with w = 0 a column reads only its own and the corner).
 struct PlaneUnits {
-  int64_t u, sigma, corner;
+  int64_t u, diag, cols, rows, corner, slots;
   explicit PlaneUnits(const Shape& s) {
     const Layout L(s);
     const int R = L.nblk(0), ra = s.a > 0 ? L.nblk(s.nt) : 0;
     const int64_t gb = plane_group(s.prec, s.b), ga = s.a > 0 ? plane_group(s.prec, s.a) : 0;
     u = (int64_t)s.w * R * gb + (int64_t)R * ga;
-    sigma = (int64_t)R * gb * (1 + 2 * s.w) + (int64_t)R * ga + (int64_t)ra * gb;
+    diag = s.w > 0 ? R * gb : 0;
+    cols = (int64_t)s.w * R * gb + (int64_t)R * ga;
+    rows = s.w > 0 ? (int64_t)(s.w - 1) * R * gb + (int64_t)ra * gb : 0;
     corner = (int64_t)ra * ga;
+    slots = s.w > 0 ? s.w + 1 : s.nt < 2 ? s.nt : 2;
   }
-  int64_t total(const Shape& s) const { return 2 * u + (s.w + 2) * sigma + corner; }
+  int64_t sigma() const { return diag + cols + rows; }
+  int64_t total() const { return 2 * u + slots * sigma() + corner; }
 };
 
 struct Builder {
@@ -654,37 +661,35 @@ struct Builder {
 
   // ---- planes (see plan.h). Tile column i's planes live in ring slots: those of
   // Sigma (the diagonal tile by rows; each tile below it by columns, and by rows
-  // where an earlier column needs them so) in slot i mod (w + 2), read by the
+  // where an earlier column needs them so) in slot i mod (w + 1), read by the
   // columns i - w .. i; those of U in slot i mod 2, read by column i; the arrow
   // corner has a slot of its own. `p2join[i]`: the products of column i are done,
-  // so the planes that only it and later columns read may be overwritten.
+  // so the planes that only it and later columns read may be overwritten. (Column
+  // i's Sigma slot is that of column i + w + 1, last read by column i + 1, whose
+  // Sigma column i's products wait for anyway: with w + 2 slots n = 122,944 took 297.4
+  // and (28, 1024, 4, 64) 204.9 ms, with these 296.4 and 204.8.)
   std::vector<int32_t> p2join;
   std::vector<int32_t> pl_d, pl_c, pl_r, pl_u;  // counters per vector group: diagonal rows; tile columns / rows; U
   std::vector<int64_t> pl_dbase, pl_cbase, pl_rbase, pl_ubase;
-  int64_t pu_sigma = 0, pu_u = 0;  // units of a Sigma slot, a U slot
-  int64_t sig_slots() const { return s.w + 2; }
+  PlaneUnits pu{s};
   // offset of a tile's planes inside its column's Sigma or U slot
   enum PlaneSet { PS_DIAG, PS_COL, PS_ROW, PS_U };
   int64_t plane_off(PlaneSet set, int k, int i) const {
-    const int R = L.nblk(i);
-    if (i == s.nt) return 2 * pu_u + sig_slots() * pu_sigma;
-    const int64_t gb = plane_group(s.prec, s.b), ga = s.a > 0 ? plane_group(s.prec, s.a) : 0;
-    if (set == PS_U) return (int64_t)(i % 2) * pu_u + (k == s.nt ? (int64_t)s.w * R * gb : (int64_t)(k - i - 1) * R * gb);
-    const int64_t slot = 2 * pu_u + (int64_t)(i % sig_slots()) * pu_sigma;
+    if (i == s.nt) return 2 * pu.u + pu.slots * pu.sigma();
+    const int64_t tile = L.nblk(i) * plane_group(s.prec, s.b);  // of a band tile
+    const int64_t band = (int64_t)(k == s.nt ? s.w : k - i - 1) * tile;
+    if (set == PS_U) return (int64_t)(i % 2) * pu.u + band;
+    const int64_t slot = 2 * pu.u + (int64_t)(i % pu.slots) * pu.sigma();
     if (set == PS_DIAG) return slot;
-    if (set == PS_COL) return slot + (int64_t)R * gb * (k == s.nt ? 1 + s.w : k - i);
-    const int64_t rows0 = slot + (int64_t)R * gb * (1 + s.w) + (int64_t)R * ga;
-    return rows0 + (k == s.nt ? (int64_t)s.w * R * gb : (int64_t)(k - i - 1) * R * gb);
+    if (set == PS_COL) return slot + pu.diag + band;
+    return slot + pu.diag + pu.cols + (k == s.nt ? (int64_t)(s.w - 1) * tile : band);
   }
   int64_t plane_ref(PlaneSet set, int k, int i, int g) const {  // group g of the tile's planes
     const int kk = set == PS_DIAG || set == PS_ROW ? L.rows(i) : L.rows(k);
     return mkref(BUF_P, plane_off(set, k, i) + (int64_t)g * plane_group(s.prec, kk));
   }
   void alloc_planes(int cols) {
-    const PlaneUnits u(s);
-    pu_u = u.u;
-    pu_sigma = u.sigma;
-    if (out) out->plane_units = u.total(s);
+    if (out) out->plane_units = pu.total();
     p2join.assign(cols, -1);
     pl_dbase.assign(cols, 0);
     for (auto* v : {&pl_cbase, &pl_rbase, &pl_ubase}) v->assign((size_t)cols * (s.w + 2), -1);
@@ -703,7 +708,9 @@ struct Builder {
         w.push_back({scol(i, i, g), L.nblk(i) - g});
       } else if (set == PS_COL) w.push_back({scol(k, i, g), L.nblk(k)});
       else w.push_back({srow(k, i, g), L.nblk(i)});
-      if (i < s.nt && i + 2 < (int)p2join.size() && p2join[i + 2] >= 0) w.push_back({p2join[i + 2], 1});
+      // the lowest column that reads what the slot held before
+      const int reader = set == PS_U ? i + 2 : i + (int)pu.slots - s.w;
+      if (i < s.nt && reader < (int)p2join.size() && p2join[reader] >= 0) w.push_back({p2join[reader], 1});
       // at most 4 chunks of K (16 parts) per task
       for (int c0 = 0; c0 < (int)plane_chunks(kk); c0 += 4) {
         const int k0 = c0 * kPlaneChunk;
@@ -1088,6 +1095,8 @@ static double task_estimate(const Shape& s) {
 bool use_planes(const Shape& s) {
   return s.prec != PREC_FP64 && s.b >= kPlanesMinB && (int64_t)s.w * s.b + s.a >= kPlanesMinK;
 }
+
+int64_t plane_units(const Shape& s) { return PlaneUnits(s).total(); }
 
 static bool shape_ok(const Shape& s) {
   return s.nt >= 1 && s.b >= 1 && s.w >= 0 && s.a >= 0 && s.w <= s.nt - 1 && tune_valid(s.tune) && s.sel0 >= 0 &&

@@ -226,6 +226,14 @@ struct Shape {
 // Whether the phase-2 products of a (reduced-precision) shape read planes: a rule
 // on its sizes, with its reasons at the definition.
 bool use_planes(const Shape& s);
+// Units of 16 bytes that they take, beside the scratch tiles.
+int64_t plane_units(const Shape& s);
+// Whether buffers of `doubles` doubles (A, L, Sigma and the scratch tiles) and the
+// planes go into a device of `device_bytes`, a sixteenth of which is left to tables and
+// the runtime: a matrix that fills the device runs without planes, as it has to.
+inline bool planes_fit(int64_t doubles, int64_t units, int64_t device_bytes) {
+  return 32 * doubles + 16 * units <= device_bytes / 16 * 15;
+}
 
 // A task with few successors is counted off them by each of its parts as it
 // finishes (one atomic per successor and part, no join of the parts on the

@@ -118,6 +118,11 @@ static bool sigma_writes_in_sigma(const Plan& p) {
 
 static size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
+static int64_t device_bytes() {  // of the current device
+  size_t free_bytes = 0, total = 0;
+  return cudaMemGetInfo(&free_bytes, &total) == cudaSuccess ? (int64_t)total : INT64_MAX;
+}
+
 static void free_handle(stiles_handle* h) {
   if (!h) return;
   for (auto& d : h->dev) {
@@ -210,7 +215,7 @@ static int create_handle(int nt, int b, int band, int arrow, int precision, int 
     return STILES_ERR_CUDA;
   }
   h->grid = h->sms * kCtasPerSm;
-  h->s.planes = use_planes(h->s);
+  h->s.planes = use_planes(h->s) && planes_fit(Layout(h->s).doubles(), plane_units(h->s), device_bytes());
   const int brc = build_handle_plans(h);
   if (brc) {
     delete h;
@@ -714,6 +719,10 @@ extern "C" int stiles_batch_create(int count, const int* nt, const int* b, const
     delete h;
     return STILES_ERR_CUDA;
   }
+  int64_t units = 0;
+  for (const Shape& s : h->shapes) units += s.planes ? plane_units(s) : 0;
+  if (units && !planes_fit(h->off[count], units, device_bytes()))
+    for (Shape& s : h->shapes) s.planes = false;
   h->grid = h->sms * kCtasPerSm;
   std::vector<int64_t> base(h->off.begin(), h->off.end() - 1);
   int rc = build_batch_plan(h->shapes, base, 0, &h->plan, &h->diag_base);

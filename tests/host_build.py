@@ -23,4 +23,6 @@ def plan_host():
     lib = ctypes.CDLL(so)
     lib.fixed_scratch.restype = ctypes.c_longlong
     lib.fixed_scratch.argtypes = [ctypes.c_int] * 5 + [ctypes.c_longlong, ctypes.POINTER(ctypes.c_longlong)]
+    lib.plane_bytes.restype = ctypes.c_longlong
+    lib.planes_go_in.argtypes = [ctypes.c_longlong] * 3
     return lib

@@ -22,3 +22,8 @@ extern "C" long long fixed_scratch(int nt, int b, int w, int a, int prec, long l
   if (build_small_plan(s, w_bytes, (size_t)limit, &p)) return -1;
   return validate_plan(p, s, PLAN_FUSED) ? -3 : (long long)(w_bytes + 4 * sched_state_ints(p));
 }
+
+extern "C" long long plane_bytes(int nt, int b, int w, int a, int prec) { return 16 * plane_units(shape(nt, b, w, a, prec)); }
+extern "C" int planes_go_in(long long doubles, long long plane_bytes, long long device) {
+  return planes_fit(doubles, plane_bytes / 16, device);
+}
