@@ -258,7 +258,7 @@ int stiles_status(stiles_t h, int *code, long long *info, long long *tasks_done)
  * nanoseconds (default 20 s); when it expires the launch stops with
  * STILES_ERR_TIMEOUT instead of hanging. STILES_OPT_GRID: persistent CTAs per
  * launch (0 = the default, two per SM). STILES_OPT_TRACE: 1 allocates a
- * device trace buffer (32 bytes per task) and makes every later launch record
+ * device trace buffer (512 bytes per task) and makes every later launch record
  * per-part %globaltimer stamps (read with stiles_trace); 0 frees it (default
  * off: tracing costs a few extra stores per part). Returns STILES_ERR_INVALID_ARG
  * for an unknown option or value. */
@@ -268,9 +268,10 @@ int stiles_set_option(stiles_t h, int option, long long value);
 /* Per-part trace of the last launch (tracing must be on). Waits for the
  * launch. *n_tasks receives the task count of that launch; if out_host is not
  * NULL it must hold capacity >= 16 * n_tasks words and receives 4 records of
- * 4 words per task (in queue order; record r holds the last to finish of the
- * parts r, r + 4, ..; records of parts a task does not have are zero): time the
- * worker started looking for work, time it got this part, end time (ns of the GPU's global timer), and
+ * 4 words per task (in queue order; record r holds one of the parts r, r + 4, ..:
+ * the one that completed the task, else their last to end; records of parts a task
+ * does not have are zero): time the worker started looking for work, time it got
+ * this part, end time (ns of the GPU's global timer), and
  * (sm << 32 | cta << 12 | precision << 10 | last part << 9 | urgent << 8 | op). */
 int stiles_trace(stiles_t h, unsigned long long *out_host, size_t capacity, size_t *n_tasks);
 

@@ -253,6 +253,22 @@ constexpr int kTasksPerBucket = 64;
 constexpr int kMaxParts = 16;  // parts of one task; a queue entry is kMaxParts * task + part
 constexpr int kMaxTasks = (1 << 27) - 1;  // entries stay positive 32-bit integers
 
+// Trace: a record per part on the device, four per task for the caller: record r is
+// the one of the parts r, r + 4, .. that completed the task, else their last to end.
+constexpr int kTraceWords = 4;
+constexpr unsigned long long kTraceLast = 1ull << 9;  // in a record's last word
+inline void trace_records(const unsigned long long* parts, unsigned long long* out) {
+  for (int r = 0; r < 4; ++r) {
+    const unsigned long long* best = parts + kTraceWords * r;
+    for (int q = r + 4; q < kMaxParts; q += 4) {
+      const unsigned long long* x = parts + kTraceWords * q;
+      const bool last = x[3] & kTraceLast, best_last = best[3] & kTraceLast;
+      if (last != best_last ? last : x[2] > best[2]) best = x;
+    }
+    for (int i = 0; i < kTraceWords; ++i) out[kTraceWords * r + i] = best[i];
+  }
+}
+
 struct Plan {
   int64_t plane_units = 0;  // BUF_P: units of 16 bytes (0: no product reads planes)
   std::vector<Task> tasks;  // in queue order

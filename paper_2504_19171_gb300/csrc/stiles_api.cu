@@ -77,6 +77,7 @@ int upload(const std::vector<T>& v, T** out) {
 // Table of the fused plan with a smaller scratch (build_small_plan), for
 // stiles_factor_selinv_noalloc where the ordinary one does not fit its fixed array.
 constexpr int kTableSmall = 3;
+constexpr size_t kTraceBytes = kMaxParts * kTraceWords * sizeof(unsigned long long);  // per task
 
 struct stiles_handle {
   Shape s;
@@ -289,7 +290,7 @@ static int launch(stiles_t h, int kind, const double* A, double* L, double* S, v
   p.budget_ns = h->budget_ns;
   p.use_tc = h->s.prec != PREC_FP64;
   p.trace = h->dtrace;
-  if (h->dtrace && cudaMemsetAsync(h->dtrace, 0, 16 * sizeof(unsigned long long) * h->trace_tasks, st) != cudaSuccess)
+  if (h->dtrace && cudaMemsetAsync(h->dtrace, 0, kTraceBytes * h->trace_tasks, st) != cudaSuccess)
     return STILES_ERR_CUDA;
   p.buf_len = Layout(h->s).doubles();
   h->last_stream = st;
@@ -473,7 +474,7 @@ extern "C" int stiles_set_option(stiles_t h, int option, long long value) {
       if (value) {
         size_t n = 0;
         for (auto& d : h->dev) n = (size_t)d.ntasks > n ? (size_t)d.ntasks : n;
-        if (dev_malloc((void**)&h->dtrace, 16 * sizeof(unsigned long long) * (n ? n : 1))) return STILES_ERR_OOM;
+        if (dev_malloc((void**)&h->dtrace, kTraceBytes * (n ? n : 1))) return STILES_ERR_OOM;
         h->trace_tasks = n;
       }
       return STILES_OK;
@@ -618,8 +619,14 @@ extern "C" int stiles_trace(stiles_t h, unsigned long long* out_host, size_t cap
   if (capacity < 16 * n) return STILES_ERR_INVALID_ARG;
   if (cudaSetDevice(h->device) != cudaSuccess) return STILES_ERR_CUDA;
   if (cudaStreamSynchronize(h->last_stream) != cudaSuccess) return STILES_ERR_CUDA;
-  if (n && cudaMemcpy(out_host, h->dtrace, 16 * sizeof(unsigned long long) * n, cudaMemcpyDeviceToHost) != cudaSuccess)
-    return STILES_ERR_CUDA;
+  constexpr size_t kStep = 1 << 14;  // tasks copied at a time
+  std::vector<unsigned long long> rec(kTraceBytes / 8 * (n < kStep ? n : kStep));
+  for (size_t t0 = 0; t0 < n; t0 += kStep) {
+    const size_t m = n - t0 < kStep ? n - t0 : kStep;
+    if (cudaMemcpy(rec.data(), h->dtrace + kTraceBytes / 8 * t0, kTraceBytes * m, cudaMemcpyDeviceToHost) != cudaSuccess)
+      return STILES_ERR_CUDA;
+    for (size_t t = 0; t < m; ++t) trace_records(rec.data() + kTraceBytes / 8 * t, out_host + 16 * (t0 + t));
+  }
   return STILES_OK;
 }
 

@@ -117,7 +117,7 @@ struct KParams {
                         // (a host buffer mapped into the device's address space), or null
   long long budget_ns;  // bound of one dependency wait
   int32_t* badpiv;     // optional: per POTRF task, first failing pivot (0-based in its block) or -1
-  unsigned long long* trace;  // optional: 4 words per task (claim, ready, end ns; sm/cta/op), or null
+  unsigned long long* trace;  // optional: kMaxParts records of kTraceWords per task (claim, ready, end ns; sm/cta/op), or null
   long long buf_len;          // doubles in each of buf[0..3] (self-checking builds)
   int serve;                  // 1: request server (rings and inbox instead of the static buckets)
   int use_tc;                 // 1: the plan has reduced-precision products (tensor memory and barriers held)

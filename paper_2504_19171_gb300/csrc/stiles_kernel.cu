@@ -1883,8 +1883,8 @@ __global__ void __launch_bounds__(NTHREADS, 2) persistent_kernel(const __grid_co
     if (threadIdx.x == 0) {
       if (tk.op == OP_POTRF) fence_dev();
       if (last) account_task(p, t);
-      if (p.trace) {  // one record per task part (parts 4 apart share one)
-        unsigned long long* tr = p.trace + 4 * (4 * (size_t)t + (q & 3));
+      if (p.trace) {  // one record per task part
+        unsigned long long* tr = p.trace + kTraceWords * (kMaxParts * (size_t)t + q);
         tr[0] = t_claim;
         tr[1] = t_ready;
         tr[2] = gtimer();

@@ -256,9 +256,10 @@ def stiles_debug_occupancy(tensor_parts: bool) -> int:
 
 
 def stiles_trace(h: int) -> np.ndarray:
-    """Per-part trace of the last launch as an (n_tasks, 4 parts, 4) uint64
+    """Trace of the last launch as an (n_tasks, 4 records, 4) uint64
     array: search start, got-part and end times (ns) and the packed
-    (sm, cta, precision, last part, urgent, op) word; absent parts are zero."""
+    (sm, cta, precision, last part, urgent, op) word; record r is of one of the
+    parts r, r + 4, .. (see the C header), zero if there is none."""
     n = ctypes.c_size_t()
     _check(_lib.stiles_trace(h, None, 0, ctypes.byref(n)), "stiles_trace")
     out = np.zeros((n.value, 4, 4), dtype=np.uint64)

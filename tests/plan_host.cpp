@@ -27,3 +27,5 @@ extern "C" long long plane_bytes(int nt, int b, int w, int a, int prec) { return
 extern "C" int planes_go_in(long long doubles, long long plane_bytes, long long device) {
   return planes_fit(doubles, plane_bytes / 16, device);
 }
+
+extern "C" void trace_pick(const unsigned long long* parts, unsigned long long* out) { trace_records(parts, out); }
