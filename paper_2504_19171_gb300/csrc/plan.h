@@ -105,6 +105,14 @@ inline int64_t plane_group(int prec, int k) {  // units of one group
   return plane_head(prec, k) + plane_stages(k) * 128 * plane_count(prec);
 }
 
+// The count of stages a CTA has run, kept below 128: stage g is in slot g % slots and
+// phase g / slots of its barriers, of which the parity counts, for 4 or 8 slots, and
+// whether there was a phase before.
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline uint32_t stage_count(uint32_t n) { return n < 64 ? n : 64 + n % 64; }
+
 // Sub-tile of part q of an m x n block (rm or cn <= 0: nothing to do).
 struct Sub {
   int r0, c0, rm, cn;

@@ -683,7 +683,7 @@ struct TcShared {
   uint64_t pfull[PL_SLOTS];   // products from planes: a slot's copies have landed
   uint64_t pempty[PL_SLOTS];  // ... its MMAs are done
   uint64_t pdone;             // every MMA issued before is done
-  uint32_t pstage;       // stages this CTA has run so far: stage g is slot g % NST, phase g / NST
+  uint32_t pstage;       // stages this CTA has run so far (stage_count): stage g is slot g % NST, phase g / NST
   uint32_t pdone_n;      // phases of pdone
   uint32_t tmem;         // TMEM base address of this CTA's TC_COLS columns
 };
@@ -1151,7 +1151,7 @@ __device__ __noinline__ void run_planes(const KParams& p, const Task& tk, int q,
     return;
   }
   if (tid == 0) {  // (read again only after the next part's first barrier)
-    ts.pstage = base + used;
+    ts.pstage = stage_count(base + used);  // (counted on, it wraps after an hour or more in a server)
     ts.pdone_n = ndone;
   }
   store_part(p, tk, q, smem, r16);

@@ -29,3 +29,5 @@ extern "C" int planes_go_in(long long doubles, long long plane_bytes, long long 
 }
 
 extern "C" void trace_pick(const unsigned long long* parts, unsigned long long* out) { trace_records(parts, out); }
+
+extern "C" unsigned stages_run(unsigned before, unsigned used) { return stage_count(before + used); }
