@@ -207,14 +207,15 @@ __device__ int wait_slot(const KParams& p, int* slot, unsigned long long start) 
 // Lane 0: claim one available part of a queue (avail / head pair) without a
 // compare-and-swap retry loop: many idle workers contending for the same
 // bucket each cost two fetch-and-adds, not a round trip per lost race. The
-// caller has just read avail > 0. Returns the claimed slot index, or -1 if
-// nothing was available.
-__device__ __forceinline__ int claim(int* avail, int* head) {
+// caller has just read avail > 0. False if nothing was available; else `pos` is the
+// claimed slot's index (a ring's grows over the launch, past 2^31 too).
+__device__ __forceinline__ bool claim(int* avail, int* head, unsigned& pos) {
   if (atomicSub(avail, 1) <= 0) {
     atomicAdd(avail, 1);
-    return -1;
+    return false;
   }
-  return atomicAdd(head, 1);
+  pos = (unsigned)atomicAdd(head, 1);
+  return true;
 }
 
 // Pause of a worker that found nothing. The first half of the grid (one CTA
@@ -294,9 +295,9 @@ __device__ int serve_pop(const KParams& p, unsigned long long deadline) {
       int got = -3;
       if (lane == 0) {
         const ServeRing& R = p.sv.ring[r];
-        const int h = claim(R.ctr + 16, R.ctr + 8);
-        if (h >= 0) {
-          int* slot = R.slots + ((unsigned)h & R.mask);
+        unsigned h = 0;
+        if (claim(R.ctr + 16, R.ctr + 8, h)) {
+          int* slot = R.slots + (h & R.mask);
           got = wait_slot(p, slot, gtimer());
           if (got >= 0) store_relaxed_i(slot, -1);
         }
@@ -358,11 +359,13 @@ __device__ int pop_task(const KParams& p, unsigned long long deadline) {
     if (__shfl_sync(FULL, v, 1) > 0) {  // urgent parts
       int got = -3;
       if (lane == 0) {
-        const int uh = claim(p.q.lo + 24, p.q.lo + 16);
-        if (uh >= p.ucap) {  // claimed past the urgent queue (checked in every build)
+        unsigned uh = 0;
+        if (!claim(p.q.lo + 24, p.q.lo + 16, uh)) {
+          // another worker was faster
+        } else if (uh >= (unsigned)p.ucap) {  // claimed past the urgent queue (checked in every build)
           check_fail(p, 4, uh, 0);
           got = -1;
-        } else if (uh >= 0) {
+        } else {
           got = wait_slot(p, p.q.uslots + uh, start);
         }
       }
@@ -376,12 +379,12 @@ __device__ int pop_task(const KParams& p, unsigned long long deadline) {
         const int bb = base + __ffs(rm) - 1;
         rm &= rm - 1;
         if (lane == 0) {
-          const int h = claim(p.q.avail + bb, p.q.head + bb);
-          if (h >= 0) {
+          unsigned h = 0;
+          if (claim(p.q.avail + bb, p.q.head + bb, h)) {
             atomicSub(p.q.gcnt + (bb >> 5), 1);
             atomicSub(p.q.scnt + (bb >> 10), 1);
             const int s0 = p.soff[bb];
-            if (h >= p.soff[bb + 1] - s0) {  // claimed past the bucket (checked in every build)
+            if (h >= (unsigned)(p.soff[bb + 1] - s0)) {  // claimed past the bucket (checked in every build)
               check_fail(p, 5, bb, 0);
               got = -1;
             } else {

@@ -343,8 +343,12 @@ extern "C" int stiles_server_start(stiles_server_t h, double window_s) {
   if (cudaSetDevice(h->device) != cudaSuccess) return STILES_ERR_CUDA;
   cudaStream_t cs = h->cstream;
   const unsigned ring = h->ring_mask + 1;
+  // a ring's positions (tail, head) count modulo 2^32 and begin just below 2^31, so
+  // that every window passes the change of sign that a long one comes to
+  int ctr[3 * 32] = {};
+  for (int r = 0; r < 3; ++r) ctr[32 * r] = ctr[32 * r + 8] = INT32_MAX - 20;
   if (cudaMemsetAsync(h->ring_slots, 0xff, sizeof(int) * 3 * (size_t)ring, cs) != cudaSuccess ||
-      cudaMemsetAsync(h->ring_ctr, 0, sizeof(int) * 3 * 32, cs) != cudaSuccess ||
+      cudaMemcpyAsync(h->ring_ctr, ctr, sizeof(ctr), cudaMemcpyHostToDevice, cs) != cudaSuccess ||
       cudaMemsetAsync(h->inbox_seen, 0, sizeof(int), cs) != cudaSuccess ||
       cudaMemsetAsync(h->dstatus, 0, sizeof(DevStatus), cs) != cudaSuccess ||
       cudaMemsetAsync(&h->dstatus->spd_col, 0xff, sizeof(unsigned long long), cs) != cudaSuccess ||
