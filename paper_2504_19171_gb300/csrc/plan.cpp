@@ -1244,12 +1244,8 @@ int validate_plan_len(const Plan& p, int64_t lim, int kind) {
     fprintf(stderr, "validate_plan: %s (task %d, op %d)\n", what, t, t >= 0 ? (int)p.tasks[t].op : -1);
     return STILES_ERR_PLAN;
   };
-  auto in = [&](int64_t ref, int64_t lo_off, int64_t hi_off) {  // [ref+lo, ref+hi] inside its buffer
-    if (ref < 0) return false;
-    const int64_t off = ref & OFF_MASK;
-    const int buf = (int)(ref >> BUF_SHIFT);
-    return buf >= 0 && buf < 4 && ((allowed >> buf) & 1) && off + lo_off >= 0 && off + hi_off < lim;
-  };
+  const Bounds all{lim, allowed, p.plane_units, p.ndiag};
+  auto in = [&](int64_t ref, int64_t lo, int64_t hi) { return ref_in(all, ref, lo, hi); };
   for (int t = 0; t < nt; ++t) {
     const Task& tk = p.tasks[t];
     if (tk.op == OP_PREP) {  // a whole tile column of the base and of L, and the row-sum vectors
@@ -1266,67 +1262,8 @@ int validate_plan_len(const Plan& p, int64_t lim, int kind) {
         return bad("PREP out of bounds", t);
       continue;
     }
-    if (tk.op == OP_JOIN) {  // no work, no access
-      if (tk.parts != 1 || tk.nseg != 0) return bad("join with work", t);
-      continue;
-    }
-    // units [ref, ref + len) of BUF_P
-    auto in_planes = [&](int64_t ref, int64_t len) {
-      return ref >= 0 && (ref >> BUF_SHIFT) == BUF_P && (ref & OFF_MASK) + len <= p.plane_units;
-    };
-    if (tk.op == OP_SPLIT) {
-      const int64_t kc = std::min<int64_t>(tk.zrows - tk.gcol, kPlaneChunk * (int64_t)(tk.parts / 4));
-      const bool kcont = tk.flags & TF_KCONT;
-      if (tk.m < 1 || tk.parts % 4 || tk.gcol % kPlaneChunk || kc < 1 || tk.prec == PREC_FP64 ||
-          (tk.parts / 4 - 1) * kPlaneChunk >= tk.zrows - tk.gcol ||
-          !in(tk.cin, 0, kcont ? (tk.m - 1) * (int64_t)tk.ldc + kc - 1 : tk.m - 1 + (kc - 1) * (int64_t)tk.ldc) ||
-          !in_planes(tk.out, plane_group(tk.prec, tk.zrows)))
-        return bad("split out of bounds", t);
-      continue;
-    }
-    if (tk.op == OP_ZERO) {  // zrows x n above the block
-      if (tk.parts != 1 || tk.nseg != 0 || tk.zrows < 1 || tk.n < 1 ||
-          !in(tk.out, -(int64_t)tk.zrows, -1 + (int64_t)(tk.n - 1) * tk.ldo))
-        return bad("zeroed rows out of bounds", t);
-      continue;
-    }
-    for (int q = 0; q < tk.parts; ++q) {
-      const Sub sb = part_sub(tk.pmode, tk.m, tk.n, q);
-      const int r0 = sb.r0, c0 = sb.c0, rm = sb.rm, cn = sb.cn;
-      if ((tk.pmode == PM_TRI16 || tk.pmode == PM_TRI3) && tk.m != tk.n) return bad("triangle parts on a block that is not square", t);
-      if ((tk.pmode == PM_TRI16 || tk.pmode == PM_GRID16) && tk.prec != PREC_FP64)
-        return bad("16 x 16 parts on a reduced-precision task", t);
-      if (tk.prec != PREC_FP64 && (tk.pmode != PM_COLS2 || cn > 32)) return bad("reduced-precision part larger than 64 x 32", t);
-      if (tk.prec != PREC_FP64 && tk.op != OP_UPD && tk.op != OP_NEG && tk.op != OP_STORE && tk.op != OP_SYMUPD)
-        return bad("reduced precision on a triangular task", t);
-      if (rm <= 0 || cn <= 0) continue;
-      const int r1 = r0 + rm - 1, c1 = c0 + cn - 1;
-      for (int g = tk.seg0; g < tk.seg0 + tk.nseg; ++g) {
-        const Seg& sg = p.segs[g];
-        if (sg.k <= 0) return bad("empty segment", t);
-        if (tk.flags & TF_PLANES) {
-          if (!in_planes(sg.a, plane_group(tk.prec, sg.k)) || !in_planes(sg.b, plane_group(tk.prec, sg.k)))
-            return bad("planes out of bounds", t);
-          continue;
-        }
-        const int64_t amax = (sg.trans & 1) ? (sg.k - 1) + (int64_t)r1 * sg.lda : r1 + (int64_t)(sg.k - 1) * sg.lda;
-        const int64_t amin = (sg.trans & 1) ? (int64_t)r0 * sg.lda : r0;
-        const int64_t bmax = (sg.trans & 2) ? c1 + (int64_t)(sg.k - 1) * sg.ldb : (sg.k - 1) + (int64_t)c1 * sg.ldb;
-        const int64_t bmin = (sg.trans & 2) ? c0 : (int64_t)c0 * sg.ldb;
-        if (!in(sg.a, amin, amax)) return bad("segment A out of bounds", t);
-        if (!in(sg.b, bmin, bmax)) return bad("segment B out of bounds", t);
-      }
-      if (!in(tk.out, r0 + (int64_t)c0 * tk.ldo, r1 + (int64_t)c1 * tk.ldo)) return bad("output out of bounds", t);
-      const bool uses_cin = tk.op == OP_UPD || tk.op == OP_POTRF || tk.op == OP_TRSM_RLT || tk.op == OP_SYMUPD;
-      if (uses_cin && !in(tk.cin, r0 + (int64_t)c0 * tk.ldc, r1 + (int64_t)c1 * tk.ldc)) return bad("input out of bounds", t);
-      if ((tk.op == OP_TRSM_RLT || tk.op == OP_POTRF) && !in(tk.aux, 0, (tk.n - 1) + (int64_t)(tk.n - 1) * tk.ldx)) return bad("T out of bounds", t);
-      if (tk.op == OP_TRTRI && !in(tk.aux, 0, (tk.m - 1) + (int64_t)(tk.m - 1) * tk.ldx))
-        return bad("T out of bounds", t);
-      if (tk.op == OP_SYMUPD && !(tk.flags & TF_SYM_DIAG) &&
-          !in(tk.aux, c0 + (int64_t)r0 * tk.ldx, c1 + (int64_t)r1 * tk.ldx))
-        return bad("mirror out of bounds", t);
-      if (tk.op == OP_POTRF && (tk.diag < 0 || tk.diag >= p.ndiag)) return bad("logdet slot out of range", t);
-    }
+    for (int q = 0; q < tk.parts; ++q)
+      if (const char* what = part_fault(tk, q, p.segs.data(), all)) return bad(what, t);
   }
   // queue emulation: pushes per bucket / urgent queue never exceed capacity
   std::vector<int> rem(p.rem0), tail(p.tail0), seen(nt, 0);

@@ -17,6 +17,12 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#ifdef __CUDACC__
+#define STILES_HD __host__ __device__
+#else
+#define STILES_HD
+#endif
+
 namespace stiles {
 
 constexpr int FB = 64;  // fine block order (rows and columns of one task's output)
@@ -97,31 +103,25 @@ enum TaskFlag : uint8_t {
 // Offsets in BUF_P count units of 16 bytes.
 constexpr int kPlaneChunk = 512;  // K per exponent (the most that cells sum exactly)
 constexpr int kPlaneK = 16;       // K per stage
-inline int plane_count(int prec) { return prec == PREC_EMU64 ? 8 : 3; }
-inline int64_t plane_stages(int k) { return (k + kPlaneK - 1) / kPlaneK; }
-inline int64_t plane_chunks(int k) { return (k + kPlaneChunk - 1) / kPlaneChunk; }
-inline int64_t plane_head(int prec, int k) { return prec == PREC_EMU64 ? 16 * plane_chunks(k) : 0; }
-inline int64_t plane_group(int prec, int k) {  // units of one group
+STILES_HD inline int plane_count(int prec) { return prec == PREC_EMU64 ? 8 : 3; }
+STILES_HD inline int64_t plane_stages(int k) { return (k + kPlaneK - 1) / kPlaneK; }
+STILES_HD inline int64_t plane_chunks(int k) { return (k + kPlaneChunk - 1) / kPlaneChunk; }
+STILES_HD inline int64_t plane_head(int prec, int k) { return prec == PREC_EMU64 ? 16 * plane_chunks(k) : 0; }
+STILES_HD inline int64_t plane_group(int prec, int k) {  // units of one group
   return plane_head(prec, k) + plane_stages(k) * 128 * plane_count(prec);
 }
 
 // The count of stages a CTA has run, kept below 128: stage g is in slot g % slots and
 // phase g / slots of its barriers, of which the parity counts, for 4 or 8 slots, and
 // whether there was a phase before.
-#ifdef __CUDACC__
-__host__ __device__
-#endif
-inline uint32_t stage_count(uint32_t n) { return n < 64 ? n : 64 + n % 64; }
+STILES_HD inline uint32_t stage_count(uint32_t n) { return n < 64 ? n : 64 + n % 64; }
 
 // Sub-tile of part q of an m x n block (rm or cn <= 0: nothing to do).
 struct Sub {
   int r0, c0, rm, cn;
 };
 
-#ifdef __CUDACC__
-__host__ __device__
-#endif
-inline Sub part_sub(int pmode, int m, int n, int q) {
+STILES_HD inline Sub part_sub(int pmode, int m, int n, int q) {
   Sub s{0, 0, m, n};
   int dim = 0;  // sub-tile order of the grid modes
   switch (pmode) {
@@ -192,6 +192,79 @@ struct Task {        // 80 bytes
 };
 static_assert(sizeof(Task) == 80 && offsetof(Task, op) % 4 == 0, "task layout");
 
+// ---- bounds of a task's accesses -----------------------------------------
+// The buffers of a launch: doubles in each of A, L, Sigma, scratch tiles, which of
+// them are there (a bit each), units of planes, logdet slots.
+struct Bounds {
+  int64_t doubles;
+  unsigned present;
+  int64_t plane_units;
+  int ndiag;
+};
+STILES_HD inline bool ref_in(const Bounds& b, int64_t ref, int64_t lo, int64_t hi) {  // [ref + lo, ref + hi]
+  const int buf = (int)(ref >> BUF_SHIFT);
+  const int64_t off = ref & OFF_MASK;
+  return ref >= 0 && buf < 4 && ((b.present >> buf) & 1) && off + lo >= 0 && off + hi < b.doubles;
+}
+STILES_HD inline bool planes_in(const Bounds& b, int64_t ref, int64_t len) {
+  return ref >= 0 && (ref >> BUF_SHIFT) == BUF_P && (ref & OFF_MASK) + len <= b.plane_units;
+}
+
+// What is wrong with part q of a task (every kind but OP_PREP): an access outside the
+// launch's buffers, or a part mode that its kernel does not take; null if nothing is.
+// The host validates whole tables with it, the self-checking device build every
+// part before it runs.
+STILES_HD inline const char* part_fault(const Task& t, int q, const Seg* segs, const Bounds& b) {
+  if (t.op == OP_JOIN) return t.parts != 1 || t.nseg != 0 ? "join with work" : nullptr;  // no access
+  if (t.m < 1 || t.n < 1 || t.m > FB || t.n > FB || t.op > OP_SPLIT || t.op == OP_PREP) return "unknown task";
+  if (t.op == OP_SPLIT) {
+    const int64_t left = t.zrows - t.gcol, most = kPlaneChunk * (int64_t)(t.parts / 4), kc = left < most ? left : most;
+    const bool kcont = t.flags & TF_KCONT;
+    return t.parts % 4 || t.gcol % kPlaneChunk || kc < 1 || t.prec == PREC_FP64 || most - kPlaneChunk >= left ||
+                   !ref_in(b, t.cin, 0,
+                           kcont ? (t.m - 1) * (int64_t)t.ldc + kc - 1 : t.m - 1 + (kc - 1) * (int64_t)t.ldc) ||
+                   !planes_in(b, t.out, plane_group(t.prec, t.zrows))
+               ? "split out of bounds"
+               : nullptr;
+  }
+  if (t.op == OP_ZERO)  // zrows x n above the block
+    return t.parts != 1 || t.nseg != 0 || t.zrows < 1 ||
+                   !ref_in(b, t.out, -(int64_t)t.zrows, -1 + (int64_t)(t.n - 1) * t.ldo)
+               ? "zeroed rows out of bounds"
+               : nullptr;
+  const Sub s = part_sub(t.pmode, t.m, t.n, q);
+  if ((t.pmode == PM_TRI16 || t.pmode == PM_TRI3) && t.m != t.n) return "triangle parts on a block that is not square";
+  if (t.prec != PREC_FP64 && (t.pmode != PM_COLS2 || s.cn > 32)) return "reduced-precision part other than 64 x 32";
+  if (t.prec != PREC_FP64 && t.op != OP_UPD && t.op != OP_NEG && t.op != OP_STORE && t.op != OP_SYMUPD)
+    return "reduced precision on a triangular task";
+  if (s.rm <= 0 || s.cn <= 0) return nullptr;
+  const int r0 = s.r0, c0 = s.c0, r1 = r0 + s.rm - 1, c1 = c0 + s.cn - 1;
+  for (int g = t.seg0; g < t.seg0 + t.nseg; ++g) {
+    const Seg x = segs[g];
+    if (x.k <= 0) return "empty segment";
+    if (t.flags & TF_PLANES) {
+      const int64_t len = plane_group(t.prec, x.k);
+      if (t.prec == PREC_FP64 || !planes_in(b, x.a, len) || !planes_in(b, x.b, len)) return "planes out of bounds";
+      continue;
+    }
+    const int64_t amax = (x.trans & 1) ? (x.k - 1) + (int64_t)r1 * x.lda : r1 + (int64_t)(x.k - 1) * x.lda;
+    const int64_t amin = (x.trans & 1) ? (int64_t)r0 * x.lda : r0;
+    const int64_t bmax = (x.trans & 2) ? c1 + (int64_t)(x.k - 1) * x.ldb : (x.k - 1) + (int64_t)c1 * x.ldb;
+    const int64_t bmin = (x.trans & 2) ? c0 : (int64_t)c0 * x.ldb;
+    if (!ref_in(b, x.a, amin, amax)) return "segment A out of bounds";
+    if (!ref_in(b, x.b, bmin, bmax)) return "segment B out of bounds";
+  }
+  if (!ref_in(b, t.out, r0 + (int64_t)c0 * t.ldo, r1 + (int64_t)c1 * t.ldo)) return "output out of bounds";
+  const bool cin = t.op == OP_UPD || t.op == OP_POTRF || t.op == OP_TRSM_RLT || t.op == OP_SYMUPD;
+  if (cin && !ref_in(b, t.cin, r0 + (int64_t)c0 * t.ldc, r1 + (int64_t)c1 * t.ldc)) return "input out of bounds";
+  const int tri = t.op == OP_TRSM_RLT || t.op == OP_POTRF ? t.n : t.op == OP_TRTRI ? t.m : 0;  // order of aux
+  if (tri && !ref_in(b, t.aux, 0, (tri - 1) + (int64_t)(tri - 1) * t.ldx)) return "T out of bounds";
+  if (t.op == OP_SYMUPD && !(t.flags & TF_SYM_DIAG) && !ref_in(b, t.aux, c0 + (int64_t)r0 * t.ldx, c1 + (int64_t)r1 * t.ldx))
+    return "mirror out of bounds";
+  if (t.op == OP_POTRF && (t.diag < 0 || t.diag >= b.ndiag)) return "logdet slot out of range";
+  return nullptr;
+}
+
 }  // namespace stiles
 
 #ifndef __CUDACC_RTC__
@@ -247,10 +320,7 @@ inline bool planes_fit(int64_t doubles, int64_t units, int64_t device_bytes) {
 // finishes (one atomic per successor and part, no join of the parts on the
 // critical path); one with many by the last of its parts.
 constexpr int kPartSucc = 16;
-#ifdef __CUDACC__
-__host__ __device__
-#endif
-inline bool counts_parts(const Task& t) { return t.nsucc <= kPartSucc; }
+STILES_HD inline bool counts_parts(const Task& t) { return t.nsucc <= kPartSucc; }
 
 // Dynamic schedule: a task becomes ready when the last part of its last
 // predecessor finishes (device counter rem[t], initialised to rem0[t]) and is

@@ -286,6 +286,7 @@ static int launch(stiles_t h, int kind, const double* A, double* L, double* S, v
   p.buf[BUF_S] = S;
   p.buf[BUF_W] = (double*)scr;
   p.planes = (uint8_t*)scr + h->w_bytes;
+  p.plane_units = noalloc_table ? 0 : h->plans[kind].plane_units;
   p.smirror = smirror;
   p.budget_ns = h->budget_ns;
   p.use_tc = h->s.prec != PREC_FP64;
@@ -821,6 +822,7 @@ static int build_batch_graph(stiles_batch* h, const double* A, double* L, double
   p.buf[BUF_S] = S;
   p.buf[BUF_W] = (double*)scr;
   p.planes = (uint8_t*)scr + h->w_bytes;
+  p.plane_units = h->plan.plane_units;
   p.budget_ns = h->budget_ns;
   p.use_tc = h->prec != PREC_FP64;
   p.trace = nullptr;

@@ -119,6 +119,7 @@ struct KParams {
   int32_t* badpiv;     // optional: per POTRF task, first failing pivot (0-based in its block) or -1
   unsigned long long* trace;  // optional: kMaxParts records of kTraceWords per task (claim, ready, end ns; sm/cta/op), or null
   long long buf_len;          // doubles in each of buf[0..3] (self-checking builds)
+  long long plane_units;      // units behind `planes` (self-checking builds)
   int serve;                  // 1: request server (rings and inbox instead of the static buckets)
   int use_tc;                 // 1: the plan has reduced-precision products (tensor memory and barriers held)
   ServeDev sv;

@@ -1690,62 +1690,33 @@ __device__ void run_sub(const KParams& p, const Task& tk, const Sub& sb, double*
   }
 }
 
-// Run part q of task tk (the planner only splits operations whose parts are
-// independent: products, the row-wise TRSM and the mirrored Sigma_ii store).
-#ifdef STILES_CHECKED
-// [ref + lo, ref + hi] inside its buffer
-__device__ bool ref_ok(const KParams& p, int64_t ref, int64_t lo, int64_t hi) {
-  if (ref < 0) return false;
-  const int buf = (int)(ref >> BUF_SHIFT);
-  const int64_t off = ref & OFF_MASK;
-  return buf >= 0 && buf < 4 && p.buf[buf] != nullptr && off + lo >= 0 && off + hi < p.buf_len;
-}
-
-__device__ bool task_part_ok(const KParams& p, const Task& tk, const Sub& sb) {
-  const int r0 = sb.r0, c0 = sb.c0, r1 = sb.r0 + sb.rm - 1, c1 = sb.c0 + sb.cn - 1;
-  if (tk.m < 1 || tk.n < 1 || tk.m > FB || tk.n > FB || tk.op > OP_SYMUPD) return false;
-  for (int s = 0; s < tk.nseg; ++s) {
-    const Seg g = load_seg(p, tk.seg0 + s);
-    const int64_t amax = (g.trans & 1) ? (g.k - 1) + (int64_t)r1 * g.lda : r1 + (int64_t)(g.k - 1) * g.lda;
-    const int64_t amin = (g.trans & 1) ? (int64_t)r0 * g.lda : r0;
-    const int64_t bmax = (g.trans & 2) ? c1 + (int64_t)(g.k - 1) * g.ldb : (g.k - 1) + (int64_t)c1 * g.ldb;
-    const int64_t bmin = (g.trans & 2) ? c0 : (int64_t)c0 * g.ldb;
-    if (g.k < 1 || !ref_ok(p, g.a, amin, amax) || !ref_ok(p, g.b, bmin, bmax)) return false;
-  }
-  if (!ref_ok(p, tk.out, r0 + (int64_t)c0 * tk.ldo, r1 + (int64_t)c1 * tk.ldo)) return false;
-  const bool cin = tk.op == OP_UPD || tk.op == OP_POTRF || tk.op == OP_TRSM_RLT || tk.op == OP_SYMUPD;
-  if (cin && !ref_ok(p, tk.cin, r0 + (int64_t)c0 * tk.ldc, r1 + (int64_t)c1 * tk.ldc)) return false;
-  if ((tk.op == OP_TRSM_RLT || tk.op == OP_POTRF) && !ref_ok(p, tk.aux, 0, (tk.n - 1) + (int64_t)(tk.n - 1) * tk.ldx))
-    return false;
-  if (tk.op == OP_TRTRI && !ref_ok(p, tk.aux, 0, (tk.m - 1) + (int64_t)(tk.m - 1) * tk.ldx))
-    return false;
-  if (tk.op == OP_SYMUPD && !(tk.flags & TF_SYM_DIAG) && !ref_ok(p, tk.aux, c0 + (int64_t)r0 * tk.ldx, c1 + (int64_t)r1 * tk.ldx))
-    return false;
-  return true;
-}
-#endif
-
 // OP_ZERO: the zrows x n block above the task's output block (column-major,
 // leading dimension ldo) set to zero.
-__device__ void run_zero(const KParams& p, const Task& tk, int t) {
-#ifdef STILES_CHECKED
-  if (tk.zrows < 1 || tk.n < 1 || !ref_ok(p, tk.out, -(int64_t)tk.zrows, (int64_t)(tk.n - 1) * tk.ldo)) {
-    if (threadIdx.x == 0) check_fail(p, 7, t, 0);
-    return;
-  }
-#endif
+__device__ void run_zero(const KParams& p, const Task& tk) {
   double* Z = resolve(p, tk.out) - tk.zrows;
   for (int e = threadIdx.x; e < tk.zrows * tk.n; e += NTHREADS) Z[e % tk.zrows + (int64_t)(e / tk.zrows) * tk.ldo] = 0.0;
 }
 
+// Run part q of task tk (the planner only splits operations whose parts are
+// independent: products, the row-wise TRSM and the mirrored Sigma_ii store).
 template <bool TC>
 __device__ void run_task(const KParams& p, const Task& tk, int t, int q, double* smem, TcShared* ts) {
+#ifdef STILES_CHECKED
+  // every part's accesses inside the launch's buffers (OP_PREP's bases have a layout of their own)
+  unsigned present = 0;
+  for (int x = 0; x < 4; ++x) present |= (p.buf[x] != nullptr) << x;
+  const Bounds all{p.buf_len, present, p.planes ? p.plane_units : 0, INT32_MAX};
+  if (tk.op != OP_PREP && part_fault(tk, q, p.segs, all)) {
+    if (threadIdx.x == 0) check_fail(p, 7, t, q);
+    return;
+  }
+#endif
   if (tk.op == OP_PREP) {
     run_prep(p, tk, t);
     return;
   }
   if (tk.op == OP_ZERO) {
-    run_zero(p, tk, t);
+    run_zero(p, tk);
     return;
   }
   if (tk.op == OP_JOIN) return;  // a dependency point only
@@ -1761,12 +1732,6 @@ __device__ void run_task(const KParams& p, const Task& tk, int t, int q, double*
       return;
     }
     if (tk.prec != PREC_FP64) {
-#ifdef STILES_CHECKED
-      if (!task_part_ok(p, tk, part_sub(tk.pmode, tk.m, tk.n, q))) {
-        if (threadIdx.x == 0) check_fail(p, 7, t, q);
-        return;
-      }
-#endif
       if (tk.prec == PREC_EMU64) run_tc<8>(p, tk, q, smem, *ts);
       else run_tc<4>(p, tk, q, smem, *ts);
       return;
@@ -1774,12 +1739,6 @@ __device__ void run_task(const KParams& p, const Task& tk, int t, int q, double*
   }
   const Sub sb = part_sub(tk.pmode, tk.m, tk.n, q);
   if (sb.rm <= 0 || sb.cn <= 0) return;
-#ifdef STILES_CHECKED
-  if (!task_part_ok(p, tk, sb)) {
-    if (threadIdx.x == 0) check_fail(p, 7, t, q);
-    return;
-  }
-#endif
   switch (tk.pmode) {
     case PM_ROWS2: run_sub<2, 8>(p, tk, sb, smem); break;
     case PM_ROWS4:

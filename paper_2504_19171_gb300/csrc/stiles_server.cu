@@ -372,6 +372,7 @@ extern "C" int stiles_server_start(stiles_server_t h, double window_s) {
   p.buf[BUF_S] = h->data;
   p.buf[BUF_W] = h->data;
   p.planes = h->planes;
+  p.plane_units = h->plane_units * h->max_req;
   p.budget_ns = h->budget_ns;
   p.buf_len = h->data_doubles;
   p.serve = 1;

@@ -31,3 +31,28 @@ extern "C" int planes_go_in(long long doubles, long long plane_bytes, long long 
 extern "C" void trace_pick(const unsigned long long* parts, unsigned long long* out) { trace_records(parts, out); }
 
 extern "C" unsigned stages_run(unsigned before, unsigned used) { return stage_count(before + used); }
+
+// Plants one fault in the fused plan's tasks that work on planes, and counts the
+// parts in which the part check (that of the self-checking device build) finds it.
+// which: 0 none, 1 a split's planes past the end, 2 a split's source past the end, 3 a
+// product's planes past the end, 4 a product's output, 5 its input block, 6 its mirror.
+extern "C" int plane_faults(int nt, int b, int w, int a, int prec, int which) {
+  const Shape s = shape(nt, b, w, a, prec);
+  Plan p;
+  if (build_plan(s, PLAN_FUSED, 0, &p) || !p.plane_units) return -1;
+  const int64_t n = Layout(s).doubles();
+  const Bounds all{n, 15, p.plane_units, p.ndiag};
+  for (Task& t : p.tasks) {
+    const bool split = t.op == OP_SPLIT, product = t.flags & TF_PLANES;
+    if (which == 1 && split) t.out = mkref(BUF_P, p.plane_units - plane_group(t.prec, t.zrows) + 1);
+    if (which == 2 && split) t.cin = mkref((int)(t.cin >> BUF_SHIFT), n - 1);
+    if (which == 3 && product) p.segs[t.seg0].b = mkref(BUF_P, p.plane_units);
+    if (which == 4 && product) t.out = mkref(BUF_S, n - 1);
+    if (which == 5 && product && t.op == OP_SYMUPD) t.cin = mkref(BUF_S, n - 1);
+    if (which == 6 && product && t.op == OP_SYMUPD && !(t.flags & TF_SYM_DIAG)) t.aux = mkref(BUF_S, n - 1);
+  }
+  int found = 0;
+  for (const Task& t : p.tasks)
+    for (int q = 0; q < t.parts; ++q) found += part_fault(t, q, p.segs.data(), all) != nullptr;
+  return found;
+}
