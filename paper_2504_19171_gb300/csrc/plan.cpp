@@ -1398,24 +1398,26 @@ class RaceCheck {
       return len > 0 ? rect(tk.out, (int)len, 0, (int)len, 0, 1, id, true) : true;
     }
     if (tk.op == OP_SPLIT) {
-      // 16 vectors x one chunk of K read; the chunk's stages written (the four
-      // vector parts of a chunk write disjoint slices: recorded once)
+      // 16 vectors x one chunk of K read; the chunk's exponents and stages written (the
+      // four vector parts of a chunk write disjoint slices: recorded once)
       const int v0 = 16 * (q & 3), nv = std::min(16, tk.m - v0), k0 = kPlaneChunk * (q >> 2);
       const int kc = std::min(kPlaneChunk, tk.zrows - tk.gcol - k0);
       const bool kcont = tk.flags & TF_KCONT;
       if (nv > 0 && (kcont ? !rect(tk.cin, tk.ldc, k0, kc, v0, nv, id, false) : !rect(tk.cin, tk.ldc, v0, nv, k0, kc, id, false)))
         return false;
       if (q & 3) return true;
-      const int64_t st = 128 * plane_count(tk.prec);
-      return planes(tk.out, plane_head(tk.prec, tk.zrows) + st * ((tk.gcol + k0) / kPlaneK), st * plane_stages(kc), id, true);
+      const int64_t st = 128 * plane_count(tk.prec), head = plane_head(tk.prec, tk.zrows);
+      const int64_t exps = head / plane_chunks(tk.zrows), chunk = (tk.gcol + k0) / kPlaneChunk;  // this chunk's exponents
+      return (exps == 0 || planes(tk.out, exps * chunk, exps, id, true)) &&
+             planes(tk.out, head + st * ((tk.gcol + k0) / kPlaneK), st * plane_stages(kc), id, true);
     }
     const Sub x = part_sub(tk.pmode, tk.m, tk.n, q);
     if (x.rm <= 0 || x.cn <= 0) return true;
     if (tk.flags & TF_PLANES) {
       for (int g = tk.seg0; g < tk.seg0 + tk.nseg; ++g) {
         const Seg& sg = p_.segs[g];
-        const int64_t hd = plane_head(tk.prec, sg.k), len = plane_group(tk.prec, sg.k) - hd;
-        if (!planes(sg.a, hd, len, id, false) || !planes(sg.b, hd, len, id, false)) return false;
+        const int64_t len = plane_group(tk.prec, sg.k);  // exponents and stages
+        if (!planes(sg.a, 0, len, id, false) || !planes(sg.b, 0, len, id, false)) return false;
       }
     }
     for (int g = tk.flags & TF_PLANES ? tk.seg0 + tk.nseg : tk.seg0; g < tk.seg0 + tk.nseg; ++g) {

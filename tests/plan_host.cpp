@@ -1,6 +1,8 @@
 // Planner internals for host tests, built together with csrc/plan.cpp.
 #include "plan.h"
 
+#include <string.h>
+
 using namespace stiles;
 
 static Shape shape(int nt, int b, int w, int a, int prec) {
@@ -55,4 +57,30 @@ extern "C" int plane_faults(int nt, int b, int w, int a, int prec, int which) {
   for (const Task& t : p.tasks)
     for (int q = 0; q < t.parts; ++q) found += part_fault(t, q, p.segs.data(), all) != nullptr;
   return found;
+}
+
+// Two splits without an order between them. apart: of their groups (units of 16 bytes;
+// the first at `apart`, the second at 0, 64 vectors x 16 of K each). Returns the race
+// check's verdict.
+extern "C" int two_splits(int prec, int apart) {
+  Plan p;
+  const int64_t group = plane_group(prec, kPlaneK);
+  p.plane_units = group + apart;
+  for (int k = 0; k < 2; ++k) {
+    Task t;
+    memset(&t, 0, sizeof(t));
+    t.op = OP_SPLIT;
+    t.out = mkref(BUF_P, k == 0 ? apart : 0);
+    t.cin = mkref(BUF_S, 0);
+    t.aux = -1;
+    t.ldc = t.m = FB;
+    t.n = 1;
+    t.zrows = kPlaneK;
+    t.parts = 4;
+    t.pmode = PM_SPLIT;
+    t.prec = (uint8_t)prec;
+    p.tasks.push_back(t);
+  }
+  p.succ_off.assign(3, 0);
+  return race_check_plan(p, FB * kPlaneK, 0);
 }
