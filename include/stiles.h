@@ -440,9 +440,11 @@ int stiles_batch_stats(stiles_batch_t h, long long stats[9]);
  * L, Sigma and scratch (3 x stiles_layout_doubles of its shape, rounded up to
  * 32 doubles; stiles_server_request_bytes), task-table arenas for
  * max(4, max_requests) copies of the largest shape, for the reduced precisions
- * room for split operands beside the arena (per request slot; at most a quarter of
- * data_bytes, none when it cannot be had), ready rings and a pinned, host-mapped
- * control block. stiles_server_submit returns STILES_ERR_BUSY if
+ * room for split operands beside the arena (max_requests times the largest need of a
+ * shape; where that is more than a quarter of data_bytes, or cannot be had, every
+ * shape goes without: its results are then the same up to rounding only, and slower),
+ * ready rings and a pinned, host-mapped control block.
+ * stiles_server_submit returns STILES_ERR_BUSY if
  * the request does not fit now (admission by HBM footprint): retry after a
  * stiles_server_release.
  *

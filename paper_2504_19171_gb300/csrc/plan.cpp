@@ -1090,8 +1090,10 @@ static double task_estimate(const Shape& s) {
 // 7446, 112 (1/20) 11897 -> 11274, 96 (1/64) 11389 -> 10517, 80 (2/33) 14692 ->
 // 12465, 64 (4/64) 11161 -> 10229, 128 (4/64) 20963 -> 15753; FP32-class products
 // gain from 48 (1/20) on: 5760 -> 5631. So the line lies at an inner length
-// (w b + arrow) of 112, between 80 and 132. (A rule on the shape alone, so that a
-// matrix gets the same arithmetic in every form of call.)
+// (w b + arrow) of 112, between 80 and 132. (A rule on the shape alone: a matrix
+// gets the same arithmetic alone, in a batch and in a server, unless the memory
+// that the call has leaves no room for the planes: planes_fit, the allocation-free
+// call's array, a server's quarter of its arena.)
 bool use_planes(const Shape& s) {
   return s.prec != PREC_FP64 && s.b >= kPlanesMinB && (int64_t)s.w * s.b + s.a >= kPlanesMinK;
 }
