@@ -3,7 +3,7 @@
 
 The planner cuts the work into tasks in several legal ways (tuning code bit
 fields, see include/stiles.h): how many source block columns one factor
-update task applies, and into how many CTA parts phase-2 and factor update
+update task applies, and into how many CTA parts FP64 phase-2 and factor update
 blocks are split. Which cut is fastest depends on the tile order b, the
 bandwidth w, the number of arrow block rows, the precision -- and on the
 regime the matrix runs in:
@@ -33,6 +33,8 @@ from . import workloads as W
 
 # chunk of old update terms (bits 0-1) x phase-2 split (bits 2-3) x newest-update split (bits 4-5)
 CANDIDATES = (0, 1, 2, 4, 8, 16, 4 + 16, 2 + 8 + 16)
+# bits 2-3 cut FP64 phase-2 blocks only: the reduced precisions always run 64 x 32 parts
+P2_SPLIT_BITS = 0b1100
 GRID_PER_SM = (2, 1)  # persistent CTAs per SM tried in the single regime
 FB = 64
 # A short probe stands in for a long matrix only roughly: in the single
@@ -52,6 +54,11 @@ def default_cache_path() -> str:
 def key_of(b: int, w: int, a: int, precision: int, regime: str = "batch") -> str:
     base = f"{b}:{w}:{(a + FB - 1) // FB}:{precision}"
     return base if regime == "batch" else f"{base}:{regime}"
+
+
+def same_plan_as(code: int, precision: int) -> int:
+    """The lowest code with the plan of `code` in a precision."""
+    return code if precision == S.STILES_FP64 else code & ~P2_SPLIT_BITS
 
 
 class Autotuner:
@@ -102,7 +109,8 @@ class Autotuner:
         return self.cache.get(key_of(b, w, a, precision, regime))
 
     def tune(self, b: int, w: int, a: int, precision: int) -> Tuple[int, Dict[int, float]]:
-        """Time every candidate code on the probe batch; returns (best code,
+        """Time every candidate plan on the probe batch (a code whose plan is
+        another's in this precision once, under same_plan_as); returns (best code,
         {code: seconds per launch})."""
         import torch
 
@@ -110,7 +118,7 @@ class Autotuner:
         shapes = [(nt, b, w, a)] * self.copies
         A = None
         times: Dict[int, float] = {}
-        for code in self.candidates:
+        for code in dict.fromkeys(same_plan_as(c, precision) for c in self.candidates):
             bt = S.StilesBatch(shapes, device=self.device, precision=precision, tuning=[code] * self.copies)
             try:
                 if A is None:
@@ -147,7 +155,7 @@ class Autotuner:
         return best
 
     def tune_single(self, b: int, w: int, a: int, precision: int) -> Tuple[Tuple[int, int], Dict]:
-        """Time every (code, CTAs per SM) on one matrix of nt_single tile
+        """Time every (plan code as in tune, CTAs per SM) on one matrix of nt_single tile
         columns launched alone; returns ((code, grid per SM), {(code, grid):
         seconds per launch})."""
         import torch
@@ -156,7 +164,7 @@ class Autotuner:
         M = None
         A = None
         times: Dict[Tuple[int, int], float] = {}
-        for code in self.candidates:
+        for code in dict.fromkeys(same_plan_as(c, precision) for c in self.candidates):
             st = S.Stiles(nt, b, w, a, device=self.device, precision=precision, tuning=code)
             try:
                 if A is None:
