@@ -60,7 +60,6 @@ enum PartMode : uint8_t {
   PM_QUAD4 = 2,  // the four 32 x 32 quadrants
   PM_TRI3 = 3,   // quadrants (0,0), (1,0), (1,1): a diagonal block's lower part
   PM_ROWS4 = 4,  // rows [0,16), [16,32), ..
-  PM_TILE32 = 5, // a grid of at most 2 x 2 sub-tiles of at most 32 x 32 (parts = row tiles x column tiles)
   PM_ROWS8 = 6,  // rows [0,8), [8,16), ..
   PM_ROWS4F = 11, // rows [0,4), [4,8), ..
   PM_GRID16 = 7, // a grid of at most 4 x 4 sub-tiles of at most 16 x 16 (parts = row tiles x column tiles)
@@ -72,7 +71,7 @@ enum PartMode : uint8_t {
 // Arithmetic of a task's block products (its epilogue is always FP64).
 enum Precision : uint8_t {
   PREC_FP64 = 0,   // FP64 FMA pipe
-  PREC_EMU64 = 1,  // split-precision emulated FP64: 8 fixed-point digits of 8 bits per operand (bf16
+  PREC_EMU64 = 1,  // split-precision emulated FP64: 8 fixed-point digits of 8 bits per operand (fp16
                    // planes) against per-row / per-column exponents, products on the tensor cores
   PREC_FP32X = 2,  // FP32-class: each operand's FP32 value as three bf16 pieces, products on the
                    // tensor cores with FP32 sums
@@ -101,7 +100,7 @@ enum TaskFlag : uint8_t {
 // left-hand: plane order of the MMA's row stacks, 64 vectors each; right-hand:
 // two halves of 32 vectors, planes in order.
 // Offsets in BUF_P count units of 16 bytes.
-constexpr int kPlaneChunk = 512;  // K per exponent (the most that cells sum exactly)
+constexpr int kPlaneChunk = 512;  // K per exponent (two stretches of the 256 that cells sum exactly)
 constexpr int kPlaneK = 16;       // K per stage
 STILES_HD inline int plane_count(int prec) { return prec == PREC_EMU64 ? 8 : 3; }
 STILES_HD inline int64_t plane_stages(int k) { return (k + kPlaneK - 1) / kPlaneK; }
@@ -132,13 +131,6 @@ STILES_HD inline Sub part_sub(int pmode, int m, int n, int q) {
     case PM_COLS2: s.c0 = 32 * q; s.cn = 32; break;
     case PM_QUAD4: dim = 32; s.r0 = 32 * (q & 1); s.c0 = 32 * (q >> 1); break;
     case PM_TRI3: dim = 32; s.r0 = q == 0 ? 0 : 32; s.c0 = q == 2 ? 32 : 0; break;
-    case PM_TILE32: {
-      const int pr = m > 32 ? 2 : 1;
-      dim = 32;
-      s.r0 = 32 * (q % pr);
-      s.c0 = 32 * (q / pr);
-      break;
-    }
     case PM_GRID16: {
       const int pr = (m + 15) / 16;
       dim = 16;
@@ -237,6 +229,7 @@ STILES_HD inline const char* part_fault(const Task& t, int q, const Seg* segs, c
   if (t.prec != PREC_FP64 && (t.pmode != PM_COLS2 || s.cn > 32)) return "reduced-precision part other than 64 x 32";
   if (t.prec != PREC_FP64 && t.op != OP_UPD && t.op != OP_NEG && t.op != OP_STORE && t.op != OP_SYMUPD)
     return "reduced precision on a triangular task";
+  if (t.prec != PREC_FP64 && (t.flags & TF_NEG)) return "negated reduced-precision store";
   if (s.rm <= 0 || s.cn <= 0) return nullptr;
   const int r0 = s.r0, c0 = s.c0, r1 = r0 + s.rm - 1, c1 = c0 + s.cn - 1;
   for (int g = t.seg0; g < t.seg0 + t.nseg; ++g) {

@@ -1501,15 +1501,13 @@ __device__ __forceinline__ void trsm_rows(double* X, const double* Tn, int m, in
   }
 }
 
-// X (m x n) <- T^{-1} X, T lower m x m, rcp[j*LDS] = 1 / T[j][j]. Columns are
-// independent; warp w owns columns 4q + w (interleaved, so that the
-// triangular work of an inverse is balanced). `lower` skips the columns c > j
-// that stay zero when X starts as the identity.
-__device__ __forceinline__ void trsm_cols_ln(double* X, const double* T, const double* rcp, int m, int n, bool lower) {
+// X (m x m) <- T^{-1} X for X the identity, T lower m x m, rcp[j*LDS] = 1 / T[j][j].
+// Columns are independent; warp w owns columns 4q + w (interleaved, so that the
+// triangular work is balanced), and the columns c > j, still zero in row j, are skipped.
+__device__ __forceinline__ void invert_cols(double* X, const double* T, const double* rcp, int m) {
   const int lane = threadIdx.x & 31, c = 4 * (lane & 15) + (threadIdx.x >> 5), half = lane >> 4;
-  const bool own = c < n;
   for (int j = 0; j < m; ++j) {
-    const bool act = own && (!lower || c <= j);
+    const bool act = c <= j;
     if (act && half == 0) X[j * LDS + c] *= rcp[j * LDS];
     __syncwarp();
     if (act) {
@@ -1677,7 +1675,7 @@ __device__ void run_sub(const KParams& p, const Task& tk, const Sub& sb, double*
             double* rcp = T + FB;
             if (tid < m) rcp[tid * LDS] = 1.0 / T[tid * LDS + tid];
             __syncthreads();
-            trsm_cols_ln(X, T, rcp, m, m, true);
+            invert_cols(X, T, rcp, m);
             __syncthreads();
             store_sub(p, tk, sb, X, true);
             break;
@@ -1747,8 +1745,7 @@ __device__ void run_task(const KParams& p, const Task& tk, int t, int q, double*
     case PM_TRI16:
     case PM_GRID16: run_sub<1, 2>(p, tk, sb, smem); break;
     case PM_QUAD4:
-    case PM_TRI3:
-    case PM_TILE32: run_sub<2, 4>(p, tk, sb, smem); break;
+    case PM_TRI3: run_sub<2, 4>(p, tk, sb, smem); break;
     default: run_sub<4, 8>(p, tk, sb, smem); break;
   }
 }
@@ -1856,7 +1853,9 @@ __global__ void __launch_bounds__(NTHREADS, 2) persistent_kernel(const __grid_co
       }
     }
   }
-  if constexpr (TC) {  // every part waited for its MMAs before it returned
+  // every part waited for its MMAs before it returned; after a timeout those of the
+  // part that raised it have had a whole wait budget
+  if constexpr (TC) {
     tc::fence_before_sync();
     __syncthreads();
     if (threadIdx.x < 32) {

@@ -37,7 +37,8 @@ extern "C" unsigned stages_run(unsigned before, unsigned used) { return stage_co
 // Plants one fault in the fused plan's tasks that work on planes, and counts the
 // parts in which the part check (that of the self-checking device build) finds it.
 // which: 0 none, 1 a split's planes past the end, 2 a split's source past the end, 3 a
-// product's planes past the end, 4 a product's output, 5 its input block, 6 its mirror.
+// product's planes past the end, 4 a product's output, 5 its input block, 6 its mirror, 7 TF_NEG on a reduced-precision
+// store (whose epilogue does not negate).
 extern "C" int plane_faults(int nt, int b, int w, int a, int prec, int which) {
   const Shape s = shape(nt, b, w, a, prec);
   Plan p;
@@ -52,6 +53,7 @@ extern "C" int plane_faults(int nt, int b, int w, int a, int prec, int which) {
     if (which == 4 && product) t.out = mkref(BUF_S, n - 1);
     if (which == 5 && product && t.op == OP_SYMUPD) t.cin = mkref(BUF_S, n - 1);
     if (which == 6 && product && t.op == OP_SYMUPD && !(t.flags & TF_SYM_DIAG)) t.aux = mkref(BUF_S, n - 1);
+    if (which == 7 && t.op == OP_STORE && t.prec != PREC_FP64) t.flags |= TF_NEG;
   }
   int found = 0;
   for (const Task& t : p.tasks)

@@ -11,5 +11,5 @@ from tests.host_build import plan_host
 def test_planted_faults_are_found(shape, prec):
     find = plan_host().plane_faults
     assert find(*shape, prec, 0) == 0
-    for which in range(1, 7):
+    for which in range(1, 8):
         assert find(*shape, prec, which) > 0, which
