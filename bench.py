@@ -51,11 +51,11 @@ VARIANT_PRODUCTS = {"emu64": {"pipe": "bf16 tensor (tcgen05)", "digits": 8, "pro
                     "fp32x": {"pipe": "bf16 tensor (tcgen05)", "digits": 3, "products": 8}}
 
 # DRAM traffic of the persistent kernel per launch, from ncu captures of the
-# nt = 8 and nt = 16 cases of the same matrix family (0.791 GB and 2.086 GB):
+# nt = 8 and nt = 16 cases of the same matrix family (0.592 GB and 1.344 GB):
 # the nt = 8 figure plus 192 more tile columns at the marginal 8 -> 16 rate.
 # Valid only for the kernel source it was measured on (sha256 prefix of
-# stiles_kernel.cu + plan.cpp); otherwise reported as null.
-TRAFFIC = {"sources_sha": "372d1de158642877", "bytes_per_launch": 31.87e9}
+# stiles_kernel.cu, block_potrf.cuh, plan.h, plan.cpp); otherwise reported as null.
+TRAFFIC = {"sources_sha": "d5159135d748fbad", "bytes_per_launch": 18.65e9}
 
 
 def measured_peaks() -> dict:
@@ -122,7 +122,7 @@ def kernel_sources_sha() -> str:
     """sha256 prefix of the kernel and planner code, comments and blank lines
     left out (they do not change what runs)."""
     h = hashlib.sha256()
-    for f in ("stiles_kernel.cu", "plan.cpp"):
+    for f in ("stiles_kernel.cu", "block_potrf.cuh", "plan.h", "plan.cpp"):
         with open(os.path.join(ROOT, "paper_2504_19171_gb300", "csrc", f)) as fh:
             for line in fh:
                 code = line.split("//", 1)[0].rstrip()

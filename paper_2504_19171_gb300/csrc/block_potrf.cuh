@@ -34,9 +34,15 @@ constexpr int NTHREADS = 128;  // 4 warps: one per SM sub-partition
 //     apply the rest (batches of 32 2 x 2 elements of the packed lower triangle,
 //     shared out by their FP64 time; single elements claimed from a counter,
 //     their rows found by a division, took three times as long).
-// A block POTRF task takes 42 us (51 with a column and a barrier per step); a panel
-// about 2.8k cycles, the early ones bound by the trailing update. Factor and logdet
-// of (60, 250, 2, 50): 36.6 ms before, 17.2 ms with the other links of the chain.
+// A block POTRF task takes 47 us in the median (43 to 52, the 10th and 90th percentiles)
+// on a GPU that runs a factorization alone, (60, 256, 2, 50), 66 us beside the parts of
+// n = 24,640 in emulated FP64 (stamped: 94k cycles): 5k until the block is in shared
+// memory, 3k the first panel, 5.7k for each of the first eight of the fifteen steps and
+// 2.9k for each of the last seven (the first have trailing updates of up to 13 batches, a
+// panel alone is about 2.8k), 1.4k the scales, 7.4k the stores, 8k until the successors
+// are released, 3k for the logdet after that. Factor and logdet of (60, 250, 2, 50):
+// 36.6 ms with a column and a barrier per step and the other links of the chain as they
+// were, 17.3 ms now.
 
 constexpr int PNB = 4;           // panel width
 constexpr int PROWS = 32 - PNB;  // rows below the panel's own per warp

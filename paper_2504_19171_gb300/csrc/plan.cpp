@@ -1135,7 +1135,11 @@ int build_serve_template(const Shape& s, int workers, Plan* out) {
   out->plane_units = 0;
   Builder B(s, PLAN_FUSED, out);
   B.serve = true;
-  B.crowd = 2;  // requests run side by side
+  // Requests run side by side; how many is not known here. Cut for one / two / four (ms
+  // per pass): 9 FP64 requests of (40,128,1,20), (24,256,1,64), (30,200,2,33) 41.7 / 51.2 /
+  // 57.6; 4 of (30,200,1,64) 22.6 / 31.7 / 35.2; but a full server, 10 of (60,300,2,128)
+  // 455 / 428 / 438, and 6 of (120,512,2,64) in emulated FP64 534 / 507 / 535.
+  B.crowd = 2;
   B.build_factor();
   B.build_selinv();
   B.flops = tile_flops(s, PLAN_FUSED);

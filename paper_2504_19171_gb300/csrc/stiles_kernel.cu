@@ -1037,14 +1037,18 @@ __device__ __forceinline__ void store_part(const KParams& p, const Task& tk, int
 // epilogue. Thread (warp, lane) owns row 32 (warp & 1) + lane, columns
 // 16 (warp >> 1) + 0..15 of it. Thread 32 copies, thread 0 multiplies: one
 // thread doing both waits for the MMAs of the stage before in between. What bounds
-// it: the stages' way out of L2 (24 KB per 1055 cycles and SM, 7.1 TB/s in all). A
-// part of inner length 1088 takes 63 us in emulated FP64, 26 in the FP32-class mode;
-// 146 and 64 us for half the outputs when each part split its operands itself.
+// it, stamped at an inner length of 1088 in a loaded launch: in emulated FP64 the
+// drains, 59k of 120k cycles (11.7k per 256 of K), then the MMAs, whose pipe the SM's
+// two CTAs share, with 7.5k cycles of waiting for copies; in the FP32-class mode the
+// MMAs, 31k of 45k cycles, with 9.6k of waiting and one drain of 4.5k. (L2 is at 19 %
+// of its rate over the selected inversion of (10, 1024, 4, 64).) Such a part takes 65
+// us in emulated FP64, 26 in the FP32-class mode; 146 and 64 us for half the outputs
+// when each part split its operands itself.
 template <int S>
 __device__ __noinline__ void run_planes(const KParams& p, const Task& tk, int q, double* smem, TcShared& ts) {
   using F = PlaneFmt<S>;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int side = warp >> 1, row = 32 * (warp & 1) + lane;
+  const int row = 32 * (warp & 1) + lane;
   uint8_t* stage = reinterpret_cast<uint8_t*>(smem);
   const uint32_t stage_a = tc::smem_addr(stage);
   double r16[16];
@@ -1240,7 +1244,6 @@ __device__ __noinline__ void run_tc(const KParams& p, const Task& tk, int q, dou
   using F = PlaneFmt<S>;
   static_assert(4 * F::STAGE <= PL_STAGE_BYTES, "64 of K in the staging region");
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int side = warp >> 1;
   uint8_t* stage = reinterpret_cast<uint8_t*>(smem);
   const uint32_t stage_a = tc::smem_addr(stage);
   // column exponents, partial exponents [4 warps][64 rows, then 32 columns]
