@@ -195,9 +195,15 @@ struct Builder {
     else if (mode == 1) split(t, PM_ROWS2);
   }
 
-  // Mark a bulk product task with the plan's reduced precision: parts of 64 x 32.
+  // Mark a bulk product task with the plan's reduced precision: parts of 64 x 32. Tiles
+  // of at most 32 leave at least half of a part empty and run in an instance of it that
+  // skips that: the selected inversion of (300, 2, 2, 1) 16.3 -> 9.6, (64, 5, 3, 3) 4.4
+  // -> 3.3, (500, 16, 2, 8) 28.9 -> 24.9 ms in emulated FP64. Chosen for a whole matrix:
+  // with every part that is not full in it, the two instances took turns in the
+  // instruction cache (8 uneven matrices 73.7 -> 75.4 ms, (400, 40, 1, 10) 19.2 -> 20.9).
   void lower_precision(Task& t) const {
     if (s.prec == PREC_FP64) return;
+    if (s.b <= 32) t.flags |= TF_SMALL;
     t.prec = (uint8_t)s.prec;
     t.pmode = PM_COLS2;
     t.parts = t.n > 32 ? 2 : 1;

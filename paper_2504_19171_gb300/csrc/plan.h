@@ -86,6 +86,7 @@ enum TaskFlag : uint8_t {
   TF_KCONT = 16,    // OP_SPLIT: K is the contiguous dimension of the source tile
   TF_BSIDE = 32,    // OP_SPLIT: planes of a right-hand operand
   TF_NEG = 64,      // OP_STORE: out = -acc
+  TF_SMALL = 128,   // reduced-precision product of a matrix of small tiles (padding left out)
 };
 
 // Planes. The reduced-precision products of phase 2 read their operands as 16-bit

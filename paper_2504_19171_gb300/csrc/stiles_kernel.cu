@@ -735,15 +735,13 @@ __device__ __forceinline__ void digit_pairs(double v0, double v1, int emax, uint
 // 23 fraction bits are taken. Below the FP32 normal range it is zero, above
 // it infinity; an infinity or NaN in gives NaN.
 __device__ __forceinline__ uint32_t fp32_bits_of(double v) {
-  const unsigned long long b0 = (unsigned long long)__double_as_longlong(v);
-  if (((b0 >> 52) & 0x7ff) == 0x7ff) return 0x7fc00000u;
-  const unsigned long long b = b0 + (1ull << 28);
-  const uint32_t hi = (uint32_t)(b >> 32), lo = (uint32_t)b;
+  const unsigned long long b0 = (unsigned long long)__double_as_longlong(v), b = b0 + (1ull << 28);
+  const uint32_t hi = (uint32_t)(b >> 32), lo = (uint32_t)b, sgn = hi & 0x80000000u;
   const int e = (int)((hi >> 20) & 0x7ff);
-  const uint32_t sgn = hi & 0x80000000u;
-  if (e < 1023 - 126) return sgn;
-  if (e > 1023 + 127) return sgn | 0x7f800000u;
-  return sgn | ((uint32_t)(e - 1023 + 127) << 23) | ((hi & 0xfffffu) << 3) | (lo >> 29);
+  // exponent and the top 23 fraction bits, rebiased
+  uint32_t r = __funnelshift_l(lo, hi & 0x7fffffffu, 3) - ((1023u - 127u) << 23);
+  r = e < 1023 - 126 ? 0u : e > 1023 + 127 ? 0x7f800000u : r;
+  return ((b0 >> 52) & 0x7ff) == 0x7ff ? 0x7fc00000u : sgn | r;
 }
 
 // The FP32 values of a pair of K-adjacent operands (v0 at k, v1 at k + 1) as
@@ -756,7 +754,7 @@ __device__ __forceinline__ void piece_pairs(double v0, double v1, uint32_t (&w)[
 #pragma unroll
   for (int t = 0; t < 3; ++t) {
     const uint32_t p0 = __float_as_uint(r0) & 0xffff0000u, p1 = __float_as_uint(r1) & 0xffff0000u;
-    w[t] = (p0 >> 16) | p1;
+    w[t] = __byte_perm(p0, p1, 0x7632);
     r0 -= __uint_as_float(p0);
     r1 -= __uint_as_float(p1);
   }
@@ -854,6 +852,9 @@ __device__ __forceinline__ void add_cell(long long& acc, uint32_t cell, int sh) 
 // Read the cells and add the part's sums of this stretch of K to r16. er: the
 // biased exponent of the thread's row, cexp: of the 32 columns (shared memory;
 // emulated FP64). SMALL: at most 64 of K in the cells.
+// rows, cols: the part's. Unless WHOLE, a group of columns or a warp's 32 rows beyond
+// them is left out: with all of them drained, parts of small tiles took 4 to 7k cycles
+// more; the tests for it in every part cost (28, 1024, 4, 64) in emulated FP64 2 %.
 // Each warp reads the cells of all 32 columns in its lane block (warps 0, 1: the
 // low levels / planes 0 and 2; warps 2, 3: the high levels / plane 1), 4 columns
 // of the other side's, handed over through shared memory, and 4 of its own at a
@@ -861,105 +862,120 @@ __device__ __forceinline__ void add_cell(long long& acc, uint32_t cell, int sh) 
 // four steps): straight-line code of this size ran at the instruction cache's
 // rate, 13k cycles a drain (n = 122,944 in emulated FP64: 345 against 321 ms, with
 // the splits of run_tc, which had the same fault).
-template <int S, bool SMALL>
-__device__ __forceinline__ void drain_cells(uint32_t tmem, uint8_t* xch, int er, const int* cexp, double (&r16)[16]) {
+template <int S, bool SMALL, bool WHOLE>
+__device__ __forceinline__ void drain_cells(uint32_t tmem, uint8_t* xch, int er, const int* cexp, int rows, int cols,
+                                            double (&r16)[16]) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int side = warp >> 1, row = 32 * (warp & 1) + lane;
   const uint32_t trow = tmem + ((uint32_t)(32 * warp) << 16);
 #pragma unroll 1
   for (int i = 0; i < 4; ++i) {
-    uint8_t* buf = xch + (i & 1) * (PL_XCH_BYTES / 2);  // free since the barrier of the step before
-    if constexpr (S == 8) {
-      constexpr int kScale = 2044 + 2 * 62 - 8 * 7;
-      long long* xhl = reinterpret_cast<long long*>(buf);  // [4 c][64 r] x (hi, lo) for side 1
-      long long* xlo = xhl + 2 * 4 * 64;                    // [4 c][64 r] lo for side 0
-      // level sums of 4 columns from col: hi (levels 0-3), lo (levels 4-7)
-      auto sums = [&](int col, long long (&hi)[4], long long (&lo)[4]) {
+    if (WHOLE || 4 * i < cols) {
+      uint8_t* buf = xch + (i & 1) * (PL_XCH_BYTES / 2);  // free since the barrier of the step before
+      // this warp's columns and the other side's that lie in the part (warp-uniform)
+      const bool live = 32 * (warp & 1) < rows;
+      const bool own = WHOLE || (live && 16 * side + 4 * i < cols);
+      const bool other = WHOLE || (live && 16 * (1 - side) + 4 * i < cols);
+      if constexpr (S == 8) {
+        constexpr int kScale = 2044 + 2 * 62 - 8 * 7;
+        long long* xhl = reinterpret_cast<long long*>(buf);  // [4 c][64 r] x (hi, lo) for side 1
+        long long* xlo = xhl + 2 * 4 * 64;                    // [4 c][64 r] lo for side 0
+        // level sums of 4 columns from col: hi (levels 0-3), lo (levels 4-7)
+        auto sums = [&](int col, long long (&hi)[4], long long (&lo)[4]) {
 #pragma unroll
-        for (int x = 0; x < 4; ++x) hi[x] = lo[x] = SMALL ? -kCellBias : 0;
-        if (side == 0) {
+          for (int x = 0; x < 4; ++x) hi[x] = lo[x] = SMALL ? -kCellBias : 0;
+          if (side == 0) {
+            uint32_t cell[8][4];
+            tc::ld_cells(trow + col, cell);
+#pragma unroll
+            for (int c = 0; c < 8; ++c)
+#pragma unroll
+              for (int x = 0; x < 4; ++x) {
+                if (c <= 3) add_cell<SMALL>(hi[x], cell[c][x], 8 * (3 - c));
+                else add_cell<SMALL>(lo[x], cell[c][x], 8 * (7 - c));
+              }
+          } else {
+            uint32_t cell[4][4];
+            tc::ld_cells(trow + col, cell);
+#pragma unroll
+            for (int c = 0; c < 4; ++c)
+#pragma unroll
+              for (int x = 0; x < 4; ++x) add_cell<SMALL>(lo[x], cell[c][x], 8 * (3 - c));
+          }
+        };
+        long long hi[4], lo[4];
+        if (other) {
+          sums(16 * (1 - side) + 4 * i, hi, lo);
+#pragma unroll
+          for (int x = 0; x < 4; ++x) {
+            const int e = x * 64 + row;
+            if (side == 0) {
+              xhl[2 * e] = hi[x];
+              xhl[2 * e + 1] = lo[x];
+            } else {
+              xlo[e] = lo[x];
+            }
+          }
+        }
+        __syncthreads();
+        if (own) {
+          sums(16 * side + 4 * i, hi, lo);
+          bool slow = false;
+          double v[4];
+          int k2[4];
+#pragma unroll
+          for (int x = 0; x < 4; ++x) {
+            const int e = x * 64 + row, ec = cexp[16 * side + 4 * i + x];
+            hi[x] = side == 0 ? hi[x] : xhl[2 * e];
+            lo[x] += side == 0 ? xlo[e] : xhl[2 * e + 1];
+            k2[x] = max(er, 1) + max(ec, 1) - kScale;
+            v[x] = scaled_sum(hi[x], lo[x], k2[x], slow);
+            if (er == 0x7ff || ec == 0x7ff) v[x] = __longlong_as_double(0x7ff8000000000000ll);
+          }
+          if (slow) {
+#pragma unroll
+            for (int x = 0; x < 4; ++x)
+              if (v[x] == v[x]) v[x] = scaled_sum_any(hi[x], lo[x], k2[x]);
+          }
+#pragma unroll
+          for (int x = 0; x < 4; ++x) r16[x] += v[x];
+        }
+      } else {
+        float* x0 = reinterpret_cast<float*>(buf);  // [4 c][64 r] plane 0, then plane 2, for side 1
+        float* x1 = x0 + 2 * 4 * 64;                // [4 c][64 r] plane 1, for side 0
+        auto pieces = [&](int col, float (&v)[4], float (&v2)[4]) {  // lane block's sums of 4 columns
           uint32_t cell[8][4];
           tc::ld_cells(trow + col, cell);
 #pragma unroll
-          for (int c = 0; c < 8; ++c)
+          for (int x = 0; x < 4; ++x) {
+            v[x] = ((0.0f + __uint_as_float(cell[0][x])) + __uint_as_float(cell[1][x])) + __uint_as_float(cell[2][x]);
+            v2[x] = (0.0f + __uint_as_float(cell[3][x])) + __uint_as_float(cell[4][x]);
+          }
+        };
+        float v[4], v2[4];
+        if (other) {
+          pieces(16 * (1 - side) + 4 * i, v, v2);
 #pragma unroll
-            for (int x = 0; x < 4; ++x) {
-              if (c <= 3) add_cell<SMALL>(hi[x], cell[c][x], 8 * (3 - c));
-              else add_cell<SMALL>(lo[x], cell[c][x], 8 * (7 - c));
+          for (int x = 0; x < 4; ++x) {
+            const int e = x * 64 + row;
+            if (side == 0) {
+              x0[e] = v[x];
+              x0[4 * 64 + e] = v2[x];
+            } else {
+              x1[e] = v[x];
             }
-        } else {
-          uint32_t cell[4][4];
-          tc::ld_cells(trow + col, cell);
-#pragma unroll
-          for (int c = 0; c < 4; ++c)
-#pragma unroll
-            for (int x = 0; x < 4; ++x) add_cell<SMALL>(lo[x], cell[c][x], 8 * (3 - c));
+          }
         }
-      };
-      long long hi[4], lo[4];
-      sums(16 * (1 - side) + 4 * i, hi, lo);
+        __syncthreads();
+        if (own) {
+          pieces(16 * side + 4 * i, v, v2);
 #pragma unroll
-      for (int x = 0; x < 4; ++x) {
-        const int e = x * 64 + row;
-        if (side == 0) {
-          xhl[2 * e] = hi[x];
-          xhl[2 * e + 1] = lo[x];
-        } else {
-          xlo[e] = lo[x];
+          for (int x = 0; x < 4; ++x) {
+            const int e = x * 64 + row;
+            const float p0 = side == 0 ? v[x] : x0[e], p1 = side == 0 ? x1[e] : v[x], p2 = side == 0 ? v2[x] : x0[4 * 64 + e];
+            r16[x] += (double)(((0.0f + p0) + p1) + p2);
+          }
         }
-      }
-      __syncthreads();
-      sums(16 * side + 4 * i, hi, lo);
-      bool slow = false;
-      double v[4];
-      int k2[4];
-#pragma unroll
-      for (int x = 0; x < 4; ++x) {
-        const int e = x * 64 + row, ec = cexp[16 * side + 4 * i + x];
-        hi[x] = side == 0 ? hi[x] : xhl[2 * e];
-        lo[x] += side == 0 ? xlo[e] : xhl[2 * e + 1];
-        k2[x] = max(er, 1) + max(ec, 1) - kScale;
-        v[x] = scaled_sum(hi[x], lo[x], k2[x], slow);
-        if (er == 0x7ff || ec == 0x7ff) v[x] = __longlong_as_double(0x7ff8000000000000ll);
-      }
-      if (slow) {
-#pragma unroll
-        for (int x = 0; x < 4; ++x)
-          if (v[x] == v[x]) v[x] = scaled_sum_any(hi[x], lo[x], k2[x]);
-      }
-#pragma unroll
-      for (int x = 0; x < 4; ++x) r16[x] += v[x];
-    } else {
-      float* x0 = reinterpret_cast<float*>(buf);  // [4 c][64 r] plane 0, then plane 2, for side 1
-      float* x1 = x0 + 2 * 4 * 64;                // [4 c][64 r] plane 1, for side 0
-      auto pieces = [&](int col, float (&v)[4], float (&v2)[4]) {  // lane block's sums of 4 columns
-        uint32_t cell[8][4];
-        tc::ld_cells(trow + col, cell);
-#pragma unroll
-        for (int x = 0; x < 4; ++x) {
-          v[x] = ((0.0f + __uint_as_float(cell[0][x])) + __uint_as_float(cell[1][x])) + __uint_as_float(cell[2][x]);
-          v2[x] = (0.0f + __uint_as_float(cell[3][x])) + __uint_as_float(cell[4][x]);
-        }
-      };
-      float v[4], v2[4];
-      pieces(16 * (1 - side) + 4 * i, v, v2);
-#pragma unroll
-      for (int x = 0; x < 4; ++x) {
-        const int e = x * 64 + row;
-        if (side == 0) {
-          x0[e] = v[x];
-          x0[4 * 64 + e] = v2[x];
-        } else {
-          x1[e] = v[x];
-        }
-      }
-      __syncthreads();
-      pieces(16 * side + 4 * i, v, v2);
-#pragma unroll
-      for (int x = 0; x < 4; ++x) {
-        const int e = x * 64 + row;
-        const float p0 = side == 0 ? v[x] : x0[e], p1 = side == 0 ? x1[e] : v[x], p2 = side == 0 ? v2[x] : x0[4 * 64 + e];
-        r16[x] += (double)(((0.0f + p0) + p1) + p2);
       }
     }
     double t[4];
@@ -1008,12 +1024,14 @@ __device__ __forceinline__ void store_part(const KParams& p, const Task& tk, int
   const int ldm = dblk ? tk.ldo : tk.ldx;
   double* Om = p.smirror ? p.smirror + (O - p.buf[BUF_S]) : nullptr;
   double* Mm = p.smirror ? p.smirror + (M - p.buf[BUF_S]) : nullptr;
-  double v[16];
+  double v[16];  // (every load in flight before the first subtraction)
 #pragma unroll
   for (int x = 0; x < 16; ++x) {
     const bool in = row < m && c0 + x < n && (!dblk || row >= c0 + x);
-    v[x] = in ? __ldcg(C + row + (int64_t)(c0 + x) * tk.ldc) - r16[x] : 0.0;
+    v[x] = in ? __ldcg(C + row + (int64_t)(c0 + x) * tk.ldc) : 0.0;
   }
+#pragma unroll
+  for (int x = 0; x < 16; ++x) v[x] -= r16[x];
   double* X = smem;  // [64 rows][33]: the staging region, every copy of which has been used
 #pragma unroll
   for (int x = 0; x < 16; ++x) {
@@ -1145,7 +1163,7 @@ __device__ __noinline__ void run_planes(const KParams& p, const Task& tk, int q,
       tc::fence_after_sync();
       if (copier)  // every slot is free: the next stages load while the cells are read
         while (ls < tk.nseg && issued < end + F::NST && issue()) {}
-      drain_cells<S, false>(ts.tmem, stage + PL_XCH_OFF, er, cexp, r16);
+      drain_cells<S, false, true>(ts.tmem, stage + PL_XCH_OFF, er, cexp, tk.m, tk.n - 32 * q, r16);
       tc::fence_before_sync();
       __syncthreads();  // TMEM and exchange reads done before the next MMAs
     }
@@ -1182,27 +1200,77 @@ __device__ __forceinline__ void load_octet(const double* P, int64_t step, bool p
 }
 __device__ __forceinline__ bool pairs_ok(const double* P, int ld) { return ((((uintptr_t)P) & 15) | (ld & 1)) == 0; }
 
-// (x[0 .. 3]: op(A), x[4], x[5]: op(B))
-__device__ __forceinline__ void tc_load(const KParams& p, const Task& tk, const Seg& g, int k0, int kc, int q,
-                                        double (&x)[6][8]) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+// A chunk of a part's inner length: at most four stages from segment s, K k0 on. In
+// emulated FP64 of one segment (it has one exponent per vector); in the FP32-class mode
+// whole segments after it too while they fit, as long as the cells may go on summing
+// (kacc of K so far): with a chunk per segment of 16 of K the parts of tiles of 16 took
+// 7k cycles more per segment.
+// x[3 h + 0], x[3 h + 1], x[3 h + 2]: the K octet warp + 4 h of rows lane and lane + 32
+// of op(A) and of column lane of op(B).
+struct TcChunk {
+  int nst, kadd;  // stages; what the chunk adds to kacc
+  int s, k0;      // the next chunk's start
+};
+// octet h: K from k on of segment g, `left` of it to the segment's (or chunk's) end
+__device__ __forceinline__ void tc_octets(const KParams& p, const Task& tk, const Seg& g, int k, int left, int q, int h,
+                                          double (&x)[6][8]) {
+  const int lane = threadIdx.x & 31;
   const bool ta = g.trans & 1, tb = g.trans & 2;
   const int64_t sa = ta ? 1 : g.lda, sb = tb ? g.ldb : 1;
-  const double* A = resolve(p, g.a) + (int64_t)k0 * sa;
-  const double* B = resolve(p, g.b) + (int64_t)k0 * sb + (int64_t)(32 * q) * (tb ? 1 : g.ldb);
+  const double* A = resolve(p, g.a) + (int64_t)k * sa;
+  const double* B = resolve(p, g.b) + (int64_t)k * sb + (int64_t)(32 * q) * (tb ? 1 : g.ldb);
   const bool va = ta && pairs_ok(A, g.lda), vb = !tb && pairs_ok(B, g.ldb);
 #pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    const int v = lane + 32 * (u & 1), k = 8 * (warp + 4 * (u >> 1));
-    const double* P = A + (int64_t)v * (ta ? g.lda : 1) + (int64_t)k * sa;
-    load_octet(P, sa, va, v < tk.m ? kc - k : 0, x[u]);
+  for (int u = 0; u < 2; ++u) {
+    const int v = lane + 32 * u;
+    load_octet(A + (int64_t)v * (ta ? g.lda : 1), sa, va, v < tk.m ? left : 0, x[3 * h + u]);
+  }
+  load_octet(B + (int64_t)lane * (tb ? 1 : g.ldb), sb, vb, 32 * q + lane < tk.n ? left : 0, x[3 * h + 2]);
+}
+template <int S>
+__device__ __forceinline__ TcChunk tc_load(const KParams& p, const Task& tk, int s, int k0, int kacc, int q,
+                                           double (&x)[6][8]) {
+  const int warp = threadIdx.x >> 5;
+  TcChunk c{0, 0, s, k0};
+  Seg cur = load_seg(p, tk.seg0 + s);
+  if constexpr (S == 8) {
+    const int kc = min(64, cur.k - k0);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) tc_octets(p, tk, cur, k0 + 8 * (warp + 4 * h), kc - 8 * (warp + 4 * h), q, h, x);
+    c.nst = (kc + kPlaneK - 1) / kPlaneK;
+    c.k0 += kc;
+    if (c.k0 >= cur.k) {
+      c.k0 = 0;
+      ++c.s;
+    }
+    return c;
+  }
+  Seg g[2] = {cur, cur};  // of this warp's octets, their first K in it and what is left from there
+  int k[2] = {0, 0}, left[2] = {0, 0};
+  for (;;) {
+    const int kc = min(min(16 * (4 - c.nst), cur.k - c.k0), PlaneFmt<S>::KMAX - kacc - c.kadd);
+    const int n = (kc + kPlaneK - 1) / kPlaneK;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int st = (warp >> 1) + 2 * h - c.nst;  // of the octet, from the first of these
+      if (st >= 0 && st < n) {
+        g[h] = cur;
+        k[h] = c.k0 + kPlaneK * st + 8 * (warp & 1);
+        left[h] = kc - kPlaneK * st - 8 * (warp & 1);
+      }
+    }
+    c.nst += n;
+    c.kadd += (kc + 31) / 32 * 32;
+    c.k0 += kc;
+    if (c.k0 < cur.k) break;
+    c.k0 = 0;
+    if (++c.s >= tk.nseg || c.nst >= 4 || kacc + c.kadd + 32 > PlaneFmt<S>::KMAX) break;
+    cur = load_seg(p, tk.seg0 + c.s);
+    if (cur.k > 16 * (4 - c.nst)) break;
   }
 #pragma unroll
-  for (int u = 0; u < 2; ++u) {
-    const int k = 8 * (warp + 4 * u);
-    const double* P = B + (int64_t)lane * (tb ? 1 : g.ldb) + (int64_t)k * sb;
-    load_octet(P, sb, vb, 32 * q + lane < tk.n ? kc - k : 0, x[4 + u]);
-  }
+  for (int h = 0; h < 2; ++h) tc_octets(p, tk, g[h], k[h], left[h], q, h, x);
+  return c;
 }
 
 // The planes of 8 K-adjacent values, 16 bytes each: plane t at dst + (t % 4) s1 + (t / 4) s2.
@@ -1239,7 +1307,7 @@ struct PlaneStep {
 // operand twice as often and scanned the whole K for exponents first: factor +
 // selected inversion of (28, 1024, 4, 64) in emulated FP64 464 ms then, 205 ms
 // with these parts and phase 2 from planes (454 ms with phase 2 in these parts).
-template <int S>
+template <int S, bool WHOLE>
 __device__ __noinline__ void run_tc(const KParams& p, const Task& tk, int q, double* smem, TcShared& ts) {
   using F = PlaneFmt<S>;
   static_assert(4 * F::STAGE <= PL_STAGE_BYTES, "64 of K in the staging region");
@@ -1260,20 +1328,18 @@ __device__ __noinline__ void run_tc(const KParams& p, const Task& tk, int q, dou
   uint32_t ndone = ts.pdone_n;
   int kacc = 0;
   double x[6][8];
-  Seg g = load_seg(p, tk.seg0);
-  int kc = min(64, g.k);
-  tc_load(p, tk, g, 0, kc, q, x);
-  for (int s = 0, k0 = 0; s < tk.nseg;) {
+  TcChunk next = tc_load<S>(p, tk, 0, 0, 0, q, x);
+  for (bool last = false; !last;) {
     int er = 0, ea[2] = {0, 0}, eb = 0;
     if constexpr (S == 8) {
 #pragma unroll
-      for (int u = 0; u < 4; ++u)
+      for (int h = 0; h < 6; h += 3)
 #pragma unroll
-        for (int y = 0; y < 8; ++y) ea[u & 1] = max(ea[u & 1], biased_exp(x[u][y]));
-#pragma unroll
-      for (int u = 4; u < 6; ++u)
-#pragma unroll
-        for (int y = 0; y < 8; ++y) eb = max(eb, biased_exp(x[u][y]));
+        for (int y = 0; y < 8; ++y) {
+          ea[0] = max(ea[0], biased_exp(x[h][y]));
+          ea[1] = max(ea[1], biased_exp(x[h + 1][y]));
+          eb = max(eb, biased_exp(x[h + 2][y]));
+        }
       int* mine = pexp + 96 * warp;
       mine[lane] = ea[0];
       mine[32 + lane] = ea[1];
@@ -1289,15 +1355,18 @@ __device__ __noinline__ void run_tc(const KParams& p, const Task& tk, int q, dou
       er = warp & 1 ? ea[1] : ea[0];
       if (warp == 0) cexp[lane] = eb;
     }
-    // octet o of the chunk: stage o / 2, half o % 2 (a loop over the six octets,
-    // their values rotated through x[0], for the instruction cache)
-    const int nst = (kc + kPlaneK - 1) / kPlaneK;
+    // octet o of the chunk: stage o / 2, half o % 2 (a loop over the six octets, their
+    // values rotated through x[0], for the instruction cache). A part that is not whole
+    // leaves out the second three where K has no more of them, and rows 32-63 where the
+    // block has none: those keep what was there, and their outputs are not read.
+    const int nst = next.nst, nu = !WHOLE && nst <= 2 ? 3 : 6;
 #pragma unroll 1
-    for (int u = 0; u < 6; ++u) {
-      const bool isa = u < 4;
-      const int v = isa ? lane + 32 * (u & 1) : lane, o = warp + 4 * (isa ? u >> 1 : u - 4);
-      if (o < 2 * nst)
-        store_planes<S, false>(x[0], !isa ? eb : u & 1 ? ea[1] : ea[0],
+    for (int u = 0; u < nu; ++u) {
+      const int o = warp + (u < 3 ? 0 : 4), t = u < 3 ? u : u - 3;
+      const bool isa = t < 2;
+      const int v = t == 1 ? lane + 32 : lane;
+      if (o < 2 * nst && (WHOLE || t != 1 || tk.m > 32))
+        store_planes<S, false>(x[0], t == 0 ? ea[0] : t == 1 ? ea[1] : eb,
                                stage + (o >> 1) * F::STAGE + (isa ? 0 : F::A_BYTES) + (o & 1) * 128 + (v >> 3) * 256 + (v & 7) * 16,
                                isa ? PlaneStep<S>::A1 : PlaneStep<S>::B1, isa ? PlaneStep<S>::A2 : PlaneStep<S>::B2);
 #pragma unroll
@@ -1305,15 +1374,9 @@ __device__ __noinline__ void run_tc(const KParams& p, const Task& tk, int q, dou
 #pragma unroll
         for (int y = 0; y < 8; ++y) x[w][y] = x[w + 1][y];
     }
-    // the next stretch of K
     const bool fresh = S == 8 || kacc == 0;
-    kacc += (kc + 31) / 32 * 32;
-    k0 += kc;
-    if (k0 >= g.k) {
-      k0 = 0;
-      if (++s < tk.nseg) g = load_seg(p, tk.seg0 + s);
-    }
-    const bool last = s >= tk.nseg;
+    kacc += next.kadd;
+    last = next.s >= tk.nseg;
     const bool drain = S == 8 || last || kacc + 32 > F::KMAX;
     tc::fence_smem_to_async();
     __syncthreads();
@@ -1324,18 +1387,14 @@ __device__ __noinline__ void run_tc(const KParams& p, const Task& tk, int q, dou
     }
     __syncwarp();
     if (drain) kacc = 0;
-    if (!last) {
-      kc = min(64, g.k - k0);
-      if constexpr (S == 4) kc = min(kc, F::KMAX - kacc);
-      tc_load(p, tk, g, k0, kc, q, x);
-    }
+    if (!last) next = tc_load<S>(p, tk, next.s, next.k0, kacc, q, x);
     bool ok = tc_wait(p, tc::smem_addr(&ts.pdone), ndone & 1);
     ++ndone;
     ok = !__syncthreads_or(!ok);
     if (!ok) return;
     if (!drain) continue;
     tc::fence_after_sync();
-    drain_cells<S, true>(ts.tmem, stage + PL_XCH_OFF, er, cexp, r16);
+    drain_cells<S, true, WHOLE>(ts.tmem, stage + PL_XCH_OFF, er, cexp, tk.m, tk.n - 32 * q, r16);
     tc::fence_before_sync();
     __syncthreads();  // TMEM and exchange reads done before the next MMAs
   }
@@ -1733,8 +1792,9 @@ __device__ void run_task(const KParams& p, const Task& tk, int t, int q, double*
       return;
     }
     if (tk.prec != PREC_FP64) {
-      if (tk.prec == PREC_EMU64) run_tc<8>(p, tk, q, smem, *ts);
-      else run_tc<4>(p, tk, q, smem, *ts);
+      const bool whole = !(tk.flags & TF_SMALL);
+      if (tk.prec == PREC_EMU64) whole ? run_tc<8, true>(p, tk, q, smem, *ts) : run_tc<8, false>(p, tk, q, smem, *ts);
+      else whole ? run_tc<4, true>(p, tk, q, smem, *ts) : run_tc<4, false>(p, tk, q, smem, *ts);
       return;
     }
   }
