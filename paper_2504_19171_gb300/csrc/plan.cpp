@@ -43,25 +43,24 @@ namespace {
 constexpr double kFlopPerNs = 7.6 / kCtasPerSm;
 constexpr double kTaskOverheadNs = 2500.0;
 constexpr int kGpuSms = 152;  // of a GB300
-constexpr int kPlanesMinB = 64, kPlanesMinK = 112;
+constexpr int kPlanesMinB = 32, kPlanesMinK = 112;
 constexpr double kSweepStepNs = 120.0;  // one step of an in-shared-memory triangular sweep
 
 // Units (16 bytes) of a tile column's planes of Sigma and of U, and of the corner's:
 // the tiles that products read. Of Sigma the diagonal tile by rows and the arrow and
 // band tiles by columns, and by rows those that an earlier column reads so (all but
-// the w-th band tile; with w = 0 a column reads only its own and the corner).
+// the w-th band tile). (w >= 1, as use_planes has it.)
 struct PlaneUnits {
   int64_t u, diag, cols, rows, corner, slots;
   explicit PlaneUnits(const Shape& s) {
     const Layout L(s);
     const int R = L.nblk(0), ra = s.a > 0 ? L.nblk(s.nt) : 0;
-    const int64_t gb = plane_group(s.prec, s.b), ga = s.a > 0 ? plane_group(s.prec, s.a) : 0;
-    u = (int64_t)s.w * R * gb + (int64_t)R * ga;
-    diag = s.w > 0 ? R * gb : 0;
-    cols = (int64_t)s.w * R * gb + (int64_t)R * ga;
-    rows = s.w > 0 ? (int64_t)(s.w - 1) * R * gb + (int64_t)ra * gb : 0;
+    const int64_t tile = R * plane_group(s.prec, s.b), ga = s.a > 0 ? plane_group(s.prec, s.a) : 0;
+    u = cols = s.w * tile + (int64_t)R * ga;
+    diag = tile;
+    rows = (s.w - 1) * tile + ra * plane_group(s.prec, s.b);
     corner = (int64_t)ra * ga;
-    slots = s.w > 0 ? s.w + 1 : s.nt < 2 ? s.nt : 2;
+    slots = s.w + 1;
   }
   int64_t sigma() const { return diag + cols + rows; }
   int64_t total() const { return 2 * u + slots * sigma() + corner; }
@@ -714,8 +713,7 @@ struct Builder {
         w.push_back({scol(i, i, g), L.nblk(i) - g});
       } else if (set == PS_COL) w.push_back({scol(k, i, g), L.nblk(k)});
       else w.push_back({srow(k, i, g), L.nblk(i)});
-      // the lowest column that reads what the slot held before
-      const int reader = set == PS_U ? i + 2 : i + (int)pu.slots - s.w;
+      const int reader = set == PS_U ? i + 2 : i + 1;  // the lowest column that reads what the slot held before
       if (i < s.nt && reader < (int)p2join.size() && p2join[reader] >= 0) w.push_back({p2join[reader], 1});
       // at most 4 chunks of K (16 parts) per task
       for (int c0 = 0; c0 < (int)plane_chunks(kk); c0 += 4) {
@@ -739,7 +737,7 @@ struct Builder {
   }
   int split_tasks(int kk) const { return (int)((plane_chunks(kk) + 3) / 4); }  // per vector group
   // Does a column before i need tile (k, i) by rows (S_ki with k > i)?
-  bool need_rows(int k, int i) const { return i > s.sel0 && s.w > 0 && i < s.nt && (k == s.nt || k - i < s.w); }
+  bool need_rows(int k, int i) const { return i > s.sel0 && i < s.nt && (k == s.nt || k - i < s.w); }
   // segment of A = S_jk (group r) and B = U_ki (group c), and what it waits for
   void plane_seg(int j, int k, int r, int i, int c, std::vector<Seg>& segs, std::vector<Wait>& w) {
     int64_t a;
@@ -869,7 +867,7 @@ struct Builder {
       }
     tile_gemms += (long long)st.size();
     if (s.planes) {
-      if (i > s.sel0 && (s.w > 0 || i == s.nt)) split_tile(PS_DIAG, i, i, pl_d, pl_dbase[i]);
+      if (i > s.sel0) split_tile(PS_DIAG, i, i, pl_d, pl_dbase[i]);
       p2join[i] = newctr(true);
       emit(blank(OP_JOIN, 0, 0), {}, {{done[0], nprod}}, {p2join[i]}, 0.0);
     }
@@ -1096,12 +1094,19 @@ static double task_estimate(const Shape& s) {
 // 7446, 112 (1/20) 11897 -> 11274, 96 (1/64) 11389 -> 10517, 80 (2/33) 14692 ->
 // 12465, 64 (4/64) 11161 -> 10229, 128 (4/64) 20963 -> 15753; FP32-class products
 // gain from 48 (1/20) on: 5760 -> 5631. So the line lies at an inner length
-// (w b + arrow) of 112, between 80 and 132. (A rule on the shape alone: a matrix
+// (w b + arrow) of 112, between 80 and 132. Smaller tiles pad the planes' 64 vectors,
+// but reach that length in several segments, which a part that splits its operands
+// takes one after the other; us of the selected inversion in emulated FP64 / the
+// FP32-class mode: 63 (4/64) 8396 -> 6297 / 5681 -> 2949, 48 (4/20, 40 columns) 4351 ->
+// 3856 / 2658 -> 1789, 33 (3/20) 5392 -> 4998 / 3444 -> 2512; 24 (4/64) 5376 -> 5407 /
+// 2753 -> 2597, so from an order of 32 on. Without a band there is no chain and no tile
+// that many products read: (100, 128, 0, 128) 615 -> 2928 / 540 -> 2457, (40, 64, 0, 512)
+// 698 -> 2070, (10, 512, 0, 128) 1489 -> 1613. (A rule on the shape alone: a matrix
 // gets the same arithmetic alone, in a batch and in a server, unless the memory
 // that the call has leaves no room for the planes: planes_fit, the allocation-free
 // call's array, a server's quarter of its arena.)
 bool use_planes(const Shape& s) {
-  return s.prec != PREC_FP64 && s.b >= kPlanesMinB && (int64_t)s.w * s.b + s.a >= kPlanesMinK;
+  return s.prec != PREC_FP64 && s.w >= 1 && s.b >= kPlanesMinB && (int64_t)s.w * s.b + s.a >= kPlanesMinK;
 }
 
 int64_t plane_units(const Shape& s) { return PlaneUnits(s).total(); }

@@ -13,14 +13,14 @@ def group(prec, k):
 
 
 @pytest.mark.parametrize("prec", [1, 2])
-@pytest.mark.parametrize("shape", [(6, 1024, 4, 64), (20, 1024, 10, 64), (200, 1024, 1, 64), (40, 100, 2, 37), (9, 130, 0, 20),
+@pytest.mark.parametrize("shape", [(6, 1024, 4, 64), (20, 1024, 10, 64), (200, 1024, 1, 64), (40, 100, 2, 37), (9, 33, 4, 20),
                                    (5, 160, 3, 0)])
 def test_ring(shape, prec):
     nt, b, w, a = shape
     R, ra = -(-b // 64), -(-a // 64)
     tile, arrow, arrow_rows = R * group(prec, b), R * group(prec, a) if a else 0, ra * group(prec, b)
-    column = 2 * w * tile + arrow + arrow_rows if w else arrow  # diagonal, w by columns, w - 1 by rows
-    want = (w + 1 if w else 2) * column + 2 * (w * tile + arrow) + (ra * group(prec, a) if a else 0)
+    column = 2 * w * tile + arrow + arrow_rows  # diagonal, w by columns, w - 1 by rows
+    want = (w + 1) * column + 2 * (w * tile + arrow) + (ra * group(prec, a) if a else 0)
     assert plan_host().plane_bytes(*shape, prec) == want
     for kind in (S.PLAN_SELINV, S.PLAN_FUSED):
         small = (min(nt, w + 4), min(b, 192), w, a) if w < 5 else (8, 80, 6, 9)
@@ -40,3 +40,13 @@ def test_a_matrix_that_fills_the_device_has_none():
     packed = device // 4 // 8  # four buffers of it are the device
     assert not fit(packed, 1 << 30, device)
     assert not fit(int(0.93 * packed), 5 << 30, device) and fit(int(0.93 * packed), 1 << 30, device)
+
+
+@pytest.mark.parametrize("prec", [1, 2])
+def test_which_shapes_take_planes(prec):
+    """From a tile order of 32 and an inner length (w b + arrow) of 112 on, with a band:
+    a plan that takes them splits tiles (more tasks than the FP64 plan's products)."""
+    from tests.host_build import plan_host
+    takes = lambda *shape: plan_host().plane_faults(*shape, prec, 0) == 0
+    assert takes(6, 32, 3, 16) and takes(6, 64, 1, 48) and takes(6, 48, 2, 16) and takes(6, 112, 1, 0)
+    assert not takes(6, 31, 3, 64) and not takes(6, 32, 3, 15) and not takes(6, 64, 1, 47) and not takes(6, 128, 0, 512)
