@@ -51,11 +51,11 @@ VARIANT_PRODUCTS = {"emu64": {"pipe": "bf16 tensor (tcgen05)", "digits": 8, "pro
                     "fp32x": {"pipe": "bf16 tensor (tcgen05)", "digits": 3, "products": 8}}
 
 # DRAM traffic of the persistent kernel per launch, from ncu captures of the
-# nt = 8 and nt = 16 cases of the same matrix family (0.592 GB and 1.344 GB):
+# nt = 8 and nt = 16 cases of the same matrix family (0.601 GB and 1.346 GB):
 # the nt = 8 figure plus 192 more tile columns at the marginal 8 -> 16 rate.
 # Valid only for the kernel source it was measured on (sha256 prefix of
 # stiles_kernel.cu, block_potrf.cuh, plan.h, plan.cpp); otherwise reported as null.
-TRAFFIC = {"sources_sha": "d5159135d748fbad", "bytes_per_launch": 18.65e9}
+TRAFFIC = {"sources_sha": "017da76acb6e6325", "bytes_per_launch": 18.47e9}
 
 
 def measured_peaks() -> dict:

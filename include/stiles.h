@@ -150,10 +150,11 @@ int stiles_layout_doubles(stiles_t h, size_t *doubles);
 /* Bytes the caller must provide: L and Sigma buffers (equal to the packed
  * size * 8) and a scratch buffer (device, 256-byte aligned) that holds
  * L_ii^{-1}, the scaled off-diagonal tiles L_ki L_ii^{-1}, for the reduced
- * precisions a ring of band + 1 tile columns' operands split for the tensor cores
- * (STILES_EMU64: 16 bytes per entry of 2 band + 2 tiles each, STILES_FP32X: 6;
- * none where they and four buffers of the packed size together leave less than a
- * sixteenth of the device's memory), and the device scheduler's state (dependency
+ * precisions, where their products are long enough to pay for it, a ring of band + 1
+ * tile columns' operands split for the tensor cores (STILES_EMU64: 16 bytes per entry
+ * of 2 band + 2 tiles each, STILES_FP32X: 6; none where they and four buffers of the
+ * packed size together leave less than a sixteenth of the device's memory), and the
+ * device scheduler's state (dependency
  * counters and ready queues). Any pointer may be NULL to skip it. */
 int stiles_workspace_bytes(stiles_t h, size_t *L_bytes, size_t *sigma_bytes, size_t *scratch_bytes);
 
