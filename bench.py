@@ -55,7 +55,7 @@ VARIANT_PRODUCTS = {"emu64": {"pipe": "bf16 tensor (tcgen05)", "digits": 8, "pro
 # the nt = 8 figure plus 192 more tile columns at the marginal 8 -> 16 rate.
 # Valid only for the kernel source it was measured on (sha256 prefix of
 # stiles_kernel.cu, block_potrf.cuh, plan.h, plan.cpp); otherwise reported as null.
-TRAFFIC = {"sources_sha": "017da76acb6e6325", "bytes_per_launch": 18.47e9}
+TRAFFIC = {"sources_sha": "ac6b83dd0cc7eacf", "bytes_per_launch": 18.47e9}
 
 
 def measured_peaks() -> dict:

@@ -43,7 +43,7 @@ namespace {
 constexpr double kFlopPerNs = 7.6 / kCtasPerSm;
 constexpr double kTaskOverheadNs = 2500.0;
 constexpr int kGpuSms = 152;  // of a GB300
-constexpr int kPlanesMinB = 32, kPlanesMinK = 112;
+constexpr int kPlanesMinB64 = 32, kPlanesMinB32 = 24, kPlanesMinK = 112;  // (use_planes)
 constexpr double kSweepStepNs = 120.0;  // one step of an in-shared-memory triangular sweep
 
 // Units (16 bytes) of a tile column's planes of Sigma and of U, and of the corner's:
@@ -1098,15 +1098,20 @@ static double task_estimate(const Shape& s) {
 // but reach that length in several segments, which a part that splits its operands
 // takes one after the other; us of the selected inversion in emulated FP64 / the
 // FP32-class mode: 63 (4/64) 8396 -> 6297 / 5681 -> 2949, 48 (4/20, 40 columns) 4351 ->
-// 3856 / 2658 -> 1789, 33 (3/20) 5392 -> 4998 / 3444 -> 2512; 24 (4/64) 5376 -> 5407 /
-// 2753 -> 2597, so from an order of 32 on. Without a band there is no chain and no tile
-// that many products read: (100, 128, 0, 128) 615 -> 2928 / 540 -> 2457, (40, 64, 0, 512)
+// 3856 / 2658 -> 1789, 33 (3/20) 5392 -> 4998 / 3444 -> 2512, 31 (4/20) 5688 -> 5426 / 2964
+// -> 2488, 24 (4/64) 5387 -> 5642 / 2772 -> 2552; 16 (8/20, 100 columns) 12340 -> 11783 / 4163
+// -> 4391: from an order of 32 and 24 on. Without a band there is no chain and no tile that many
+// products read: (100, 128, 0, 128) 615 -> 2928 / 540 -> 2457, (40, 64, 0, 512)
 // 698 -> 2070, (10, 512, 0, 128) 1489 -> 1613. (A rule on the shape alone: a matrix
 // gets the same arithmetic alone, in a batch and in a server, unless the memory
 // that the call has leaves no room for the planes: planes_fit, the allocation-free
 // call's array, a server's quarter of its arena.)
 bool use_planes(const Shape& s) {
-  return s.prec != PREC_FP64 && s.w >= 1 && s.b >= kPlanesMinB && (int64_t)s.w * s.b + s.a >= kPlanesMinK;
+  if (s.w < 1 || (int64_t)s.w * s.b + s.a < kPlanesMinK) return false;
+  // (emulated FP64: planes have an exponent for 512 of a tile's K, parts that split their
+  // own operands for 64: tiles below 64 take planes where that is no coarser)
+  if (s.prec == PREC_EMU64) return s.b >= kPlanesMinB64 && (s.b >= 64 || s.a <= 64);
+  return s.prec == PREC_FP32X && s.b >= kPlanesMinB32;
 }
 
 int64_t plane_units(const Shape& s) { return PlaneUnits(s).total(); }

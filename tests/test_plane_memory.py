@@ -44,9 +44,10 @@ def test_a_matrix_that_fills_the_device_has_none():
 
 @pytest.mark.parametrize("prec", [1, 2])
 def test_which_shapes_take_planes(prec):
-    """From a tile order of 32 and an inner length (w b + arrow) of 112 on, with a band:
-    a plan that takes them splits tiles (more tasks than the FP64 plan's products)."""
-    from tests.host_build import plan_host
+    """With a band, from an inner length (w b + a) of 112 and a tile order of 24
+    (FP32-class) or 32 (emulated FP64) on; in emulated FP64 with tiles below 64 for arrows
+    of up to 64 only (no tile's K beyond one exponent of either kind of part)."""
     takes = lambda *shape: plan_host().plane_faults(*shape, prec, 0) == 0
-    assert takes(6, 32, 3, 16) and takes(6, 64, 1, 48) and takes(6, 48, 2, 16) and takes(6, 112, 1, 0)
-    assert not takes(6, 31, 3, 64) and not takes(6, 32, 3, 15) and not takes(6, 64, 1, 47) and not takes(6, 128, 0, 512)
+    assert all(takes(*s) for s in [(6, 32, 3, 16), (6, 64, 1, 48), (6, 48, 2, 16), (6, 112, 1, 0), (6, 63, 1, 64), (6, 64, 1, 65)])
+    assert not any(takes(*s) for s in [(6, 23, 3, 64), (6, 32, 3, 15), (6, 64, 1, 47), (6, 128, 0, 512)])
+    assert all(takes(*s) == (prec == 2) for s in [(6, 24, 3, 40), (6, 31, 3, 40), (6, 63, 1, 65)])
